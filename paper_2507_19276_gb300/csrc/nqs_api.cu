@@ -991,67 +991,92 @@ extern "C" int nqs_set_ansatz(nqs_ctx* c, const double* site_tensors, int n_edge
     }
     c->has_ans = false;
     const size_t nt = (size_t)n_edges * 4 * D * D;
-    std::vector<double> hA(nt), hAT(nt);
-    if (is_device_ptr(site_tensors)) CK(cudaMemcpy(hA.data(), site_tensors, nt * 8, cudaMemcpyDeviceToHost));
-    else memcpy(hA.data(), site_tensors, nt * 8);
-    for (size_t m = 0; m < (size_t)n_edges * 4; ++m)
-        for (int r = 0; r < D; ++r)
-            for (int q = 0; q < D; ++q) hAT[m * D * D + (size_t)q * D + r] = hA[m * D * D + (size_t)r * D + q];
+    // the parameters are read on the context's stream, after the work already on
+    // the legacy default stream (which a synchronous copy would wait for)
+    if (c->stream) {
+        cudaEvent_t ev = get_event(c);
+        CK(cudaEventRecord(ev, cudaStreamLegacy));
+        CK(cudaStreamWaitEvent(c->stream, ev, 0));
+        c->free_events.push_back(ev);
+    }
     TRY(ensure(c, c->A, nt * 8));
     TRY(ensure(c, c->AT, nt * 8));
-    CK(cudaMemcpy(c->A.p, hA.data(), nt * 8, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->AT.p, hAT.data(), nt * 8, cudaMemcpyHostToDevice));
+    TRY(ensure(c, c->Af, nt * 4));
+    TRY(ensure(c, c->ATf, nt * 4));
+    CK(cudaMemcpyAsync(c->A.p, site_tensors, nt * 8, cudaMemcpyDefault, c->stream));
     if (!chain) {
         TRY(ensure(c, c->pred_ptr, (K + 1) * 4));
         TRY(ensure(c, c->pred_idx, (size_t)n_edges * 4));
-        CK(cudaMemcpy(c->pred_ptr.p, ptr.data(), (K + 1) * 4, cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(c->pred_idx.p, idx.data(), (size_t)n_edges * 4, cudaMemcpyHostToDevice));
+        CK(cudaMemcpyAsync(c->pred_ptr.p, ptr.data(), (K + 1) * 4, cudaMemcpyHostToDevice, c->stream));
+        CK(cudaMemcpyAsync(c->pred_idx.p, idx.data(), (size_t)n_edges * 4, cudaMemcpyHostToDevice, c->stream));
     }
+    AnsatzForms fm{};
+    fm.D = D;
+    fm.n_mats = n_edges * 4;
+    fm.A = (const double*)c->A.p;
+    fm.AT = (double*)c->AT.p;
+    fm.Af = (float*)c->Af.p;
+    fm.ATf = (float*)c->ATf.p;
+    c->has_tc = false;
+    c->has_gtc = false;
+    c->gtc_why[0] = 0;
+    GraphTcPlan gp;
+    if (chain) {
+        // (hi, lo) pairs of both copies for the double-FP32 arithmetic
+        TRY(ensure(c, c->ATdf, nt * 8));
+        TRY(ensure(c, c->Adf, nt * 8));
+        fm.Adf = (float2*)c->Adf.p;
+        fm.ATdf = (float2*)c->ATdf.p;
+        // tensor-core batches: D % 16 == 0 up to 128 in one reduction chunk, or
+        // 192 / 256 in chunks of 64 (N = D <= 256 accumulator columns)
+        if (D % 16 == 0 && (D <= 128 || (D % 64 == 0 && D <= 256))) {
+            TRY(ensure(c, c->tc_img, fam_tc_image_bytes(K, D)));
+            TRY(ensure(c, c->tc_exps, (size_t)2 * fm.n_mats * 4));
+            fm.exps = (int*)c->tc_exps.p;
+            fm.exps2 = fm.exps + fm.n_mats;
+            fm.chain_img = (unsigned char*)c->tc_img.p;
+            fm.kc = fam_tc_kc(D);
+            c->has_tc = true;
+        }
+    } else {
+        const char* why = nullptr;
+        if (graph_tc_plan(ptr.data(), idx.data(), K, D, n_hidden, gp, &why)) {
+            TRY(ensure(c, c->g_img, (size_t)n_edges * 16 * D * D));
+            TRY(ensure(c, c->g_bexp, (size_t)fm.n_mats * 4));
+            TRY(ensure(c, c->g_col0, (size_t)fm.n_mats * D * 4));
+            TRY(ensure(c, c->g_slot, (size_t)K * 4));
+            TRY(ensure(c, c->g_last, (size_t)K * 4));
+            CK(cudaMemcpyAsync(c->g_slot.p, gp.slot.data(), (size_t)K * 4, cudaMemcpyHostToDevice, c->stream));
+            CK(cudaMemcpyAsync(c->g_last.p, gp.last_use.data(), (size_t)K * 4, cudaMemcpyHostToDevice, c->stream));
+            fm.exps = (int*)c->g_bexp.p;
+            fm.graph_img = (unsigned char*)c->g_img.p;
+            fm.col0 = (float*)c->g_col0.p;
+            c->g_slots = gp.n_slots;
+            c->g_maxdeg = gp.max_deg;
+            c->g_nbuf = gp.nbuf;
+            c->has_gtc = true;
+        } else {
+            snprintf(c->gtc_why, sizeof(c->gtc_why), "%s", why ? why : "unsupported graph");
+        }
+    }
+    LAUNCH(NQS_STAGE_OTHER, launch_ansatz_forms(fm, c->stream));
+    CK(cudaGetLastError());
     if (n_hidden > 0) {
-        const size_t nw = (size_t)n_hidden * 2 * K;
+        const size_t nw = (size_t)n_hidden * 2 * K, np = (size_t)((n_hidden + 3) & ~3);
         TRY(ensure(c, c->W, nw * 8));
         TRY(ensure(c, c->b, (size_t)n_hidden * 8));
-        CK(cudaMemcpy(c->W.p, rbm_W, nw * 8, cudaMemcpyDefault));
-        CK(cudaMemcpy(c->b.p, rbm_b, (size_t)n_hidden * 8, cudaMemcpyDefault));
-    }
-    {
-        std::vector<float> fA(nt), fAT(nt);
-        for (size_t i = 0; i < nt; ++i) { fA[i] = (float)hA[i]; fAT[i] = (float)hAT[i]; }
-        TRY(ensure(c, c->Af, nt * 4));
-        TRY(ensure(c, c->ATf, nt * 4));
-        CK(cudaMemcpy(c->Af.p, fA.data(), nt * 4, cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(c->ATf.p, fAT.data(), nt * 4, cudaMemcpyHostToDevice));
-        if (chain) {
-            // (hi, lo) with hi = fl32(x), lo = fl32(x - hi): 48 of the entry's 53 bits
-            std::vector<float2> dAT(nt), dA(nt);
-            for (size_t i = 0; i < nt; ++i) {
-                const float h = (float)hAT[i], g = (float)hA[i];
-                dAT[i] = make_float2(h, (float)(hAT[i] - (double)h));
-                dA[i] = make_float2(g, (float)(hA[i] - (double)g));
-            }
-            TRY(ensure(c, c->ATdf, nt * 8));
-            TRY(ensure(c, c->Adf, nt * 8));
-            CK(cudaMemcpy(c->ATdf.p, dAT.data(), nt * 8, cudaMemcpyHostToDevice));
-            CK(cudaMemcpy(c->Adf.p, dA.data(), nt * 8, cudaMemcpyHostToDevice));
-        }
-        if (n_hidden > 0) {
-            // transposed FP32 copy for the graph tiles' correlator: lanes over hidden
-            // units read consecutive words of one spin-orbital's column
-            const size_t nw = (size_t)n_hidden * 2 * K, np = (size_t)((n_hidden + 3) & ~3);
-            std::vector<double> hW(nw);
-            CK(cudaMemcpy(hW.data(), c->W.p, nw * 8, cudaMemcpyDeviceToHost));
-            std::vector<float> fWT((size_t)2 * K * np, 0.0f);
-            for (int k = 0; k < n_hidden; ++k)
-                for (int q = 0; q < 2 * K; ++q) fWT[(size_t)q * np + k] = (float)hW[(size_t)k * 2 * K + q];
-            TRY(ensure(c, c->WTf, fWT.size() * 4));
-            CK(cudaMemcpy(c->WTf.p, fWT.data(), fWT.size() * 4, cudaMemcpyHostToDevice));
-            TRY(ensure(c, c->csite, (size_t)K * 12 * np * 16));
-            TRY(ensure(c, c->csite64, (size_t)K * 12 * np * 32));
-            fam_corr_sites((const double*)c->W.p, K, n_hidden, (float4*)c->csite.p, (double4_32a*)c->csite64.p,
-                           c->stream);
-            CK(cudaGetLastError());
-            CK(cudaStreamSynchronize(c->stream));
-        }
+        CK(cudaMemcpyAsync(c->W.p, rbm_W, nw * 8, cudaMemcpyDefault, c->stream));
+        CK(cudaMemcpyAsync(c->b.p, rbm_b, (size_t)n_hidden * 8, cudaMemcpyDefault, c->stream));
+        // transposed FP32 copy for the graph tiles' correlator: lanes over hidden
+        // units read consecutive words of one spin-orbital's column
+        TRY(ensure(c, c->WTf, (size_t)2 * K * np * 4));
+        LAUNCH(NQS_STAGE_OTHER, launch_corr_transpose((const double*)c->W.p, n_hidden, (int)np, 2 * K,
+                                                      (float*)c->WTf.p, c->stream));
+        TRY(ensure(c, c->csite, (size_t)K * 12 * np * 16));
+        TRY(ensure(c, c->csite64, (size_t)K * 12 * np * 32));
+        LAUNCH(NQS_STAGE_OTHER, fam_corr_sites((const double*)c->W.p, K, n_hidden, (float4*)c->csite.p,
+                                               (double4_32a*)c->csite64.p, c->stream));
+        CK(cudaGetLastError());
     }
     AnsatzView a{};
     a.K = K; a.D = D; a.n_edges = n_edges; a.chain = chain ? 1 : 0;
@@ -1067,43 +1092,6 @@ extern "C" int nqs_set_ansatz(nqs_ctx* c, const double* site_tensors, int n_edge
     a.mask_nb = c->nb;
     a.corr = 0;
     c->av = a;
-    c->has_tc = false;
-    // tensor-core batches: D % 16 == 0 up to 128 in one reduction chunk, or
-    // 192 / 256 in chunks of 64 (N = D <= 256 accumulator columns)
-    if (chain && D % 16 == 0 && (D <= 128 || (D % 64 == 0 && D <= 256))) {
-        std::vector<unsigned char> img;
-        std::vector<int> ex;
-        fam_tc_images(hA.data(), K, D, img, ex);
-        TRY(ensure(c, c->tc_img, img.size()));
-        TRY(ensure(c, c->tc_exps, ex.size() * 4));
-        CK(cudaMemcpy(c->tc_img.p, img.data(), img.size(), cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(c->tc_exps.p, ex.data(), ex.size() * 4, cudaMemcpyHostToDevice));
-        c->has_tc = true;
-    }
-    c->has_gtc = false;
-    c->gtc_why[0] = 0;
-    if (!chain) {
-        GraphTcPlan gp;
-        const char* why = nullptr;
-        if (graph_tc_plan(hA.data(), ptr.data(), idx.data(), K, D, n_hidden, gp, &why)) {
-            TRY(ensure(c, c->g_img, gp.img.size()));
-            TRY(ensure(c, c->g_bexp, gp.bexp.size() * 4));
-            TRY(ensure(c, c->g_col0, gp.col0.size() * 4));
-            TRY(ensure(c, c->g_slot, (size_t)K * 4));
-            TRY(ensure(c, c->g_last, (size_t)K * 4));
-            CK(cudaMemcpy(c->g_img.p, gp.img.data(), gp.img.size(), cudaMemcpyHostToDevice));
-            CK(cudaMemcpy(c->g_bexp.p, gp.bexp.data(), gp.bexp.size() * 4, cudaMemcpyHostToDevice));
-            CK(cudaMemcpy(c->g_col0.p, gp.col0.data(), gp.col0.size() * 4, cudaMemcpyHostToDevice));
-            CK(cudaMemcpy(c->g_slot.p, gp.slot.data(), (size_t)K * 4, cudaMemcpyHostToDevice));
-            CK(cudaMemcpy(c->g_last.p, gp.last_use.data(), (size_t)K * 4, cudaMemcpyHostToDevice));
-            c->g_slots = gp.n_slots;
-            c->g_maxdeg = gp.max_deg;
-            c->g_nbuf = gp.nbuf;
-            c->has_gtc = true;
-        } else {
-            snprintf(c->gtc_why, sizeof(c->gtc_why), "%s", why ? why : "unsupported graph");
-        }
-    }
     CK(cudaStreamSynchronize(c->stream));
     c->has_ans = true;
     return NQS_OK;
@@ -1492,7 +1480,7 @@ int le_core(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, uint64
                          deabs ? &c->part_draw_abs : nullptr, graph ? &c->mv_draw : nullptr));
         }
     }
-    TRY(ensure(c, c->summary, 8 * 8));
+    TRY(ensure(c, c->summary, kSummaryDoubles * 8));
     FinalArgs f{};
     f.Ns = Ns;
     f.h_diag = (const double*)c->hdiag.p;
@@ -1641,7 +1629,7 @@ int refine_pass(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, ui
     c->audit_rel = observed;
     c->err_factor = f;
     c->n_audited = (int64_t)audit.size();
-    TRY(ensure(c, c->summary2, 8 * 8));
+    TRY(ensure(c, c->summary2, kSummaryDoubles * 8));
     FinalArgs fa{};
     fa.Ns = Ns;
     fa.counts = dc;
@@ -1743,7 +1731,7 @@ int vjp_core(nqs_ctx* c, const uint64_t* ds, const double* du, int64_t Ns, doubl
         return NQS_OK;
     }
     const int64_t ch = c->grad_chunk > 0 ? c->grad_chunk : Ns;
-    TRY(ensure(c, c->grad_scr, grad_scratch_bytes(c->av, ch < Ns ? ch : Ns)));
+    TRY(ensure(c, c->grad_scr, grad_scratch_bytes(c->av, ch < Ns ? ch : Ns) + 256));
     for (int64_t s0 = 0; s0 < Ns; s0 += ch) {
         const int64_t n = Ns - s0 < ch ? Ns - s0 : ch;
         const uint64_t* cs = ds + 2 * s0;
@@ -1776,6 +1764,8 @@ int vjp_core(nqs_ctx* c, const uint64_t* ds, const double* du, int64_t Ns, doubl
         g.sidx = (int32_t*)scr;
         g.soff = (int64_t*)(scr + (((size_t)K * n * 4 + 255) & ~(size_t)255));
         g.part = (double*)((char*)g.soff + (((size_t)K * 5 * 8 + 255) & ~(size_t)255));
+        g.vcorr = (double*)(scr + ((grad_corr_offset(c->av, n) + 255) & ~(size_t)255));
+        g.cpart = g.vcorr + (size_t)n * NH;
         LAUNCH(NQS_STAGE_OTHER, launch_grad_fp64(g, c->stream));
         CK(cudaGetLastError());
     }

@@ -1690,40 +1690,6 @@ int fam_launch_rows(const FamArgs<T>& f, const RowSet& rows, int64_t grid, doubl
     return 1;
 }
 
-void fam_tc_images(const double* A, int K, int D, std::vector<unsigned char>& images, std::vector<int>& exps)
-{
-    const size_t blk = (size_t)4 * D * D;
-    images.assign((size_t)2 * K * 4 * blk, 0);
-    exps.assign((size_t)2 * K * 4, 0);
-    for (int side = 0; side < 2; ++side)
-        for (int t = 0; t < K; ++t)
-            for (int sg = 0; sg < 4; ++sg) {
-                const double* M = A + ((size_t)t * 4 + sg) * D * D;
-                double mx = 0.0;
-                for (size_t i = 0; i < (size_t)D * D; ++i) mx = std::max(mx, std::fabs(M[i]));
-                int e = 0;
-                if (mx > 0.0) std::frexp(mx, &e);
-                const size_t id = ((size_t)side * K + t) * 4 + sg;
-                exps[id] = e;
-                const int kc = fam_tc_kc(D);
-                const size_t chunk = (size_t)4 * D * kc;     // hi + lo of one reduction chunk
-                for (int n = 0; n < D; ++n)
-                    for (int k = 0; k < D; ++k) {
-                        // B[n][k]: side 0 -> M[n][k] (y = M x), side 1 -> M[k][n] (y = x^T M)
-                        const double m = std::ldexp(side == 0 ? M[(size_t)n * D + k] : M[(size_t)k * D + n], -e);
-                        const float mf = (float)m;
-                        const __half h = __float2half_rn(mf);
-                        const __half l = __float2half_rn(mf - __half2float(h));
-                        const int ck = k / kc, kk = k - ck * kc;
-                        unsigned char* hi = images.data() + id * blk + (size_t)ck * chunk;
-                        unsigned char* lo = hi + (size_t)2 * D * kc;
-                        const size_t off = ((size_t)(n >> 3) * (kc >> 3) + (kk >> 3)) * 128 + (n & 7) * 16 + (kk & 7) * 2;
-                        std::memcpy(hi + off, &h, 2);
-                        std::memcpy(lo + off, &l, 2);
-                    }
-            }
-}
-
 #define NQS_FAM_INST(T)                                                                    \
     template int fam_launch_mark<T>(const FamArgs<T>&, const RowSet&, int, uint32_t*, cudaStream_t);  \
     template int fam_launch_compact<T>(const FamArgs<T>&, int, cudaStream_t);              \

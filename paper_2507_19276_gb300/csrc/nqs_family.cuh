@@ -2,8 +2,6 @@
 // (see nqs_family.cu for the decomposition).
 #pragma once
 
-#include <vector>
-
 #include "nqs_kernels.cuh"
 
 namespace nqs {
@@ -18,7 +16,7 @@ struct FamArgs {
     size_t batch_bytes;       // shared memory of one batch (see fam_batch_bytes)
     int tc;                   // 1: tensor-core batches (FP32; D % 16 == 0 up to 128, or 192 / 256)
     int tc_cols;              // tensor-memory columns allocated per block
-    const uint4* tc_mats;     // [2][K][4] split-FP16 operand images, see fam_tc_images
+    const uint4* tc_mats;     // [2][K][4] split-FP16 operand images, see fam_tc_image_bytes
     const int* tc_exp;        // [2][K][4] power-of-two scale of each image
     DevError* err;
     const T* A;               // [K][4][D][D] site tensors in T, A[a][b]
@@ -122,9 +120,9 @@ __host__ __device__ inline size_t fam_batch_bytes(int D, int nmax, size_t elem, 
 // batches: for side 0 the matrix A_t^s, for side 1 its transpose, each scaled
 // by 2^-e (max |entry| in [0.5, 1)). Each image is D / kc reduction chunks
 // (kc = fam_tc_kc(D)), each chunk its hi then its lo half, D rows x kc columns
-// in the K-major core-matrix layout. images holds 2*K*4 blocks of 4*D*D bytes;
-// exps the e.
-void fam_tc_images(const double* A, int K, int D, std::vector<unsigned char>& images, std::vector<int>& exps);
+// in the K-major core-matrix layout: 2 sides x 4 K blocks of 4*D*D bytes
+// (written by launch_ansatz_forms).
+inline size_t fam_tc_image_bytes(int K, int D) { return (size_t)2 * K * 4 * 4 * D * D; }
 
 // bytes of the per-sample tables (G, H, their exponents, cluster maps)
 // elements of one correlator-factor row: N_h rounded up to 4, one more for the

@@ -29,9 +29,27 @@ constexpr int kStage = 16;        // samples staged per round
 
 int64_t grad_chunks(int64_t Ns) { return (Ns + kGradChunk - 1) / kGradChunk; }
 
+// samples per block of the correlator gradient: at most 128 chunks, at least
+// 32 samples each (about two blocks per SM for N_h = 100, 4096 samples)
+int64_t corr_chunk(int64_t Ns)
+{
+    const int64_t c = (Ns + 127) / 128;
+    return c < 32 ? 32 : c;
+}
+
+// bound on corr_chunks over every count up to Ns (a shorter last pass may have more chunks)
+int64_t max_corr_chunks(int64_t Ns) { return (Ns + 31) / 32 < 128 ? (Ns + 31) / 32 : 128; }
+
+int64_t corr_chunks(int64_t Ns) { return (Ns + corr_chunk(Ns) - 1) / corr_chunk(Ns); }
+
 }  // namespace
 
 size_t grad_scratch_bytes(const AnsatzView& an, int64_t Ns)
+{
+    return grad_corr_offset(an, Ns) + ((size_t)Ns + (size_t)max_corr_chunks(Ns) * (2 * an.K + 1)) * an.n_hidden * 8;
+}
+
+size_t grad_corr_offset(const AnsatzView& an, int64_t Ns)
 {
     return (size_t)an.K * Ns * 4 + (size_t)an.K * 5 * 8 + 512 +     // two 256-byte alignments
            (size_t)grad_chunks(Ns) * an.n_edges * 4 * an.D * an.D * 8;
@@ -169,25 +187,63 @@ __global__ void k_grad_reduce(GradArgs a)
     a.grad_sites[q] = acc;
 }
 
-__global__ void k_grad_rbm(GradArgs a)
+// v[s][k] = u_s d log|f(s)| / d theta_k
+__global__ void k_grad_corr_v(GradArgs a)
 {
-    const int k = blockIdx.x, K = a.an.K, NH = a.an.n_hidden;
-    const int col = threadIdx.x;             // 0..2K-1: W[k][col]; 2K: b[k]
-    if (col > 2 * K) return;
-    double acc = 0.0;
-    for (int64_t s = 0; s < a.Ns; ++s) {
-        const double t = corr_dlog(a.an.corr, a.theta[(size_t)s * NH + k]);
-        if (col == 2 * K) acc += a.u[s] * t;
-        else {
-            const uint64_t w = a.samples[2 * s + (col & 1)];
-            if ((w >> (col >> 1)) & 1ull) acc += a.u[s] * t;
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= a.Ns * a.an.n_hidden) return;
+    a.vcorr[q] = a.u[q / a.an.n_hidden] * corr_dlog(a.an.corr, a.theta[q]);
+}
+
+// One chunk of samples and 32 hidden units per block (one per lane): warp w
+// sums the columns w, w + 8, ... (spin orbitals 0..2K-1, then b at 2K). The
+// samples' words are uniform over a warp, so an unoccupied column costs no FP64
+// add. With one thread per parameter over all samples, each re-evaluating
+// tanh, the same sums took 4.2 ms for H50 (4096 samples, N_h = 100); the FP64
+// adds alone need 0.04 ms.
+constexpr int kCorrCols = 2 * kMaxOrb / 8 + 1;
+
+__global__ void __launch_bounds__(256) k_grad_rbm(GradArgs a, int64_t chunk)
+{
+    const int K2 = 2 * a.an.K, NH = a.an.n_hidden;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int k = blockIdx.y * 32 + lane;
+    const int64_t s0 = (int64_t)blockIdx.x * chunk;
+    const int64_t s1 = s0 + chunk < a.Ns ? s0 + chunk : a.Ns;
+    double acc[kCorrCols];
+    #pragma unroll
+    for (int j = 0; j < kCorrCols; ++j) acc[j] = 0.0;
+    for (int64_t s = s0; s < s1; ++s) {
+        const uint64_t w0 = __ldg(a.samples + 2 * s), w1 = __ldg(a.samples + 2 * s + 1);
+        const double v = k < NH ? a.vcorr[s * NH + k] : 0.0;
+        #pragma unroll
+        for (int j = 0; j < kCorrCols; ++j) {
+            const int col = warp + 8 * j;
+            if (col > K2) continue;
+            if (col == K2 || (((col & 1) ? w1 : w0) >> (col >> 1)) & 1ull) acc[j] += v;
         }
     }
-    if (col == 2 * K) { if (a.grad_b) a.grad_b[k] = (a.accumulate ? a.grad_b[k] : 0.0) + acc; }
-    else if (a.grad_W) {
-        double* g = a.grad_W + (size_t)k * 2 * K + col;
-        *g = (a.accumulate ? *g : 0.0) + acc;
+    if (k >= NH) return;
+    double* out = a.cpart + ((size_t)blockIdx.x * (K2 + 1)) * NH + k;
+    #pragma unroll
+    for (int j = 0; j < kCorrCols; ++j) {
+        const int col = warp + 8 * j;
+        if (col <= K2) out[(size_t)col * NH] = acc[j];
     }
+}
+
+__global__ void k_grad_rbm_reduce(GradArgs a, int64_t chunks)
+{
+    const int K2 = 2 * a.an.K, NH = a.an.n_hidden;
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= (K2 + 1) * NH) return;
+    const int col = q / NH, k = q - col * NH;
+    double* g = col == K2 ? (a.grad_b ? a.grad_b + k : nullptr)
+                          : (a.grad_W ? a.grad_W + (size_t)k * K2 + col : nullptr);
+    if (!g) return;
+    double acc = a.accumulate ? *g : 0.0;
+    for (int64_t c = 0; c < chunks; ++c) acc += a.cpart[(size_t)c * (K2 + 1) * NH + q];
+    *g = acc;
 }
 
 __global__ void k_grad_w2(GradArgs a)
@@ -199,7 +255,7 @@ __global__ void k_grad_w2(GradArgs a)
         for (int64_t s = 0; s < a.Ns; ++s) {
             const uint64_t w1 = a.samples[2 * s + (s1 & 1)], w2 = a.samples[2 * s + (s2 & 1)];
             if (((w1 >> (s1 >> 1)) & 1ull) && ((w2 >> (s2 >> 1)) & 1ull))
-                acc += a.u[s] * (0.5 * corr_dlog(a.an.corr, a.theta[(size_t)s * NH + k]));
+                acc += 0.5 * a.vcorr[s * NH + k];
         }
         double* g = a.grad_W2 + ((size_t)k * N + s1) * N + s2;
         *g = (a.accumulate ? *g : 0.0) + acc;
@@ -244,11 +300,19 @@ int launch_grad_fp64(const GradArgs& a, cudaStream_t st)
         k_grad_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(a);
         n += 3;
     }
-    if (a.an.n_hidden > 0 && (a.grad_W || a.grad_b)) {
-        k_grad_rbm<<<a.an.n_hidden, ((2 * a.an.K + 1 + 31) / 32) * 32, 0, st>>>(a);
+    const int NH = a.an.n_hidden;
+    const bool w2 = a.grad_W2 && a.an.corr == 2;
+    if (NH > 0 && a.Ns > 0 && (a.grad_W || a.grad_b || w2)) {
+        k_grad_corr_v<<<(unsigned)((a.Ns * NH + 255) / 256), 256, 0, st>>>(a);
         ++n;
     }
-    if (a.an.n_hidden > 0 && a.grad_W2 && a.an.corr == 2) {
+    if (NH > 0 && a.Ns > 0 && (a.grad_W || a.grad_b)) {
+        const int64_t nc = corr_chunks(a.Ns);
+        k_grad_rbm<<<dim3((unsigned)nc, (unsigned)((NH + 31) / 32)), 256, 0, st>>>(a, corr_chunk(a.Ns));
+        k_grad_rbm_reduce<<<(unsigned)(((2 * a.an.K + 1) * NH + 255) / 256), 256, 0, st>>>(a, nc);
+        n += 2;
+    }
+    if (NH > 0 && a.Ns > 0 && w2) {
         k_grad_w2<<<a.an.n_hidden, 256, 0, st>>>(a);
         ++n;
     }

@@ -544,7 +544,7 @@ size_t graph_tiles_smem(int D, int K, int n_slots, int max_deg, int n_hidden, in
            (((size_t)2 * K * n_hidden + 3) & ~(size_t)3) * 4 + np * 4;
 }
 
-bool graph_tc_plan(const double* A, const int* ptr, const int* idx, int K, int D, int n_hidden,
+bool graph_tc_plan(const int* ptr, const int* idx, int K, int D, int n_hidden,
                    GraphTcPlan& p, const char** why)
 {
     *why = nullptr;
@@ -589,37 +589,6 @@ bool graph_tc_plan(const double* A, const int* ptr, const int* idx, int K, int D
         *why = "the tile's states and matrix images exceed the shared memory";
         return false;
     }
-    // split images of every M_e^sigma scaled by 2^-x (max |M| 2^-x in [0.5, 1)):
-    // per edge B[sigma D + n][k] = M_e^sigma[n][k] in the K-major core-matrix
-    // layout (4D rows), hi then lo; column 0 in FP32 for the e_0 sources
-    const int E = ptr[K];
-    const size_t img = (size_t)16 * D * D;
-    p.img.assign((size_t)E * img, 0);
-    p.bexp.assign((size_t)E * 4, 0);
-    p.col0.assign((size_t)E * 4 * D, 0.f);
-    for (int e = 0; e < E; ++e)
-        for (int sg = 0; sg < 4; ++sg) {
-            const double* M = A + ((size_t)e * 4 + sg) * D * D;
-            double m = 0.0;
-            for (size_t q = 0; q < (size_t)D * D; ++q) m = std::max(m, std::fabs(M[q]));
-            int x = 0;
-            if (m > 0.0) std::frexp(m, &x);
-            const size_t id = (size_t)e * 4 + sg;
-            p.bexp[id] = x;
-            unsigned char* hi = p.img.data() + (size_t)e * img + (size_t)sg * 2 * D * D;
-            unsigned char* lo = hi + (size_t)8 * D * D;
-            for (int n = 0; n < D; ++n) {
-                p.col0[id * D + n] = (float)M[(size_t)n * D];
-                for (int k = 0; k < D; ++k) {
-                    const float v = (float)std::ldexp(M[(size_t)n * D + k], -x);
-                    const __half h = __float2half_rn(v);
-                    const __half l = __float2half_rn(v - __half2float(h));
-                    const size_t off = ((size_t)(n >> 3) * (D >> 3) + (k >> 3)) * 128 + (n & 7) * 16 + (k & 7) * 2;
-                    std::memcpy(hi + off, &h, 2);
-                    std::memcpy(lo + off, &l, 2);
-                }
-            }
-        }
     return true;
 }
 

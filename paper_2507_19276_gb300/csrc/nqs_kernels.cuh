@@ -100,6 +100,30 @@ int launch_scan_i64_wide(const int64_t* in, int64_t* out, int64_t n, int64_t* tm
 // chunk bases for row sets: out[s] = sum_{s'<s} ceil(cnt[s'] / rows), out[Ns] total
 int launch_chunk_base(const int64_t* cnt, int rows, int64_t* out, int64_t Ns, cudaStream_t st);
 
+// ---- parameter forms (nqs_ansatz.cu) ----------------------------------------
+
+// Working forms of n_mats D x D site matrices A (device, FP64, row-major).
+struct AnsatzForms {
+    int D, n_mats;                       // n_mats = 4 n_edges (below 65536)
+    const double* A;
+    double* AT;                          // [n_mats][D][D] transposed
+    float* Af; float* ATf;               // FP32 copies of both
+    float2* Adf; float2* ATdf;           // chain: (hi, lo) float pairs of both (NULL: none)
+    int* exps; int* exps2;               // [n_mats] powers of two of the images (exps2: a second
+                                         // copy, may be NULL); exps NULL: no images
+    unsigned char* chain_img;            // split images of both sides, see fam_tc_image_bytes
+    int kc;                              // reduction chunk of the chain images
+    unsigned char* graph_img;            // [E] split images of the four local states, hi then lo:
+                                         // B[sigma D + n][k] = M_e^sigma[n][k], K-major core matrices
+    float* col0;                         // [n_mats][D] column 0 of each matrix (e_0 sources)
+};
+int launch_ansatz_forms(const AnsatzForms& f, cudaStream_t st);
+// W [n_hidden][K2] -> FP32 [K2][np], zero-padded
+int launch_corr_transpose(const double* W, int n_hidden, int np, int K2, float* WTf, cudaStream_t st);
+
+constexpr int kSummaryBlocks = 128;
+constexpr int kSummaryDoubles = 8 + 9 * kSummaryBlocks;
+
 struct FinalArgs {
     int64_t Ns;
     const double* h_diag;                // [Ns]
@@ -116,7 +140,8 @@ struct FinalArgs {
     double* e_stoch;                     // [Ns] (optional)
     const int64_t* span_det;             // [chunks] from the amplitude kernels
     const int64_t* span_draw;
-    double* summary;                     // [8] e_mean, sum_c, log_B, e_tilde_mean, n_det, n_uniq, span
+    double* summary;                     // [8] e_mean, sum_c, log_B, e_tilde_mean, n_det, n_uniq, span,
+                                         // products; then the blocks' partial sums (kSummaryDoubles)
     const double* part_det_abs;          // chunk sums of |term| (NULL: no e_abs)
     const double* part_draw_abs;
     double* e_abs;                       // [Ns] |H_nn| + sum |terms| (optional)
@@ -320,16 +345,13 @@ constexpr int kGtMaxSlots = 16;          // vertex states a tile keeps at once
 constexpr int kGtMaxDeg = 8;             // in-degree bound of the graph ansatz
 
 struct GraphTcPlan {
-    std::vector<unsigned char> img;      // [E][4] split images of M_e^sigma (hi, lo)
-    std::vector<int> bexp;               // [E][4] power of two taken out of each image
-    std::vector<float> col0;             // [E][4][D] column 0 of each matrix (e_0 sources)
     std::vector<int> slot;               // [K] state slot of each vertex (-1: never read)
     std::vector<int> last_use;           // [K] last vertex reading each state (-1: none)
     int n_slots = 0, max_deg = 0;
     int nbuf = 1;                        // matrix-image buffers that fit next to the slots
 };
 // false (with the reason) when the graph does not fit the tile kernel
-bool graph_tc_plan(const double* A, const int* ptr, const int* idx, int K, int D, int n_hidden,
+bool graph_tc_plan(const int* ptr, const int* idx, int K, int D, int n_hidden,
                    GraphTcPlan& p, const char** why);
 size_t graph_tiles_smem(int D, int K, int n_slots, int max_deg, int n_hidden, int nbuf);
 
@@ -344,9 +366,9 @@ struct GraphTcArgs {
     float* tts;                          // [Ns][np] tanh (cos form: tan) of theta_k(n) (written here)
     const double* theta;                 // [Ns][n_hidden]
     const double* psi_mant; const int* psi_exp;
-    const unsigned char* bimg;           // GraphTcPlan::img on the device
-    const int* bexp;
-    const float* col0;
+    const unsigned char* bimg;           // AnsatzForms::graph_img
+    const int* bexp;                     // [E][4] power of two taken out of each image
+    const float* col0;                   // [E][4][D] column 0 of each matrix (e_0 sources)
     const int* slot;
     const int* last_use;
     int n_slots, max_deg, nbuf;
@@ -390,9 +412,14 @@ struct GradArgs {
     int32_t* sidx;                        // [K][Ns]
     int64_t* soff;                        // [K][5]
     double* part;                         // [n_chunks][E][4][D][D]
+    // scratch of the correlator part: u_n d log|f(n)| / d theta_k, and per chunk
+    // of samples the partial sums of every (column, hidden unit)
+    double* vcorr;                        // [Ns][n_hidden]
+    double* cpart;                        // [chunks][2K + 1][n_hidden]
 };
-// scratch bytes of the tensor-part gradient for Ns samples
+// scratch bytes of the gradient for Ns samples, and the offset of vcorr in them
 size_t grad_scratch_bytes(const AnsatzView& an, int64_t Ns);
+size_t grad_corr_offset(const AnsatzView& an, int64_t Ns);
 int launch_grad_fp64(const GradArgs& a, cudaStream_t st);
 
 // d log|f| / d theta_k of the correlator: tanh (2cosh), -tan (cos, Ising)

@@ -200,25 +200,38 @@ int launch_chunk_base(const int64_t* cnt, int rows, int64_t* out, int64_t Ns, cu
 
 // ---------------------------------------------------------------------------
 // E_loc per sample = H_nn + sum of det-row partials + sum of draw-row partials
-// (fixed order), then the weighted summary in one block (fixed tree order).
+// (one warp per sample, lanes strided over the chunks, then the shuffle tree),
+// then the weighted summary: per-block partial sums over strided samples and
+// chunks, combined by one warp in block order (fixed order throughout). One
+// block for all of it took 1.1 ms on 16 384 samples with 1.2 M chunks; spread
+// over the chip it is launch-bound (~10 us).
 // ---------------------------------------------------------------------------
 
-__global__ void k_final_samples(FinalArgs a)
+__device__ double chunk_sum_warp(const double* v, int64_t b0, int64_t b1, int lane)
 {
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    double x = 0.0;
+    for (int64_t b = b0 + lane; b < b1; b += 32) x += v[b];
+    return warp_sum_f64(x);                                   // lane 0
+}
+
+__global__ void __launch_bounds__(256) k_final_samples(FinalArgs a)
+{
+    const int64_t s = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
     if (s >= a.Ns) return;
-    double ed = 0.0, es = 0.0;
-    for (int64_t b = a.base_det[s]; b < a.base_det[s + 1]; ++b) ed += a.part_det[b];
-    if (a.base_draw)
-        for (int64_t b = a.base_draw[s]; b < a.base_draw[s + 1]; ++b) es += a.part_draw[b];
-    a.e_loc[s] = a.h_diag[s] + ed + es;
+    const int64_t d0 = a.base_det[s], d1 = a.base_det[s + 1];
+    int64_t w0 = 0, w1 = 0;
+    if (a.base_draw) { w0 = a.base_draw[s]; w1 = a.base_draw[s + 1]; }
+    const double ed = chunk_sum_warp(a.part_det, d0, d1, lane);
+    const double es = w1 > w0 ? chunk_sum_warp(a.part_draw, w0, w1, lane) : 0.0;
+    double ea = 0.0;
     if (a.e_abs) {
-        double ea = fabs(a.h_diag[s]);
-        for (int64_t b = a.base_det[s]; b < a.base_det[s + 1]; ++b) ea += a.part_det_abs[b];
-        if (a.base_draw && a.part_draw_abs)
-            for (int64_t b = a.base_draw[s]; b < a.base_draw[s + 1]; ++b) ea += a.part_draw_abs[b];
-        a.e_abs[s] = ea;
+        ea = chunk_sum_warp(a.part_det_abs, d0, d1, lane);
+        if (a.part_draw_abs && w1 > w0) ea += chunk_sum_warp(a.part_draw_abs, w0, w1, lane);
     }
+    if (lane) return;
+    a.e_loc[s] = a.h_diag[s] + ed + es;
+    if (a.e_abs) a.e_abs[s] = fabs(a.h_diag[s]) + ea;
     if (a.e_det) a.e_det[s] = ed;
     if (a.e_stoch) a.e_stoch[s] = es;
 }
@@ -236,12 +249,15 @@ __device__ double block_reduce_sum(double v, double* sh)
     return r;   // valid in thread 0
 }
 
-__global__ void __launch_bounds__(256) k_summary(FinalArgs a)
+// Block b's partial sums at summary[8 + 9 b]: the reference m_b = max 2 log f,
+// then sum c, sum c E, sum c f^2 e^{-m_b}, sum c f^2 e^{-m_b} E, and the counts.
+__global__ void __launch_bounds__(256) k_summary_part(FinalArgs a)
 {
     __shared__ double sh[32];
     __shared__ double bc;
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
     double m = -INFINITY;
-    for (int64_t s = threadIdx.x; s < a.Ns; s += blockDim.x) m = fmax(m, 2.0 * a.log_f[s]);
+    for (int64_t s = t0; s < a.Ns; s += step) m = fmax(m, 2.0 * a.log_f[s]);
     m = warp_max_f64(m);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
     __syncthreads();
@@ -252,59 +268,63 @@ __global__ void __launch_bounds__(256) k_summary(FinalArgs a)
     }
     __syncthreads();
     m = bc;
-    __syncthreads();
-    double sc = 0.0, sce = 0.0, scf = 0.0, ndet = 0.0, nu = 0.0;
-    for (int64_t s = threadIdx.x; s < a.Ns; s += blockDim.x) {
-        const double c = a.counts ? a.counts[s] : 1.0;
-        sc += c;
-        sce += c * a.e_loc[s];
-        scf += c * exp(2.0 * a.log_f[s] - m);
-        if (a.det_off) ndet += (double)(a.det_off[s + 1] - a.det_off[s]);
-        if (a.n_unique) nu += (double)a.n_unique[s];
+    double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int64_t s = t0; s < a.Ns; s += step) {
+        const double c = a.counts ? a.counts[s] : 1.0, e = a.e_loc[s];
+        // a block whose f all vanish adds nothing (unless every block's do)
+        const double f2 = m == -INFINITY ? 0.0 : exp(2.0 * a.log_f[s] - m);
+        v[0] += c;
+        v[1] += c * e;
+        v[2] += c * f2;
+        v[3] += c * f2 * e;
+        if (a.det_off) v[4] += (double)(a.det_off[s + 1] - a.det_off[s]);
+        if (a.n_unique) v[5] += (double)a.n_unique[s];
     }
-    double sp = 0.0;
     if (a.span_det)
-        for (int64_t b = threadIdx.x; b < a.base_det[a.Ns]; b += blockDim.x) sp += (double)a.span_det[b];
+        for (int64_t b = t0; b < a.base_det[a.Ns]; b += step) v[6] += (double)a.span_det[b];
     if (a.span_draw && a.base_draw)
-        for (int64_t b = threadIdx.x; b < a.base_draw[a.Ns]; b += blockDim.x) sp += (double)a.span_draw[b];
-    double mv = 0.0;
+        for (int64_t b = t0; b < a.base_draw[a.Ns]; b += step) v[6] += (double)a.span_draw[b];
     if (a.mv_det)
-        for (int64_t b = threadIdx.x; b < a.base_det[a.Ns]; b += blockDim.x) mv += (double)a.mv_det[b];
+        for (int64_t b = t0; b < a.base_det[a.Ns]; b += step) v[7] += (double)a.mv_det[b];
     if (a.mv_draw && a.base_draw)
-        for (int64_t b = threadIdx.x; b < a.base_draw[a.Ns]; b += blockDim.x) mv += (double)a.mv_draw[b];
-    sp = block_reduce_sum(sp, sh);
-    mv = block_reduce_sum(mv, sh);
-    sc = block_reduce_sum(sc, sh);
-    sce = block_reduce_sum(sce, sh);
-    scf = block_reduce_sum(scf, sh);
-    ndet = block_reduce_sum(ndet, sh);
-    nu = block_reduce_sum(nu, sh);
-    if (threadIdx.x == 0) bc = m + log(scf / sc);
-    __syncthreads();
-    const double logB = bc;
-    double set = 0.0;
-    for (int64_t s = threadIdx.x; s < a.Ns; s += blockDim.x) {
-        const double c = a.counts ? a.counts[s] : 1.0;
-        set += c * exp(2.0 * a.log_f[s] - logB) * a.e_loc[s];
+        for (int64_t b = t0; b < a.base_draw[a.Ns]; b += step) v[7] += (double)a.mv_draw[b];
+    double* out = a.summary + 8 + 9 * blockIdx.x;
+    for (int k = 0; k < 8; ++k) {
+        const double r = block_reduce_sum(v[k], sh);
+        if (threadIdx.x == 0) out[k + 1] = r;
     }
-    set = block_reduce_sum(set, sh);
+    if (threadIdx.x == 0) out[0] = m;
+}
+
+__global__ void __launch_bounds__(32) k_summary_final(double* summary, int blocks)
+{
+    const double* p = summary + 8;
+    double m = -INFINITY;
+    for (int b = threadIdx.x; b < blocks; b += 32) m = fmax(m, p[9 * b]);
+    m = warp_max_f64(m);
+    double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int b = threadIdx.x; b < blocks; b += 32) {
+        const double mb = p[9 * b];
+        const double f = mb == -INFINITY && m != -INFINITY ? 0.0 : exp(mb - m);
+        for (int k = 0; k < 8; ++k) v[k] += (k == 2 || k == 3) ? f * p[9 * b + 1 + k] : p[9 * b + 1 + k];
+    }
+    for (int k = 0; k < 8; ++k) v[k] = warp_sum_f64(v[k]);
     if (threadIdx.x == 0) {
-        a.summary[0] = sce / sc;
-        a.summary[1] = sc;
-        a.summary[2] = logB;
-        a.summary[3] = set / sc;
-        a.summary[4] = ndet;
-        a.summary[5] = nu;
-        a.summary[6] = sp;
-        a.summary[7] = mv;
+        summary[0] = v[1] / v[0];
+        summary[1] = v[0];
+        summary[2] = m + log(v[2] / v[0]);        // log B
+        summary[3] = v[3] / v[2];                 // sum c f^2 E / sum c f^2 = (1 / sum c) sum c (f^2 / B) E
+        for (int k = 4; k < 8; ++k) summary[k] = v[k];
     }
 }
 
 int launch_summary(const FinalArgs& a, cudaStream_t st)
 {
     if (a.Ns == 0 || !a.summary) return 0;
-    k_summary<<<1, 256, 0, st>>>(a);
-    return 1;
+    const int blocks = a.Ns >= 64 ? kSummaryBlocks : 16;
+    k_summary_part<<<blocks, 256, 0, st>>>(a);
+    k_summary_final<<<1, 32, 0, st>>>(a.summary, blocks);
+    return 2;
 }
 
 // samples picked for re-evaluation: their words, counts and global positions
@@ -346,9 +366,8 @@ int launch_scatter_picked(const int64_t* idx, int64_t n, const double* v, double
 int launch_finalize(const FinalArgs& a, cudaStream_t st)
 {
     if (a.Ns == 0) return 0;
-    k_final_samples<<<(unsigned)((a.Ns + 255) / 256), 256, 0, st>>>(a);
-    if (a.summary) k_summary<<<1, 256, 0, st>>>(a);
-    return a.summary ? 2 : 1;
+    k_final_samples<<<(unsigned)((a.Ns + 7) / 8), 256, 0, st>>>(a);
+    return 1 + launch_summary(a, st);
 }
 
 }  // namespace nqs

@@ -1,0 +1,74 @@
+"""Kernels at the edges of their tiles and ranges, against plain float64
+references. Tolerances are a multiple of 2^-53 times the sum of the magnitudes
+added (the bound of a sum taken in any order)."""
+import numpy as np
+import pytest
+
+from paper_2507_19276_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_2507_19276_gb300 import nqs  # noqa: E402
+
+U = 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = nqs.Context(0)
+    yield c
+    c.close()
+
+
+def _occ(s, K):
+    b = (np.asarray(s, np.uint64)[:, None, :] >> np.arange(K, dtype=np.uint64)[None, :, None]) & np.uint64(1)
+    return b.reshape(len(s), 2 * K).astype(np.float64)
+
+
+@pytest.mark.parametrize("nh,ns", [(1, 1), (3, 31), (32, 33), (33, 4097 // 16), (36, 4900)])
+def test_correlator_gradient_chunks(ctx, nh, ns):
+    """Chunks of samples x 32 hidden units: remainders on both sides, a last
+    chunked pass (grad_chunk) whose chunk count differs from the full passes'."""
+    s = W.tiny_system(K=8, na=4, nb=4, D=3, n_hidden=nh, seed=nh + ns, n_samples=ns)
+    u = np.random.default_rng(ns).normal(size=len(s.samples))
+    n = _occ(s.samples, s.K)
+    t = np.tanh(s.rbm_b + n @ s.rbm_W.T)
+    ref_W, ref_b = (u[:, None] * t).T @ n, (u[:, None] * t).sum(0)
+    size = np.abs(u)[:, None] * np.abs(t)
+    ctx.set_system(s)
+    for chunk in (0, max(1, ns // 2 + 1)):
+        ctx.set_precision(nqs.NQS_PREC_FP64, grad_chunk=chunk)
+        _, gW, gb = ctx.grad_log_psi_vjp(s.samples, u)
+        tol = (len(u) + 64) * U
+        assert np.all(np.abs(gb - ref_b) <= tol * size.sum(0) + 1e-300)
+        assert np.all(np.abs(gW - ref_W) <= tol * size.sum(0)[:, None] + 1e-300)
+    ctx.set_precision(nqs.NQS_PREC_FP64)
+
+
+@pytest.mark.parametrize("graph,D", [(False, 1), (False, 16), (False, 33), (False, 80), (False, 192), (True, 16), (True, 33)])
+def test_ansatz_forms_from_host_and_device(ctx, graph, D):
+    """The device-made parameter forms (tiles of 32, one or several reduction
+    chunks) serve every precision form; host and device parameters agree bitwise."""
+    s = W.tiny_system(K=6, na=3, nb=3, D=D, n_hidden=5, seed=D, graph=graph, n_samples=40)
+    ctx.set_system(s)
+    got = {}
+    for where in ("host", "device"):
+        args = [s.tensors, s.rbm_W, s.rbm_b]
+        if where == "device":
+            args = [torch.from_numpy(x).cuda() for x in args]
+        ctx.set_ansatz(args[0], s.pred_ptr, s.pred_idx, args[1], args[2])
+        for prec in (nqs.NQS_PREC_FP64, nqs.NQS_PREC_MIXED):
+            if graph and prec == nqs.NQS_PREC_MIXED and D != 16:
+                continue
+            ctx.set_precision(prec)
+            got[where, prec] = ctx.local_energy(s.samples, s.counts, 0.0, 0, 1)[0]
+    for prec in (nqs.NQS_PREC_FP64, nqs.NQS_PREC_MIXED):
+        if ("host", prec) in got:
+            assert np.array_equal(got["host", prec], got["device", prec])
+            ref = got["host", nqs.NQS_PREC_FP64]
+            assert np.all(np.abs(got["host", prec] - ref) <= 1e-5 * np.maximum(np.abs(ref), np.abs(ref).max()))
+    ctx.set_precision(nqs.NQS_PREC_FP64)
