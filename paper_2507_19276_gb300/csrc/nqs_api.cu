@@ -97,7 +97,7 @@ struct nqs_ctx {
     int table_mb = 0;          // cap on one sample batch's shared-prefix tables (0: none)
     // autoregressive sampler levels
     std::vector<DevBuf> smp_pa, smp_pb, smp_off, smp_cnt, smp_par, smp_cell;
-    DevBuf smp_cand, smp_ccnt, smp_cpos, smp_tabs;
+    DevBuf smp_cand, smp_ccnt, smp_cpos, smp_tabs, smp_tree;
     struct Pending { int stage; cudaEvent_t a, b; };
     std::vector<Pending> pending;
     std::vector<cudaEvent_t> free_events;
@@ -814,7 +814,7 @@ extern "C" int nqs_destroy(nqs_ctx* c)
     for (DevBuf* b : bufs) release(*b);
     DevBuf* more[] = {&c->rv, &c->reta, &c->rw, &c->rc, &c->W2, &c->rnn_cells, &c->rnn_lp, &c->rnn_sg,
                       &c->grad_scr, &c->u_dev, &c->ebar_dev, &c->smp_cand, &c->smp_ccnt, &c->smp_cpos,
-                      &c->smp_tabs, &c->tk_rank, &c->tk_off, &c->tk, &c->g_img, &c->g_bexp,
+                      &c->smp_tabs, &c->smp_tree, &c->tk_rank, &c->tk_off, &c->tk, &c->g_img, &c->g_bexp,
                       &c->g_col0, &c->g_slot, &c->g_last, &c->mv_det, &c->mv_draw, &c->g_simg,
                       &c->g_tts, &c->g_rank, &c->g_coef};
     for (DevBuf* b : more) release(*b);
@@ -1862,6 +1862,64 @@ extern "C" int nqs_energy_gradient(nqs_ctx* c, const uint64_t* samples, const do
     return NQS_OK;
 }
 
+namespace {
+
+// nqs_sample in one launch: lays the node arrays out in c->smp_tree, runs the
+// descent, reads the node count back, then writes the determinants.
+int sample_tree(nqs_ctx* c, int64_t n_samples, uint64_t seed, uint64_t* samples, double* counts,
+                int64_t capacity, int64_t* n_unique)
+{
+    const int K = c->K, D = c->av.D;
+    SampleTree t{};
+    t.an = c->av;
+    t.n_samples = n_samples;
+    t.cap = (n_samples + 3) & ~(int64_t)3;
+    t.seed = seed;
+    t.keep = c->av.chain ? 0 : 1;
+    const size_t cap = (size_t)t.cap;
+    const size_t nl = t.keep ? (size_t)K + 1 : 2, nc = t.keep ? (size_t)K : 2;
+    const size_t b_words = 2 * cap * 8, b_int = 2 * cap * 4, b_child = 2 * cap * 16, b_thr = cap * 48;
+    const size_t b_link = nl * cap * 4, b_cand = nc * cap * 4 * D * 8, b_stat = 512;
+    TRY(ensure(c, c->smp_tree, 2 * b_words + 2 * b_int + b_int / 2 + b_child + b_thr + b_link + b_cand + b_stat));
+    char* p = (char*)c->smp_tree.p;
+    t.status = (int*)p; p += b_stat;
+    t.cand = (double*)p; p += b_cand;
+    t.thr = (double*)p; p += b_thr;
+    t.child = (int*)p; p += b_child;
+    t.pa = (uint64_t*)p; p += b_words;
+    t.pb = (uint64_t*)p; p += b_words;
+    t.off = (int*)p; p += b_int;
+    t.cnt = (int*)p; p += b_int;
+    t.node = (int*)p; p += b_int / 2;
+    t.link = (int*)p;
+    CK(cudaMemsetAsync(t.status, 0, b_stat, c->stream));
+    LAUNCH(NQS_STAGE_OTHER, launch_sample_tree(t, c->n_sm, c->stream));
+    CK(cudaGetLastError());
+    int st[4 + kMaxOrb + 1];
+    CK(cudaMemcpyAsync(st, t.status, sizeof(st), cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    if (st[1] == 1) return set_err(c, NQS_ERR_TIMEOUT, "the sampler's grid barrier gave up");
+    if (st[1] >= 2) return set_err(c, NQS_ERR_INVALID_ARG, "no local state is allowed at vertex %d", st[1] - 2);
+    const int64_t n = st[4 + K];
+    *n_unique = n;
+    if (capacity < n)
+        return set_err(c, NQS_ERR_INVALID_ARG, "capacity %lld < %lld unique samples (n_unique written)",
+                       (long long)capacity, (long long)n);
+    uint64_t* dsm;
+    double* dcn;
+    bool hs, hc;
+    TRY(stage_out(c, c->st_out0, samples, (size_t)n * 2, &dsm, &hs));
+    TRY(stage_out(c, c->st_out1, counts, (size_t)n, &dcn, &hc));
+    LAUNCH(NQS_STAGE_OTHER, launch_sample_tree_output(t, n, dsm, dcn, c->stream));
+    CK(cudaGetLastError());
+    TRY(copy_back(c, samples, dsm, (size_t)n * 2, hs));
+    TRY(copy_back(c, counts, dcn, (size_t)n, hc));
+    CK(cudaStreamSynchronize(c->stream));
+    return NQS_OK;
+}
+
+}  // namespace
+
 extern "C" int nqs_sample(nqs_ctx* c, int64_t n_samples, uint64_t seed, uint64_t* samples, double* counts,
                           int64_t capacity, int64_t* n_unique)
 {
@@ -1876,6 +1934,14 @@ extern "C" int nqs_sample(nqs_ctx* c, int64_t n_samples, uint64_t seed, uint64_t
     *n_unique = 0;
     if (n_samples == 0) return NQS_OK;
     const int K = c->K, D = c->av.D;
+    // up to 2^17 draws (and 2 GiB of kept cells): one cooperative launch. Every block
+    // counts the children before its own nodes, O(draws) per block and level, and
+    // the node arrays hold one entry per draw; the descent by levels, whose
+    // buffers follow the distinct prefixes, serves larger batches.
+    const size_t keep_rows = c->av.chain ? 2 : (size_t)K;
+    if (n_samples <= (1 << 17) && (double)n_samples * keep_rows * 32.0 * D <= 2147483648.0 &&
+        sample_tree_fits(c->av, c->n_sm))
+        return sample_tree(c, n_samples, seed, samples, counts, capacity, n_unique);
     c->smp_pa.resize(K + 1); c->smp_pb.resize(K + 1); c->smp_off.resize(K + 1);
     c->smp_cnt.resize(K + 1); c->smp_par.resize(K + 1); c->smp_cell.resize(K + 1);
     // level 0: the empty prefix holds every draw

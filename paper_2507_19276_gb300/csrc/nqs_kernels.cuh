@@ -597,6 +597,33 @@ struct SampleChildren {
 int launch_sample_children(const SampleChildren& a, cudaStream_t st);
 int launch_sample_output(const uint64_t* pa, const uint64_t* pb, const int64_t* cnt, int64_t n,
                          uint64_t* dets, double* counts, cudaStream_t st);
+// The whole breadth-first descent in one cooperative launch (see k_sample_tree).
+// Node arrays of the levels alternate between two halves of `cap` entries; the
+// candidate cells and links of every level are kept for a graph (keep = 1),
+// alternate for a chain.
+struct SampleTree {
+    AnsatzView an;
+    int64_t n_samples;
+    int64_t cap;                          // node bound: min over the levels' needs, <= n_samples
+    uint64_t seed;
+    uint64_t* pa; uint64_t* pb;           // [2][cap]
+    int* off; int* cnt;                   // [2][cap] draw offsets and counts
+    int* child;                           // [2][cap][4] draws per local state
+    double* thr;                          // [cap][6] cumulative P of the allowed states (-1: not
+                                          // allowed), Z, last allowed state
+    int* node;                            // [cap] node of each draw
+    int* link;                            // [K + 1 or 2][cap] candidate (parent * 4 + state) of a node
+    double* cand;                         // [K or 2][cap][4][D]
+    int keep;
+    int* status;                          // [0] barrier arrivals, [1] stop flag (0 ok, 1 timeout,
+                                          // 2 + i: no child at vertex i), [2] nodes of the last level,
+                                          // [4 + i] nodes of level i
+    DevError* err;
+};
+// false when the tree's kernel cannot run resident on this device
+bool sample_tree_fits(const AnsatzView& an, int n_sm);
+int launch_sample_tree(const SampleTree& a, int n_sm, cudaStream_t st);
+int launch_sample_tree_output(const SampleTree& a, int64_t n, uint64_t* dets, double* counts, cudaStream_t st);
 // u_n of the energy gradient (nqs_grad.cu)
 int launch_energy_weights(const double* e_loc, const double* counts, const double* log_f, int64_t Ns,
                           double e_mean, double sum_c, double log_B, bool reweighted, double* u,

@@ -590,6 +590,247 @@ int launch_sample_children(const SampleChildren& a, cudaStream_t st)
     return 1;
 }
 
+// ---------------------------------------------------------------------------
+// The descent in one launch (up to 2^17 draws, no tensor term): one
+// 512-thread block per SM, two grid barriers per level and no host in between.
+// Launch by launch (cells + draws, scan, children, and a wait for the node count
+// per level) the H50 sampler spent 2.2 of its 3.3 ms in 150 kernels bound by
+// their latency, the first levels in one warp that picked every draw of the one
+// node.
+//   phase 1: a block numbers the children of its run of level i - 1's nodes (it
+//     counts the children before them: at most 4 cap integers from L2), writes
+//     their words, offsets and links and the node of every draw, then forms the
+//     candidate cells of vertex i: the 4 D entries of all its nodes dealt out
+//     one per thread, eight lanes per P. FP64 bounds this (2 lanes per clock and
+//     SM), so full warps matter: a warp per node with 40 entries at D = 10 and
+//     32-lane sums took 60 FP64 warp instructions per node instead of ~25;
+//   phase 2: a thread per draw picks its node's local state and adds to the
+//     node's counts (integers: any order).
+// The decisions are those of k_sample_level up to the order of P's sum.
+// ---------------------------------------------------------------------------
+
+constexpr int kTreeThreads = 512;
+
+// Grid barrier of a cooperative launch; `gen` counts the barriers passed. Gives
+// up (stop flag 1) after ~2^24 polls, then every block leaves.
+__device__ bool tree_barrier(int* status, int gen)
+{
+    __shared__ int s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(status, 1);
+        const int want = gen * (int)gridDim.x;
+        int ok = 0;
+        for (int it = 0; it < (1 << 24); ++it) {
+            int v;
+            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(status) : "memory");
+            if (v >= want) { ok = 1; break; }
+        }
+        if (!ok) atomicExch(status + 1, 1);
+        int stop;
+        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(stop) : "l"(status + 1) : "memory");
+        s_ok = ok && stop != 1;
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
+__global__ void __launch_bounds__(kTreeThreads) k_sample_tree(SampleTree a)
+{
+    constexpr int NW = kTreeThreads / 32;
+    __shared__ int s_part[NW];
+    __shared__ int s_link[kTreeThreads], s_off[kTreeThreads];
+    __shared__ uint64_t s_wa[kTreeThreads], s_wb[kTreeThreads];
+    __shared__ int s_end;
+    const AnsatzView& an = a.an;
+    const int K = an.K, D = an.D;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const size_t cap = (size_t)a.cap;
+    auto cand_of = [&](int l) { return a.cand + (size_t)(a.keep ? l : l & 1) * cap * 4 * D; };   // cells of vertex l
+    auto link_of = [&](int l) { return a.link + (size_t)(a.keep ? l : l & 1) * cap; };
+    int gen = 0;
+    for (int i = 0; i <= K; ++i) {
+        const int cur = i & 1, prv = cur ^ 1;
+        uint64_t* pa = a.pa + cur * cap;
+        uint64_t* pb = a.pb + cur * cap;
+        int* off = a.off + cur * cap;
+        int* cnt = a.cnt + cur * cap;
+        int* child = a.child + cur * cap * 4;
+        // level 0 is the child of a node that holds every draw
+        const int np = i == 0 ? 1 : *(volatile int*)(a.status + 4 + i - 1);
+        const int* pc = a.child + prv * cap * 4;
+        const int per = (np + (int)gridDim.x - 1) / (int)gridDim.x;
+        const int q0 = min(np, (int)blockIdx.x * per), q1 = min(np, q0 + per);
+        int base = 0;
+        if (q0 < q1) {
+            int before = 0;
+            for (int g = tid; g < q0; g += kTreeThreads) {
+                const int4 c = __ldcg((const int4*)pc + g);
+                before += (c.x > 0) + (c.y > 0) + (c.z > 0) + (c.w > 0);
+            }
+            before = (int)__reduce_add_sync(kFull, (unsigned)before);
+            if (lane == 0) s_part[warp] = before;
+            __syncthreads();
+            for (int w = 0; w < NW; ++w) base += s_part[w];
+        }
+        for (int g0 = q0; g0 < q1; g0 += kTreeThreads / 4) {       // block-uniform
+            // (parent, local state) per thread; the block's scan of the existing children
+            const int g = g0 + (tid >> 2), s = tid & 3;
+            int c = 0;
+            if (g < q1) c = i == 0 ? (s == 0 ? (int)a.n_samples : 0) : __ldcg(pc + 4 * (size_t)g + s);
+            const unsigned bal = __ballot_sync(kFull, c > 0);
+            int pre = c;                                             // draws of the quad up to s
+            for (int o = 1; o < 4; o <<= 1) {
+                const int u = __shfl_up_sync(kFull, pre, o, 4);
+                if (s >= o) pre += u;
+            }
+            __syncthreads();                                         // s_part and the lists are free
+            if (lane == 0) s_part[warp] = __popc(bal);
+            __syncthreads();
+            int at = __popc(bal & ((1u << lane) - 1u)), nch = 0;
+            for (int w = 0; w < NW; ++w) { if (w < warp) at += s_part[w]; nch += s_part[w]; }
+            if (c > 0) {
+                uint64_t wa = 0, wb = 0;
+                int o = 0;
+                if (i > 0) {
+                    wa = __ldcg(a.pa + prv * cap + g) | ((uint64_t)(s & 1) << (i - 1));
+                    wb = __ldcg(a.pb + prv * cap + g) | ((uint64_t)(s >> 1) << (i - 1));
+                    o = __ldcg(a.off + prv * cap + g) + pre - c;
+                }
+                const int q = base + at;
+                pa[q] = wa;
+                pb[q] = wb;
+                off[q] = o;
+                cnt[q] = c;
+                link_of(i)[q] = g * 4 + s;
+                *(int4*)(child + 4 * (size_t)q) = make_int4(0, 0, 0, 0);
+                s_link[at] = g * 4 + s;
+                s_wa[at] = wa;
+                s_wb[at] = wb;
+                s_off[at] = o;
+                if (at == nch - 1) s_end = o + c;
+            }
+            __syncthreads();
+            if (i < K && nch > 0) {
+                // the node of every draw of these children (their draws are contiguous)
+                for (int j = s_off[0] + tid; j < s_end; j += kTreeThreads) {
+                    int lo = 0, hi = nch - 1;
+                    while (lo < hi) {
+                        const int mid = (lo + hi + 1) >> 1;
+                        if (s_off[mid] <= j) lo = mid; else hi = mid - 1;
+                    }
+                    a.node[j] = base + lo;
+                }
+                // candidate cells of vertex i (as in rnn_vertex_warp)
+                const int e0 = an.chain ? i : an.pred_ptr[i], e1 = an.chain ? i + 1 : an.pred_ptr[i + 1];
+                double* cand = cand_of(i) + (size_t)base * 4 * D;
+                for (int q = tid; q < nch * 4 * D; q += kTreeThreads) {
+                    const int x = q / (4 * D), sr = q - x * 4 * D, ss = sr / D, r = sr - ss * D;
+                    double acc = __ldg(an.rv + ((size_t)i * 4 + ss) * D + r);
+                    for (int e = e0; e < e1; ++e) {
+                        const int j = an.chain ? e - 1 : an.pred_idx[e];
+                        const double* AT = an.AT + ((size_t)e * 4 + ss) * D * D;
+                        if (j < 0) {
+                            acc += __ldg(AT + r);
+                        } else {
+                            int lk = s_link[x];                      // candidate of vertex i - 1
+                            for (int l = i - 1; l > j; --l) lk = link_of(l)[lk >> 2];
+                            acc += dot_col4(AT, cand_of(j) + (size_t)lk * D, D, r);
+                        }
+                    }
+                    cand[q] = acc;
+                }
+                __syncthreads();
+                // P and the thresholds, a warp per node, eight lanes per local state
+                for (int x = warp; x < nch; x += NW) {
+                    const double* h = cand + ((size_t)x * 4 + (lane >> 3)) * D;
+                    double p = 0.0;
+                    for (int r = lane & 7; r < D; r += 8) p = fma(__ldg(an.reta + (size_t)i * D + r) * h[r], h[r], p);
+                    for (int o = 4; o; o >>= 1) p += __shfl_xor_sync(kFull, p, o);
+                    const int nad = __popcll(s_wa[x]), nbd = __popcll(s_wb[x]);
+                    int last = -1;
+                    double Z = 0.0, thr = -1.0;
+                    for (int t = 0; t < 4; ++t) {
+                        const double pt = __shfl_sync(kFull, p, 8 * t);
+                        if (!rnn_allowed(an, i, nad, nbd, t)) continue;
+                        Z += pt;
+                        if (lane == t) thr = Z;
+                        last = t;
+                    }
+                    if (lane == 4) thr = Z;
+                    if (lane == 5) thr = (double)last;
+                    if (lane < 6) a.thr[6 * (size_t)(base + x) + lane] = thr;
+                }
+            }
+            base += nch;
+        }
+        if (q0 < q1 && q1 == np && tid == 0) {               // the last node's block knows the total
+            a.status[4 + i] = base;
+            if (base == 0) atomicExch(a.status + 1, 1 + i);
+        }
+        if (!tree_barrier(a.status, ++gen)) return;
+        if (*(volatile int*)(a.status + 4 + i) <= 0) return;
+        if (i == K) break;
+        const int64_t step = (int64_t)gridDim.x * kTreeThreads;
+        for (int64_t j0 = (int64_t)blockIdx.x * kTreeThreads + warp * 32; j0 < a.n_samples; j0 += step) {
+            const int64_t j = j0 + lane;                     // whole warps: the match below needs them
+            int key = -1;
+            if (j < a.n_samples) {
+                const int q = __ldcg(a.node + j);
+                const double* t = a.thr + 6 * (size_t)q;
+                const double t0 = __ldcg(t), t1 = __ldcg(t + 1), t2 = __ldcg(t + 2), t3 = __ldcg(t + 3);
+                const double Z = __ldcg(t + 4), last = __ldcg(t + 5);
+                const uint64_t x = philox_first4((uint64_t)j, (uint64_t)i, 1ull, a.seed);
+                const double tt = (double)(x >> 11) * 0x1.0p-53 * Z;
+                // the first allowed state above tt
+                const int pick = tt < t0 ? 0 : tt < t1 ? 1 : tt < t2 ? 2 : tt < t3 ? 3 : (int)last;
+                if (pick >= 0) key = q * 4 + pick;
+            }
+            const unsigned same = __match_any_sync(kFull, key);
+            if (key >= 0 && lane == __ffs(same) - 1) atomicAdd(child + key, __popc(same));
+        }
+        if (!tree_barrier(a.status, ++gen)) return;
+    }
+}
+
+bool sample_tree_fits(const AnsatzView& an, int n_sm)
+{
+    int dev = 0, coop = 0, occ = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    if (!coop || n_sm < 1 || an.tk_rank) return false;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sample_tree, kTreeThreads, 0) == cudaSuccess && occ >= 1;
+}
+
+int launch_sample_tree(const SampleTree& a, int n_sm, cudaStream_t st)
+{
+    // blocks beyond one thread per draw would only wait
+    const int64_t want = (a.n_samples + 31) / 32;
+    const unsigned grid = (unsigned)(want < n_sm ? want : n_sm);
+    SampleTree args = a;
+    void* p[] = {&args};
+    cudaLaunchCooperativeKernel(k_sample_tree, dim3(grid), dim3(kTreeThreads), p, 0, st);
+    return 1;
+}
+
+__global__ void k_sample_tree_output(SampleTree a, int64_t n, uint64_t* dets, double* counts)
+{
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= n) return;
+    const size_t at = (size_t)(a.an.K & 1) * a.cap + q;
+    dets[2 * q] = a.pa[at];
+    dets[2 * q + 1] = a.pb[at];
+    counts[q] = (double)a.cnt[at];
+}
+
+int launch_sample_tree_output(const SampleTree& a, int64_t n, uint64_t* dets, double* counts, cudaStream_t st)
+{
+    if (n == 0) return 0;
+    k_sample_tree_output<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(a, n, dets, counts);
+    return 1;
+}
+
 // The last level's nodes as determinants [n][2] and counts (as doubles).
 __global__ void k_sample_output(const uint64_t* pa, const uint64_t* pb, const int64_t* cnt, int64_t n,
                                 uint64_t* dets, double* counts)

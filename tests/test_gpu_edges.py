@@ -72,3 +72,19 @@ def test_ansatz_forms_from_host_and_device(ctx, graph, D):
             ref = got["host", nqs.NQS_PREC_FP64]
             assert np.all(np.abs(got["host", prec] - ref) <= 1e-5 * np.maximum(np.abs(ref), np.abs(ref).max()))
     ctx.set_precision(nqs.NQS_PREC_FP64)
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 4097, 140000])
+@pytest.mark.parametrize("graph", [False, True])
+def test_sampler_sizes(ctx, n, graph):
+    """One draw, part warps, several blocks, and the descent by levels (above
+    2^17 draws): determinants and counts bit-equal to the oracle's."""
+    from oracle import oracle as O
+    s = W.with_readout(W.tiny_system(K=8, na=4, nb=3, D=5, n_hidden=3, seed=n % 97, graph=graph, n_samples=4), seed=2)
+    if graph and n in (33, 4097):
+        s = W.with_tensor_term(s, seed=1)        # the descent by levels at small sizes
+    ctx.set_system(s)
+    dets, counts = ctx.sample(n, 11 + n)
+    ref, ref_c, _ = O.sample(O.Problem(s), n, 11 + n)
+    assert counts.sum() == n
+    assert np.array_equal(dets, ref) and np.array_equal(counts, ref_c)
