@@ -12,6 +12,7 @@
 #include "../../include/nqs.h"
 #include "nqs_kernels.cuh"
 #include "nqs_family.cuh"
+#include "nqs_tree.cuh"
 
 using namespace nqs;
 
@@ -85,6 +86,10 @@ struct nqs_ctx {
     DevBuf tk_rank, tk_off, tk;   // tensor term (Tucker form) of the graph ansatz
     // mixed form of the graph ansatz: matrix images, e_0 columns, state slots
     DevBuf g_img, g_bexp, g_col0, g_slot, g_last, mv_det, mv_draw, g_simg, g_tts, g_rank, g_coef;
+    // prefix trees (graphs, the normalised chain readout)
+    DevBuf tr_rows, tr_build, tr_items, tr_pool, tr_close, g_live;
+    std::vector<int> pred_ptr_h, pred_idx_h;
+    int n_live = 0;           // entries of g_live past its K + 1 offsets
     int g_slots = 0, g_maxdeg = 0, g_nbuf = 1;
     bool has_gtc = false;
     char gtc_why[160] = {0};   // why the graph does not fit the tensor-core tiles
@@ -764,6 +769,221 @@ int family_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, i
     return NQS_OK;
 }
 
+// ---- prefix trees (nqs_tree.cu) ----------------------------------------------
+
+// Carves aligned pieces out of one buffer; the first pass (p = NULL) sizes it.
+struct Carve {
+    char* p;
+    size_t n = 0;
+    template <typename T>
+    T* take(size_t count)
+    {
+        n = (n + 255) & ~(size_t)255;
+        T* r = p ? (T*)(p + n) : nullptr;
+        n += count * sizeof(T);
+        return r;
+    }
+};
+
+enum TreeKind { kTreeGraph64, kTreeGraphTc, kTreeRnn };
+
+// Amplitudes of the deterministic and drawn rows over the prefix trees of
+// sample batches: partial sums per kTreeRows-row chunk of a sample's rows
+// (deterministic, then drawn) into part_det, chunk bases in base_det.
+int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int n_draws, TreeKind kind, bool want_abs)
+{
+    const int K = c->K, D = c->av.D, NH = c->av.n_hidden, T = 3 * K, np = (NH + 3) & ~3;
+    const bool full = kind != kTreeGraph64;
+    const int stage = NQS_STAGE_AMP_DET;
+    StageScope sc(c, stage);
+    TRY(ensure(c, c->tr_rows, (size_t)(2 * Ns + 1) * 8));
+    TRY(ensure(c, c->base_det, (size_t)(Ns + 1) * 8));
+    int64_t* row_cnt = (int64_t*)c->tr_rows.p;
+    int64_t* row_base = row_cnt + Ns;
+    const int64_t* dcnt = n_draws > 0 ? (const int64_t*)c->n_unique.p : nullptr;
+    LAUNCH(stage, launch_tree_row_counts((const int64_t*)c->det_tot.p, dcnt, Ns, row_cnt, c->stream));
+    LAUNCH(stage, launch_scan_i64(row_cnt, row_base, Ns, c->stream));
+    LAUNCH(stage, launch_chunk_base(row_cnt, kTreeRows, (int64_t*)c->base_det.p, Ns, c->stream));
+    const int64_t rows_bound = total_det + Ns * (int64_t)n_draws;
+    const int64_t chunks_all = rows_bound / kTreeRows + Ns;
+    TRY(ensure(c, c->part_det, (size_t)(chunks_all + 1) * 8));
+    TRY(ensure(c, c->span_det, (size_t)(chunks_all + 1) * 8));
+    if (kind != kTreeRnn) TRY(ensure(c, c->mv_det, (size_t)(chunks_all + 1) * 8));
+    if (want_abs) TRY(ensure(c, c->part_det_abs, (size_t)(chunks_all + 1) * 8));
+
+    size_t free_b = 0, total_b = 0;
+    cudaMemGetInfo(&free_b, &total_b);
+    free_b += c->tr_build.n + c->tr_pool.n + c->tr_items.n;     // kept from earlier calls
+    size_t budget = std::min<size_t>(c->table_mb > 0 ? (size_t)c->table_mb << 20 : (size_t)16 << 30, free_b / 3);
+    if (c->fam_budget > 0) budget = std::min(budget, c->fam_budget);
+    const int n2max = 9 * K * (K - 1) / 2 > 0 ? 9 * K * (K - 1) / 2 : 1, W = (T + 31) / 32;
+    const size_t state = kind == kTreeGraph64 ? (size_t)D * 8 + 4 : (size_t)D * 4 + 4;
+    const size_t node_b = kind == kTreeRnn ? 16 + 2 * ((size_t)D * 8 + 16) : 16 + (full ? 8 : 0);
+    // bytes of a sample with r rows: tables, nodes, and about 0.4 K levels per row
+    auto bytes_of = [&](int64_t r) {
+        const size_t nodes = 1 + T + n2max + (size_t)r * (full ? 2 : 1);
+        const size_t lv = (size_t)r * K * 2 / 5 + K;
+        return (size_t)4 * T * (T + 1) + (size_t)8 * n2max * W + nodes * node_b + (size_t)8 * r +
+               lv * (4 + (kind == kTreeRnn ? 0 : state)) + (kind == kTreeGraph64 ? (size_t)3 * c->n_live * (D * 8 + 4) : 0);
+    };
+    for (int64_t s0 = 0; s0 < Ns;) {
+        int64_t s1 = s0;
+        size_t want = 0;
+        while (s1 < Ns && s1 - s0 < 32768) {
+            const int64_t r = c->det_off_h[s1 + 1] - c->det_off_h[s1] + n_draws;
+            const size_t add = bytes_of(r);
+            if (s1 > s0 && want + add > budget) break;
+            want += add;
+            ++s1;
+        }
+        // equal batches
+        const int64_t parts = (Ns - s0 + (s1 - s0) - 1) / (s1 - s0);
+        if (parts > 1) s1 = s0 + std::max<int64_t>(1, std::min(s1 - s0, (Ns - s0 + parts - 1) / parts));
+    retry:
+        const int nb = (int)(s1 - s0);
+        const int64_t R = c->det_off_h[s1] - c->det_off_h[s0] + (int64_t)nb * n_draws;
+        const int64_t max_chunks = R / kTreeRows + nb;
+        TreeArgs a{};
+        a.h = c->hv;
+        a.samples = ds;
+        a.s0 = s0;
+        a.nb = nb;
+        a.K = K;
+        a.full = full ? 1 : 0;
+        a.det_rank = (const uint32_t*)c->det_rank.p;
+        a.det_off = (const int64_t*)c->det_off.p;
+        a.det_cnt = (const int64_t*)c->det_tot.p;
+        a.det_coef = (const double*)c->det_coef.p;
+        if (n_draws > 0) {
+            a.draw_rank = (const uint32_t*)c->draw_rank.p;
+            a.draw_stride = n_draws;
+            a.draw_cnt = dcnt;
+            a.draw_coef = (const double*)c->draw_coef.p;
+        }
+        a.row_base = row_base;
+        a.chunk_base = (const int64_t*)c->base_det.p;
+        a.n2max = n2max;
+        a.W = W;
+        a.pool0 = kind == kTreeRnn ? 0u : (uint32_t)nb * (uint32_t)K;
+        const int64_t nodes = (int64_t)nb * (1 + T + n2max) + R * (full ? 2 : 1);
+        if (nodes >= ((int64_t)1 << 32))
+            return set_err(c, NQS_ERR_UNSUPPORTED, "prefix trees of %lld nodes exceed 2^32", (long long)nodes);
+        a.id1 = (uint32_t)nb;
+        a.id2 = a.id1 + (uint32_t)(nb * T);
+        a.id3 = a.id2 + (uint32_t)((int64_t)nb * n2max);
+        a.id4 = a.id3 + (uint32_t)R;
+        const int64_t ncnt = (int64_t)4 * K * nb;
+        int64_t *scan_tmp = nullptr, *pool_off = nullptr;
+        float* mant = nullptr;
+        int* mexp = nullptr;
+        TreeRnn rn{};
+        for (int pass = 0; pass < 2; ++pass) {
+            Carve v{pass ? (char*)c->tr_build.p : nullptr};
+            a.word = v.take<uint32_t>((size_t)R + 1);
+            a.rnode = v.take<uint32_t>((size_t)R + 1);
+            a.e1 = v.take<int>((size_t)nb * T);
+            a.e2 = v.take<int>((size_t)nb * T * T);
+            a.n2 = v.take<int>((size_t)nb);
+            a.n3 = v.take<int>((size_t)nb);
+            a.bits = v.take<uint32_t>((size_t)nb * n2max * W);
+            a.bits_base = v.take<uint32_t>((size_t)nb * n2max * W);
+            a.parent = v.take<uint32_t>((size_t)nodes);
+            a.end = v.take<int>((size_t)nodes);
+            a.start = v.take<uint32_t>((size_t)nodes);
+            a.base = v.take<uint32_t>((size_t)nodes);
+            a.pool_tot = v.take<int64_t>((size_t)nb + 1);
+            pool_off = v.take<int64_t>((size_t)nb + 1);
+            a.level_cnt = v.take<int64_t>((size_t)ncnt);
+            a.level_off = v.take<int64_t>((size_t)ncnt + 1);
+            scan_tmp = v.take<int64_t>((size_t)scan_i64_tmp_elems(ncnt));
+            if (kind == kTreeGraphTc) {
+                mant = v.take<float>((size_t)nodes);
+                mexp = v.take<int>((size_t)nodes);
+            }
+            if (kind == kTreeRnn) {
+                rn.cell = v.take<double>((size_t)2 * nodes * D);
+                rn.prod = v.take<double>((size_t)2 * nodes);
+                rn.pex = v.take<int>((size_t)2 * nodes);
+                rn.flag = v.take<uint32_t>((size_t)2 * nodes);
+            }
+            if (!pass) TRY(ensure(c, c->tr_build, v.n));
+        }
+        LAUNCH(stage, launch_tree_nodes(a, max_chunks, c->stream));
+        LAUNCH(stage, launch_scan_i64(a.pool_tot, pool_off, nb, c->stream));
+        LAUNCH(stage, launch_scan_i64_wide(a.level_cnt, a.level_off, ncnt, scan_tmp, c->stream));
+        CK(cudaGetLastError());
+        std::vector<int64_t> bounds((size_t)4 * K + 1);
+        int64_t pool_rows = 0;
+        CK(cudaMemcpy2DAsync(bounds.data(), 8, a.level_off, (size_t)nb * 8, 8, (size_t)4 * K + 1, cudaMemcpyDeviceToHost,
+                             c->stream));
+        CK(cudaMemcpyAsync(&pool_rows, pool_off + nb, 8, cudaMemcpyDeviceToHost, c->stream));
+        CK(cudaStreamSynchronize(c->stream));
+        const int64_t rows_total = pool_rows + a.pool0;
+        const size_t pool_b = kind == kTreeRnn ? 0 : (size_t)rows_total * state;
+        if (nb > 1 && (rows_total >= ((int64_t)1 << 32) ||
+                       (double)pool_b + 4.0 * (double)bounds.back() > 2.0 * (double)budget)) {
+            s1 = s0 + (nb + 1) / 2;       // more levels per row than estimated
+            goto retry;
+        }
+        if (rows_total >= ((int64_t)1 << 32))
+            return set_err(c, NQS_ERR_UNSUPPORTED, "prefix trees of %lld states exceed 2^32", (long long)rows_total);
+        TRY(ensure(c, c->tr_items, (size_t)(bounds.back() + 1) * 4));
+        a.items = (uint32_t*)c->tr_items.p;
+        a.pool_tot = pool_off;
+        LAUNCH(stage, launch_tree_items(a, c->stream));
+        if (kind == kTreeGraph64) {
+            TreeGraph64 g{};
+            TreeClose q{};
+            for (int pass = 0; pass < 2; ++pass) {
+                Carve v{pass ? (char*)c->tr_pool.p : nullptr};
+                g.pool = v.take<double>((size_t)rows_total * D);
+                g.pool_e = v.take<int>((size_t)rows_total);
+                if (!pass) TRY(ensure(c, c->tr_pool, v.n));
+            }
+            for (int pass = 0; pass < 2; ++pass) {
+                Carve v{pass ? (char*)c->tr_close.p : nullptr};
+                q.Q = v.take<double>((size_t)nb * c->n_live * 3 * D);
+                q.Qe = v.take<int>((size_t)nb * c->n_live * 3);
+                q.c = v.take<double>((size_t)nb * K * 3);
+                q.ce = v.take<int>((size_t)nb * K * 3);
+                if (!pass) TRY(ensure(c, c->tr_close, v.n));
+            }
+            CK(cudaMemcpyAsync(g.pool, (const double*)c->Hst.p + (size_t)s0 * K * D, (size_t)nb * K * D * 8,
+                               cudaMemcpyDeviceToDevice, c->stream));
+            CK(cudaMemcpyAsync(g.pool_e, (const int*)c->Hexp.p + (size_t)s0 * K, (size_t)nb * K * 4,
+                               cudaMemcpyDeviceToDevice, c->stream));
+            g.an = c->av;
+            g.items = a.items;
+            g.parent = a.parent; g.start = a.start; g.base = a.base;
+            for (int t = 0; t < K; ++t) LAUNCH(stage, launch_tree_graph64(g, t, bounds.data(), c->stream));
+            q.an = c->av;
+            q.samples = ds;
+            q.s0 = s0;
+            q.nb = nb;
+            q.Gst = (const double*)c->Gst.p; q.Gexp = (const int*)c->Gexp.p;
+            q.live_ptr = (const int*)c->g_live.p;
+            q.live_idx = q.live_ptr + K + 1;
+            q.n_live = c->n_live;
+            LAUNCH(stage, launch_tree_close(q, c->stream));
+            TreeRows64 r{};
+            r.t = a;
+            r.q = q;
+            r.pool = g.pool; r.pool_e = g.pool_e;
+            r.theta = (const double*)c->theta.p;
+            r.lc = (const double*)c->lc.p;
+            r.psi_mant = (const double*)c->pmant.p;
+            r.psi_exp = (const int*)c->pexp.p;
+            r.partial = (double*)c->part_det.p;
+            r.span = (int64_t*)c->span_det.p;
+            r.mv = (int64_t*)c->mv_det.p;
+            LAUNCH(stage, launch_tree_rows64(r, max_chunks, c->stream));
+        }
+        CK(cudaGetLastError());
+        s0 = s1;
+    }
+    return NQS_OK;
+}
+
 }  // namespace
 
 // ============================================================================
@@ -816,7 +1036,8 @@ extern "C" int nqs_destroy(nqs_ctx* c)
                       &c->grad_scr, &c->u_dev, &c->ebar_dev, &c->smp_cand, &c->smp_ccnt, &c->smp_cpos,
                       &c->smp_tabs, &c->smp_tree, &c->tk_rank, &c->tk_off, &c->tk, &c->g_img, &c->g_bexp,
                       &c->g_col0, &c->g_slot, &c->g_last, &c->mv_det, &c->mv_draw, &c->g_simg,
-                      &c->g_tts, &c->g_rank, &c->g_coef};
+                      &c->g_tts, &c->g_rank, &c->g_coef, &c->tr_rows, &c->tr_build, &c->tr_items,
+                      &c->tr_pool, &c->tr_close, &c->g_live};
     for (DevBuf* b : more) release(*b);
     for (auto* v : {&c->smp_pa, &c->smp_pb, &c->smp_off, &c->smp_cnt, &c->smp_par, &c->smp_cell})
         for (DevBuf& b : *v) release(b);
@@ -1039,6 +1260,23 @@ extern "C" int nqs_set_ansatz(nqs_ctx* c, const double* site_tensors, int n_edge
             c->has_tc = true;
         }
     } else {
+        // per vertex q, the earlier vertices whose states q or a later vertex reads
+        std::vector<int> lp((size_t)K + 1, 0), li;
+        for (int q = 0; q < K; ++q) {
+            for (int j = 0; j < q; ++j) {
+                bool live = false;
+                for (int e = ptr[q]; e < n_edges && !live; ++e) live = idx[e] == j;
+                if (live) li.push_back(j);
+            }
+            lp[(size_t)q + 1] = (int)li.size();
+        }
+        TRY(ensure(c, c->g_live, (size_t)(K + 1 + li.size()) * 4));
+        CK(cudaMemcpyAsync(c->g_live.p, lp.data(), lp.size() * 4, cudaMemcpyHostToDevice, c->stream));
+        if (!li.empty())
+            CK(cudaMemcpyAsync((int*)c->g_live.p + K + 1, li.data(), li.size() * 4, cudaMemcpyHostToDevice, c->stream));
+        c->n_live = (int)li.size();
+        c->pred_ptr_h = ptr;
+        c->pred_idx_h = idx;
         const char* why = nullptr;
         if (graph_tc_plan(ptr.data(), idx.data(), K, D, n_hidden, gp, &why)) {
             TRY(ensure(c, c->g_img, (size_t)n_edges * 16 * D * D));
@@ -1397,6 +1635,9 @@ int le_core(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, uint64
     const bool shared = c->av.chain && (prec == NQS_PREC_MIXED || prec == NQS_PREC_FP64_SHARED);
     const bool gtc = !c->av.chain && prec == NQS_PREC_MIXED;
     const bool graph = !c->av.chain && !rnn;
+    // psi is linear in the states of a graph without the tensor term: its rows
+    // share prefixes and close with n's adjoints (the tensor term's are re-run)
+    const bool tree64 = graph && !gtc && !c->av.tk_rank;
     if (!c->av.chain && prec == NQS_PREC_FP64_SHARED)
         return set_err(c, NQS_ERR_UNSUPPORTED,
                        "graph ansatze have no shared-prefix form (NQS_PREC_FP64 or NQS_PREC_MIXED)");
@@ -1417,7 +1658,7 @@ int le_core(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, uint64
         StageScope sc(c, NQS_STAGE_ENV);
         LAUNCH(NQS_STAGE_ENV, launch_validate(ds, Ns, c->K, c->na, c->nb, (DevError*)c->derr.p, c->stream));
         // the mixed form takes psi(n) in double-FP32 arithmetic, the FP64 forms in FP64
-        TRY(env_pass(c, ds, Ns, false, rnn ? 0 : (shared ? (prec == NQS_PREC_MIXED ? 3 : 2) : 1)));
+        TRY(env_pass(c, ds, Ns, tree64, rnn ? 0 : (shared ? (prec == NQS_PREC_MIXED ? 3 : 2) : 1)));
         if (rnn) TRY(rnn_env_pass(c, ds, Ns));
         k_check_psi<<<(unsigned)((Ns + 255) / 256), 256, 0, c->stream>>>((const double*)c->pmant.p, Ns,
                                                                        (DevError*)c->derr.p);
@@ -1425,7 +1666,7 @@ int le_core(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, uint64
     }
     int64_t total = 0;
     TRY(count_pass(c, ds, Ns, eb, &total, n_draws > 0));
-    if (shared) {
+    if (shared || tree64) {
         c->det_off_h.resize(Ns + 1);
         CK(cudaMemcpyAsync(c->det_off_h.data(), c->det_off.p, (size_t)(Ns + 1) * 8, cudaMemcpyDeviceToHost, c->stream));
     }
@@ -1460,6 +1701,8 @@ int le_core(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, uint64
     if (shared) {
         if (prec == NQS_PREC_MIXED) TRY(family_pass<float>(c, ds, Ns, total, n_draws, deabs != nullptr));
         else TRY(family_pass<double>(c, ds, Ns, total, n_draws, deabs != nullptr));
+    } else if (tree64) {
+        TRY(tree_pass(c, ds, Ns, total, n_draws, kTreeGraph64, false));
     } else {
         // amplitudes: deterministic rows, then the distinct drawn rows
         RowSet rd{};
@@ -1481,26 +1724,27 @@ int le_core(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, uint64
         }
     }
     TRY(ensure(c, c->summary, kSummaryDoubles * 8));
+    const bool draws_apart = n_draws > 0 && !tree64;     // drawn rows in their own partial sums
     FinalArgs f{};
     f.Ns = Ns;
     f.h_diag = (const double*)c->hdiag.p;
     f.part_det = (const double*)c->part_det.p;
     f.base_det = (const int64_t*)c->base_det.p;
-    f.part_draw = n_draws > 0 ? (const double*)c->part_draw.p : nullptr;
-    f.base_draw = n_draws > 0 ? (const int64_t*)c->base_draw.p : nullptr;
+    f.part_draw = draws_apart ? (const double*)c->part_draw.p : nullptr;
+    f.base_draw = draws_apart ? (const int64_t*)c->base_draw.p : nullptr;
     f.counts = dc;
     f.log_f = (const double*)c->logf.p;
     f.det_off = (const int64_t*)c->det_off.p;
     f.n_unique = n_draws > 0 ? (const int64_t*)c->n_unique.p : nullptr;
     f.e_loc = de;
     f.span_det = (const int64_t*)c->span_det.p;
-    f.span_draw = n_draws > 0 ? (const int64_t*)c->span_draw.p : nullptr;
+    f.span_draw = draws_apart ? (const int64_t*)c->span_draw.p : nullptr;
     f.summary = want_summary ? (double*)c->summary.p : nullptr;
     f.e_abs = deabs;
     f.part_det_abs = deabs ? (const double*)c->part_det_abs.p : nullptr;
-    f.part_draw_abs = deabs && n_draws > 0 ? (const double*)c->part_draw_abs.p : nullptr;
+    f.part_draw_abs = deabs && draws_apart ? (const double*)c->part_draw_abs.p : nullptr;
     f.mv_det = graph ? (const int64_t*)c->mv_det.p : nullptr;
-    f.mv_draw = graph && n_draws > 0 ? (const int64_t*)c->mv_draw.p : nullptr;
+    f.mv_draw = graph && draws_apart ? (const int64_t*)c->mv_draw.p : nullptr;
     {
         StageScope sc(c, NQS_STAGE_FINAL);
         LAUNCH(NQS_STAGE_FINAL, launch_finalize(f, c->stream));

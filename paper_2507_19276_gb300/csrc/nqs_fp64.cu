@@ -227,7 +227,11 @@ __global__ void k_env_fp64(EnvArgs a)
             if (threadIdx.x == 0) gset[K - 1] = 1;
             __syncthreads();
             for (int i = K - 1; i >= 0; --i) {
-                if (!gset[i]) continue;
+                if (!gset[i]) {                  // no later vertex reads h_i
+                    for (int r = threadIdx.x; r < D; r += blockDim.x) Gs[(size_t)i * D + r] = 0.0;
+                    if (threadIdx.x == 0) Ge[i] = -1000000;
+                    continue;
+                }
                 for (int r = threadIdx.x; r < D; r += blockDim.x) x[r] = Gs[(size_t)i * D + r];
                 __syncthreads();
                 const int ge = block_renorm(x, D, sh);

@@ -1,0 +1,821 @@
+// nqs_tree.cu -- prefix trees of the connected determinants of a sample.
+//
+// A connected m differs from n on two to four sites. Everything an ansatz
+// computes vertex by vertex up to vertex t depends on m's local states at the
+// vertices up to t, so rows that share their first changes share the work up to
+// the next one. A node is a distinct prefix of changes (site, new local state)
+// together with n's states in between; it lives on the levels (vertices) from
+// its last change to the last level some row needs it at, and continues its
+// parent (the prefix without the last change; n itself is the root). On H18 at
+// eps = 0 a sample's 9 315 rows re-run 139 700 vertices from their first change
+// to the end; their tree has 51 900 (node, level) pairs, and 15 200 when a row
+// stops before its last change (a linear readout: the rest is one covector per
+// (site, alternative), see k_tree_close). H50 at eps = 0.01: 908 000 against
+// 444 000.
+//
+// Building a batch's trees: the rows mark one- and two-change prefixes in
+// tables indexed by change pairs, the two-change ones are numbered, third
+// changes become bits of a row of 3K per two-change node (their rank is a
+// popcount), and four-change rows are nodes of their own. Node ids are fixed
+// regions per sample, so no count is read back before the pool of states is
+// sized. Per level the nodes' ids are grouped by local state (one matrix per
+// in-edge and group).
+#include "nqs_tree.cuh"
+
+namespace nqs {
+
+namespace {
+
+constexpr uint32_t kNoNode = 0xffffffffu;
+
+// sample (call index) of chunk b of the batch, -1 past its end
+__device__ __forceinline__ int64_t tree_sample(const TreeArgs& a, int64_t b)
+{
+    if (b >= a.chunk_base[a.s0 + a.nb]) return -1;
+    int64_t lo = a.s0, hi = a.s0 + a.nb - 1;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi + 1) >> 1;
+        if (a.chunk_base[mid] <= b) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
+struct TreeWord {
+    int c;                    // changes
+    int x[4];
+};
+
+__device__ __forceinline__ TreeWord tree_unpack(uint32_t w)
+{
+    TreeWord r;
+    for (int k = 0; k < 4; ++k) r.x[k] = (int)((w >> (8 * k)) & 255u);
+    r.c = r.x[1] == r.x[0] ? 1 : (r.x[2] == r.x[1] ? 2 : (r.x[3] == r.x[2] ? 3 : 4));
+    return r;
+}
+
+// Words of the rows, and the levels their one- and two-change prefixes are
+// needed to (a prefix that a later change follows: one level before it; a
+// whole row, full form: K - 1).
+__global__ void __launch_bounds__(kTreeRows) k_tree_mark(TreeArgs a)
+{
+    __shared__ OrbLists lists;
+    __shared__ int64_t s_s;
+    if (threadIdx.x == 0) s_s = tree_sample(a, a.chunk_base[a.s0] + blockIdx.x);
+    __syncthreads();
+    const int64_t s = s_s;
+    if (s < 0) return;
+    const int64_t b = a.chunk_base[a.s0] + blockIdx.x;
+    const uint64_t na = a.samples[2 * s], nb = a.samples[2 * s + 1];
+    if (threadIdx.x < 32) build_lists_warp(na, nb, a.h.K, lists, threadIdx.x);
+    __syncthreads();
+    const int64_t r = (b - a.chunk_base[s]) * kTreeRows + threadIdx.x;
+    if (r >= a.row_base[s + 1] - a.row_base[s]) return;
+    const int64_t nd = a.det_cnt[s];
+    const uint32_t rank = r < nd ? a.det_rank[a.det_off[s] + r] : a.draw_rank[s * a.draw_stride + (r - nd)];
+    const Exc e = decode_rank<false>(a.h, lists, rank);
+    uint64_t ma = na, mb = nb;
+    flip(ma, mb, e.i); flip(ma, mb, e.a);
+    if (e.kind == 2) { flip(ma, mb, e.j); flip(ma, mb, e.b); }
+    uint64_t ch = (na ^ ma) | (nb ^ mb);
+    int x[4], c = 0;
+    #pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (ch) {
+            const int p = __ffsll((long long)ch) - 1;
+            ch &= ch - 1;
+            const int own = sigma_at(na, nb, p), nw = sigma_at(ma, mb, p);
+            x[k] = 3 * p + nw - (nw > own ? 1 : 0);
+            ++c;
+        } else {
+            x[k] = k ? x[k - 1] : 0;
+        }
+    }
+    a.word[a.row_base[s] - a.row_base[a.s0] + r] =
+        (uint32_t)x[0] | ((uint32_t)x[1] << 8) | ((uint32_t)x[2] << 16) | ((uint32_t)x[3] << 24);
+    const int T = 3 * a.K, sl = (int)(s - a.s0);
+    int* e1 = a.e1 + (size_t)sl * T + x[0];
+    const int n1 = c >= 2 ? x[1] / 3 - 1 : (a.full ? a.K - 1 : -1);
+    if (*(volatile int*)e1 < n1) atomicMax(e1, n1);
+    const int n2 = c >= 3 ? x[2] / 3 - 1 : (c == 2 && a.full ? a.K - 1 : -1);
+    if (n2 >= 0) {
+        int* e2 = a.e2 + ((size_t)sl * T + x[0]) * T + x[1];
+        if (*(volatile int*)e2 < n2) atomicMax(e2, n2);
+    }
+}
+
+// block-wide exclusive scan (one value per thread), total in *tot
+__device__ __forceinline__ int block_excl(int v, int* sh, int* tot)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    int incl = v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += u;
+    }
+    __syncthreads();
+    if (lane == 31) sh[warp] = incl;
+    __syncthreads();
+    int before = 0, t = 0;
+    for (int w = 0; w < nw; ++w) { if (w < warp) before += sh[w]; t += sh[w]; }
+    *tot = t;
+    return before + incl - v;
+}
+
+// One block per sample: roots, one-change nodes, and the two-change nodes in
+// the order of their changes (their table entries become indices).
+__global__ void __launch_bounds__(512) k_tree_two(TreeArgs a)
+{
+    __shared__ int sh[16];
+    const int sl = blockIdx.x, T = 3 * a.K;
+    const int64_t s = a.s0 + sl;
+    const uint64_t na = a.samples[2 * s], nb = a.samples[2 * s + 1];
+    if (threadIdx.x == 0) {
+        a.parent[sl] = kNoNode;
+        a.start[sl] = 0;
+        a.end[sl] = -1;
+        a.base[sl] = (uint32_t)(sl * a.K);
+    }
+    for (int x = threadIdx.x; x < T; x += blockDim.x) {
+        const uint32_t id = a.id1 + (uint32_t)(sl * T + x);
+        const int p = x / 3;
+        a.parent[id] = (uint32_t)sl;
+        a.start[id] = (uint32_t)p | ((uint32_t)tree_alt_state(sigma_at(na, nb, p), x - 3 * p) << 8);
+        a.end[id] = a.e1[(size_t)sl * T + x];
+    }
+    int* e2 = a.e2 + (size_t)sl * T * T;
+    const uint32_t first = a.id2 + (uint32_t)sl * (uint32_t)a.n2max;
+    int carry = 0;
+    for (int q0 = 0; q0 < T * T; q0 += 512 * 4) {
+        int e[4], cnt = 0;
+        #pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int q = q0 + 4 * (int)threadIdx.x + k;
+            e[k] = q < T * T ? e2[q] : -1;
+            cnt += e[k] >= 0;
+        }
+        int tot;
+        int at = carry + block_excl(cnt, sh, &tot);
+        carry += tot;
+        #pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (e[k] < 0) continue;
+            const int q = q0 + 4 * (int)threadIdx.x + k;
+            const int x1 = q / T, x2 = q - x1 * T, p = x2 / 3;
+            const uint32_t id = first + (uint32_t)at;
+            a.parent[id] = a.id1 + (uint32_t)(sl * T + x1);
+            a.start[id] = (uint32_t)p | ((uint32_t)tree_alt_state(sigma_at(na, nb, p), x2 - 3 * p) << 8);
+            a.end[id] = e[k];
+            e2[q] = at++;
+        }
+    }
+    if (threadIdx.x == 0) a.n2[sl] = carry;
+}
+
+// rows -> (sample, row of the sample, batch row); false past the end
+__device__ __forceinline__ bool tree_row(const TreeArgs& a, int64_t& s, int64_t& r, int64_t& g)
+{
+    __shared__ int64_t s_s;
+    const int64_t b = a.chunk_base[a.s0] + blockIdx.x;
+    if (threadIdx.x == 0) s_s = tree_sample(a, b);
+    __syncthreads();
+    s = s_s;
+    if (s < 0) return false;
+    r = (b - a.chunk_base[s]) * kTreeRows + threadIdx.x;
+    g = a.row_base[s] - a.row_base[a.s0] + r;
+    return r < a.row_base[s + 1] - a.row_base[s];
+}
+
+// third changes
+__global__ void __launch_bounds__(kTreeRows) k_tree_bits(TreeArgs a)
+{
+    int64_t s, r, g;
+    if (!tree_row(a, s, r, g)) return;
+    const TreeWord w = tree_unpack(a.word[g]);
+    if (w.c < (a.full ? 3 : 4)) return;
+    const int T = 3 * a.K, sl = (int)(s - a.s0);
+    const int i2 = a.e2[((size_t)sl * T + w.x[0]) * T + w.x[1]];
+    uint32_t* bits = a.bits + ((size_t)sl * a.n2max + i2) * a.W + (w.x[2] >> 5);
+    const uint32_t m = 1u << (w.x[2] & 31);
+    if (!(*(volatile uint32_t*)bits & m)) atomicOr(bits, m);
+}
+
+// One block per sample: ranks of the third changes' bits, the three-change nodes.
+__global__ void __launch_bounds__(512) k_tree_three(TreeArgs a)
+{
+    __shared__ int sh[16];
+    const int sl = blockIdx.x;
+    const int64_t s = a.s0 + sl;
+    const uint64_t na = a.samples[2 * s], nb = a.samples[2 * s + 1];
+    const int words = a.n2[sl] * a.W;
+    const uint32_t* bits = a.bits + (size_t)sl * a.n2max * a.W;
+    uint32_t* base = a.bits_base + (size_t)sl * a.n2max * a.W;
+    const uint32_t first = a.id3 + (uint32_t)(a.row_base[s] - a.row_base[a.s0]);
+    int carry = 0;
+    for (int q0 = 0; q0 < words; q0 += 512) {
+        const int q = q0 + threadIdx.x;
+        uint32_t m = q < words ? bits[q] : 0u;
+        int tot;
+        int at = carry + block_excl(__popc(m), sh, &tot);
+        carry += tot;
+        if (q < words) base[q] = (uint32_t)at;
+        const int i2 = q / a.W, x0 = (q - i2 * a.W) * 32;
+        while (m) {
+            const int x = x0 + __ffs((int)m) - 1, p = x / 3;
+            m &= m - 1;
+            const uint32_t id = first + (uint32_t)at++;
+            a.parent[id] = a.id2 + (uint32_t)sl * (uint32_t)a.n2max + (uint32_t)i2;
+            a.start[id] = (uint32_t)p | ((uint32_t)tree_alt_state(sigma_at(na, nb, p), x - 3 * p) << 8);
+            a.end[id] = -1;
+        }
+    }
+    if (threadIdx.x == 0) a.n3[sl] = carry;
+}
+
+// The node each row ends on, the levels three-change nodes are needed to, and
+// (full form) the four-change rows' own nodes.
+__global__ void __launch_bounds__(kTreeRows) k_tree_rows(TreeArgs a)
+{
+    int64_t s, r, g;
+    if (!tree_row(a, s, r, g)) return;
+    const TreeWord w = tree_unpack(a.word[g]);
+    const int T = 3 * a.K, sl = (int)(s - a.s0);
+    const int depth = a.full ? w.c : w.c - 1;             // changes of the node the row ends on
+    uint32_t id1 = depth <= 0 ? (uint32_t)sl : a.id1 + (uint32_t)(sl * T + w.x[0]);
+    uint32_t node = id1;
+    if (depth >= 2) {
+        const int i2 = a.e2[((size_t)sl * T + w.x[0]) * T + w.x[1]];
+        node = a.id2 + (uint32_t)sl * (uint32_t)a.n2max + (uint32_t)i2;
+        if (depth >= 3) {
+            const size_t q = ((size_t)sl * a.n2max + i2) * a.W + (w.x[2] >> 5);
+            const uint32_t below = a.bits[q] & ((1u << (w.x[2] & 31)) - 1u);
+            node = a.id3 + (uint32_t)(a.row_base[s] - a.row_base[a.s0]) + a.bits_base[q] + (uint32_t)__popc(below);
+            const int n3 = w.c == 4 ? w.x[3] / 3 - 1 : a.K - 1;
+            int* e3 = a.end + node;
+            if (*(volatile int*)e3 < n3) atomicMax(e3, n3);
+        }
+    }
+    if (a.full) {
+        const uint32_t id = a.id4 + (uint32_t)g;
+        if (depth == 4) {
+            const int p = w.x[3] / 3;
+            const uint64_t na = a.samples[2 * s], nb = a.samples[2 * s + 1];
+            a.parent[id] = node;
+            a.start[id] = (uint32_t)p | ((uint32_t)tree_alt_state(sigma_at(na, nb, p), w.x[3] - 3 * p) << 8);
+            a.end[id] = a.K - 1;
+            node = id;
+        } else {
+            a.end[id] = -1;
+        }
+    }
+    a.rnode[g] = node;
+}
+
+// the q-th node slot of a sample (one-, two-, three-, then four-change)
+struct TreeSlots {
+    int T, n2, n3, rows;
+    uint32_t f1, f2, f3, f4;
+    __device__ TreeSlots(const TreeArgs& a, int sl)
+    {
+        const int64_t s = a.s0 + sl;
+        const uint32_t rb = (uint32_t)(a.row_base[s] - a.row_base[a.s0]);
+        T = 3 * a.K;
+        n2 = a.n2[sl];
+        n3 = a.n3[sl];
+        rows = a.full ? (int)(a.row_base[s + 1] - a.row_base[s]) : 0;
+        f1 = a.id1 + (uint32_t)(sl * T);
+        f2 = a.id2 + (uint32_t)sl * (uint32_t)a.n2max;
+        f3 = a.id3 + rb;
+        f4 = a.id4 + rb;
+    }
+    __device__ int total() const { return T + n2 + n3 + rows; }
+    __device__ uint32_t id(int q) const
+    {
+        if (q < T) return f1 + (uint32_t)q;
+        q -= T;
+        if (q < n2) return f2 + (uint32_t)q;
+        q -= n2;
+        return q < n3 ? f3 + (uint32_t)q : f4 + (uint32_t)(q - n3);
+    }
+};
+
+// One block per sample: pool rows (relative) of its nodes, their number, and
+// the nodes per (level, local state): those that start there with their new
+// state, the others with n's.
+__global__ void __launch_bounds__(512) k_tree_count(TreeArgs a)
+{
+    __shared__ int sh[16];
+    __shared__ int s_cnt[4 * kMaxOrb], s_diff[kMaxOrb + 1];
+    const int sl = blockIdx.x, K = a.K;
+    const int64_t s = a.s0 + sl;
+    for (int q = threadIdx.x; q < 4 * K; q += blockDim.x) s_cnt[q] = 0;
+    for (int q = threadIdx.x; q <= K; q += blockDim.x) s_diff[q] = 0;
+    __syncthreads();
+    const TreeSlots sl_(a, sl);
+    const int n = sl_.total();
+    int carry = 0;
+    for (int q0 = 0; q0 < n; q0 += 512) {
+        const int q = q0 + threadIdx.x;
+        int len = 0;
+        uint32_t id = 0;
+        if (q < n) {
+            id = sl_.id(q);
+            const uint32_t st = a.start[id];
+            const int p = (int)(st & 255u), e = a.end[id];
+            if (e >= p) {
+                len = e - p + 1;
+                atomicAdd(&s_cnt[4 * p + (int)(st >> 8)], 1);
+                if (e > p) { atomicAdd(&s_diff[p + 1], 1); atomicAdd(&s_diff[e + 1], -1); }
+            }
+        }
+        int tot;
+        const int at = carry + block_excl(len, sh, &tot);
+        carry += tot;
+        if (len) a.base[id] = (uint32_t)at;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        a.pool_tot[sl] = carry;
+        const uint64_t na = a.samples[2 * s], nb = a.samples[2 * s + 1];
+        int alive = 0;
+        for (int t = 0; t < K; ++t) {
+            alive += s_diff[t];
+            s_cnt[4 * t + sigma_at(na, nb, t)] += alive;
+        }
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < 4 * K; q += blockDim.x) a.level_cnt[(size_t)q * a.nb + sl] = s_cnt[q];
+}
+
+// One block per sample: absolute pool rows, and the items of every level. A
+// warp walks its nodes' levels together: one atomic per level and local state.
+__global__ void __launch_bounds__(512) k_tree_items(TreeArgs a)
+{
+    __shared__ uint32_t cur[4 * kMaxOrb];
+    const int sl = blockIdx.x, K = a.K;
+    const int lane = threadIdx.x & 31;
+    const int64_t s = a.s0 + sl;
+    const uint64_t na = a.samples[2 * s], nb = a.samples[2 * s + 1];
+    for (int q = threadIdx.x; q < 4 * K; q += blockDim.x) cur[q] = (uint32_t)a.level_off[(size_t)q * a.nb + sl];
+    __syncthreads();
+    const TreeSlots sl_(a, sl);
+    const int n = sl_.total();
+    const uint32_t pool = a.pool0 + (uint32_t)a.pool_tot[sl];
+    for (int q0 = (int)(threadIdx.x & ~31u); q0 < n; q0 += blockDim.x) {
+        const int q = q0 + lane;
+        uint32_t id = 0;
+        int p = kMaxOrb, e = -1, nw = 0;
+        if (q < n) {
+            id = sl_.id(q);
+            const uint32_t st = a.start[id];
+            const int en = a.end[id];
+            if (en >= (int)(st & 255u)) {
+                p = (int)(st & 255u);
+                e = en;
+                nw = (int)(st >> 8);
+                a.base[id] += pool;
+            }
+        }
+        const int t0 = __reduce_min_sync(kFull, p), t1 = __reduce_max_sync(kFull, e);
+        for (int t = t0; t <= t1; ++t) {
+            const bool on = t >= p && t <= e;
+            const int sg = t == p ? nw : sigma_at(na, nb, t);
+            #pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                const unsigned bal = __ballot_sync(kFull, on && sg == g);
+                if (!bal) continue;
+                uint32_t at = 0;
+                if (lane == __ffs((int)bal) - 1) at = atomicAdd(&cur[4 * t + g], (uint32_t)__popc(bal));
+                at = __shfl_sync(kFull, at, __ffs((int)bal) - 1);
+                if (on && sg == g) a.items[at + (uint32_t)__popc(bal & ((1u << lane) - 1u))] = id;
+            }
+        }
+    }
+}
+
+__global__ void k_tree_row_counts(const int64_t* det, const int64_t* draw, int64_t n, int64_t* cnt)
+{
+    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s < n) cnt[s] = det[s] + (draw ? draw[s] : 0);
+}
+
+// pool row of vertex j's state seen from `node` (the node or an ancestor of it
+// that lived at level j)
+__device__ __forceinline__ uint32_t tree_source(const uint32_t* __restrict__ parent, const uint32_t* __restrict__ start,
+                                                const uint32_t* __restrict__ base, uint32_t node, int j)
+{
+    int p = (int)(__ldg(start + node) & 255u);
+    while (p > j) {
+        node = __ldg(parent + node);
+        const uint32_t st = __ldg(start + node);
+        p = (int)(st & 255u);
+    }
+    return __ldg(base + node) + (uint32_t)(j - p);
+}
+
+// 2^d as a double, 0 below the normal range (d <= 0)
+__device__ __forceinline__ double pow2_neg64(int d)
+{
+    return d >= -1022 ? __longlong_as_double((long long)(1023 + d) << 52) : 0.0;
+}
+
+}  // namespace
+
+int launch_tree_row_counts(const int64_t* det_cnt, const int64_t* draw_cnt, int64_t Ns, int64_t* cnt, cudaStream_t st)
+{
+    if (Ns == 0) return 0;
+    k_tree_row_counts<<<(unsigned)((Ns + 255) / 256), 256, 0, st>>>(det_cnt, draw_cnt, Ns, cnt);
+    return 1;
+}
+
+int launch_tree_nodes(const TreeArgs& a, int64_t max_chunks, cudaStream_t st)
+{
+    const size_t T = (size_t)3 * a.K;
+    cudaMemsetAsync(a.e1, 0xff, a.nb * T * 4, st);
+    cudaMemsetAsync(a.e2, 0xff, a.nb * T * T * 4, st);
+    cudaMemsetAsync(a.bits, 0, (size_t)a.nb * a.n2max * a.W * 4, st);
+    if (max_chunks > 0) k_tree_mark<<<(unsigned)max_chunks, kTreeRows, 0, st>>>(a);
+    k_tree_two<<<a.nb, 512, 0, st>>>(a);
+    if (max_chunks > 0) k_tree_bits<<<(unsigned)max_chunks, kTreeRows, 0, st>>>(a);
+    k_tree_three<<<a.nb, 512, 0, st>>>(a);
+    if (max_chunks > 0) k_tree_rows<<<(unsigned)max_chunks, kTreeRows, 0, st>>>(a);
+    k_tree_count<<<a.nb, 512, 0, st>>>(a);
+    return max_chunks > 0 ? 6 : 3;
+}
+
+int launch_tree_items(const TreeArgs& a, cudaStream_t st)
+{
+    k_tree_items<<<a.nb, 512, 0, st>>>(a);
+    return 1;
+}
+
+// ---------------------------------------------------------------------------
+// FP64 states of a graph ansatz, one vertex of the nodes of a group
+// ---------------------------------------------------------------------------
+
+namespace {
+
+struct TreeGroups {
+    int64_t b[5];             // item bounds of the four local states
+    int tile[5];              // their tiles
+};
+
+// A tile of IT items: per in-edge the sources' vectors in shared memory, a
+// column for four items per thread (the matrix entries come through L1, one
+// load per four FMAs; FP64 at 2 lanes per clock and SM bounds this), the edges'
+// sums aligned by powers of two, one warp per item renormalising.
+__global__ void __launch_bounds__(256) k_tree_graph64(TreeGraph64 a, int t, TreeGroups gr, int IT)
+{
+    extern __shared__ double sm[];
+    __shared__ uint32_t s_src[32];
+    __shared__ int s_ex[32], s_er[32];
+    __shared__ uint32_t s_node[32];
+    const int D = a.an.D;
+    double* xs = sm;                                  // [IT][D] sources, then the sums
+    int g = 0;
+    while (g < 3 && (int)blockIdx.x >= gr.tile[g + 1]) ++g;
+    const int64_t i0 = gr.b[g] + (int64_t)(blockIdx.x - gr.tile[g]) * IT;
+    const int n = (int)(gr.b[g + 1] - i0 < IT ? gr.b[g + 1] - i0 : IT);
+    const int e0 = a.an.pred_ptr[t], e1 = a.an.pred_ptr[t + 1];
+    if ((int)threadIdx.x < n) {
+        const uint32_t node = a.items[i0 + threadIdx.x];
+        s_node[threadIdx.x] = node;
+        int er = -1000000;
+        for (int e = e0; e < e1; ++e) {
+            const int j = a.an.pred_idx[e];
+            const int ej = j < 0 ? 0 : a.pool_e[tree_source(a.parent, a.start, a.base, node, j)];
+            er = ej > er ? ej : er;
+        }
+        s_er[threadIdx.x] = er;
+    }
+    // (group of four items, column) tasks of this thread
+    const int tasks = (IT / 4) * D;
+    double y[2][4];
+    #pragma unroll
+    for (int u = 0; u < 2; ++u)
+        #pragma unroll
+        for (int v = 0; v < 4; ++v) y[u][v] = 0.0;
+    for (int e = e0; e < e1; ++e) {
+        const int j = a.an.pred_idx[e];
+        const double* AT = a.an.AT + ((size_t)e * 4 + g) * D * D;
+        __syncthreads();
+        if (j >= 0) {
+            if ((int)threadIdx.x < n) {
+                const uint32_t r = tree_source(a.parent, a.start, a.base, s_node[threadIdx.x], j);
+                s_src[threadIdx.x] = r;
+                s_ex[threadIdx.x] = a.pool_e[r];
+            }
+            __syncthreads();
+            for (int q = threadIdx.x; q < n * D; q += 256) {
+                const int it = q / D, c = q - it * D;
+                xs[q] = a.pool[(size_t)s_src[it] * D + c];
+            }
+            __syncthreads();
+        }
+        #pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int q = threadIdx.x + 256 * u;
+            if (q >= tasks) continue;
+            const int it = 4 * (q / D), c = q - (it >> 2) * D;
+            if (it >= n) continue;
+            double acc[4] = {0.0, 0.0, 0.0, 0.0};
+            if (j < 0) {
+                const double m = __ldg(AT + c);
+                for (int v = 0; v < 4; ++v) acc[v] = m;
+            } else {
+                // (the tile's rows past n hold older numbers: their sums are not stored)
+                const double* x = xs + (size_t)it * D;
+                for (int k = 0; k < D; ++k) {
+                    const double m = __ldg(AT + (size_t)k * D + c);
+                    #pragma unroll
+                    for (int v = 0; v < 4; ++v) acc[v] = fma(m, x[v * D + k], acc[v]);
+                }
+            }
+            #pragma unroll
+            for (int v = 0; v < 4; ++v)
+                if (it + v < n) y[u][v] += acc[v] * pow2_neg64((j < 0 ? 0 : s_ex[it + v]) - s_er[it + v]);
+        }
+    }
+    __syncthreads();
+    #pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int q = threadIdx.x + 256 * u;
+        if (q >= tasks) continue;
+        const int it = 4 * (q / D), c = q - (it >> 2) * D;
+        #pragma unroll
+        for (int v = 0; v < 4; ++v)
+            if (it + v < n) xs[(size_t)(it + v) * D + c] = y[u][v];
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int it = threadIdx.x >> 5; it < n; it += 8) {
+        const double* v = xs + (size_t)it * D;
+        double m = 0.0;
+        for (int c = lane; c < D; c += 32) m = fmax(m, fabs(v[c]));
+        m = warp_max_f64(m);
+        int ex = 0;
+        if (m != 0.0) frexp(m, &ex);
+        const uint32_t node = s_node[it];
+        const uint32_t row = a.base[node] + (uint32_t)(t - (int)(a.start[node] & 255u));
+        for (int c = lane; c < D; c += 32) a.pool[(size_t)row * D + c] = ldexp(v[c], -ex);
+        if (lane == 0) a.pool_e[row] = s_er[it] + ex;
+    }
+}
+
+}  // namespace
+
+int launch_tree_graph64(const TreeGraph64& a, int t, const int64_t* bounds, cudaStream_t st)
+{
+    const int D = a.an.D;
+    // at most two (four items, column) tasks per thread
+    int IT = 2048 / D / 4 * 4;
+    IT = IT < 4 ? 4 : (IT > 32 ? 32 : IT);
+    TreeGroups g;
+    g.tile[0] = 0;
+    for (int k = 0; k < 5; ++k) g.b[k] = bounds[4 * t + k];
+    for (int k = 0; k < 4; ++k) g.tile[k + 1] = g.tile[k] + (int)((g.b[k + 1] - g.b[k] + IT - 1) / IT);
+    if (g.tile[4] == 0) return 0;
+    k_tree_graph64<<<(unsigned)g.tile[4], 256, (size_t)IT * D * 8, st>>>(a, t, g, IT);
+    return 1;
+}
+
+// ---------------------------------------------------------------------------
+// Closing covectors. With the linear readout psi is linear in the states of the
+// vertices below q given the local states from q on: for m equal to n above q
+// and local state s at q,
+//   psi(m) = sum_{j < q} h_j . [ sum_{e: j->i, i > q} M_e^{s_i(n) T} g_i(n)
+//                               + sum_{e: j->q} M_e^{s T} g_q(n) ] + e_0 sources,
+// g_i(n) = d psi / d h_i at n's states above (the adjoints). One block per
+// (sample, q).
+// ---------------------------------------------------------------------------
+
+namespace {
+
+// z[c] += 2^? M^T g in shared memory with a running power of two (block-wide)
+__device__ void close_add(double* z, int* zx, const double* M, const double* g, int gx, int D, bool first)
+{
+    const int e = first ? gx : (*zx > gx ? *zx : gx);
+    const double fz = first ? 0.0 : pow2_neg64(*zx - e), fg = pow2_neg64(gx - e);
+    for (int c = threadIdx.x; c < D; c += blockDim.x) {
+        double acc = 0.0;
+        for (int r = 0; r < D; ++r) acc = fma(g[r], __ldg(M + (size_t)r * D + c), acc);
+        z[c] = (first ? 0.0 : z[c] * fz) + acc * fg;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) *zx = e;
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(64) k_tree_close(TreeClose a)
+{
+    extern __shared__ double sm[];
+    __shared__ int zx, cx;
+    __shared__ double cv;
+    const AnsatzView& an = a.an;
+    const int K = an.K, D = an.D;
+    double* z = sm;                                   // n's part of the current j
+    double* g = sm + D;                               // an adjoint
+    const int sl = blockIdx.x / K, q = blockIdx.x - sl * K;
+    const int64_t s = a.s0 + sl;
+    const uint64_t na = a.samples[2 * s], nb = a.samples[2 * s + 1];
+    const int own = sigma_at(na, nb, q);
+    auto load_g = [&](int i) {
+        __syncthreads();
+        for (int c = threadIdx.x; c < D; c += blockDim.x) g[c] = a.Gst[((size_t)s * K + i) * D + c];
+        __syncthreads();
+        return a.Gexp[(size_t)s * K + i];
+    };
+    for (int lj = a.live_ptr[q]; lj < a.live_ptr[q + 1]; ++lj) {
+        const int j = a.live_idx[lj];
+        bool first = true;
+        for (int i = q + 1; i < K; ++i)
+            for (int e = an.pred_ptr[i]; e < an.pred_ptr[i + 1]; ++e) {
+                if (an.pred_idx[e] != j) continue;
+                const int gx = load_g(i);
+                close_add(z, &zx, an.A + ((size_t)e * 4 + sigma_at(na, nb, i)) * D * D, g, gx, D, first);
+                first = false;
+            }
+        for (int alt = 0; alt < 3; ++alt) {
+            const int sg = tree_alt_state(own, alt);
+            double* out = a.Q + (((size_t)sl * a.n_live + lj) * 3 + alt) * D;
+            // the alternative's part on top of n's, aligned
+            int ex = first ? -1000000 : zx;
+            for (int e = an.pred_ptr[q]; e < an.pred_ptr[q + 1]; ++e)
+                if (an.pred_idx[e] == j) { const int gx = a.Gexp[(size_t)s * K + q]; ex = gx > ex ? gx : ex; }
+            const int gx = load_g(q);
+            for (int c = threadIdx.x; c < D; c += blockDim.x) {
+                double v = first ? 0.0 : z[c] * pow2_neg64(zx - ex);
+                for (int e = an.pred_ptr[q]; e < an.pred_ptr[q + 1]; ++e) {
+                    if (an.pred_idx[e] != j) continue;
+                    const double* M = an.A + ((size_t)e * 4 + sg) * D * D;
+                    double acc = 0.0;
+                    for (int r = 0; r < D; ++r) acc = fma(g[r], __ldg(M + (size_t)r * D + c), acc);
+                    v += acc * pow2_neg64(gx - ex);
+                }
+                out[c] = v;
+            }
+            if (threadIdx.x == 0) a.Qe[((size_t)sl * a.n_live + lj) * 3 + alt] = ex;
+        }
+        __syncthreads();
+    }
+    // e_0 sources: of q with the alternative, of later vertices with n's states
+    for (int alt = 0; alt < 3; ++alt) {
+        __syncthreads();
+        if (threadIdx.x == 0) { cv = 0.0; cx = -1000000; }
+        for (int i = q; i < K; ++i)
+            for (int e = an.pred_ptr[i]; e < an.pred_ptr[i + 1]; ++e) {
+                if (an.pred_idx[e] >= 0) continue;
+                const int gx = load_g(i);
+                if (threadIdx.x < 32) {
+                    const int sg = i == q ? tree_alt_state(own, alt) : sigma_at(na, nb, i);
+                    const double* col = an.AT + ((size_t)e * 4 + sg) * D * D;      // row 0 of the transpose
+                    double acc = 0.0;
+                    for (int r = threadIdx.x; r < D; r += 32) acc = fma(g[r], __ldg(col + r), acc);
+                    acc = warp_sum_f64(acc);
+                    if (threadIdx.x == 0) {
+                        const int x = gx > cx ? gx : cx;
+                        cv = cv * pow2_neg64(cx - x) + acc * pow2_neg64(gx - x);
+                        cx = x;
+                    }
+                }
+                __syncthreads();
+            }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            a.c[((size_t)sl * K + q) * 3 + alt] = cv;
+            a.ce[((size_t)sl * K + q) * 3 + alt] = cx;
+        }
+    }
+}
+
+// x 2^e with the exponent field where the result stays normal
+__device__ __forceinline__ double scale_pow2(double x, int e)
+{
+    const long long bits = __double_as_longlong(x);
+    const int ex = (int)((bits >> 52) & 0x7FF), ne = ex + e;
+    if (ex != 0 && ex != 0x7FF && ne > 0 && ne < 0x7FF) return __longlong_as_double(bits + ((long long)e << 52));
+    return ldexp(x, e);
+}
+
+// determinant of a row from its word
+__device__ __forceinline__ void tree_det(const TreeWord& w, uint64_t na, uint64_t nb, uint64_t& ma, uint64_t& mb)
+{
+    ma = na;
+    mb = nb;
+    for (int k = 0; k < w.c; ++k) {
+        const int p = w.x[k] / 3, sg = tree_alt_state(sigma_at(na, nb, p), w.x[k] - 3 * p);
+        ma = (ma & ~(1ull << p)) | ((uint64_t)(sg & 1) << p);
+        mb = (mb & ~(1ull << p)) | ((uint64_t)(sg >> 1) << p);
+    }
+}
+
+__device__ __forceinline__ double tree_coef(const TreeArgs& t, int64_t s, int64_t r)
+{
+    const int64_t nd = t.det_cnt[s];
+    return r < nd ? t.det_coef[t.det_off[s] + r] : t.draw_coef[s * t.draw_stride + (r - nd)];
+}
+
+constexpr int kRowLanes = 8;
+
+// Rows of the FP64 graph form: eight lanes per row dot the live states of the
+// row's node with the closing covectors, then form the correlator ratio.
+__global__ void __launch_bounds__(256) k_tree_rows64(TreeRows64 a)
+{
+    __shared__ int64_t s_s;
+    __shared__ double s_term[kTreeRows];
+    __shared__ int s_span[kTreeRows], s_mv[kTreeRows];
+    const TreeArgs& t = a.t;
+    const AnsatzView& an = a.q.an;
+    const int64_t b = t.chunk_base[t.s0] + blockIdx.x;
+    if (threadIdx.x == 0) s_s = tree_sample(t, b);
+    __syncthreads();
+    const int64_t s = s_s;
+    if (s < 0) return;
+    const int K = an.K, D = an.D, sl = (int)(s - t.s0);
+    const uint64_t na = t.samples[2 * s], nb = t.samples[2 * s + 1];
+    const int64_t r0 = (b - t.chunk_base[s]) * kTreeRows, g0 = t.row_base[s] - t.row_base[t.s0] + r0;
+    const int64_t left = t.row_base[s + 1] - t.row_base[s] - r0;
+    const int nr = (int)(left < kTreeRows ? left : kTreeRows);
+    const int l8 = threadIdx.x & 7, lane = threadIdx.x & 31;
+    const double rpsi = a.psi_mant[s];
+    const int pex = a.psi_exp[s];
+    for (int rr = threadIdx.x >> 3; rr < kTreeRows; rr += 32) {      // whole warps: the shuffles need them
+        const bool on = rr < nr;
+        double tn = 0.0;
+        if (on) {
+            const TreeWord w = tree_unpack(t.word[g0 + rr]);
+            const uint32_t node = t.rnode[g0 + rr];
+            const int x = w.x[w.c - 1], q = x / 3, alt = x - 3 * q;
+            const size_t ci = ((size_t)sl * K + q) * 3 + alt;
+            const int v0 = a.q.live_ptr[q], v1 = a.q.live_ptr[q + 1];
+            int er = a.q.ce[ci];
+            for (int v = v0; v < v1; ++v) {
+                const uint32_t row = tree_source(t.parent, t.start, t.base, node, a.q.live_idx[v]);
+                const int e = a.pool_e[row] + a.q.Qe[((size_t)sl * a.q.n_live + v) * 3 + alt];
+                er = e > er ? e : er;
+            }
+            double acc = l8 == 0 ? a.q.c[ci] * pow2_neg64(a.q.ce[ci] - er) : 0.0;
+            for (int v = v0; v < v1; ++v) {
+                const uint32_t row = tree_source(t.parent, t.start, t.base, node, a.q.live_idx[v]);
+                const size_t qi = ((size_t)sl * a.q.n_live + v) * 3 + alt;
+                const double* hj = a.pool + (size_t)row * D;
+                const double* Qj = a.q.Q + qi * D;
+                double d = 0.0;
+                for (int c = l8; c < D; c += kRowLanes) d = fma(__ldg(Qj + c), hj[c], d);
+                acc = fma(d, pow2_neg64(a.pool_e[row] + a.q.Qe[qi] - er), acc);
+            }
+            tn = acc;
+            // exponent of the sum against psi(n)
+            s_span[rr] = er - pex;
+        }
+        for (int o = 4; o; o >>= 1) tn += __shfl_xor_sync(kFull, tn, o);
+        __syncwarp();
+        if (on && l8 == 0) s_term[rr] = scale_pow2(tn / rpsi, s_span[rr]);
+        __syncwarp();
+    }
+    __syncthreads();
+    // correlator ratio, one warp per row
+    for (int rr = threadIdx.x >> 5; rr < nr; rr += 8) {
+        const TreeWord w = tree_unpack(t.word[g0 + rr]);
+        uint64_t ma, mb;
+        tree_det(w, na, nb, ma, mb);
+        int neg;
+        const double lr = corr_log_ratio_warp(an, s, a.theta, a.lc, na, nb, ma, mb, lane, &neg);
+        if (lane == 0) {
+            const int p = w.x[0] / 3;
+            s_term[rr] = tree_coef(t, s, r0 + rr) * s_term[rr] * ((neg ? -1.0 : 1.0) * exp(lr));
+            s_span[rr] = K - p;
+            s_mv[rr] = graph_matvecs(an, p);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        double term = 0.0;
+        int sp = 0, mv = 0;
+        for (int rr = lane; rr < nr; rr += 32) { term += s_term[rr]; sp += s_span[rr]; mv += s_mv[rr]; }
+        term = warp_sum_f64(term);
+        sp = (int)__reduce_add_sync(kFull, (unsigned)sp);
+        mv = (int)__reduce_add_sync(kFull, (unsigned)mv);
+        if (lane == 0) {
+            a.partial[b] = term;
+            if (a.span) a.span[b] = sp;
+            if (a.mv) a.mv[b] = mv;
+        }
+    }
+}
+
+}  // namespace
+
+int launch_tree_close(const TreeClose& a, cudaStream_t st)
+{
+    k_tree_close<<<(unsigned)(a.nb * a.an.K), 64, (size_t)2 * a.an.D * 8, st>>>(a);
+    return 1;
+}
+
+int launch_tree_rows64(const TreeRows64& a, int64_t max_chunks, cudaStream_t st)
+{
+    if (max_chunks == 0) return 0;
+    k_tree_rows64<<<(unsigned)max_chunks, 256, 0, st>>>(a);
+    return 1;
+}
+
+}  // namespace nqs

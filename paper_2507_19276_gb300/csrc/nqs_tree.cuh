@@ -1,0 +1,145 @@
+// nqs_tree.cuh -- prefix trees of connected determinants (see nqs_tree.cu).
+#pragma once
+
+#include "nqs_kernels.cuh"
+
+namespace nqs {
+
+constexpr int kTreeRows = 128;            // rows per chunk of the row kernels
+
+// A row's changed sites ascending, each as x = 3 site + alternative (the
+// alternatives of a site are the three local states n does not have there, in
+// ascending order), one byte each, the last repeated up to four.
+__host__ __device__ __forceinline__ int tree_alt_state(int own, int a) { return a + (a >= own ? 1 : 0); }
+
+struct TreeArgs {
+    HamView h;
+    const uint64_t* samples;              // all samples of the call
+    int64_t s0;                           // batch = samples [s0, s0 + nb)
+    int nb;
+    int K;
+    int full;                             // 1: every row is re-run to vertex K - 1 (a row is a node
+                                          // itself); 0: a row ends on the node before its last change
+    // rows: each sample's deterministic rows, then its drawn rows
+    const uint32_t* det_rank; const int64_t* det_off; const int64_t* det_cnt; const double* det_coef;
+    const uint32_t* draw_rank; int64_t draw_stride; const int64_t* draw_cnt; const double* draw_coef;   // or NULL
+    const int64_t* row_base;              // [Ns+1] prefix of the samples' row counts
+    const int64_t* chunk_base;            // [Ns+1] prefix of their chunks of kTreeRows
+    // per batch row
+    uint32_t* word;                       // changes (see above)
+    uint32_t* rnode;                      // the node the row ends on
+    // per batch sample
+    int* e1;                              // [nb][3K] last level of the one-change nodes (-1 unused)
+    int* e2;                              // [nb][3K][3K] the same of two-change nodes, then their index
+    int* n2; int* n3;                     // [nb] two- and three-change nodes
+    uint32_t* bits;                       // [nb][n2max][W] third changes of each two-change node
+    uint32_t* bits_base;                  // [nb][n2max][W] three-change nodes before each word
+    int n2max, W;
+    // nodes: ids are roots [nb], one-change [nb][3K], two-change [nb][n2max],
+    // three-change [rows], four-change [rows] (full)
+    uint32_t id1, id2, id3, id4;          // first id of each kind
+    uint32_t* parent;
+    int* end;                             // last level the node is needed at (-1: none)
+    uint32_t* start;                      // first level | new local state << 8
+    uint32_t* base;                       // row of the state pool at level `start`
+    // levels
+    int64_t* pool_tot;                    // [nb + 1] pool rows per sample, then their prefix
+    int64_t* level_cnt;                   // [K][4][nb] nodes per (level, local state, sample)
+    int64_t* level_off;                   // their exclusive prefix (one more entry)
+    uint32_t* items;                      // node ids by (level, local state)
+    uint32_t pool0;                       // first pool row after the roots' rows [nb][K]
+};
+
+// rows of every sample (deterministic + drawn)
+int launch_tree_row_counts(const int64_t* det_cnt, const int64_t* draw_cnt, int64_t Ns, int64_t* cnt, cudaStream_t st);
+// words, marks and nodes of the batch; fills pool_tot and level_cnt
+int launch_tree_nodes(const TreeArgs& a, int64_t max_chunks, cudaStream_t st);
+// pool rows of the nodes (pool_tot scanned) and the items (level_off scanned)
+int launch_tree_items(const TreeArgs& a, cudaStream_t st);
+
+// ---- node evaluations -------------------------------------------------------
+
+// FP64 states of a graph ansatz (linear readout): one vertex of every node of
+// the items [i0, i1), whose local state there is sg.
+struct TreeGraph64 {
+    AnsatzView an;
+    const uint32_t* items;
+    const uint32_t* parent; const uint32_t* start; const uint32_t* base;
+    double* pool;                         // [rows][D]
+    int* pool_e;                          // [rows]
+};
+int launch_tree_graph64(const TreeGraph64& a, int t, const int64_t* bounds, cudaStream_t st);
+
+// Covectors that close a row at its last changed vertex: for each (q,
+// alternative a) and each vertex j < q read at or after q, Q_j with
+// psi(m) = c + sum_j Q_j . h_j(node).
+struct TreeClose {
+    AnsatzView an;
+    const uint64_t* samples; int64_t s0; int nb;
+    const double* Gst; const int* Gexp;   // adjoints of n [Ns][K][D]
+    const int* live_ptr; const int* live_idx;   // [K+1], vertices read at or after q
+    int n_live;                           // live_ptr[K]
+    double* Q; int* Qe;                   // [nb][n_live][3][D], [nb][n_live][3]
+    double* c; int* ce;                   // [nb][K][3] the e_0 sources' part
+};
+int launch_tree_close(const TreeClose& a, cudaStream_t st);
+
+struct TreeRows64 {
+    TreeArgs t;
+    TreeClose q;
+    const double* pool; const int* pool_e;
+    const double* theta; const double* lc;
+    const double* psi_mant; const int* psi_exp;
+    double* partial; int64_t* span; int64_t* mv;
+};
+int launch_tree_rows64(const TreeRows64& a, int64_t max_chunks, cudaStream_t st);
+
+// Mixed form of a graph ansatz: split-FP16 states, one vertex per launch.
+struct TreeGraphTc {
+    AnsatzView an;
+    const uint32_t* items;
+    const uint32_t* parent; const uint32_t* start; const uint32_t* base;
+    unsigned char* pool;                  // [rows][hi D | lo D] FP16
+    int* pool_e;
+    const unsigned char* bimg; const int* bexp; const float* col0;
+    float* mant; int* mexp;               // [nodes] psi_TN of the nodes of level K - 1
+    DevError* err;
+};
+int launch_tree_graph_tc(const TreeGraphTc& a, int t, int deg, const int64_t* bounds, int n_sm, cudaStream_t st);
+
+struct TreeRowsTc {
+    TreeArgs t;
+    AnsatzView an;
+    const float* mant; const int* mexp;
+    const float* tts; const float* WT; int np;
+    const double* psi_mant; const int* psi_exp;
+    double* partial; double* partial_abs; int64_t* span; int64_t* mv;
+};
+int launch_tree_rows_tc(const TreeRowsTc& a, int64_t max_chunks, cudaStream_t st);
+// split images and exponents of the roots' states into the pool, tanh theta
+int launch_tree_graph_prep(const double* Hst, const int* Hexp, const double* theta, int64_t s0, int nb, int K, int D,
+                           int NH, int NP, int corr, unsigned char* pool, int* pool_e, float* tts, cudaStream_t st);
+
+// Normalised readout on a chain: the nodes' running cell, weight and sign
+// (two buffers by level parity).
+struct TreeRnn {
+    AnsatzView an;
+    TreeArgs t;
+    const double* cells;                  // n's cells [Ns][K][D]
+    double* cell;                         // [2][nodes][D]
+    double* prod;                         // [2][nodes] prod P / Z = prod * 2^pex since the first change
+    int* pex;                             // [2][nodes]
+    uint32_t* flag;                       // [2][nodes] N_alpha | N_beta << 8 | odd << 16 | dead << 17
+    uint32_t n_nodes;
+};
+int launch_tree_rnn(const TreeRnn& a, int t, const int64_t* bounds, int n_sm, cudaStream_t st);
+
+struct TreeRowsRnn {
+    TreeRnn r;
+    const double* lp; const int8_t* sg;
+    const double* theta; const double* lc;
+    double* partial; int64_t* span;
+};
+int launch_tree_rows_rnn(const TreeRowsRnn& a, int64_t max_chunks, cudaStream_t st);
+
+}  // namespace nqs

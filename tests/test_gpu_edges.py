@@ -88,3 +88,41 @@ def test_sampler_sizes(ctx, n, graph):
     ref, ref_c, _ = O.sample(O.Problem(s), n, 11 + n)
     assert counts.sum() == n
     assert np.array_equal(dets, ref) and np.array_equal(counts, ref_c)
+
+
+def _dag(seed, K, D, n_hidden=4, n_samples=None, eps=0.0, n_draws=0):
+    """A graph system whose edges skip vertices: e_0 sources in the middle, a
+    vertex nothing reads, repeated sources."""
+    import dataclasses
+    rng = np.random.default_rng(seed)
+    s = W.tiny_system(K=K, na=K // 2, nb=(K + 1) // 2, D=D, n_hidden=n_hidden, seed=seed, eps=eps, n_draws=n_draws,
+                      n_samples=n_samples)
+    ptr, idx = [0], []
+    for i in range(K):
+        src = [-1] if i == 0 else sorted(rng.integers(-1, i, size=rng.integers(1, 4)).tolist())
+        if i == K - 1:
+            src = sorted(set(src + [i - 1, max(0, i - 3)]))
+        idx += src
+        ptr.append(len(idx))
+    T = rng.normal(size=(len(idx), 4, D, D)) / np.sqrt(D) + 0.3 * np.eye(D)
+    return dataclasses.replace(s, pred_ptr=np.array(ptr, np.int32), pred_idx=np.array(idx, np.int32),
+                               tensors=np.ascontiguousarray(T))
+
+
+@pytest.mark.parametrize("seed,K,D,ns,eps,draws", [
+    (1, 7, 5, None, 0.0, 0), (2, 7, 33, 40, 0.05, 50), (3, 5, 1, None, 0.0, 0), (4, 9, 8, 300, 1e3, 200),
+    (5, 6, 130, 7, 0.0, 0), (6, 8, 16, 1, 0.02, 7), (7, 2, 4, None, 0.0, 0)])
+def test_graph_prefix_tree_fp64(ctx, seed, K, D, ns, eps, draws):
+    """FP64 form of graphs over the prefix trees: tiles and remainders of every
+    kind, drawn rows alone (eps above every element), against the oracle within
+    the FP64 bar of the other parity tests."""
+    from oracle import oracle as O
+    s = _dag(seed, K, D, n_samples=ns, eps=eps, n_draws=draws)
+    ctx.set_system(s)
+    ctx.set_precision(nqs.NQS_PREC_FP64)
+    ref = O.local_energy(O.Problem(s), cond=True)
+    ok = np.isfinite(ref["e_loc"])
+    e, summ = ctx.local_energy(s.samples, s.counts, s.eps, s.n_draws, s.seed)
+    scale = np.maximum(np.abs(ref["e_loc"]), ref["e_abs"]) + (2.0 ** -52 / 1e-12) * ref["e_cond"]
+    assert np.all(np.abs(e - ref["e_loc"])[ok] <= 1e-12 * scale[ok])
+    assert summ["n_det"] == int(ref["n_det"].sum())
