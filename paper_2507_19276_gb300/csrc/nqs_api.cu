@@ -87,8 +87,7 @@ struct nqs_ctx {
     // mixed form of the graph ansatz: matrix images, e_0 columns, state slots
     DevBuf g_img, g_bexp, g_col0, g_slot, g_last, mv_det, mv_draw, g_simg, g_tts, g_rank, g_coef;
     // prefix trees (graphs, the normalised chain readout)
-    DevBuf tr_rows, tr_build, tr_items, tr_pool, tr_close, g_live;
-    std::vector<int> pred_ptr_h, pred_idx_h;
+    DevBuf tr_rows, tr_build, tr_items, tr_pool, tr_close, g_live, cexp, corr_ab;
     int n_live = 0;           // entries of g_live past its K + 1 offsets
     int g_slots = 0, g_maxdeg = 0, g_nbuf = 1;
     bool has_gtc = false;
@@ -519,8 +518,6 @@ int amp_pass(nqs_ctx* c, const uint64_t* samples, int64_t Ns, RowSet rows, int64
     a.Ns = Ns;
     a.rows = rows;
     a.rows_per_block = R;
-    a.Lenv = (const double*)c->Lenv.p; a.Lexp = (const int*)c->Lexp.p;
-    a.Renv = (const double*)c->Renv.p; a.Rexp = (const int*)c->Rexp.p;
     a.Hst = (const double*)c->Hst.p; a.Hexp = (const int*)c->Hexp.p;
     a.theta = (const double*)c->theta.p;
     a.lc = (const double*)c->lc.p;
@@ -948,19 +945,28 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
                 q.ce = v.take<int>((size_t)nb * K * 3);
                 if (!pass) TRY(ensure(c, c->tr_close, v.n));
             }
-            CK(cudaMemcpyAsync(g.pool, (const double*)c->Hst.p + (size_t)s0 * K * D, (size_t)nb * K * D * 8,
-                               cudaMemcpyDeviceToDevice, c->stream));
-            CK(cudaMemcpyAsync(g.pool_e, (const int*)c->Hexp.p + (size_t)s0 * K, (size_t)nb * K * 4,
-                               cudaMemcpyDeviceToDevice, c->stream));
+            // the roots' states h_j(n): a chain keeps L_{j+1} behind L_0 and R_{i+1} as g_i
+            const bool chain = c->av.chain != 0;
+            const size_t srow = (size_t)K + (chain ? 1 : 0);
+            const double* h0 = chain ? (const double*)c->Lenv.p + D : (const double*)c->Hst.p;
+            const int* x0 = chain ? (const int*)c->Lexp.p + 1 : (const int*)c->Hexp.p;
+            CK(cudaMemcpy2DAsync(g.pool, (size_t)K * D * 8, h0 + (size_t)s0 * srow * D, srow * D * 8, (size_t)K * D * 8,
+                                 (size_t)nb, cudaMemcpyDeviceToDevice, c->stream));
+            CK(cudaMemcpy2DAsync(g.pool_e, (size_t)K * 4, x0 + (size_t)s0 * srow, srow * 4, (size_t)K * 4, (size_t)nb,
+                                 cudaMemcpyDeviceToDevice, c->stream));
             g.an = c->av;
+            g.an.pred_ptr = (const int*)c->pred_ptr.p;
+            g.an.pred_idx = (const int*)c->pred_idx.p;
             g.items = a.items;
             g.parent = a.parent; g.start = a.start; g.base = a.base;
             for (int t = 0; t < K; ++t) LAUNCH(stage, launch_tree_graph64(g, t, bounds.data(), c->stream));
-            q.an = c->av;
+            q.an = g.an;
             q.samples = ds;
             q.s0 = s0;
             q.nb = nb;
-            q.Gst = (const double*)c->Gst.p; q.Gexp = (const int*)c->Gexp.p;
+            q.Gst = chain ? (const double*)c->Renv.p + D : (const double*)c->Gst.p;
+            q.Gexp = chain ? (const int*)c->Rexp.p + 1 : (const int*)c->Gexp.p;
+            q.g_stride = (int)srow;
             q.live_ptr = (const int*)c->g_live.p;
             q.live_idx = q.live_ptr + K + 1;
             q.n_live = c->n_live;
@@ -968,7 +974,15 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
             TreeRows64 r{};
             r.t = a;
             r.q = q;
+            r.chain = chain ? 1 : 0;
             r.pool = g.pool; r.pool_e = g.pool_e;
+            if (NH > 0 && c->av.corr == NQS_CORR_COSH) {
+                TRY(ensure(c, c->corr_ab, (size_t)nb * NH * 16));
+                LAUNCH(stage, launch_corr_ab((const double*)c->theta.p + (size_t)s0 * NH, (int64_t)nb * NH,
+                                             (double2*)c->corr_ab.p, c->stream));
+                r.expd = (const double2*)c->cexp.p;
+                r.ab = (const double2*)c->corr_ab.p;
+            }
             r.theta = (const double*)c->theta.p;
             r.lc = (const double*)c->lc.p;
             r.psi_mant = (const double*)c->pmant.p;
@@ -1037,7 +1051,7 @@ extern "C" int nqs_destroy(nqs_ctx* c)
                       &c->smp_tabs, &c->smp_tree, &c->tk_rank, &c->tk_off, &c->tk, &c->g_img, &c->g_bexp,
                       &c->g_col0, &c->g_slot, &c->g_last, &c->mv_det, &c->mv_draw, &c->g_simg,
                       &c->g_tts, &c->g_rank, &c->g_coef, &c->tr_rows, &c->tr_build, &c->tr_items,
-                      &c->tr_pool, &c->tr_close, &c->g_live};
+                      &c->tr_pool, &c->tr_close, &c->g_live, &c->cexp, &c->corr_ab};
     for (DevBuf* b : more) release(*b);
     for (auto* v : {&c->smp_pa, &c->smp_pb, &c->smp_off, &c->smp_cnt, &c->smp_par, &c->smp_cell})
         for (DevBuf& b : *v) release(b);
@@ -1225,11 +1239,32 @@ extern "C" int nqs_set_ansatz(nqs_ctx* c, const double* site_tensors, int n_edge
     TRY(ensure(c, c->Af, nt * 4));
     TRY(ensure(c, c->ATf, nt * 4));
     CK(cudaMemcpyAsync(c->A.p, site_tensors, nt * 8, cudaMemcpyDefault, c->stream));
-    if (!chain) {
-        TRY(ensure(c, c->pred_ptr, (K + 1) * 4));
-        TRY(ensure(c, c->pred_idx, (size_t)n_edges * 4));
-        CK(cudaMemcpyAsync(c->pred_ptr.p, ptr.data(), (K + 1) * 4, cudaMemcpyHostToDevice, c->stream));
-        CK(cudaMemcpyAsync(c->pred_idx.p, idx.data(), (size_t)n_edges * 4, cudaMemcpyHostToDevice, c->stream));
+    if (chain) {
+        // a chain's edge lists, for the kernels that take any graph
+        ptr.resize(K + 1);
+        idx.resize(K);
+        for (int i = 0; i < K; ++i) { ptr[i] = i; idx[i] = i - 1; }
+        ptr[K] = K;
+    }
+    TRY(ensure(c, c->pred_ptr, (K + 1) * 4));
+    TRY(ensure(c, c->pred_idx, (size_t)n_edges * 4));
+    CK(cudaMemcpyAsync(c->pred_ptr.p, ptr.data(), (K + 1) * 4, cudaMemcpyHostToDevice, c->stream));
+    CK(cudaMemcpyAsync(c->pred_idx.p, idx.data(), (size_t)n_edges * 4, cudaMemcpyHostToDevice, c->stream));
+    {
+        // per vertex q, the earlier vertices whose states q or a later vertex reads
+        std::vector<int> lp((size_t)K + 1, 0), li;
+        for (int q = 0; q < K; ++q) {
+            for (int j = 0; j < q; ++j) {
+                bool live = false;
+                for (int e = ptr[q]; e < n_edges && !live; ++e) live = idx[e] == j;
+                if (live) li.push_back(j);
+            }
+            lp[(size_t)q + 1] = (int)li.size();
+        }
+        lp.insert(lp.end(), li.begin(), li.end());
+        TRY(ensure(c, c->g_live, lp.size() * 4));
+        CK(cudaMemcpyAsync(c->g_live.p, lp.data(), lp.size() * 4, cudaMemcpyHostToDevice, c->stream));
+        c->n_live = (int)li.size();
     }
     AnsatzForms fm{};
     fm.D = D;
@@ -1260,23 +1295,6 @@ extern "C" int nqs_set_ansatz(nqs_ctx* c, const double* site_tensors, int n_edge
             c->has_tc = true;
         }
     } else {
-        // per vertex q, the earlier vertices whose states q or a later vertex reads
-        std::vector<int> lp((size_t)K + 1, 0), li;
-        for (int q = 0; q < K; ++q) {
-            for (int j = 0; j < q; ++j) {
-                bool live = false;
-                for (int e = ptr[q]; e < n_edges && !live; ++e) live = idx[e] == j;
-                if (live) li.push_back(j);
-            }
-            lp[(size_t)q + 1] = (int)li.size();
-        }
-        TRY(ensure(c, c->g_live, (size_t)(K + 1 + li.size()) * 4));
-        CK(cudaMemcpyAsync(c->g_live.p, lp.data(), lp.size() * 4, cudaMemcpyHostToDevice, c->stream));
-        if (!li.empty())
-            CK(cudaMemcpyAsync((int*)c->g_live.p + K + 1, li.data(), li.size() * 4, cudaMemcpyHostToDevice, c->stream));
-        c->n_live = (int)li.size();
-        c->pred_ptr_h = ptr;
-        c->pred_idx_h = idx;
         const char* why = nullptr;
         if (graph_tc_plan(ptr.data(), idx.data(), K, D, n_hidden, gp, &why)) {
             TRY(ensure(c, c->g_img, (size_t)n_edges * 16 * D * D));
@@ -1314,6 +1332,8 @@ extern "C" int nqs_set_ansatz(nqs_ctx* c, const double* site_tensors, int n_edge
         TRY(ensure(c, c->csite64, (size_t)K * 12 * np * 32));
         LAUNCH(NQS_STAGE_OTHER, fam_corr_sites((const double*)c->W.p, K, n_hidden, (float4*)c->csite.p,
                                                (double4_32a*)c->csite64.p, c->stream));
+        TRY(ensure(c, c->cexp, (size_t)K * 12 * n_hidden * 16));
+        LAUNCH(NQS_STAGE_OTHER, launch_corr_exp((const double*)c->W.p, K, n_hidden, (double2*)c->cexp.p, c->stream));
         CK(cudaGetLastError());
     }
     AnsatzView a{};
@@ -1635,9 +1655,9 @@ int le_core(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, uint64
     const bool shared = c->av.chain && (prec == NQS_PREC_MIXED || prec == NQS_PREC_FP64_SHARED);
     const bool gtc = !c->av.chain && prec == NQS_PREC_MIXED;
     const bool graph = !c->av.chain && !rnn;
-    // psi is linear in the states of a graph without the tensor term: its rows
-    // share prefixes and close with n's adjoints (the tensor term's are re-run)
-    const bool tree64 = graph && !gtc && !c->av.tk_rank;
+    // the plain FP64 form: psi is linear in the states without the tensor term, so
+    // the rows share prefixes and close with n's adjoints (the tensor term's are re-run)
+    const bool tree64 = !rnn && !gtc && !shared && !c->av.tk_rank;
     if (!c->av.chain && prec == NQS_PREC_FP64_SHARED)
         return set_err(c, NQS_ERR_UNSUPPORTED,
                        "graph ansatze have no shared-prefix form (NQS_PREC_FP64 or NQS_PREC_MIXED)");

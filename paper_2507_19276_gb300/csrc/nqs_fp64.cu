@@ -7,10 +7,10 @@
 //
 // Environments (per sample n): left states L_t = A_t^{s_t(n)} ... A_0 l and
 // right covectors R_t = r^T A_{K-1} ... A_t (chain), forward states h_i(n) and
-// adjoints g_i(n) = d psi_TN / d h_i (graph). An amplitude psi(m) for m that
-// differs from n on sites p..q is R_{q+1} A_q^{s_q(m)} ... A_p^{s_p(m)} L_{p-1}
-// (chain), or the graph recursion re-run from the first changed vertex p with
-// the stored h_j(n), j < p.
+// adjoints g_i(n) = d psi_TN / d h_i (graph). The amplitudes of the connected m
+// continue them over prefix trees (nqs_tree.cu); with the tensor term, which is
+// not linear in the states, the recursion is re-run here from the first changed
+// vertex p with the stored h_j(n), j < p.
 #include "nqs_kernels.cuh"
 
 namespace nqs {
@@ -322,15 +322,12 @@ int launch_env_fp64(const EnvArgs& a, cudaStream_t st)
 }
 
 // ---------------------------------------------------------------------------
-// Span-limited amplitudes of the connected rows, FP64
+// Amplitudes of the connected rows of a graph with the tensor term, FP64 (the
+// other plain forms share prefixes, see nqs_tree.cu)
 // ---------------------------------------------------------------------------
 
 int amp_fp64_rows_per_block(const AnsatzView& an)
 {
-    if (an.chain) {
-        int r = 4096 / an.D;
-        return r < 4 ? 4 : (r > 64 ? 64 : r);
-    }
     // rows of the states kept in shared memory ([R][K][D] doubles): about 32 KB,
     // so that several blocks share an SM and their FMA chains overlap
     int r = 4096 / (an.K * an.D);
@@ -339,8 +336,8 @@ int amp_fp64_rows_per_block(const AnsatzView& an)
 
 size_t amp_fp64_smem(const AnsatzView& an, int R)
 {
-    size_t st = an.chain ? (size_t)2 * R * an.D : (size_t)R * an.K * an.D;
-    size_t ints = (size_t)R * (an.chain ? 1 : an.K);
+    size_t st = (size_t)R * an.K * an.D;
+    size_t ints = (size_t)R * an.K;
     ints = (ints + 1) & ~(size_t)1;                       // the tensor-term scratch after is 8-byte aligned
     return st * sizeof(double) + ints * sizeof(int) + (size_t)R * an.tk_zy * sizeof(double);
 }
@@ -370,106 +367,6 @@ __device__ double rbm_log_ratio_warp(const AnsatzView& an, int64_t s, const doub
     const double lr = corr_log_ratio_warp(an, s, theta, lc, na, nb, ma, mb, lane, &neg);
     *sign = neg ? -1.0 : 1.0;
     return lr;
-}
-
-__global__ void k_amp_chain_fp64(AmpArgs a)
-{
-    extern __shared__ double sm[];
-    __shared__ OrbLists lists;
-    __shared__ RowInfo info[64];
-    __shared__ int s_range[2];
-    const int R = a.rows_per_block, D = a.an.D;
-    const int64_t b = blockIdx.x;
-    const int64_t* cb = a.rows.chunk_base;
-    if (b >= cb[a.Ns]) return;
-    const int64_t s = find_sample(cb, a.Ns, b);
-    const int64_t j = b - cb[s];
-    const int64_t beg = a.rows.begin ? a.rows.begin[s] : s * a.rows.stride;
-    const int64_t cnt = a.rows.count[s];
-    const int64_t r0 = beg + j * R;
-    const int nr = (int)((cnt - j * R) < R ? (cnt - j * R) : R);
-    const uint64_t na = a.samples[2 * s], nb = a.samples[2 * s + 1];
-    double* X = sm;
-    double* Y = sm + (size_t)R * D;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    if (warp == 0) build_lists_warp(na, nb, a.h.K, lists, lane);
-    if (threadIdx.x == 0) { s_range[0] = 1 << 30; s_range[1] = -1; }
-    __syncthreads();
-    for (int r = threadIdx.x; r < nr; r += blockDim.x) {
-        const Exc e = decode_rank<false>(a.h, lists, a.rows.rank[r0 + r]);   // sites only
-        uint64_t ma = na, mb = nb;
-        flip(ma, mb, e.i); flip(ma, mb, e.a);
-        if (e.kind == 2) { flip(ma, mb, e.j); flip(ma, mb, e.b); }
-        const uint64_t ch = (na ^ ma) | (nb ^ mb);
-        RowInfo ri;
-        ri.ma = ma; ri.mb = mb;
-        ri.coef = a.rows.coef[r0 + r];
-        ri.tn = 0.0;
-        ri.p = __ffsll((long long)ch) - 1;
-        ri.q = 63 - __clzll((long long)ch);
-        ri.ex = 0;
-        info[r] = ri;
-        atomicMin(&s_range[0], ri.p);
-        atomicMax(&s_range[1], ri.q);
-    }
-    __syncthreads();
-    const int tmin = s_range[0], tmax = s_range[1];
-    const double mant_n = a.psi_mant[s];
-    const int exp_n = a.psi_exp[s];
-    const int K = a.an.K;
-    const double* Ls = a.Lenv + (size_t)s * (K + 1) * D;
-    const double* Rs = a.Renv + (size_t)s * (K + 1) * D;
-    for (int t = tmin; t <= tmax; ++t) {
-        // rows entering at t start from L_{t-1}(n)
-        for (int q = threadIdx.x; q < nr * D; q += blockDim.x) {
-            const int r = q / D, c = q - r * D;
-            if (info[r].p == t) X[(size_t)r * D + c] = Ls[(size_t)t * D + c];
-        }
-        for (int r = threadIdx.x; r < nr; r += blockDim.x)
-            if (info[r].p == t) info[r].ex = a.Lexp[(size_t)s * (K + 1) + t];
-        __syncthreads();
-        for (int q = threadIdx.x; q < nr * D; q += blockDim.x) {
-            const int r = q / D, c = q - r * D;
-            if (t < info[r].p || t > info[r].q) continue;
-            const double* AT = tens(a.an.AT, t, sigma_at(info[r].ma, info[r].mb, t), D);
-            const double* x = X + (size_t)r * D;
-            const double acc = dot_col4(AT, x, D, c);
-            Y[(size_t)r * D + c] = acc;
-        }
-        __syncthreads();
-        for (int r = warp; r < nr; r += nw) {
-            if (t < info[r].p || t > info[r].q) continue;
-            double* y = Y + (size_t)r * D;
-            const int e = warp_renorm(y, D, lane);
-            const int exn = info[r].ex + e;
-            __syncwarp();
-            for (int c = lane; c < D; c += 32) X[(size_t)r * D + c] = y[c];
-            if (lane == 0) info[r].ex = exn;
-            if (t == info[r].q) {
-                double dot = 0.0;
-                for (int c = lane; c < D; c += 32) dot = fma(Rs[(size_t)(t + 1) * D + c], y[c], dot);
-                dot = warp_sum_f64(dot);
-                if (lane == 0) {
-                    const int em = exn + a.Rexp[(size_t)s * (K + 1) + t + 1];
-                    info[r].tn = ldexp(dot / mant_n, em - exp_n);
-                }
-            }
-        }
-        __syncthreads();
-    }
-    for (int r = warp; r < nr; r += nw) {
-        double fsg;
-        const double lr = rbm_log_ratio_warp(a.an, s, a.theta, a.lc, na, nb, info[r].ma, info[r].mb, lane, &fsg);
-        if (lane == 0) info[r].tn = info[r].coef * info[r].tn * (fsg * exp(lr));
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double acc = 0.0;
-        int64_t sp = 0;
-        for (int r = 0; r < nr; ++r) { acc += info[r].tn; sp += info[r].q - info[r].p + 1; }
-        a.partial[b] = acc;
-        if (a.span) a.span[b] = sp;
-    }
 }
 
 __global__ void k_amp_graph_fp64(AmpArgs a)
@@ -602,13 +499,8 @@ int launch_amp_fp64(const AmpArgs& a, cudaStream_t st)
 {
     if (a.rows.max_chunks == 0) return 0;
     const size_t smem = amp_fp64_smem(a.an, a.rows_per_block);
-    if (a.an.chain) {
-        allow_max_smem(k_amp_chain_fp64);
-        k_amp_chain_fp64<<<(unsigned)a.rows.max_chunks, 256, smem, st>>>(a);
-    } else {
-        allow_max_smem(k_amp_graph_fp64);
-        k_amp_graph_fp64<<<(unsigned)a.rows.max_chunks, 256, smem, st>>>(a);
-    }
+    allow_max_smem(k_amp_graph_fp64);
+    k_amp_graph_fp64<<<(unsigned)a.rows.max_chunks, 256, smem, st>>>(a);
     return 1;
 }
 

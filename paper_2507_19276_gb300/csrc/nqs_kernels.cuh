@@ -326,8 +326,6 @@ struct AmpArgs {
     int64_t Ns;
     RowSet rows;
     int rows_per_block;
-    const double* Lenv; const int* Lexp;
-    const double* Renv; const int* Rexp;
     const double* Hst; const int* Hexp;
     const double* theta; const double* lc;
     const double* psi_mant; const int* psi_exp;

@@ -620,9 +620,9 @@ __global__ void __launch_bounds__(64) k_tree_close(TreeClose a)
     const int own = sigma_at(na, nb, q);
     auto load_g = [&](int i) {
         __syncthreads();
-        for (int c = threadIdx.x; c < D; c += blockDim.x) g[c] = a.Gst[((size_t)s * K + i) * D + c];
+        for (int c = threadIdx.x; c < D; c += blockDim.x) g[c] = a.Gst[((size_t)s * a.g_stride + i) * D + c];
         __syncthreads();
-        return a.Gexp[(size_t)s * K + i];
+        return a.Gexp[(size_t)s * a.g_stride + i];
     };
     for (int lj = a.live_ptr[q]; lj < a.live_ptr[q + 1]; ++lj) {
         const int j = a.live_idx[lj];
@@ -640,7 +640,7 @@ __global__ void __launch_bounds__(64) k_tree_close(TreeClose a)
             // the alternative's part on top of n's, aligned
             int ex = first ? -1000000 : zx;
             for (int e = an.pred_ptr[q]; e < an.pred_ptr[q + 1]; ++e)
-                if (an.pred_idx[e] == j) { const int gx = a.Gexp[(size_t)s * K + q]; ex = gx > ex ? gx : ex; }
+                if (an.pred_idx[e] == j) { const int gx = a.Gexp[(size_t)s * a.g_stride + q]; ex = gx > ex ? gx : ex; }
             const int gx = load_g(q);
             for (int c = threadIdx.x; c < D; c += blockDim.x) {
                 double v = first ? 0.0 : z[c] * pow2_neg64(zx - ex);
@@ -716,13 +716,17 @@ __device__ __forceinline__ double tree_coef(const TreeArgs& t, int64_t s, int64_
 
 constexpr int kRowLanes = 8;
 
-// Rows of the FP64 graph form: eight lanes per row dot the live states of the
-// row's node with the closing covectors, then form the correlator ratio.
+// Rows of the FP64 form: eight lanes per row dot the live states of the row's
+// node with the closing covectors and take the correlator ratio as a product
+// (9 FP64 operations per hidden unit; log 2cosh of every unit and row was ~80
+// and 40% of the H18 time). A ratio outside the normal range is redone as a sum
+// of logarithms, as the cos forms are.
 __global__ void __launch_bounds__(256) k_tree_rows64(TreeRows64 a)
 {
     __shared__ int64_t s_s;
     __shared__ double s_term[kTreeRows];
     __shared__ int s_span[kTreeRows], s_mv[kTreeRows];
+    __shared__ unsigned char s_log[kTreeRows];
     const TreeArgs& t = a.t;
     const AnsatzView& an = a.q.an;
     const int64_t b = t.chunk_base[t.s0] + blockIdx.x;
@@ -730,30 +734,32 @@ __global__ void __launch_bounds__(256) k_tree_rows64(TreeRows64 a)
     __syncthreads();
     const int64_t s = s_s;
     if (s < 0) return;
-    const int K = an.K, D = an.D, sl = (int)(s - t.s0);
+    const int K = an.K, D = an.D, NH = an.n_hidden, sl = (int)(s - t.s0);
     const uint64_t na = t.samples[2 * s], nb = t.samples[2 * s + 1];
     const int64_t r0 = (b - t.chunk_base[s]) * kTreeRows, g0 = t.row_base[s] - t.row_base[t.s0] + r0;
     const int64_t left = t.row_base[s + 1] - t.row_base[s] - r0;
     const int nr = (int)(left < kTreeRows ? left : kTreeRows);
     const int l8 = threadIdx.x & 7, lane = threadIdx.x & 31;
-    const double rpsi = a.psi_mant[s];
+    const double mant = a.psi_mant[s];
     const int pex = a.psi_exp[s];
     for (int rr = threadIdx.x >> 3; rr < kTreeRows; rr += 32) {      // whole warps: the shuffles need them
         const bool on = rr < nr;
-        double tn = 0.0;
+        double tn = 0.0, ratio = 1.0;
+        int er = 0;
+        TreeWord w{};
         if (on) {
-            const TreeWord w = tree_unpack(t.word[g0 + rr]);
+            w = tree_unpack(t.word[g0 + rr]);
             const uint32_t node = t.rnode[g0 + rr];
             const int x = w.x[w.c - 1], q = x / 3, alt = x - 3 * q;
             const size_t ci = ((size_t)sl * K + q) * 3 + alt;
             const int v0 = a.q.live_ptr[q], v1 = a.q.live_ptr[q + 1];
-            int er = a.q.ce[ci];
+            er = a.q.ce[ci];
             for (int v = v0; v < v1; ++v) {
                 const uint32_t row = tree_source(t.parent, t.start, t.base, node, a.q.live_idx[v]);
                 const int e = a.pool_e[row] + a.q.Qe[((size_t)sl * a.q.n_live + v) * 3 + alt];
                 er = e > er ? e : er;
             }
-            double acc = l8 == 0 ? a.q.c[ci] * pow2_neg64(a.q.ce[ci] - er) : 0.0;
+            tn = l8 == 0 ? a.q.c[ci] * pow2_neg64(a.q.ce[ci] - er) : 0.0;
             for (int v = v0; v < v1; ++v) {
                 const uint32_t row = tree_source(t.parent, t.start, t.base, node, a.q.live_idx[v]);
                 const size_t qi = ((size_t)sl * a.q.n_live + v) * 3 + alt;
@@ -761,31 +767,50 @@ __global__ void __launch_bounds__(256) k_tree_rows64(TreeRows64 a)
                 const double* Qj = a.q.Q + qi * D;
                 double d = 0.0;
                 for (int c = l8; c < D; c += kRowLanes) d = fma(__ldg(Qj + c), hj[c], d);
-                acc = fma(d, pow2_neg64(a.pool_e[row] + a.q.Qe[qi] - er), acc);
+                tn = fma(d, pow2_neg64(a.pool_e[row] + a.q.Qe[qi] - er), tn);
             }
-            tn = acc;
-            // exponent of the sum against psi(n)
-            s_span[rr] = er - pex;
+            if (a.expd) {
+                const double2* ex[4];
+                for (int k = 0; k < 4; ++k) {
+                    const int p = w.x[k] / 3;
+                    ex[k] = a.expd + (size_t)((p * 4 + sigma_at(na, nb, p)) * 3 + w.x[k] - 3 * p) * NH;
+                }
+                const double2* ab = a.ab + (size_t)sl * NH;
+                for (int k = l8; k < NH; k += kRowLanes) {
+                    const double2 h = __ldg(ab + k);
+                    double2 e = __ldg(ex[0] + k);
+                    for (int c = 1; c < w.c; ++c) {
+                        const double2 f = __ldg(ex[c] + k);
+                        e.x *= f.x;
+                        e.y *= f.y;
+                    }
+                    ratio *= fma(h.x, e.x, h.y * e.y);
+                }
+            }
         }
-        for (int o = 4; o; o >>= 1) tn += __shfl_xor_sync(kFull, tn, o);
-        __syncwarp();
-        if (on && l8 == 0) s_term[rr] = scale_pow2(tn / rpsi, s_span[rr]);
-        __syncwarp();
+        for (int o = 4; o; o >>= 1) {
+            tn += __shfl_xor_sync(kFull, tn, o);
+            ratio *= __shfl_xor_sync(kFull, ratio, o);
+        }
+        if (on && l8 == 0) {
+            const int p = w.x[0] / 3;
+            const bool by_log = NH > 0 && (!a.expd || !(ratio > 1e-290 && ratio < 1e290));
+            const double coef = tree_coef(t, s, r0 + rr);
+            s_term[rr] = coef * scale_pow2(tn / mant, er - pex) * (by_log ? 1.0 : ratio);
+            s_span[rr] = a.chain ? w.x[w.c - 1] / 3 - p + 1 : K - p;
+            s_mv[rr] = graph_matvecs(an, p);
+            s_log[rr] = by_log;
+        }
     }
     __syncthreads();
-    // correlator ratio, one warp per row
     for (int rr = threadIdx.x >> 5; rr < nr; rr += 8) {
+        if (!s_log[rr]) continue;                                    // uniform over the warp
         const TreeWord w = tree_unpack(t.word[g0 + rr]);
         uint64_t ma, mb;
         tree_det(w, na, nb, ma, mb);
         int neg;
         const double lr = corr_log_ratio_warp(an, s, a.theta, a.lc, na, nb, ma, mb, lane, &neg);
-        if (lane == 0) {
-            const int p = w.x[0] / 3;
-            s_term[rr] = tree_coef(t, s, r0 + rr) * s_term[rr] * ((neg ? -1.0 : 1.0) * exp(lr));
-            s_span[rr] = K - p;
-            s_mv[rr] = graph_matvecs(an, p);
-        }
+        if (lane == 0) s_term[rr] *= (neg ? -1.0 : 1.0) * exp(lr);
     }
     __syncthreads();
     if (threadIdx.x < 32) {
@@ -803,7 +828,41 @@ __global__ void __launch_bounds__(256) k_tree_rows64(TreeRows64 a)
     }
 }
 
+__global__ void k_corr_exp(const double* __restrict__ W, int K, int NH, double2* expd)
+{
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= K * 12 * NH) return;
+    const int k = idx % NH, row = idx / NH;
+    const int p = row / 12, own = (row % 12) / 3, to = tree_alt_state(own, row % 3);
+    const double wa = W[(size_t)k * 2 * K + 2 * p], wb = W[(size_t)k * 2 * K + 2 * p + 1];
+    const double d = ((to & 1) - (own & 1)) * wa + ((to >> 1) - (own >> 1)) * wb;
+    expd[idx] = make_double2(exp(d), exp(-d));
+}
+
+__global__ void k_corr_ab(const double* __restrict__ theta, int64_t n, double2* ab)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double e = exp(-2.0 * fabs(theta[i])), big = 1.0 / (1.0 + e), small = e * big;
+    ab[i] = theta[i] >= 0.0 ? make_double2(big, small) : make_double2(small, big);
+}
+
 }  // namespace
+
+int launch_corr_exp(const double* W, int K, int n_hidden, double2* expd, cudaStream_t st)
+{
+    const int n = K * 12 * n_hidden;
+    if (n == 0) return 0;
+    k_corr_exp<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(W, K, n_hidden, expd);
+    return 1;
+}
+
+int launch_corr_ab(const double* theta, int64_t n, double2* ab, cudaStream_t st)
+{
+    if (n == 0) return 0;
+    k_corr_ab<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(theta, n, ab);
+    return 1;
+}
 
 int launch_tree_close(const TreeClose& a, cudaStream_t st)
 {

@@ -59,10 +59,10 @@ int launch_tree_items(const TreeArgs& a, cudaStream_t st);
 
 // ---- node evaluations -------------------------------------------------------
 
-// FP64 states of a graph ansatz (linear readout): one vertex of every node of
-// the items [i0, i1), whose local state there is sg.
+// FP64 states of a chain or graph ansatz (linear readout): vertex t of every
+// node of level t.
 struct TreeGraph64 {
-    AnsatzView an;
+    AnsatzView an;                        // with the edge lists (a chain's too)
     const uint32_t* items;
     const uint32_t* parent; const uint32_t* start; const uint32_t* base;
     double* pool;                         // [rows][D]
@@ -76,7 +76,8 @@ int launch_tree_graph64(const TreeGraph64& a, int t, const int64_t* bounds, cuda
 struct TreeClose {
     AnsatzView an;
     const uint64_t* samples; int64_t s0; int nb;
-    const double* Gst; const int* Gexp;   // adjoints of n [Ns][K][D]
+    const double* Gst; const int* Gexp;   // adjoints of n: sample s's vertex i at row s * g_stride + i
+    int g_stride;
     const int* live_ptr; const int* live_idx;   // [K+1], vertices read at or after q
     int n_live;                           // live_ptr[K]
     double* Q; int* Qe;                   // [nb][n_live][3][D], [nb][n_live][3]
@@ -84,9 +85,18 @@ struct TreeClose {
 };
 int launch_tree_close(const TreeClose& a, cudaStream_t st);
 
+// 2cosh correlator on the rows: cosh(theta + d) / cosh theta = A e^d + B e^-d
+// with A = 1 / (1 + e^(-2 theta)), B = 1 - A, and e^d a product over the changed
+// sites: expd [K][4 own][3 alternatives][n_hidden] = {e^d, e^-d} of one site's
+// change d of theta_k, ab [samples][n_hidden] = {A, B}.
+int launch_corr_exp(const double* W, int K, int n_hidden, double2* expd, cudaStream_t st);
+int launch_corr_ab(const double* theta, int64_t n, double2* ab, cudaStream_t st);
+
 struct TreeRows64 {
     TreeArgs t;
     TreeClose q;
+    int chain;                            // the span of a chain's row ends at its last change
+    const double2* expd; const double2* ab;   // NULL: no 2cosh correlator (ab: batch samples)
     const double* pool; const int* pool_e;
     const double* theta; const double* lc;
     const double* psi_mant; const int* psi_exp;
