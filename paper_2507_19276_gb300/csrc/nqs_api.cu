@@ -84,12 +84,12 @@ struct nqs_ctx {
     // normalised readout, correlator kind, gradient and audit options
     DevBuf rv, reta, rw, rc, W2, rnn_cells, rnn_lp, rnn_sg, grad_scr, u_dev, ebar_dev;
     DevBuf tk_rank, tk_off, tk;   // tensor term (Tucker form) of the graph ansatz
-    // mixed form of the graph ansatz: matrix images, e_0 columns, state slots
-    DevBuf g_img, g_bexp, g_col0, g_slot, g_last, mv_det, mv_draw, g_simg, g_tts, g_rank, g_coef;
+    // mixed form of the graph ansatz: matrix images, e_0 columns, tanh theta
+    DevBuf g_img, g_bexp, g_col0, mv_det, mv_draw, g_tts;
     // prefix trees (graphs, the normalised chain readout)
     DevBuf tr_rows, tr_build, tr_items, tr_pool, tr_close, g_live, cexp, corr_ab;
     int n_live = 0;           // entries of g_live past its K + 1 offsets
-    int g_slots = 0, g_maxdeg = 0, g_nbuf = 1;
+    std::vector<int> deg_h;   // in-degree of every vertex
     bool has_gtc = false;
     char gtc_why[160] = {0};   // why the graph does not fit the tensor-core tiles
     int grad_chunk = 0;        // samples whose environments live at once in the gradient (0: all)
@@ -424,17 +424,16 @@ int env_pass(nqs_ctx* c, const uint64_t* samples, int64_t Ns, bool adjoints, int
     return NQS_OK;
 }
 
-// Amplitudes over one row set, accumulated into per-chunk partial sums.
-// gtc: the mixed form of the graph ansatz (tensor-core tiles of 128 rows),
-// which also sums the magnitudes of the terms into *pabs when it is non-NULL.
+// Amplitudes over one row set, accumulated into per-chunk partial sums: the
+// forms that re-run each row from its first change (normalised readout of a
+// graph or a wide chain, tensor term).
 int amp_pass(nqs_ctx* c, const uint64_t* samples, int64_t Ns, RowSet rows, int64_t total_rows,
              const int64_t* count_dev, DevBuf& base, DevBuf& part, DevBuf& span,
-             int64_t max_rows_per_sample, int stage, bool gtc = false, DevBuf* pabs = nullptr,
-             DevBuf* mvb = nullptr)
+             int64_t max_rows_per_sample, int stage, DevBuf* mvb = nullptr)
 {
     StageScope sc(c, stage);
     const bool rnn = c->av.readout == 1;
-    const int R = gtc ? 128 : (rnn ? rnn_rows_per_block() : amp_fp64_rows_per_block(c->av));
+    const int R = rnn ? rnn_rows_per_block() : amp_fp64_rows_per_block(c->av);
     int64_t max_chunks = total_rows / R + Ns;
     if (max_rows_per_sample >= 0) max_chunks = Ns * ((max_rows_per_sample + R - 1) / R);
     TRY(ensure(c, base, (size_t)(Ns + 1) * 8));
@@ -445,53 +444,6 @@ int amp_pass(nqs_ctx* c, const uint64_t* samples, int64_t Ns, RowSet rows, int64
     rows.chunk_base = (const int64_t*)base.p;
     rows.max_chunks = max_chunks;
     if (mvb) TRY(ensure(c, *mvb, (size_t)(max_chunks ? max_chunks : 1) * 8));
-    if (gtc) {
-        if (pabs) TRY(ensure(c, *pabs, (size_t)(max_chunks ? max_chunks : 1) * 8));
-        // rows with the same first changed vertex side by side: a tile re-runs
-        // the vertices its rows need, not those of its earliest row
-        const size_t span_rows = rows.begin ? (size_t)total_rows : (size_t)Ns * rows.stride;
-        TRY(ensure(c, c->g_rank, (span_rows ? span_rows : 1) * 4));
-        TRY(ensure(c, c->g_coef, (span_rows ? span_rows : 1) * 8));
-        LAUNCH(stage, launch_graph_sort(c->hv, samples, rows, Ns, c->K, (uint32_t*)c->g_rank.p,
-                                        (double*)c->g_coef.p, c->stream));
-        rows.rank = (const uint32_t*)c->g_rank.p;
-        rows.coef = (const double*)c->g_coef.p;
-        GraphTcArgs g{};
-        g.an = c->av;
-        g.h = c->hv;
-        g.samples = samples;
-        g.Ns = Ns;
-        g.rows = rows;
-        g.Hst = (const double*)c->Hst.p; g.Hexp = (const int*)c->Hexp.p;
-        TRY(ensure(c, c->g_simg, (size_t)Ns * c->K * 4 * c->av.D));
-        TRY(ensure(c, c->g_tts, (size_t)Ns * (((c->av.n_hidden + 3) & ~3) ? ((c->av.n_hidden + 3) & ~3) : 1) * 4));
-        g.simg = (unsigned char*)c->g_simg.p;
-        g.tts = (float*)c->g_tts.p;
-        g.theta = (const double*)c->theta.p;
-        g.psi_mant = (const double*)c->pmant.p;
-        g.psi_exp = (const int*)c->pexp.p;
-        g.bimg = (const unsigned char*)c->g_img.p;
-        g.bexp = (const int*)c->g_bexp.p;
-        g.col0 = (const float*)c->g_col0.p;
-        g.slot = (const int*)c->g_slot.p;
-        g.last_use = (const int*)c->g_last.p;
-        g.n_slots = c->g_slots;
-        g.max_deg = c->g_maxdeg;
-        g.nbuf = c->g_nbuf;
-        uint32_t cols = 32;
-        while (cols < (uint32_t)(c->g_maxdeg * 4 * c->av.D)) cols <<= 1;
-        g.tmem_cols = cols;
-        g.WT = c->av.n_hidden ? (const float*)c->WTf.p : nullptr;
-        g.np = (c->av.n_hidden + 3) & ~3;
-        g.partial = (double*)part.p;
-        g.partial_abs = pabs ? (double*)pabs->p : nullptr;
-        g.span = (int64_t*)span.p;
-        g.mv = mvb ? (int64_t*)mvb->p : nullptr;
-        g.err = (DevError*)c->derr.p;
-        LAUNCH(stage, launch_graph_tiles(g, c->n_sm, c->stream));
-        CK(cudaGetLastError());
-        return NQS_OK;
-    }
     if (rnn) {
         RnnAmpArgs r{};
         r.an = c->av;
@@ -924,10 +876,24 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
         }
         if (rows_total >= ((int64_t)1 << 32))
             return set_err(c, NQS_ERR_UNSUPPORTED, "prefix trees of %lld states exceed 2^32", (long long)rows_total);
-        TRY(ensure(c, c->tr_items, (size_t)(bounds.back() + 1) * 4));
+        TreeLevels lv{};
+        lv.sources = kind != kTreeRnn ? 1 : 0;
+        int64_t n_items = 0;
+        for (int t = 0; t < K; ++t) {
+            const int64_t n = bounds[(size_t)4 * t + 4] - bounds[(size_t)4 * t];
+            lv.at[t] = (uint32_t)n_items;
+            lv.first[t] = (uint32_t)bounds[(size_t)4 * t];
+            lv.n[t] = (uint32_t)n;
+            n_items += n * (1 + (lv.sources ? c->deg_h[(size_t)t] : 0));
+        }
+        if (n_items >= ((int64_t)1 << 32)) {
+            if (nb > 1) { s1 = s0 + (nb + 1) / 2; goto retry; }
+            return set_err(c, NQS_ERR_UNSUPPORTED, "prefix trees of %lld items exceed 2^32", (long long)n_items);
+        }
+        TRY(ensure(c, c->tr_items, (size_t)(n_items + 1) * 4));
         a.items = (uint32_t*)c->tr_items.p;
         a.pool_tot = pool_off;
-        LAUNCH(stage, launch_tree_items(a, c->stream));
+        LAUNCH(stage, launch_tree_items(a, lv, (const int*)c->pred_ptr.p, (const int*)c->pred_idx.p, c->stream));
         if (kind == kTreeGraph64) {
             TreeGraph64 g{};
             TreeClose q{};
@@ -958,8 +924,7 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
             g.an.pred_ptr = (const int*)c->pred_ptr.p;
             g.an.pred_idx = (const int*)c->pred_idx.p;
             g.items = a.items;
-            g.parent = a.parent; g.start = a.start; g.base = a.base;
-            for (int t = 0; t < K; ++t) LAUNCH(stage, launch_tree_graph64(g, t, bounds.data(), c->stream));
+            for (int t = 0; t < K; ++t) LAUNCH(stage, launch_tree_graph64(g, t, lv, bounds.data(), c->stream));
             q.an = g.an;
             q.samples = ds;
             q.s0 = s0;
@@ -991,6 +956,45 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
             r.span = (int64_t*)c->span_det.p;
             r.mv = (int64_t*)c->mv_det.p;
             LAUNCH(stage, launch_tree_rows64(r, max_chunks, c->stream));
+        }
+        if (kind == kTreeGraphTc) {
+            TreeGraphTc g{};
+            for (int pass = 0; pass < 2; ++pass) {
+                Carve v{pass ? (char*)c->tr_pool.p : nullptr};
+                g.pool = v.take<unsigned char>((size_t)rows_total * 4 * D);
+                g.pool_e = v.take<int>((size_t)rows_total);
+                if (!pass) TRY(ensure(c, c->tr_pool, v.n));
+            }
+            TRY(ensure(c, c->g_tts, (size_t)nb * (np ? np : 1) * 4));
+            LAUNCH(stage, launch_tree_graph_prep((const double*)c->Hst.p, (const int*)c->Hexp.p, (const double*)c->theta.p,
+                                                 s0, nb, K, D, NH, np, c->av.corr, g.pool, g.pool_e, (float*)c->g_tts.p,
+                                                 c->stream));
+            g.an = c->av;
+            g.items = a.items;
+            g.bimg = (const unsigned char*)c->g_img.p;
+            g.bexp = (const int*)c->g_bexp.p;
+            g.col0 = (const float*)c->g_col0.p;
+            g.mant = mant;
+            g.mexp = mexp;
+            g.err = (DevError*)c->derr.p;
+            for (int t = 0; t < K; ++t)
+                LAUNCH(stage, launch_tree_graph_tc(g, t, c->deg_h[(size_t)t], lv, bounds.data(), c->n_sm,
+                                                   c->stream));
+            TreeRowsTc r{};
+            r.t = a;
+            r.an = c->av;
+            r.mant = mant;
+            r.mexp = mexp;
+            r.tts = (const float*)c->g_tts.p;
+            r.WT = NH ? (const float*)c->WTf.p : nullptr;
+            r.np = np;
+            r.psi_mant = (const double*)c->pmant.p;
+            r.psi_exp = (const int*)c->pexp.p;
+            r.partial = (double*)c->part_det.p;
+            r.partial_abs = want_abs ? (double*)c->part_det_abs.p : nullptr;
+            r.span = (int64_t*)c->span_det.p;
+            r.mv = (int64_t*)c->mv_det.p;
+            LAUNCH(stage, launch_tree_rows_tc(r, max_chunks, c->n_sm, c->stream));
         }
         CK(cudaGetLastError());
         s0 = s1;
@@ -1049,8 +1053,7 @@ extern "C" int nqs_destroy(nqs_ctx* c)
     DevBuf* more[] = {&c->rv, &c->reta, &c->rw, &c->rc, &c->W2, &c->rnn_cells, &c->rnn_lp, &c->rnn_sg,
                       &c->grad_scr, &c->u_dev, &c->ebar_dev, &c->smp_cand, &c->smp_ccnt, &c->smp_cpos,
                       &c->smp_tabs, &c->smp_tree, &c->tk_rank, &c->tk_off, &c->tk, &c->g_img, &c->g_bexp,
-                      &c->g_col0, &c->g_slot, &c->g_last, &c->mv_det, &c->mv_draw, &c->g_simg,
-                      &c->g_tts, &c->g_rank, &c->g_coef, &c->tr_rows, &c->tr_build, &c->tr_items,
+                      &c->g_col0, &c->mv_det, &c->mv_draw, &c->g_tts, &c->tr_rows, &c->tr_build, &c->tr_items,
                       &c->tr_pool, &c->tr_close, &c->g_live, &c->cexp, &c->corr_ab};
     for (DevBuf* b : more) release(*b);
     for (auto* v : {&c->smp_pa, &c->smp_pb, &c->smp_off, &c->smp_cnt, &c->smp_par, &c->smp_cell})
@@ -1265,6 +1268,8 @@ extern "C" int nqs_set_ansatz(nqs_ctx* c, const double* site_tensors, int n_edge
         TRY(ensure(c, c->g_live, lp.size() * 4));
         CK(cudaMemcpyAsync(c->g_live.p, lp.data(), lp.size() * 4, cudaMemcpyHostToDevice, c->stream));
         c->n_live = (int)li.size();
+        c->deg_h.resize(K);
+        for (int i = 0; i < K; ++i) c->deg_h[i] = ptr[i + 1] - ptr[i];
     }
     AnsatzForms fm{};
     fm.D = D;
@@ -1276,7 +1281,6 @@ extern "C" int nqs_set_ansatz(nqs_ctx* c, const double* site_tensors, int n_edge
     c->has_tc = false;
     c->has_gtc = false;
     c->gtc_why[0] = 0;
-    GraphTcPlan gp;
     if (chain) {
         // (hi, lo) pairs of both copies for the double-FP32 arithmetic
         TRY(ensure(c, c->ATdf, nt * 8));
@@ -1296,20 +1300,13 @@ extern "C" int nqs_set_ansatz(nqs_ctx* c, const double* site_tensors, int n_edge
         }
     } else {
         const char* why = nullptr;
-        if (graph_tc_plan(ptr.data(), idx.data(), K, D, n_hidden, gp, &why)) {
+        if (graph_tc_fits(ptr.data(), idx.data(), K, D, n_hidden, &why)) {
             TRY(ensure(c, c->g_img, (size_t)n_edges * 16 * D * D));
             TRY(ensure(c, c->g_bexp, (size_t)fm.n_mats * 4));
             TRY(ensure(c, c->g_col0, (size_t)fm.n_mats * D * 4));
-            TRY(ensure(c, c->g_slot, (size_t)K * 4));
-            TRY(ensure(c, c->g_last, (size_t)K * 4));
-            CK(cudaMemcpyAsync(c->g_slot.p, gp.slot.data(), (size_t)K * 4, cudaMemcpyHostToDevice, c->stream));
-            CK(cudaMemcpyAsync(c->g_last.p, gp.last_use.data(), (size_t)K * 4, cudaMemcpyHostToDevice, c->stream));
             fm.exps = (int*)c->g_bexp.p;
             fm.graph_img = (unsigned char*)c->g_img.p;
             fm.col0 = (float*)c->g_col0.p;
-            c->g_slots = gp.n_slots;
-            c->g_maxdeg = gp.max_deg;
-            c->g_nbuf = gp.nbuf;
             c->has_gtc = true;
         } else {
             snprintf(c->gtc_why, sizeof(c->gtc_why), "%s", why ? why : "unsupported graph");
@@ -1658,6 +1655,7 @@ int le_core(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, uint64
     // the plain FP64 form: psi is linear in the states without the tensor term, so
     // the rows share prefixes and close with n's adjoints (the tensor term's are re-run)
     const bool tree64 = !rnn && !gtc && !shared && !c->av.tk_rank;
+    const bool tree = tree64 || gtc;
     if (!c->av.chain && prec == NQS_PREC_FP64_SHARED)
         return set_err(c, NQS_ERR_UNSUPPORTED,
                        "graph ansatze have no shared-prefix form (NQS_PREC_FP64 or NQS_PREC_MIXED)");
@@ -1686,7 +1684,7 @@ int le_core(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, uint64
     }
     int64_t total = 0;
     TRY(count_pass(c, ds, Ns, eb, &total, n_draws > 0));
-    if (shared || tree64) {
+    if (shared || tree) {
         c->det_off_h.resize(Ns + 1);
         CK(cudaMemcpyAsync(c->det_off_h.data(), c->det_off.p, (size_t)(Ns + 1) * 8, cudaMemcpyDeviceToHost, c->stream));
     }
@@ -1721,8 +1719,8 @@ int le_core(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, uint64
     if (shared) {
         if (prec == NQS_PREC_MIXED) TRY(family_pass<float>(c, ds, Ns, total, n_draws, deabs != nullptr));
         else TRY(family_pass<double>(c, ds, Ns, total, n_draws, deabs != nullptr));
-    } else if (tree64) {
-        TRY(tree_pass(c, ds, Ns, total, n_draws, kTreeGraph64, false));
+    } else if (tree) {
+        TRY(tree_pass(c, ds, Ns, total, n_draws, gtc ? kTreeGraphTc : kTreeGraph64, deabs != nullptr));
     } else {
         // amplitudes: deterministic rows, then the distinct drawn rows
         RowSet rd{};
@@ -1730,8 +1728,7 @@ int le_core(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, uint64
         rd.coef = (const double*)c->det_coef.p;
         rd.begin = (const int64_t*)c->det_off.p;
         TRY(amp_pass(c, ds, Ns, rd, total, (const int64_t*)c->det_tot.p, c->base_det, c->part_det,
-                     c->span_det, -1, NQS_STAGE_AMP_DET, gtc, deabs ? &c->part_det_abs : nullptr,
-                     graph ? &c->mv_det : nullptr));
+                     c->span_det, -1, NQS_STAGE_AMP_DET, graph ? &c->mv_det : nullptr));
         if (n_draws > 0) {
             RowSet rs{};
             rs.rank = (const uint32_t*)c->draw_rank.p;
@@ -1739,12 +1736,12 @@ int le_core(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, uint64
             rs.begin = nullptr;
             rs.stride = n_draws;
             TRY(amp_pass(c, ds, Ns, rs, (int64_t)Ns * n_draws, (const int64_t*)c->n_unique.p,
-                         c->base_draw, c->part_draw, c->span_draw, n_draws, NQS_STAGE_AMP_DRAW, gtc,
-                         deabs ? &c->part_draw_abs : nullptr, graph ? &c->mv_draw : nullptr));
+                         c->base_draw, c->part_draw, c->span_draw, n_draws, NQS_STAGE_AMP_DRAW,
+                         graph ? &c->mv_draw : nullptr));
         }
     }
     TRY(ensure(c, c->summary, kSummaryDoubles * 8));
-    const bool draws_apart = n_draws > 0 && !tree64;     // drawn rows in their own partial sums
+    const bool draws_apart = n_draws > 0 && !tree;     // drawn rows in their own partial sums
     FinalArgs f{};
     f.Ns = Ns;
     f.h_diag = (const double*)c->hdiag.p;

@@ -339,50 +339,11 @@ int launch_amp_fp64(const AmpArgs& a, cudaStream_t st);
 
 // ---- mixed form of the graph ansatz on the tensor cores (nqs_graph.cu) ------
 
-constexpr int kGtMaxSlots = 16;          // vertex states a tile keeps at once
+constexpr int kGtMaxSlots = 16;          // vertex states alive at once
 constexpr int kGtMaxDeg = 8;             // in-degree bound of the graph ansatz
 
-struct GraphTcPlan {
-    std::vector<int> slot;               // [K] state slot of each vertex (-1: never read)
-    std::vector<int> last_use;           // [K] last vertex reading each state (-1: none)
-    int n_slots = 0, max_deg = 0;
-    int nbuf = 1;                        // matrix-image buffers that fit next to the slots
-};
-// false (with the reason) when the graph does not fit the tile kernel
-bool graph_tc_plan(const int* ptr, const int* idx, int K, int D, int n_hidden,
-                   GraphTcPlan& p, const char** why);
-size_t graph_tiles_smem(int D, int K, int n_slots, int max_deg, int n_hidden, int nbuf);
-
-struct GraphTcArgs {
-    AnsatzView an;
-    HamView h;
-    const uint64_t* samples;
-    int64_t Ns;
-    RowSet rows;                         // chunk_base over 128-row tiles
-    const double* Hst; const int* Hexp;  // h_j(n) and their powers of two (FP64 pass)
-    unsigned char* simg;                 // [Ns][K][4D] bytes: split images of h_j(n) (written here)
-    float* tts;                          // [Ns][np] tanh (cos form: tan) of theta_k(n) (written here)
-    const double* theta;                 // [Ns][n_hidden]
-    const double* psi_mant; const int* psi_exp;
-    const unsigned char* bimg;           // AnsatzForms::graph_img
-    const int* bexp;                     // [E][4] power of two taken out of each image
-    const float* col0;                   // [E][4][D] column 0 of each matrix (e_0 sources)
-    const int* slot;
-    const int* last_use;
-    int n_slots, max_deg, nbuf;
-    uint32_t tmem_cols;                  // power of two >= max_deg * 4 * D
-    const float* WT;                     // [2K][np] FP32 correlator weights, transposed
-    int np;
-    double* partial;                     // [tiles] sum of the terms
-    double* partial_abs;                 // [tiles] sum of their magnitudes (optional)
-    int64_t* span;                       // [tiles] vertices re-run
-    int64_t* mv;                         // [tiles] in-edge D x D products of the rows (optional)
-    DevError* err;
-};
-int launch_graph_tiles(const GraphTcArgs& a, int n_sm, cudaStream_t st);
-// each sample's rows (rank, coefficient) stably sorted by their first changed vertex
-int launch_graph_sort(const HamView& h, const uint64_t* samples, const RowSet& in, int64_t Ns, int K,
-                      uint32_t* out_rank, double* out_coef, cudaStream_t st);
+// false (with the reason) when this form does not take the graph
+bool graph_tc_fits(const int* ptr, const int* idx, int K, int D, int n_hidden, const char** why);
 
 // full K-site product for arbitrary determinants (nqs_amplitude)
 int launch_full_amp_fp64(const AnsatzView& an, const uint64_t* dets, int64_t n, double* log_abs,

@@ -26,33 +26,6 @@ namespace nqs {
 
 namespace {
 
-constexpr uint32_t kNoNode = 0xffffffffu;
-
-// sample (call index) of chunk b of the batch, -1 past its end
-__device__ __forceinline__ int64_t tree_sample(const TreeArgs& a, int64_t b)
-{
-    if (b >= a.chunk_base[a.s0 + a.nb]) return -1;
-    int64_t lo = a.s0, hi = a.s0 + a.nb - 1;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi + 1) >> 1;
-        if (a.chunk_base[mid] <= b) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-struct TreeWord {
-    int c;                    // changes
-    int x[4];
-};
-
-__device__ __forceinline__ TreeWord tree_unpack(uint32_t w)
-{
-    TreeWord r;
-    for (int k = 0; k < 4; ++k) r.x[k] = (int)((w >> (8 * k)) & 255u);
-    r.c = r.x[1] == r.x[0] ? 1 : (r.x[2] == r.x[1] ? 2 : (r.x[3] == r.x[2] ? 3 : 4));
-    return r;
-}
-
 // Words of the rows, and the levels their one- and two-change prefixes are
 // needed to (a prefix that a later change follows: one level before it; a
 // whole row, full form: K - 1).
@@ -346,39 +319,63 @@ __global__ void __launch_bounds__(512) k_tree_count(TreeArgs a)
     for (int q = threadIdx.x; q < 4 * K; q += blockDim.x) a.level_cnt[(size_t)q * a.nb + sl] = s_cnt[q];
 }
 
-// One block per sample: absolute pool rows, and the items of every level. A
-// warp walks its nodes' levels together: one atomic per level and local state.
-__global__ void __launch_bounds__(512) k_tree_items(TreeArgs a)
+// One block per sample: the items of every level. A warp walks its nodes' levels
+// together: one atomic per level and local state. The sources are resolved here,
+// where a node's ancestors sit in registers: left to the level kernels, the walk
+// (four to eight dependent loads per in-edge) was most of a tile's 13 us.
+__global__ void __launch_bounds__(512) k_tree_items(TreeArgs a, TreeLevels lv, const int* __restrict__ pred_ptr,
+                                                    const int* __restrict__ pred_idx)
 {
     __shared__ uint32_t cur[4 * kMaxOrb];
+    __shared__ int s_ptr[kMaxOrb + 1];
+    __shared__ short s_idx[kMaxOrb * 8];
     const int sl = blockIdx.x, K = a.K;
     const int lane = threadIdx.x & 31;
     const int64_t s = a.s0 + sl;
     const uint64_t na = a.samples[2 * s], nb = a.samples[2 * s + 1];
-    for (int q = threadIdx.x; q < 4 * K; q += blockDim.x) cur[q] = (uint32_t)a.level_off[(size_t)q * a.nb + sl];
+    for (int q = threadIdx.x; q < 4 * K; q += blockDim.x) cur[q] = (uint32_t)a.level_off[(size_t)q * a.nb + sl] - lv.first[q >> 2];
+    if (lv.sources) {
+        for (int q = threadIdx.x; q <= K; q += blockDim.x) s_ptr[q] = pred_ptr[q];
+        const int E = pred_ptr[K];
+        for (int q = threadIdx.x; q < E; q += blockDim.x) s_idx[q] = (short)pred_idx[q];
+    }
     __syncthreads();
-    const TreeSlots sl_(a, sl);
-    const int n = sl_.total();
+    const TreeSlots slots(a, sl);
+    const int n = slots.total();
     const uint32_t pool = a.pool0 + (uint32_t)a.pool_tot[sl];
     for (int q0 = (int)(threadIdx.x & ~31u); q0 < n; q0 += blockDim.x) {
         const int q = q0 + lane;
         uint32_t id = 0;
         int p = kMaxOrb, e = -1, nw = 0;
+        // the node and its ancestors: state of vertex j (start <= j) at row
+        // off + j; those past the root repeat it
+        int st[4] = {0, 0, 0, 0};
+        uint32_t off[5] = {0, 0, 0, 0, 0};
         if (q < n) {
-            id = sl_.id(q);
-            const uint32_t st = a.start[id];
+            id = slots.id(q);
+            const uint32_t w = a.start[id];
             const int en = a.end[id];
-            if (en >= (int)(st & 255u)) {
-                p = (int)(st & 255u);
+            if (en >= (int)(w & 255u)) {
+                p = (int)(w & 255u);
                 e = en;
-                nw = (int)(st >> 8);
-                a.base[id] += pool;
+                nw = (int)(w >> 8);
+                uint32_t x = id;
+                for (int k = 0; k < 4 && lv.sources; ++k) {
+                    if (x < a.id1) break;                  // the root: off stays to be set below
+                    st[k] = (int)(a.start[x] & 255u);
+                    off[k] = pool + a.base[x] - (uint32_t)st[k];
+                    x = a.parent[x];
+                }
+                #pragma unroll
+                for (int k = 0; k < 5; ++k)
+                    if (off[k] == 0) off[k] = (uint32_t)(sl * K);      // (a node's row is at least pool0 - start > 0)
             }
         }
         const int t0 = __reduce_min_sync(kFull, p), t1 = __reduce_max_sync(kFull, e);
         for (int t = t0; t <= t1; ++t) {
             const bool on = t >= p && t <= e;
             const int sg = t == p ? nw : sigma_at(na, nb, t);
+            uint32_t pos = 0;
             #pragma unroll
             for (int g = 0; g < 4; ++g) {
                 const unsigned bal = __ballot_sync(kFull, on && sg == g);
@@ -386,7 +383,21 @@ __global__ void __launch_bounds__(512) k_tree_items(TreeArgs a)
                 uint32_t at = 0;
                 if (lane == __ffs((int)bal) - 1) at = atomicAdd(&cur[4 * t + g], (uint32_t)__popc(bal));
                 at = __shfl_sync(kFull, at, __ffs((int)bal) - 1);
-                if (on && sg == g) a.items[at + (uint32_t)__popc(bal & ((1u << lane) - 1u))] = id;
+                if (sg == g) pos = at + (uint32_t)__popc(bal & ((1u << lane) - 1u));
+            }
+            if (!on) continue;
+            uint32_t* out = a.items + lv.at[t] + pos;
+            if (!lv.sources) {
+                *out = id;
+                continue;
+            }
+            *out = t == K - 1 ? id : off[0] + (uint32_t)t;
+            for (int k = s_ptr[t]; k < s_ptr[t + 1]; ++k) {
+                const int j = s_idx[k];
+                if (j < 0) continue;
+                out += lv.n[t];
+                const uint32_t o = j >= st[0] ? off[0] : j >= st[1] ? off[1] : j >= st[2] ? off[2] : j >= st[3] ? off[3] : off[4];
+                *out = o + (uint32_t)j;
             }
         }
     }
@@ -396,20 +407,6 @@ __global__ void k_tree_row_counts(const int64_t* det, const int64_t* draw, int64
 {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s < n) cnt[s] = det[s] + (draw ? draw[s] : 0);
-}
-
-// pool row of vertex j's state seen from `node` (the node or an ancestor of it
-// that lived at level j)
-__device__ __forceinline__ uint32_t tree_source(const uint32_t* __restrict__ parent, const uint32_t* __restrict__ start,
-                                                const uint32_t* __restrict__ base, uint32_t node, int j)
-{
-    int p = (int)(__ldg(start + node) & 255u);
-    while (p > j) {
-        node = __ldg(parent + node);
-        const uint32_t st = __ldg(start + node);
-        p = (int)(st & 255u);
-    }
-    return __ldg(base + node) + (uint32_t)(j - p);
 }
 
 // 2^d as a double, 0 below the normal range (d <= 0)
@@ -442,9 +439,9 @@ int launch_tree_nodes(const TreeArgs& a, int64_t max_chunks, cudaStream_t st)
     return max_chunks > 0 ? 6 : 3;
 }
 
-int launch_tree_items(const TreeArgs& a, cudaStream_t st)
+int launch_tree_items(const TreeArgs& a, const TreeLevels& lv, const int* pred_ptr, const int* pred_idx, cudaStream_t st)
 {
-    k_tree_items<<<a.nb, 512, 0, st>>>(a);
+    k_tree_items<<<a.nb, 512, 0, st>>>(a, lv, pred_ptr, pred_idx);
     return 1;
 }
 
@@ -454,37 +451,42 @@ int launch_tree_items(const TreeArgs& a, cudaStream_t st)
 
 namespace {
 
-struct TreeGroups {
-    int64_t b[5];             // item bounds of the four local states
-    int tile[5];              // their tiles
-};
-
 // A tile of IT items: per in-edge the sources' vectors in shared memory, a
 // column for four items per thread (the matrix entries come through L1, one
 // load per four FMAs; FP64 at 2 lanes per clock and SM bounds this), the edges'
 // sums aligned by powers of two, one warp per item renormalising.
-__global__ void __launch_bounds__(256) k_tree_graph64(TreeGraph64 a, int t, TreeGroups gr, int IT)
+__global__ void __launch_bounds__(256) k_tree_graph64(TreeGraph64 a, int t, uint32_t at, uint32_t nl, TreeGroups gr, int IT)
 {
     extern __shared__ double sm[];
-    __shared__ uint32_t s_src[32];
-    __shared__ int s_ex[32], s_er[32];
-    __shared__ uint32_t s_node[32];
+    __shared__ uint32_t s_src[8][32];
+    __shared__ int s_ex[8][32], s_er[32];
+    __shared__ uint32_t s_out[32];
     const int D = a.an.D;
     double* xs = sm;                                  // [IT][D] sources, then the sums
     int g = 0;
     while (g < 3 && (int)blockIdx.x >= gr.tile[g + 1]) ++g;
-    const int64_t i0 = gr.b[g] + (int64_t)(blockIdx.x - gr.tile[g]) * IT;
-    const int n = (int)(gr.b[g + 1] - i0 < IT ? gr.b[g + 1] - i0 : IT);
+    const uint32_t i0 = gr.b[g] + (uint32_t)((int)blockIdx.x - gr.tile[g]) * (uint32_t)IT;
+    const int n = (int)min(gr.b[g + 1] - i0, (uint32_t)IT);
     const int e0 = a.an.pred_ptr[t], e1 = a.an.pred_ptr[t + 1];
-    if ((int)threadIdx.x < n) {
-        const uint32_t node = a.items[i0 + threadIdx.x];
-        s_node[threadIdx.x] = node;
-        int er = -1000000;
-        for (int e = e0; e < e1; ++e) {
-            const int j = a.an.pred_idx[e];
-            const int ej = j < 0 ? 0 : a.pool_e[tree_source(a.parent, a.start, a.base, node, j)];
-            er = ej > er ? ej : er;
+    // one warp per in-edge: the items' sources and their powers of two
+    {
+        const int w = threadIdx.x >> 5, it = threadIdx.x & 31;
+        if (w < e1 - e0 && it < n) {
+            int x = 0, slot = 0;
+            for (int e = e0; e < e0 + w; ++e) slot += a.an.pred_idx[e] >= 0;
+            if (a.an.pred_idx[e0 + w] >= 0) {
+                const uint32_t r = __ldg(a.items + at + (size_t)(slot + 1) * nl + i0 + it);
+                s_src[w][it] = r;
+                x = a.pool_e[r];
+            }
+            s_ex[w][it] = x;
         }
+        if (w == 7 && it < n) s_out[it] = __ldg(a.items + at + i0 + it);
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < n) {
+        int er = -1000000;
+        for (int k = 0; k < e1 - e0; ++k) er = max(er, s_ex[k][threadIdx.x]);
         s_er[threadIdx.x] = er;
     }
     // (group of four items, column) tasks of this thread
@@ -499,15 +501,9 @@ __global__ void __launch_bounds__(256) k_tree_graph64(TreeGraph64 a, int t, Tree
         const double* AT = a.an.AT + ((size_t)e * 4 + g) * D * D;
         __syncthreads();
         if (j >= 0) {
-            if ((int)threadIdx.x < n) {
-                const uint32_t r = tree_source(a.parent, a.start, a.base, s_node[threadIdx.x], j);
-                s_src[threadIdx.x] = r;
-                s_ex[threadIdx.x] = a.pool_e[r];
-            }
-            __syncthreads();
             for (int q = threadIdx.x; q < n * D; q += 256) {
                 const int it = q / D, c = q - it * D;
-                xs[q] = a.pool[(size_t)s_src[it] * D + c];
+                xs[q] = a.pool[(size_t)s_src[e - e0][it] * D + c];
             }
             __syncthreads();
         }
@@ -532,7 +528,7 @@ __global__ void __launch_bounds__(256) k_tree_graph64(TreeGraph64 a, int t, Tree
             }
             #pragma unroll
             for (int v = 0; v < 4; ++v)
-                if (it + v < n) y[u][v] += acc[v] * pow2_neg64((j < 0 ? 0 : s_ex[it + v]) - s_er[it + v]);
+                if (it + v < n) y[u][v] += acc[v] * pow2_neg64(s_ex[e - e0][it + v] - s_er[it + v]);
         }
     }
     __syncthreads();
@@ -554,8 +550,7 @@ __global__ void __launch_bounds__(256) k_tree_graph64(TreeGraph64 a, int t, Tree
         m = warp_max_f64(m);
         int ex = 0;
         if (m != 0.0) frexp(m, &ex);
-        const uint32_t node = s_node[it];
-        const uint32_t row = a.base[node] + (uint32_t)(t - (int)(a.start[node] & 255u));
+        const uint32_t row = s_out[it];
         for (int c = lane; c < D; c += 32) a.pool[(size_t)row * D + c] = ldexp(v[c], -ex);
         if (lane == 0) a.pool_e[row] = s_er[it] + ex;
     }
@@ -563,18 +558,15 @@ __global__ void __launch_bounds__(256) k_tree_graph64(TreeGraph64 a, int t, Tree
 
 }  // namespace
 
-int launch_tree_graph64(const TreeGraph64& a, int t, const int64_t* bounds, cudaStream_t st)
+int launch_tree_graph64(const TreeGraph64& a, int t, const TreeLevels& lv, const int64_t* bounds, cudaStream_t st)
 {
     const int D = a.an.D;
     // at most two (four items, column) tasks per thread
     int IT = 2048 / D / 4 * 4;
     IT = IT < 4 ? 4 : (IT > 32 ? 32 : IT);
-    TreeGroups g;
-    g.tile[0] = 0;
-    for (int k = 0; k < 5; ++k) g.b[k] = bounds[4 * t + k];
-    for (int k = 0; k < 4; ++k) g.tile[k + 1] = g.tile[k] + (int)((g.b[k + 1] - g.b[k] + IT - 1) / IT);
+    const TreeGroups g = tree_groups(t, bounds, IT);
     if (g.tile[4] == 0) return 0;
-    k_tree_graph64<<<(unsigned)g.tile[4], 256, (size_t)IT * D * 8, st>>>(a, t, g, IT);
+    k_tree_graph64<<<(unsigned)g.tile[4], 256, (size_t)IT * D * 8, st>>>(a, t, lv.at[t], lv.n[t], g, IT);
     return 1;
 }
 
@@ -687,33 +679,6 @@ __global__ void __launch_bounds__(64) k_tree_close(TreeClose a)
     }
 }
 
-// x 2^e with the exponent field where the result stays normal
-__device__ __forceinline__ double scale_pow2(double x, int e)
-{
-    const long long bits = __double_as_longlong(x);
-    const int ex = (int)((bits >> 52) & 0x7FF), ne = ex + e;
-    if (ex != 0 && ex != 0x7FF && ne > 0 && ne < 0x7FF) return __longlong_as_double(bits + ((long long)e << 52));
-    return ldexp(x, e);
-}
-
-// determinant of a row from its word
-__device__ __forceinline__ void tree_det(const TreeWord& w, uint64_t na, uint64_t nb, uint64_t& ma, uint64_t& mb)
-{
-    ma = na;
-    mb = nb;
-    for (int k = 0; k < w.c; ++k) {
-        const int p = w.x[k] / 3, sg = tree_alt_state(sigma_at(na, nb, p), w.x[k] - 3 * p);
-        ma = (ma & ~(1ull << p)) | ((uint64_t)(sg & 1) << p);
-        mb = (mb & ~(1ull << p)) | ((uint64_t)(sg >> 1) << p);
-    }
-}
-
-__device__ __forceinline__ double tree_coef(const TreeArgs& t, int64_t s, int64_t r)
-{
-    const int64_t nd = t.det_cnt[s];
-    return r < nd ? t.det_coef[t.det_off[s] + r] : t.draw_coef[s * t.draw_stride + (r - nd)];
-}
-
 constexpr int kRowLanes = 8;
 
 // Rows of the FP64 form: eight lanes per row dot the live states of the row's
@@ -755,13 +720,13 @@ __global__ void __launch_bounds__(256) k_tree_rows64(TreeRows64 a)
             const int v0 = a.q.live_ptr[q], v1 = a.q.live_ptr[q + 1];
             er = a.q.ce[ci];
             for (int v = v0; v < v1; ++v) {
-                const uint32_t row = tree_source(t.parent, t.start, t.base, node, a.q.live_idx[v]);
+                const uint32_t row = tree_source(t, sl, node, a.q.live_idx[v]);
                 const int e = a.pool_e[row] + a.q.Qe[((size_t)sl * a.q.n_live + v) * 3 + alt];
                 er = e > er ? e : er;
             }
             tn = l8 == 0 ? a.q.c[ci] * pow2_neg64(a.q.ce[ci] - er) : 0.0;
             for (int v = v0; v < v1; ++v) {
-                const uint32_t row = tree_source(t.parent, t.start, t.base, node, a.q.live_idx[v]);
+                const uint32_t row = tree_source(t, sl, node, a.q.live_idx[v]);
                 const size_t qi = ((size_t)sl * a.q.n_live + v) * 3 + alt;
                 const double* hj = a.pool + (size_t)row * D;
                 const double* Qj = a.q.Q + qi * D;

@@ -41,13 +41,23 @@ struct TreeArgs {
     uint32_t* parent;
     int* end;                             // last level the node is needed at (-1: none)
     uint32_t* start;                      // first level | new local state << 8
-    uint32_t* base;                       // row of the state pool at level `start`
+    uint32_t* base;                       // row of the state pool at level `start`, within the
+                                          // sample's rows (a root: within the pool)
     // levels
     int64_t* pool_tot;                    // [nb + 1] pool rows per sample, then their prefix
     int64_t* level_cnt;                   // [K][4][nb] nodes per (level, local state, sample)
     int64_t* level_off;                   // their exclusive prefix (one more entry)
-    uint32_t* items;                      // node ids by (level, local state)
+    uint32_t* items;                      // by (level, local state), see TreeLevels
     uint32_t pool0;                       // first pool row after the roots' rows [nb][K]
+};
+
+// Items of the levels: level t holds n[t] of them from `at[t]` of the items,
+// first[t] before it in level_off's numbering. With sources, an item is the
+// pool row its state goes to (level K - 1: its node) and, in n[t]-long arrays
+// behind, the pool row of every vertex source of t's in-edges; else its node.
+struct TreeLevels {
+    uint32_t at[kMaxOrb], first[kMaxOrb], n[kMaxOrb];
+    int sources;
 };
 
 // rows of every sample (deterministic + drawn)
@@ -55,7 +65,7 @@ int launch_tree_row_counts(const int64_t* det_cnt, const int64_t* draw_cnt, int6
 // words, marks and nodes of the batch; fills pool_tot and level_cnt
 int launch_tree_nodes(const TreeArgs& a, int64_t max_chunks, cudaStream_t st);
 // pool rows of the nodes (pool_tot scanned) and the items (level_off scanned)
-int launch_tree_items(const TreeArgs& a, cudaStream_t st);
+int launch_tree_items(const TreeArgs& a, const TreeLevels& lv, const int* pred_ptr, const int* pred_idx, cudaStream_t st);
 
 // ---- node evaluations -------------------------------------------------------
 
@@ -64,11 +74,10 @@ int launch_tree_items(const TreeArgs& a, cudaStream_t st);
 struct TreeGraph64 {
     AnsatzView an;                        // with the edge lists (a chain's too)
     const uint32_t* items;
-    const uint32_t* parent; const uint32_t* start; const uint32_t* base;
     double* pool;                         // [rows][D]
     int* pool_e;                          // [rows]
 };
-int launch_tree_graph64(const TreeGraph64& a, int t, const int64_t* bounds, cudaStream_t st);
+int launch_tree_graph64(const TreeGraph64& a, int t, const TreeLevels& lv, const int64_t* bounds, cudaStream_t st);
 
 // Covectors that close a row at its last changed vertex: for each (q,
 // alternative a) and each vertex j < q read at or after q, Q_j with
@@ -108,14 +117,14 @@ int launch_tree_rows64(const TreeRows64& a, int64_t max_chunks, cudaStream_t st)
 struct TreeGraphTc {
     AnsatzView an;
     const uint32_t* items;
-    const uint32_t* parent; const uint32_t* start; const uint32_t* base;
     unsigned char* pool;                  // [rows][hi D | lo D] FP16
     int* pool_e;
     const unsigned char* bimg; const int* bexp; const float* col0;
     float* mant; int* mexp;               // [nodes] psi_TN of the nodes of level K - 1
     DevError* err;
 };
-int launch_tree_graph_tc(const TreeGraphTc& a, int t, int deg, const int64_t* bounds, int n_sm, cudaStream_t st);
+int launch_tree_graph_tc(const TreeGraphTc& a, int t, int deg, const TreeLevels& lv, const int64_t* bounds, int n_sm,
+                         cudaStream_t st);
 
 struct TreeRowsTc {
     TreeArgs t;
@@ -125,7 +134,7 @@ struct TreeRowsTc {
     const double* psi_mant; const int* psi_exp;
     double* partial; double* partial_abs; int64_t* span; int64_t* mv;
 };
-int launch_tree_rows_tc(const TreeRowsTc& a, int64_t max_chunks, cudaStream_t st);
+int launch_tree_rows_tc(const TreeRowsTc& a, int64_t max_chunks, int n_sm, cudaStream_t st);
 // split images and exponents of the roots' states into the pool, tanh theta
 int launch_tree_graph_prep(const double* Hst, const int* Hexp, const double* theta, int64_t s0, int nb, int K, int D,
                            int NH, int NP, int corr, unsigned char* pool, int* pool_e, float* tts, cudaStream_t st);
@@ -151,5 +160,87 @@ struct TreeRowsRnn {
     double* partial; int64_t* span;
 };
 int launch_tree_rows_rnn(const TreeRowsRnn& a, int64_t max_chunks, cudaStream_t st);
+
+// ---- shared device helpers ---------------------------------------------------
+
+constexpr uint32_t kNoNode = 0xffffffffu;
+
+// sample (call index) of chunk b of the batch, -1 past its end
+__device__ __forceinline__ int64_t tree_sample(const TreeArgs& a, int64_t b)
+{
+    if (b >= a.chunk_base[a.s0 + a.nb]) return -1;
+    int64_t lo = a.s0, hi = a.s0 + a.nb - 1;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi + 1) >> 1;
+        if (a.chunk_base[mid] <= b) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
+struct TreeWord {
+    int c;                    // changes
+    int x[4];
+};
+
+__device__ __forceinline__ TreeWord tree_unpack(uint32_t w)
+{
+    TreeWord r;
+    for (int k = 0; k < 4; ++k) r.x[k] = (int)((w >> (8 * k)) & 255u);
+    r.c = r.x[1] == r.x[0] ? 1 : (r.x[2] == r.x[1] ? 2 : (r.x[3] == r.x[2] ? 3 : 4));
+    return r;
+}
+
+// pool row of vertex j's state seen from a node of batch sample sl (the node or
+// an ancestor of it that lived at level j)
+__device__ __forceinline__ uint32_t tree_source(const TreeArgs& a, int sl, uint32_t node, int j)
+{
+    int p = (int)(__ldg(a.start + node) & 255u);
+    while (p > j) {
+        node = __ldg(a.parent + node);
+        p = (int)(__ldg(a.start + node) & 255u);
+    }
+    return __ldg(a.base + node) + (uint32_t)(j - p) + (node < a.id1 ? 0u : a.pool0 + (uint32_t)a.pool_tot[sl]);
+}
+
+// x 2^e with the exponent field where the result stays normal
+__device__ __forceinline__ double scale_pow2(double x, int e)
+{
+    const long long bits = __double_as_longlong(x);
+    const int ex = (int)((bits >> 52) & 0x7FF), ne = ex + e;
+    if (ex != 0 && ex != 0x7FF && ne > 0 && ne < 0x7FF) return __longlong_as_double(bits + ((long long)e << 52));
+    return ldexp(x, e);
+}
+
+// determinant of a row from its word
+__device__ __forceinline__ void tree_det(const TreeWord& w, uint64_t na, uint64_t nb, uint64_t& ma, uint64_t& mb)
+{
+    ma = na;
+    mb = nb;
+    for (int k = 0; k < w.c; ++k) {
+        const int p = w.x[k] / 3, sg = tree_alt_state(sigma_at(na, nb, p), w.x[k] - 3 * p);
+        ma = (ma & ~(1ull << p)) | ((uint64_t)(sg & 1) << p);
+        mb = (mb & ~(1ull << p)) | ((uint64_t)(sg >> 1) << p);
+    }
+}
+
+__device__ __forceinline__ double tree_coef(const TreeArgs& t, int64_t s, int64_t r)
+{
+    const int64_t nd = t.det_cnt[s];
+    return r < nd ? t.det_coef[t.det_off[s] + r] : t.draw_coef[s * t.draw_stride + (r - nd)];
+}
+
+struct TreeGroups {
+    uint32_t b[5];            // item bounds of the four local states within the level
+    int tile[5];              // their tiles
+};
+
+inline TreeGroups tree_groups(int t, const int64_t* bounds, int rows)
+{
+    TreeGroups g;
+    g.tile[0] = 0;
+    for (int k = 0; k < 5; ++k) g.b[k] = (uint32_t)(bounds[4 * t + k] - bounds[4 * t]);
+    for (int k = 0; k < 4; ++k) g.tile[k + 1] = g.tile[k] + (int)((g.b[k + 1] - g.b[k] + rows - 1) / rows);
+    return g;
+}
 
 }  // namespace nqs
