@@ -745,14 +745,31 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
     const bool full = kind != kTreeGraph64;
     const int stage = NQS_STAGE_AMP_DET;
     StageScope sc(c, stage);
-    TRY(ensure(c, c->tr_rows, (size_t)(2 * Ns + 1) * 8));
+    TRY(ensure(c, c->tr_rows, (size_t)(3 * Ns + 2) * 8));
     TRY(ensure(c, c->base_det, (size_t)(Ns + 1) * 8));
     int64_t* row_cnt = (int64_t*)c->tr_rows.p;
     int64_t* row_base = row_cnt + Ns;
     const int64_t* dcnt = n_draws > 0 ? (const int64_t*)c->n_unique.p : nullptr;
     LAUNCH(stage, launch_tree_row_counts((const int64_t*)c->det_tot.p, dcnt, Ns, row_cnt, c->stream));
     LAUNCH(stage, launch_scan_i64(row_cnt, row_base, Ns, c->stream));
-    LAUNCH(stage, launch_chunk_base(row_cnt, kTreeRows, (int64_t*)c->base_det.p, Ns, c->stream));
+    // the FP64 forms sum a sample's rows together, the mixed form the deterministic
+    // and the drawn rows apart
+    const bool apart = kind == kTreeGraphTc;
+    int64_t* chunk_base = apart ? row_base + Ns + 1 : (int64_t*)c->base_det.p;
+    LAUNCH(stage, launch_chunk_base(row_cnt, kTreeRows, chunk_base, Ns, c->stream));
+    const int64_t det_chunks = total_det / kTreeRows + Ns;
+    const int64_t draw_chunks = Ns * (((int64_t)n_draws + kTreeRows - 1) / kTreeRows);
+    if (apart) {
+        LAUNCH(stage, launch_chunk_base((const int64_t*)c->det_tot.p, kTreeRows, (int64_t*)c->base_det.p, Ns, c->stream));
+        if (n_draws > 0) {
+            TRY(ensure(c, c->base_draw, (size_t)(Ns + 1) * 8));
+            TRY(ensure(c, c->part_draw, (size_t)(draw_chunks + 1) * 8));
+            TRY(ensure(c, c->span_draw, (size_t)(draw_chunks + 1) * 8));
+            TRY(ensure(c, c->mv_draw, (size_t)(draw_chunks + 1) * 8));
+            if (want_abs) TRY(ensure(c, c->part_draw_abs, (size_t)(draw_chunks + 1) * 8));
+            LAUNCH(stage, launch_chunk_base(dcnt, kTreeRows, (int64_t*)c->base_draw.p, Ns, c->stream));
+        }
+    }
     const int64_t rows_bound = total_det + Ns * (int64_t)n_draws;
     const int64_t chunks_all = rows_bound / kTreeRows + Ns;
     TRY(ensure(c, c->part_det, (size_t)(chunks_all + 1) * 8));
@@ -810,7 +827,7 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
             a.draw_coef = (const double*)c->draw_coef.p;
         }
         a.row_base = row_base;
-        a.chunk_base = (const int64_t*)c->base_det.p;
+        a.chunk_base = chunk_base;
         a.n2max = n2max;
         a.W = W;
         a.pool0 = kind == kTreeRnn ? 0u : (uint32_t)nb * (uint32_t)K;
@@ -825,6 +842,7 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
         int64_t *scan_tmp = nullptr, *pool_off = nullptr;
         float* mant = nullptr;
         int* mexp = nullptr;
+        uint32_t* perm = nullptr;
         TreeRnn rn{};
         for (int pass = 0; pass < 2; ++pass) {
             Carve v{pass ? (char*)c->tr_build.p : nullptr};
@@ -848,6 +866,7 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
             if (kind == kTreeGraphTc) {
                 mant = v.take<float>((size_t)nodes);
                 mexp = v.take<int>((size_t)nodes);
+                perm = v.take<uint32_t>((size_t)R + 1);
             }
             if (kind == kTreeRnn) {
                 rn.cell = v.take<double>((size_t)2 * nodes * D);
@@ -990,11 +1009,39 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
             r.np = np;
             r.psi_mant = (const double*)c->pmant.p;
             r.psi_exp = (const int*)c->pexp.p;
+            LAUNCH(stage, launch_tree_perm(a, perm, c->stream));
+            r.perm = perm;
+            r.chunk_base = (const int64_t*)c->base_det.p;
             r.partial = (double*)c->part_det.p;
             r.partial_abs = want_abs ? (double*)c->part_det_abs.p : nullptr;
             r.span = (int64_t*)c->span_det.p;
             r.mv = (int64_t*)c->mv_det.p;
-            LAUNCH(stage, launch_tree_rows_tc(r, max_chunks, c->n_sm, c->stream));
+            LAUNCH(stage, launch_tree_rows_tc(r, det_chunks, c->n_sm, c->stream));
+            if (n_draws > 0) {
+                r.draws = 1;
+                r.chunk_base = (const int64_t*)c->base_draw.p;
+                r.partial = (double*)c->part_draw.p;
+                r.partial_abs = want_abs ? (double*)c->part_draw_abs.p : nullptr;
+                r.span = (int64_t*)c->span_draw.p;
+                r.mv = (int64_t*)c->mv_draw.p;
+                LAUNCH(stage, launch_tree_rows_tc(r, draw_chunks, c->n_sm, c->stream));
+            }
+        }
+        if (kind == kTreeRnn) {
+            rn.an = c->av;
+            rn.t = a;
+            rn.n_nodes = (uint32_t)nodes;
+            rn.cells = (const double*)c->rnn_cells.p;
+            for (int t = 0; t < K; ++t) LAUNCH(stage, launch_tree_rnn(rn, t, lv, bounds.data(), c->n_sm, c->stream));
+            TreeRowsRnn r{};
+            r.r = rn;
+            r.lp = (const double*)c->rnn_lp.p;
+            r.sg = (const int8_t*)c->rnn_sg.p;
+            r.theta = (const double*)c->theta.p;
+            r.lc = (const double*)c->lc.p;
+            r.partial = (double*)c->part_det.p;
+            r.span = (int64_t*)c->span_det.p;
+            LAUNCH(stage, launch_tree_rows_rnn(r, max_chunks, c->stream));
         }
         CK(cudaGetLastError());
         s0 = s1;
@@ -1655,7 +1702,8 @@ int le_core(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, uint64
     // the plain FP64 form: psi is linear in the states without the tensor term, so
     // the rows share prefixes and close with n's adjoints (the tensor term's are re-run)
     const bool tree64 = !rnn && !gtc && !shared && !c->av.tk_rank;
-    const bool tree = tree64 || gtc;
+    const bool tree_rnn = rnn && c->av.chain && c->av.D <= kTreeRnnMaxD;
+    const bool tree = tree64 || gtc || tree_rnn;
     if (!c->av.chain && prec == NQS_PREC_FP64_SHARED)
         return set_err(c, NQS_ERR_UNSUPPORTED,
                        "graph ansatze have no shared-prefix form (NQS_PREC_FP64 or NQS_PREC_MIXED)");
@@ -1720,7 +1768,8 @@ int le_core(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, uint64
         if (prec == NQS_PREC_MIXED) TRY(family_pass<float>(c, ds, Ns, total, n_draws, deabs != nullptr));
         else TRY(family_pass<double>(c, ds, Ns, total, n_draws, deabs != nullptr));
     } else if (tree) {
-        TRY(tree_pass(c, ds, Ns, total, n_draws, gtc ? kTreeGraphTc : kTreeGraph64, deabs != nullptr));
+        TRY(tree_pass(c, ds, Ns, total, n_draws, tree_rnn ? kTreeRnn : gtc ? kTreeGraphTc : kTreeGraph64,
+                      deabs != nullptr));
     } else {
         // amplitudes: deterministic rows, then the distinct drawn rows
         RowSet rd{};
@@ -1741,7 +1790,7 @@ int le_core(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, uint64
         }
     }
     TRY(ensure(c, c->summary, kSummaryDoubles * 8));
-    const bool draws_apart = n_draws > 0 && !tree;     // drawn rows in their own partial sums
+    const bool draws_apart = n_draws > 0 && (!tree || gtc);     // drawn rows in their own partial sums
     FinalArgs f{};
     f.Ns = Ns;
     f.h_diag = (const double*)c->hdiag.p;

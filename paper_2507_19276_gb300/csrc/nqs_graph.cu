@@ -342,19 +342,20 @@ __global__ void __launch_bounds__(kTreeRows) k_tree_rows_tc(TreeRowsTc a)
         const int k = q / (2 * K), f = q - k * 2 * K;
         WTs[q] = a.WT[(size_t)f * NP + k];
     }
-    const int64_t b0 = t.chunk_base[t.s0], b1 = t.chunk_base[t.s0 + t.nb];
+    const int64_t b0 = a.chunk_base[t.s0], b1 = a.chunk_base[t.s0 + t.nb];
     for (int64_t b = b0 + blockIdx.x; b < b1; b += gridDim.x) {
         __syncthreads();
-        if (tid == 0) s_s = tree_sample(t, b);
+        if (tid == 0) s_s = tree_sample(t, a.chunk_base, b);
         __syncthreads();
         const int64_t s = s_s;
         const uint64_t na = t.samples[2 * s], nb = t.samples[2 * s + 1];
-        const int64_t r0 = (b - t.chunk_base[s]) * kTreeRows;
-        const int64_t left = t.row_base[s + 1] - t.row_base[s] - r0;
+        const int64_t r0 = (b - a.chunk_base[s]) * kTreeRows, rb = t.row_base[s] - t.row_base[t.s0];
+        const int64_t first = a.draws ? t.det_cnt[s] : 0;
+        const int64_t left = (a.draws ? t.draw_cnt[s] : t.det_cnt[s]) - r0;
         double term = 0.0, ab = 0.0;
         int sp = 0, mv = 0;
         if (tid < left) {
-            const int64_t g = t.row_base[s] - t.row_base[t.s0] + r0 + tid;
+            const int64_t row = a.perm[rb + first + r0 + tid], g = rb + row;
             const TreeWord w = tree_unpack(t.word[g]);
             const uint32_t node = t.rnode[g];
             uint64_t ma, mb;
@@ -415,7 +416,7 @@ __global__ void __launch_bounds__(kTreeRows) k_tree_rows_tc(TreeRowsTc a)
             const float X = fmaf(X2[0], X2[1], X2[0] + X2[1]);
             const double rpsi = 1.0 / a.psi_mant[s];
             const double tn = scale_pow2((double)a.mant[node] * rpsi, a.mexp[node] - a.psi_exp[s]);
-            term = tree_coef(t, s, r0 + tid) * tn * (1.0 + (double)X);
+            term = tree_coef(t, s, row) * tn * (1.0 + (double)X);
             ab = fabs(term);
             const int p = w.x[0] / 3;
             sp = K - p;

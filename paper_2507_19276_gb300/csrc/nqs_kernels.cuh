@@ -122,7 +122,7 @@ int launch_ansatz_forms(const AnsatzForms& f, cudaStream_t st);
 int launch_corr_transpose(const double* W, int n_hidden, int np, int K2, float* WTf, cudaStream_t st);
 
 constexpr int kSummaryBlocks = 128;
-constexpr int kSummaryDoubles = 8 + 9 * kSummaryBlocks;
+constexpr int kSummaryDoubles = 8 + 2 * kSummaryBlocks;
 
 struct FinalArgs {
     int64_t Ns;
@@ -141,7 +141,7 @@ struct FinalArgs {
     const int64_t* span_det;             // [chunks] from the amplitude kernels
     const int64_t* span_draw;
     double* summary;                     // [8] e_mean, sum_c, log_B, e_tilde_mean, n_det, n_uniq, span,
-                                         // products; then the blocks' partial sums (kSummaryDoubles)
+                                         // products; then the blocks' counts (kSummaryDoubles)
     const double* part_det_abs;          // chunk sums of |term| (NULL: no e_abs)
     const double* part_draw_abs;
     double* e_abs;                       // [Ns] |H_nn| + sum |terms| (optional)

@@ -9,8 +9,9 @@
 // still allows, and Phi(n) = prod_i sqrt(P~_i(s_i)) sign(w_i . h_i^{s_i} + c_i).
 //
 // Local energy: a connected m shares n's prefix up to its first changed
-// vertex p, so its cells and conditionals agree with n's below p; the kernel
-// re-runs vertices p..K-1 for m (one warp per row) and divides by n's suffix
+// vertex p, so its cells and conditionals agree with n's below p; vertices
+// p..K-1 are re-run for m (chains up to D = 32 over prefix trees, k_tree_rnn;
+// else one warp per row, k_rnn_amp) and divided by n's suffix
 // of conditionals and signs. The normalisers depend on the whole prefix, so
 // there is no right environment: the cost per amplitude is (K - p) x 4 cell
 // products.
@@ -22,7 +23,9 @@
 // as the first allowed s with u_j Z < sum_{allowed s' <= s} P_i(s') (the last
 // allowed state when rounding leaves none); the children keep the offsets in
 // the order of s, so the result does not depend on how nodes are scheduled.
-#include "nqs_kernels.cuh"
+#include "nqs_tree.cuh"
+
+#include <algorithm>
 
 namespace nqs {
 
@@ -262,167 +265,217 @@ __global__ void __launch_bounds__(256) k_rnn_amp(RnnAmpArgs a)
     }
 }
 
-// Chain readout, the block's 32 rows in lockstep over the vertices: per vertex
-// the four site matrices are staged once in shared memory for every row, the
-// 4 D candidate entries of all rows spread over the block (four independent
-// FMA chains each), then one thread per (row, local state) forms P and one
-// thread per row the normaliser, the choice and the phase. The arithmetic of
-// each row is that of k_rnn_amp up to the order of the sums.
-constexpr int kRnnChainMaxD = 32;
+// ---------------------------------------------------------------------------
+// Chain readout over the prefix trees (nqs_tree.cu): one launch per vertex
+// advances every node of its level. The normalisers depend on the whole prefix,
+// so every row is continued to the last vertex; what rows share is the part up
+// to their third change (H50 at eps = 0.01: 444 000 instead of 908 000 vertex
+// updates per sample). FP64 bounds it (4 D^2 + 8 D operations per update at two
+// per clock and SM): the vertex's four matrices sit in shared memory, each
+// thread holds one candidate entry of four nodes, a thread per (node, local
+// state) forms P, a thread per node the normaliser and the choice. The weight
+// is kept as a product of P / Z (one division per update) instead of a sum of
+// logarithms (two logs, a tenth of the operations at D = 10). The 32-row blocks
+// that re-ran every row took 420 ms for 300 H50 samples (chi = 10).
+// ---------------------------------------------------------------------------
 
-__global__ void __launch_bounds__(256) k_rnn_amp_chain(RnnAmpArgs a)
+constexpr double kProdLow = 0x1p-500;
+
+__global__ void __launch_bounds__(256) k_tree_rnn(TreeRnn a, int t, uint32_t at, uint32_t nl, TreeGroups gr, int IT)
 {
     extern __shared__ double sm[];
-    __shared__ OrbLists lists;
-    __shared__ uint64_t s_ma[kRnnRows], s_mb[kRnnRows];
-    __shared__ int s_p[kRnnRows], s_nad[kRnnRows], s_nbd[kRnnRows], s_odd[kRnnRows], s_ok[kRnnRows];
-    __shared__ int s_sig[kRnnRows];
-    __shared__ double s_lpm[kRnnRows], s_term[kRnnRows];
-    __shared__ int s_tmin;
+    __shared__ const double* s_src[64];
+    __shared__ double s_prod[64];
+    __shared__ int s_pex[64], s_sig[64];
+    __shared__ uint32_t s_flag[64], s_node[64];
     const AnsatzView& an = a.an;
-    const int K = an.K, D = an.D;
-    const int64_t b = blockIdx.x;
-    const int64_t* cb = a.rows.chunk_base;
-    if (b >= cb[a.Ns]) return;
-    int64_t lo = 0, hi = a.Ns - 1;                  // largest s with cb[s] <= b
-    while (lo < hi) {
-        const int64_t mid = (lo + hi + 1) >> 1;
-        if (cb[mid] <= b) lo = mid; else hi = mid - 1;
-    }
-    const int64_t s = lo;
-    const int64_t j = b - cb[s];
-    const int64_t beg = a.rows.begin ? a.rows.begin[s] : s * a.rows.stride;
-    const int64_t cnt = a.rows.count[s];
-    const int64_t r0 = beg + j * kRnnRows;
-    const int nr = (int)((cnt - j * kRnnRows) < kRnnRows ? (cnt - j * kRnnRows) : kRnnRows);
-    const uint64_t na = a.samples[2 * s], nb = a.samples[2 * s + 1];
-    const int tid = threadIdx.x, nt = blockDim.x;
-    double* AT4 = sm;                                // [4][D][D]: AT4[s][c][a] = M_t^s[a][c]
-    double* cell = AT4 + (size_t)4 * D * D;          // [R][D] each row's previous cell
-    double* cand = cell + (size_t)kRnnRows * D;      // [R][4][D]
-    double* Pv = cand + (size_t)kRnnRows * 4 * D;    // [R][4]
-    if (tid < 32) build_lists_warp(na, nb, a.h.K, lists, tid);
-    if (tid == 0) s_tmin = K;
-    __syncthreads();
-    if (tid < nr) {
-        const Exc e = decode_rank<false>(a.h, lists, a.rows.rank[r0 + tid]);   // sites only
-        uint64_t ma = na, mb = nb;
-        flip(ma, mb, e.i); flip(ma, mb, e.a);
-        if (e.kind == 2) { flip(ma, mb, e.j); flip(ma, mb, e.b); }
-        const int p = __ffsll((long long)((na ^ ma) | (nb ^ mb))) - 1;
-        s_ma[tid] = ma; s_mb[tid] = mb; s_p[tid] = p;
-        s_nad[tid] = __popcll(na & low_mask(p));
-        s_nbd[tid] = __popcll(nb & low_mask(p));
-        s_odd[tid] = 0; s_ok[tid] = 1; s_lpm[tid] = 0.0;
-        atomicMin(&s_tmin, p);
-    }
-    __syncthreads();
-    const double* cn = a.cells + (size_t)s * K * D;  // n's cells
-    for (int t = s_tmin; t < K; ++t) {
-        // the site matrices of vertex t, and the previous cell of the rows entering at t
-        const double* ATg = an.AT + (size_t)t * 4 * D * D;
-        for (int q = tid; q < 4 * D * D; q += nt) AT4[q] = __ldg(ATg + q);
-        for (int q = tid; q < nr * D; q += nt) {
-            const int r = q / D, c = q - r * D;
-            if (s_p[r] == t) cell[q] = t == 0 ? (c == 0 ? 1.0 : 0.0) : cn[(size_t)(t - 1) * D + c];
-        }
+    const int K = an.K, D = an.D, DP = D | 1;        // padded rows: no bank conflicts across nodes
+    double* AT4 = sm;                                // [4][D][D]: AT4[s][k][c] = M^s[c][k]
+    double* rv = AT4 + (size_t)4 * D * D;            // [4][D]
+    double* eta = rv + 4 * D;                        // [D]
+    double* rw = eta + D;                            // [D]
+    double* xs = rw + D;                             // [IT][D] the nodes' previous cells
+    double* cand = xs + (size_t)IT * D;              // [IT][4][DP]
+    double* Pv = cand + (size_t)IT * 4 * DP;         // [IT][4]
+    const int tid = threadIdx.x;
+    for (int q = tid; q < 4 * D * D; q += 256) AT4[q] = __ldg(an.AT + (size_t)t * 4 * D * D + q);
+    for (int q = tid; q < 4 * D; q += 256) rv[q] = __ldg(an.rv + (size_t)t * 4 * D + q);
+    for (int q = tid; q < D; q += 256) { eta[q] = __ldg(an.reta + (size_t)t * D + q); rw[q] = __ldg(an.rw + (size_t)t * D + q); }
+    const double rc = __ldg(an.rc + t);
+    const size_t cur = (size_t)(t & 1) * a.n_nodes, prv = (size_t)((t & 1) ^ 1) * a.n_nodes;
+    const uint32_t nt = (nl + IT - 1) / IT;
+    for (uint32_t tile = blockIdx.x; tile < nt; tile += gridDim.x) {
+        const uint32_t i0 = tile * (uint32_t)IT;
+        const int n = (int)min(nl - i0, (uint32_t)IT);
         __syncthreads();
-        for (int q = tid; q < nr * 4 * D; q += nt) {
-            const int r = q / (4 * D), sa = q - r * 4 * D, sg = sa / D, c = sa - sg * D;
-            if (t < s_p[r]) continue;
-            const double* M = AT4 + (size_t)sg * D * D;
-            const double* h = cell + (size_t)r * D;
-            double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-            int k = 0;
-            for (; k + 3 < D; k += 4) {
-                s0 = fma(M[(size_t)k * D + c], h[k], s0);
-                s1 = fma(M[(size_t)(k + 1) * D + c], h[k + 1], s1);
-                s2 = fma(M[(size_t)(k + 2) * D + c], h[k + 2], s2);
-                s3 = fma(M[(size_t)(k + 3) * D + c], h[k + 3], s3);
+        if (tid < n) {
+            const uint32_t i = i0 + tid, node = __ldg(a.t.items + at + i);
+            s_node[tid] = node;
+            s_sig[tid] = (i >= gr.b[1]) + (i >= gr.b[2]) + (i >= gr.b[3]);
+            uint32_t src = node;
+            if ((int)(a.t.start[node] & 255u) == t) src = a.t.parent[node];
+            if (src < a.t.id1) {                     // n itself up to here
+                const int64_t s = a.t.s0 + src;
+                const uint64_t na = a.t.samples[2 * s], nb = a.t.samples[2 * s + 1];
+                s_src[tid] = t > 0 ? a.cells + ((size_t)s * K + t - 1) * D : nullptr;
+                s_prod[tid] = 1.0;
+                s_pex[tid] = 0;
+                s_flag[tid] = (uint32_t)__popcll(na & low_mask(t)) | ((uint32_t)__popcll(nb & low_mask(t)) << 8);
+            } else {
+                s_src[tid] = a.cell + (prv + src) * D;
+                s_prod[tid] = a.prod[prv + src];
+                s_pex[tid] = a.pex[prv + src];
+                s_flag[tid] = a.flag[prv + src];
             }
-            for (; k < D; ++k) s0 = fma(M[(size_t)k * D + c], h[k], s0);
-            cand[q] = __ldg(an.rv + ((size_t)t * 4 + sg) * D + c) + ((s0 + s1) + (s2 + s3));
         }
         __syncthreads();
-        for (int q = tid; q < nr * 4; q += nt) {
-            const int r = q >> 2, sg = q & 3;
-            if (t < s_p[r]) continue;
-            const double* h = cand + (size_t)(r * 4 + sg) * D;
+        for (int q = tid; q < n * D; q += 256) {
+            const int it = q / D, c = q - it * D;
+            const double* src = s_src[it];
+            xs[q] = src ? src[c] : (c == 0 ? 1.0 : 0.0);       // h_{-1} = e_0
+        }
+        __syncthreads();
+        for (int q = tid; q < (IT / 4) * 4 * D; q += 256) {
+            const int it = 4 * (q / (4 * D)), sc = q - it * D, sg = sc / D, c = sc - sg * D;
+            if (it >= n) continue;
+            const double* M = AT4 + (size_t)sg * D * D + c;
+            const double* x = xs + (size_t)it * D;   // (rows past n hold older numbers, not used)
+            double acc[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int k = 0; k < D; ++k) {
+                const double m = M[(size_t)k * D];
+                #pragma unroll
+                for (int v = 0; v < 4; ++v) acc[v] = fma(m, x[v * D + k], acc[v]);
+            }
+            const double v0 = rv[sc];
+            #pragma unroll
+            for (int v = 0; v < 4; ++v) cand[((size_t)(it + v) * 4 + sg) * DP + c] = v0 + acc[v];
+        }
+        __syncthreads();
+        for (int q = tid; q < n * 4; q += 256) {
+            const double* h = cand + (size_t)q * DP;
             double p = 0.0;
-            for (int c = 0; c < D; ++c) p = fma(__ldg(an.reta + (size_t)t * D + c) * h[c], h[c], p);
+            for (int c = 0; c < D; ++c) p = fma(eta[c] * h[c], h[c], p);
             Pv[q] = p;
         }
         __syncthreads();
-        if (tid < nr && t >= s_p[tid]) {
-            const int r = tid, sg = sigma_at(s_ma[r], s_mb[r], t);
+        if (tid < n) {
+            const int sg = s_sig[tid];
+            uint32_t f = s_flag[tid];
+            const int nad = (int)(f & 255u), nbd = (int)((f >> 8) & 255u);
             double Z = 0.0;
             for (int q = 0; q < 4; ++q)
-                if (rnn_allowed(an, t, s_nad[r], s_nbd[r], q)) Z += Pv[r * 4 + q];
-            const double P = Pv[r * 4 + sg];
-            double ph = __ldg(an.rc + t);
-            const double* h = cand + (size_t)(r * 4 + sg) * D;
-            for (int c = 0; c < D; ++c) ph = fma(__ldg(an.rw + (size_t)t * D + c), h[c], ph);
-            if (!rnn_allowed(an, t, s_nad[r], s_nbd[r], sg) || !(P > 0.0) || !(Z > 0.0)) s_ok[r] = 0;
+                if (rnn_allowed(an, t, nad, nbd, q)) Z += Pv[tid * 4 + q];
+            const double P = Pv[tid * 4 + sg];
+            const double* h = cand + (size_t)(tid * 4 + sg) * DP;
+            double ph = rc;
+            for (int c = 0; c < D; ++c) ph = fma(rw[c], h[c], ph);
+            double prod = s_prod[tid];
+            int pex = s_pex[tid];
+            if (!rnn_allowed(an, t, nad, nbd, sg) || !(P > 0.0) || !(Z > 0.0)) f |= 1u << 17;
             else {
-                s_lpm[r] += 0.5 * (log(P) - log(Z));
-                s_odd[r] ^= ph < 0.0;
+                prod *= P / Z;
+                if (prod < kProdLow) { prod *= 0x1p500; --pex; }
+                f ^= ph < 0.0 ? 1u << 16 : 0u;
             }
-            s_sig[r] = sg;
-            s_nad[r] += sg & 1;
-            s_nbd[r] += sg >> 1;
+            f += (uint32_t)(sg & 1) + ((uint32_t)(sg >> 1) << 8);
+            const uint32_t node = s_node[tid];
+            a.prod[cur + node] = prod;
+            a.pex[cur + node] = pex;
+            a.flag[cur + node] = f;
         }
-        __syncthreads();
-        for (int q = tid; q < nr * D; q += nt) {
-            const int r = q / D, c = q - r * D;
-            if (t >= s_p[r]) cell[q] = cand[(size_t)(r * 4 + s_sig[r]) * D + c];
-        }
-        __syncthreads();
-    }
-    // n's suffix of conditionals and signs, the correlator ratio, the term (one warp per row)
-    const int warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
-    for (int r = warp; r < nr; r += nw) {
-        const int p = s_p[r];
-        double lpn = 0.0;
-        int oddn = 0;
-        for (int i = p + lane; i < K; i += 32) {
-            lpn += a.lp[(size_t)s * K + i];
-            oddn ^= a.sg[(size_t)s * K + i] < 0;
-        }
-        for (int o = 16; o; o >>= 1) {
-            lpn += __shfl_xor_sync(kFull, lpn, o);
-            oddn ^= __shfl_xor_sync(kFull, oddn, o);
-        }
-        int negf;
-        const double lr = corr_log_ratio_warp(an, s, a.theta, a.lc, na, nb, s_ma[r], s_mb[r], lane, &negf);
-        if (lane == 0) {
-            double tv = 0.0;
-            if (s_ok[r]) {
-                tv = a.rows.coef[r0 + r] * exp(s_lpm[r] - lpn + lr);
-                if (s_odd[r] ^ oddn ^ negf) tv = -tv;
+        if (t + 1 < K)
+            for (int q = tid; q < n * D; q += 256) {
+                const int it = q / D, c = q - it * D;
+                a.cell[(cur + s_node[it]) * D + c] = cand[(size_t)(it * 4 + s_sig[it]) * DP + c];
             }
-            s_term[r] = tv;
+    }
+}
+
+int launch_tree_rnn(const TreeRnn& a, int t, const TreeLevels& lv, const int64_t* bounds, int n_sm, cudaStream_t st)
+{
+    if (lv.n[t] == 0) return 0;
+    const int D = a.an.D, IT = D <= 16 ? 64 : 32;
+    const size_t smem = ((size_t)4 * D * D + 6 * D + (size_t)IT * D + (size_t)IT * 4 * (D | 1) + 4 * IT) * sizeof(double);
+    allow_max_smem(k_tree_rnn);
+    const uint32_t nt = (lv.n[t] + IT - 1) / IT;
+    const int per = std::max(1, std::min(6, (int)((200u << 10) / smem)));
+    k_tree_rnn<<<std::min<uint32_t>(nt, (uint32_t)(per * n_sm)), 256, smem, st>>>(a, t, lv.at[t], lv.n[t],
+                                                                              tree_groups(t, bounds, IT), IT);
+    return 1;
+}
+
+// Terms of the rows: a row's node holds its weight since the first change p, n's
+// is the sum of its conditionals from p on.
+__global__ void __launch_bounds__(kTreeRows) k_tree_rows_rnn(TreeRowsRnn a)
+{
+    __shared__ int64_t s_s;
+    __shared__ double s_lp[kMaxOrb + 1], s_lr[kTreeRows], wsum[4];
+    __shared__ int s_odd[kMaxOrb + 1], s_neg[kTreeRows], wspan[4];
+    const TreeArgs& t = a.r.t;
+    const AnsatzView& an = a.r.an;
+    const int K = an.K, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t b = t.chunk_base[t.s0] + blockIdx.x;
+    if (tid == 0) s_s = tree_sample(t, b);
+    __syncthreads();
+    const int64_t s = s_s;
+    if (s < 0) return;
+    const uint64_t na = t.samples[2 * s], nb = t.samples[2 * s + 1];
+    const int64_t r0 = (b - t.chunk_base[s]) * kTreeRows, g0 = t.row_base[s] - t.row_base[t.s0] + r0;
+    const int64_t left = t.row_base[s + 1] - t.row_base[s] - r0;
+    const int nr = (int)(left < kTreeRows ? left : kTreeRows);
+    if (tid <= K) {
+        double lp = 0.0;
+        int odd = 0;
+        for (int i = K - 1; i >= tid; --i) {
+            lp += a.lp[(size_t)s * K + i];
+            odd ^= a.sg[(size_t)s * K + i] < 0;
+        }
+        s_lp[tid] = lp;
+        s_odd[tid] = odd;
+    }
+    if (an.n_hidden > 0)
+        for (int rr = warp; rr < nr; rr += kTreeRows / 32) {
+            uint64_t ma, mb;
+            tree_det(tree_unpack(t.word[g0 + rr]), na, nb, ma, mb);
+            int neg;
+            const double lr = corr_log_ratio_warp(an, s, a.theta, a.lc, na, nb, ma, mb, lane, &neg);
+            if (lane == 0) { s_lr[rr] = lr; s_neg[rr] = neg; }
+        }
+    __syncthreads();
+    double term = 0.0;
+    int sp = 0;
+    if (tid < nr) {
+        const int p = (int)(t.word[g0 + tid] & 255u) / 3;
+        const size_t at = (size_t)((K - 1) & 1) * a.r.n_nodes + t.rnode[g0 + tid];
+        const uint32_t f = a.r.flag[at];
+        sp = K - p;
+        if (!((f >> 17) & 1u)) {
+            const double lpm = 0.5 * (log(a.r.prod[at]) + (500.0 * 0.69314718055994530942) * a.r.pex[at]);
+            term = tree_coef(t, s, r0 + tid) * exp(lpm - s_lp[p] + (an.n_hidden > 0 ? s_lr[tid] : 0.0));
+            const int neg = (int)((f >> 16) & 1u) ^ s_odd[p] ^ (an.n_hidden > 0 ? s_neg[tid] : 0);
+            if (neg) term = -term;
         }
     }
+    term = warp_sum_f64(term);
+    sp = (int)__reduce_add_sync(kFull, (unsigned)sp);
+    if (lane == 0) { wsum[warp] = term; wspan[warp] = sp; }
     __syncthreads();
     if (tid == 0) {
-        double acc = 0.0;
-        int64_t sp = 0;
-        for (int r = 0; r < nr; ++r) { acc += s_term[r]; sp += K - s_p[r]; }
-        a.partial[b] = acc;
-        if (a.span) a.span[b] = sp;
+        a.partial[b] = ((wsum[0] + wsum[1]) + wsum[2]) + wsum[3];
+        if (a.span) a.span[b] = wspan[0] + wspan[1] + wspan[2] + wspan[3];
     }
+}
+
+int launch_tree_rows_rnn(const TreeRowsRnn& a, int64_t max_chunks, cudaStream_t st)
+{
+    if (max_chunks == 0) return 0;
+    k_tree_rows_rnn<<<(unsigned)max_chunks, kTreeRows, 0, st>>>(a);
+    return 1;
 }
 
 int launch_rnn_amp(const RnnAmpArgs& a, cudaStream_t st)
 {
     if (a.rows.max_chunks == 0) return 0;
-    if (a.an.chain && a.an.D <= kRnnChainMaxD) {
-        const int D = a.an.D;
-        const size_t smem = ((size_t)4 * D * D + (size_t)kRnnRows * D * 5 + (size_t)kRnnRows * 4) * sizeof(double);
-        allow_max_smem(k_rnn_amp_chain);
-        k_rnn_amp_chain<<<(unsigned)a.rows.max_chunks, 256, smem, st>>>(a);
-        return 1;
-    }
     const int w = rnn_warps(a.an);
     const size_t smem = (size_t)w * ((a.an.K + 4) * a.an.D + a.an.tk_zy) * sizeof(double);
     allow_max_smem(k_rnn_amp);

@@ -403,6 +403,55 @@ __global__ void __launch_bounds__(512) k_tree_items(TreeArgs a, TreeLevels lv, c
     }
 }
 
+// Stable counting sort by the first changed vertex, one block per (sample, kind
+// of row): the order in which the mixed form adds its terms.
+__global__ void __launch_bounds__(256) k_tree_perm(TreeArgs a, uint32_t* perm)
+{
+    __shared__ int off[kMaxOrb];                  // next position of each vertex
+    __shared__ int wc[8][kMaxOrb];                // per-warp counts of the current 256 rows
+    const int64_t s = a.s0 + blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nd = (int)a.det_cnt[s], all = (int)(a.row_base[s + 1] - a.row_base[s]);
+    const int r0 = blockIdx.y ? nd : 0, cnt = blockIdx.y ? all - nd : nd;
+    const uint32_t* word = a.word + (a.row_base[s] - a.row_base[a.s0]) + r0;
+    perm += (a.row_base[s] - a.row_base[a.s0]) + r0;
+    for (int q = tid; q < 8 * kMaxOrb; q += 256) (&wc[0][0])[q] = 0;
+    if (tid < kMaxOrb) off[tid] = 0;
+    __syncthreads();
+    for (int c0 = 0; c0 < cnt; c0 += 256) {
+        const int p = c0 + tid < cnt ? (int)(word[c0 + tid] & 255u) / 3 : -1;
+        const unsigned m = __match_any_sync(kFull, p);
+        if (p >= 0 && lane == __ffs((int)m) - 1) atomicAdd(&off[p], __popc(m));
+    }
+    __syncthreads();
+    if (tid == 0) {
+        int acc = 0;
+        for (int v = 0; v < a.K; ++v) { const int c = off[v]; off[v] = acc; acc += c; }
+    }
+    __syncthreads();
+    const unsigned below = (1u << lane) - 1u;
+    for (int c0 = 0; c0 < cnt; c0 += 256) {
+        const int r = c0 + tid;
+        const bool valid = r < cnt;
+        const int p = valid ? (int)(word[r] & 255u) / 3 : -1;
+        const unsigned m = __match_any_sync(kFull, p);
+        if (valid && lane == __ffs((int)m) - 1) wc[warp][p] = __popc(m);
+        __syncthreads();
+        if (valid) {
+            int pos = off[p] + __popc(m & below);
+            for (int w = 0; w < warp; ++w) pos += wc[w][p];
+            perm[pos] = (uint32_t)(r0 + r);
+        }
+        __syncthreads();
+        if (tid < a.K) {
+            int t = 0;
+            for (int w = 0; w < 8; ++w) { t += wc[w][tid]; wc[w][tid] = 0; }
+            off[tid] += t;
+        }
+        __syncthreads();
+    }
+}
+
 __global__ void k_tree_row_counts(const int64_t* det, const int64_t* draw, int64_t n, int64_t* cnt)
 {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -437,6 +486,12 @@ int launch_tree_nodes(const TreeArgs& a, int64_t max_chunks, cudaStream_t st)
     if (max_chunks > 0) k_tree_rows<<<(unsigned)max_chunks, kTreeRows, 0, st>>>(a);
     k_tree_count<<<a.nb, 512, 0, st>>>(a);
     return max_chunks > 0 ? 6 : 3;
+}
+
+int launch_tree_perm(const TreeArgs& a, uint32_t* perm, cudaStream_t st)
+{
+    k_tree_perm<<<dim3(a.nb, a.draw_cnt ? 2 : 1), 256, 0, st>>>(a, perm);
+    return 1;
 }
 
 int launch_tree_items(const TreeArgs& a, const TreeLevels& lv, const int* pred_ptr, const int* pred_idx, cudaStream_t st)

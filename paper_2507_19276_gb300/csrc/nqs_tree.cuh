@@ -128,30 +128,37 @@ int launch_tree_graph_tc(const TreeGraphTc& a, int t, int deg, const TreeLevels&
 
 struct TreeRowsTc {
     TreeArgs t;
+    int draws;                            // 0: the deterministic rows, 1: the drawn rows
+    const int64_t* chunk_base;            // [Ns+1] chunks of kTreeRows of those rows
+    const uint32_t* perm;                 // per batch row: the sample's rows of that kind sorted by
+                                          // their first change (launch_tree_perm)
     AnsatzView an;
     const float* mant; const int* mexp;
     const float* tts; const float* WT; int np;
     const double* psi_mant; const int* psi_exp;
     double* partial; double* partial_abs; int64_t* span; int64_t* mv;
 };
+// stable order of each sample's deterministic and drawn rows by their first changed vertex
+int launch_tree_perm(const TreeArgs& a, uint32_t* perm, cudaStream_t st);
 int launch_tree_rows_tc(const TreeRowsTc& a, int64_t max_chunks, int n_sm, cudaStream_t st);
 // split images and exponents of the roots' states into the pool, tanh theta
 int launch_tree_graph_prep(const double* Hst, const int* Hexp, const double* theta, int64_t s0, int nb, int K, int D,
                            int NH, int NP, int corr, unsigned char* pool, int* pool_e, float* tts, cudaStream_t st);
 
-// Normalised readout on a chain: the nodes' running cell, weight and sign
-// (two buffers by level parity).
+// Normalised readout on a chain (D <= kTreeRnnMaxD): the nodes' running cell,
+// weight and sign, in two buffers by level parity.
+constexpr int kTreeRnnMaxD = 32;
 struct TreeRnn {
     AnsatzView an;
     TreeArgs t;
-    const double* cells;                  // n's cells [Ns][K][D]
-    double* cell;                         // [2][nodes][D]
-    double* prod;                         // [2][nodes] prod P / Z = prod * 2^pex since the first change
-    int* pex;                             // [2][nodes]
-    uint32_t* flag;                       // [2][nodes] N_alpha | N_beta << 8 | odd << 16 | dead << 17
     uint32_t n_nodes;
+    const double* cells;                  // n's cells [Ns][K][D]
+    double* cell;                         // [2][n_nodes][D]
+    double* prod;                         // [2][n_nodes] prod of P / Z since the first change, times
+    int* pex;                             // 2^(500 pex) ([2][n_nodes])
+    uint32_t* flag;                       // [2][n_nodes] N_alpha | N_beta << 8 | odd << 16 | dead << 17
 };
-int launch_tree_rnn(const TreeRnn& a, int t, const int64_t* bounds, int n_sm, cudaStream_t st);
+int launch_tree_rnn(const TreeRnn& a, int t, const TreeLevels& lv, const int64_t* bounds, int n_sm, cudaStream_t st);
 
 struct TreeRowsRnn {
     TreeRnn r;
@@ -166,16 +173,18 @@ int launch_tree_rows_rnn(const TreeRowsRnn& a, int64_t max_chunks, cudaStream_t 
 constexpr uint32_t kNoNode = 0xffffffffu;
 
 // sample (call index) of chunk b of the batch, -1 past its end
-__device__ __forceinline__ int64_t tree_sample(const TreeArgs& a, int64_t b)
+__device__ __forceinline__ int64_t tree_sample(const TreeArgs& a, const int64_t* chunk_base, int64_t b)
 {
-    if (b >= a.chunk_base[a.s0 + a.nb]) return -1;
+    if (b >= chunk_base[a.s0 + a.nb]) return -1;
     int64_t lo = a.s0, hi = a.s0 + a.nb - 1;
     while (lo < hi) {
         const int64_t mid = (lo + hi + 1) >> 1;
-        if (a.chunk_base[mid] <= b) lo = mid; else hi = mid - 1;
+        if (chunk_base[mid] <= b) lo = mid; else hi = mid - 1;
     }
     return lo;
 }
+
+__device__ __forceinline__ int64_t tree_sample(const TreeArgs& a, int64_t b) { return tree_sample(a, a.chunk_base, b); }
 
 struct TreeWord {
     int c;                    // changes

@@ -200,18 +200,27 @@ int launch_chunk_base(const int64_t* cnt, int rows, int64_t* out, int64_t Ns, cu
 
 // ---------------------------------------------------------------------------
 // E_loc per sample = H_nn + sum of det-row partials + sum of draw-row partials
-// (one warp per sample, lanes strided over the chunks, then the shuffle tree),
-// then the weighted summary: per-block partial sums over strided samples and
-// chunks, combined by one warp in block order (fixed order throughout). One
-// block for all of it took 1.1 ms on 16 384 samples with 1.2 M chunks; spread
-// over the chip it is launch-bound (~10 us).
+// (in chunk order), then the weighted summary (fixed tree order). A heavy
+// sample's E_loc - Ebar cancels in the energy gradient, so the orders are those
+// of plain loops: a warp per sample loads 32 partials at a time and adds them
+// one after the other; the summary's sums run in one block, and only the counts
+// of the chunks (whole numbers, 1.2 M chunks on H18) are summed over the chip.
 // ---------------------------------------------------------------------------
 
-__device__ double chunk_sum_warp(const double* v, int64_t b0, int64_t b1, int lane)
+// v[b0] + v[b0 + 1] + ... in order, on every lane of the warp
+__device__ double chunk_sum_warp(const double* v, int64_t b0, int64_t b1, int lane, double x)
 {
-    double x = 0.0;
-    for (int64_t b = b0 + lane; b < b1; b += 32) x += v[b];
-    return warp_sum_f64(x);                                   // lane 0
+    for (int64_t b = b0; b < b1; b += 32) {
+        const double mine = b + lane < b1 ? v[b + lane] : 0.0;
+        const int n = (int)(b1 - b < 32 ? b1 - b : 32);
+        if (n == 32) {
+            #pragma unroll
+            for (int k = 0; k < 32; ++k) x += __shfl_sync(kFull, mine, k);
+        } else {
+            for (int k = 0; k < n; ++k) x += __shfl_sync(kFull, mine, k);
+        }
+    }
+    return x;
 }
 
 __global__ void __launch_bounds__(256) k_final_samples(FinalArgs a)
@@ -222,16 +231,16 @@ __global__ void __launch_bounds__(256) k_final_samples(FinalArgs a)
     const int64_t d0 = a.base_det[s], d1 = a.base_det[s + 1];
     int64_t w0 = 0, w1 = 0;
     if (a.base_draw) { w0 = a.base_draw[s]; w1 = a.base_draw[s + 1]; }
-    const double ed = chunk_sum_warp(a.part_det, d0, d1, lane);
-    const double es = w1 > w0 ? chunk_sum_warp(a.part_draw, w0, w1, lane) : 0.0;
+    const double ed = chunk_sum_warp(a.part_det, d0, d1, lane, 0.0);
+    const double es = chunk_sum_warp(a.part_draw, w0, w1, lane, 0.0);
     double ea = 0.0;
     if (a.e_abs) {
-        ea = chunk_sum_warp(a.part_det_abs, d0, d1, lane);
-        if (a.part_draw_abs && w1 > w0) ea += chunk_sum_warp(a.part_draw_abs, w0, w1, lane);
+        ea = chunk_sum_warp(a.part_det_abs, d0, d1, lane, fabs(a.h_diag[s]));
+        if (a.part_draw_abs) ea = chunk_sum_warp(a.part_draw_abs, w0, w1, lane, ea);
     }
     if (lane) return;
     a.e_loc[s] = a.h_diag[s] + ed + es;
-    if (a.e_abs) a.e_abs[s] = fabs(a.h_diag[s]) + ea;
+    if (a.e_abs) a.e_abs[s] = ea;
     if (a.e_det) a.e_det[s] = ed;
     if (a.e_stoch) a.e_stoch[s] = es;
 }
@@ -249,82 +258,102 @@ __device__ double block_reduce_sum(double v, double* sh)
     return r;   // valid in thread 0
 }
 
-// Block b's partial sums at summary[8 + 9 b]: the reference m_b = max 2 log f,
-// then sum c, sum c E, sum c f^2 e^{-m_b}, sum c f^2 e^{-m_b} E, and the counts.
-__global__ void __launch_bounds__(256) k_summary_part(FinalArgs a)
+// Block b's share of the chunks' vertex and product counts, at summary[8 + 2 b].
+__global__ void __launch_bounds__(256) k_summary_counts(FinalArgs a)
 {
     __shared__ double sh[32];
-    __shared__ double bc;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    double sp = 0.0, mv = 0.0;
+    const int64_t nd = a.base_det ? a.base_det[a.Ns] : 0, nw = a.base_draw ? a.base_draw[a.Ns] : 0;
+    if (a.span_det) for (int64_t b = t0; b < nd; b += step) sp += (double)a.span_det[b];
+    if (a.span_draw) for (int64_t b = t0; b < nw; b += step) sp += (double)a.span_draw[b];
+    if (a.mv_det) for (int64_t b = t0; b < nd; b += step) mv += (double)a.mv_det[b];
+    if (a.mv_draw) for (int64_t b = t0; b < nw; b += step) mv += (double)a.mv_draw[b];
+    sp = block_reduce_sum(sp, sh);
+    mv = block_reduce_sum(mv, sh);
+    if (threadIdx.x == 0) {
+        a.summary[8 + 2 * blockIdx.x] = sp;
+        a.summary[8 + 2 * blockIdx.x + 1] = mv;
+    }
+}
+
+__global__ void __launch_bounds__(256) k_summary(FinalArgs a, int count_blocks)
+{
+    __shared__ double sh[5][8];
+    __shared__ double bc;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double m = -INFINITY;
-    for (int64_t s = t0; s < a.Ns; s += step) m = fmax(m, 2.0 * a.log_f[s]);
+    #pragma unroll 4
+    for (int64_t s = threadIdx.x; s < a.Ns; s += 256) m = fmax(m, 2.0 * a.log_f[s]);
     m = warp_max_f64(m);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
+    if (lane == 0) sh[0][warp] = m;
     __syncthreads();
     if (threadIdx.x == 0) {
         double mm = -INFINITY;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) mm = fmax(mm, sh[w]);
+        for (int w = 0; w < 8; ++w) mm = fmax(mm, sh[0][w]);
         bc = mm;
     }
     __syncthreads();
     m = bc;
-    double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int64_t s = t0; s < a.Ns; s += step) {
-        const double c = a.counts ? a.counts[s] : 1.0, e = a.e_loc[s];
-        // a block whose f all vanish adds nothing (unless every block's do)
-        const double f2 = m == -INFINITY ? 0.0 : exp(2.0 * a.log_f[s] - m);
+    // sum c, sum c E, sum c f^2 e^-m, listed and drawn rows
+    double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    #pragma unroll 4
+    for (int64_t s = threadIdx.x; s < a.Ns; s += 256) {
+        const double c = a.counts ? a.counts[s] : 1.0;
         v[0] += c;
-        v[1] += c * e;
-        v[2] += c * f2;
-        v[3] += c * f2 * e;
-        if (a.det_off) v[4] += (double)(a.det_off[s + 1] - a.det_off[s]);
-        if (a.n_unique) v[5] += (double)a.n_unique[s];
+        v[1] += c * a.e_loc[s];
+        v[2] += c * exp(2.0 * a.log_f[s] - m);
+        if (a.det_off) v[3] += (double)(a.det_off[s + 1] - a.det_off[s]);
+        if (a.n_unique) v[4] += (double)a.n_unique[s];
     }
-    if (a.span_det)
-        for (int64_t b = t0; b < a.base_det[a.Ns]; b += step) v[6] += (double)a.span_det[b];
-    if (a.span_draw && a.base_draw)
-        for (int64_t b = t0; b < a.base_draw[a.Ns]; b += step) v[6] += (double)a.span_draw[b];
-    if (a.mv_det)
-        for (int64_t b = t0; b < a.base_det[a.Ns]; b += step) v[7] += (double)a.mv_det[b];
-    if (a.mv_draw && a.base_draw)
-        for (int64_t b = t0; b < a.base_draw[a.Ns]; b += step) v[7] += (double)a.mv_draw[b];
-    double* out = a.summary + 8 + 9 * blockIdx.x;
-    for (int k = 0; k < 8; ++k) {
-        const double r = block_reduce_sum(v[k], sh);
-        if (threadIdx.x == 0) out[k + 1] = r;
+    __syncthreads();
+    #pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        v[k] = warp_sum_f64(v[k]);
+        if (lane == 0) sh[k][warp] = v[k];
     }
-    if (threadIdx.x == 0) out[0] = m;
-}
-
-__global__ void __launch_bounds__(32) k_summary_final(double* summary, int blocks)
-{
-    const double* p = summary + 8;
-    double m = -INFINITY;
-    for (int b = threadIdx.x; b < blocks; b += 32) m = fmax(m, p[9 * b]);
-    m = warp_max_f64(m);
-    double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int b = threadIdx.x; b < blocks; b += 32) {
-        const double mb = p[9 * b];
-        const double f = mb == -INFINITY && m != -INFINITY ? 0.0 : exp(mb - m);
-        for (int k = 0; k < 8; ++k) v[k] += (k == 2 || k == 3) ? f * p[9 * b + 1 + k] : p[9 * b + 1 + k];
+    __syncthreads();
+    double r = 0.0;                                   // threads 0..4: one sum each, warps in order
+    if (threadIdx.x < 5)
+        for (int w = 0; w < 8; ++w) r += sh[threadIdx.x][w];
+    __syncthreads();
+    if (threadIdx.x < 5) sh[threadIdx.x][0] = r;
+    __syncthreads();
+    const double sc = sh[0][0], sce = sh[1][0], scf = sh[2][0], ndet = sh[3][0], nu = sh[4][0];
+    const double logB = m + log(scf / sc);
+    double set = 0.0;
+    #pragma unroll 4
+    for (int64_t s = threadIdx.x; s < a.Ns; s += 256) {
+        const double c = a.counts ? a.counts[s] : 1.0;
+        set += c * exp(2.0 * a.log_f[s] - logB) * a.e_loc[s];
     }
-    for (int k = 0; k < 8; ++k) v[k] = warp_sum_f64(v[k]);
+    __syncthreads();
+    set = block_reduce_sum(set, sh[0]);
+    double sp = 0.0, mv = 0.0;
+    if (warp == 0) {
+        for (int b = lane; b < count_blocks; b += 32) { sp += a.summary[8 + 2 * b]; mv += a.summary[8 + 2 * b + 1]; }
+        sp = warp_sum_f64(sp);
+        mv = warp_sum_f64(mv);
+    }
     if (threadIdx.x == 0) {
-        summary[0] = v[1] / v[0];
-        summary[1] = v[0];
-        summary[2] = m + log(v[2] / v[0]);        // log B
-        summary[3] = v[3] / v[2];                 // sum c f^2 E / sum c f^2 = (1 / sum c) sum c (f^2 / B) E
-        for (int k = 4; k < 8; ++k) summary[k] = v[k];
+        a.summary[0] = sce / sc;
+        a.summary[1] = sc;
+        a.summary[2] = logB;
+        a.summary[3] = set / sc;
+        a.summary[4] = ndet;
+        a.summary[5] = nu;
+        a.summary[6] = sp;
+        a.summary[7] = mv;
     }
 }
 
 int launch_summary(const FinalArgs& a, cudaStream_t st)
 {
     if (a.Ns == 0 || !a.summary) return 0;
-    const int blocks = a.Ns >= 64 ? kSummaryBlocks : 16;
-    k_summary_part<<<blocks, 256, 0, st>>>(a);
-    k_summary_final<<<1, 32, 0, st>>>(a.summary, blocks);
-    return 2;
+    const bool counts = a.span_det || a.mv_det;
+    if (counts) k_summary_counts<<<kSummaryBlocks, 256, 0, st>>>(a);
+    k_summary<<<1, 256, 0, st>>>(a, counts ? kSummaryBlocks : 0);
+    return counts ? 2 : 1;
 }
 
 // samples picked for re-evaluation: their words, counts and global positions

@@ -126,3 +126,45 @@ def test_graph_prefix_tree_fp64(ctx, seed, K, D, ns, eps, draws):
     scale = np.maximum(np.abs(ref["e_loc"]), ref["e_abs"]) + (2.0 ** -52 / 1e-12) * ref["e_cond"]
     assert np.all(np.abs(e - ref["e_loc"])[ok] <= 1e-12 * scale[ok])
     assert summ["n_det"] == int(ref["n_det"].sum())
+
+
+@pytest.mark.parametrize("K,D,ns,eps,draws,nh", [(8, 1, 70, 0.0, 0, 0), (7, 16, 1, 0.02, 9, 5), (6, 17, None, 1e3, 300, 0),
+                                                 (9, 32, 33, 0.05, 64, 4), (3, 33, None, 0.0, 0, 2), (1, 4, None, 0.0, 0, 0)])
+def test_normalised_chain_prefix_tree(ctx, K, D, ns, eps, draws, nh):
+    """Normalised readout of chains over the prefix trees (D up to 32) and row by
+    row (33): 32- and 64-node tiles, drawn rows alone, one sample; FP64 bar."""
+    from oracle import oracle as O
+    s = W.with_readout(W.tiny_system(K=K, na=K // 2, nb=(K + 1) // 2, D=D, n_hidden=nh, seed=K + D, eps=eps,
+                                     n_draws=draws, n_samples=ns), seed=D)
+    ctx.set_system(s)
+    ctx.set_precision(nqs.NQS_PREC_FP64)
+    ref = O.local_energy(O.Problem(s))
+    e, summ = ctx.local_energy(s.samples, s.counts, s.eps, s.n_draws, s.seed)
+    assert np.all(np.abs(e - ref["e_loc"]) <= 1e-12 * np.maximum(np.abs(ref["e_loc"]), ref["e_abs"]) + 1e-300)
+    assert summ["n_det"] == int(ref["n_det"].sum())
+
+
+@pytest.mark.parametrize("seed,K,D,ns,eps,draws", [(11, 7, 16, None, 0.0, 0), (12, 6, 32, 5, 0.05, 40), (13, 8, 16, 1, 1e3, 200),
+                                                   (14, 5, 64, None, 0.02, 16)])
+def test_graph_prefix_tree_mixed(ctx, seed, K, D, ns, eps, draws):
+    """Mixed form of graphs over the prefix trees: 128-node tiles of every local
+    state, vertices without a vertex source, drawn rows alone; mixed bar."""
+    import dataclasses
+    from oracle import oracle as O
+    s = _dag(seed, K, D, n_samples=ns, eps=eps, n_draws=draws)
+    if D == 64:                                     # in-degree x 4 D must fit 512 columns
+        ptr, idx, keep = [0], [], []
+        for i in range(K):
+            e = list(range(s.pred_ptr[i], s.pred_ptr[i + 1]))[-2:]
+            keep += e
+            idx += [int(s.pred_idx[x]) for x in e]
+            ptr.append(len(idx))
+        s = dataclasses.replace(s, pred_ptr=np.array(ptr, np.int32), pred_idx=np.array(idx, np.int32),
+                                tensors=np.ascontiguousarray(s.tensors[keep]))
+    ctx.set_system(s)
+    ctx.set_precision(nqs.NQS_PREC_MIXED)
+    ref = O.local_energy(O.Problem(s))
+    e, summ = ctx.local_energy(s.samples, s.counts, s.eps, s.n_draws, s.seed)
+    ctx.set_precision(nqs.NQS_PREC_FP64)
+    assert np.all(np.abs(e - ref["e_loc"]) <= 1e-6 * np.maximum(np.abs(ref["e_loc"]), ref["e_abs"]))
+    assert summ["n_det"] == int(ref["n_det"].sum())
