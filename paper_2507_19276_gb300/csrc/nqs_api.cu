@@ -7,12 +7,14 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/nqs.h"
 #include "nqs_kernels.cuh"
 #include "nqs_family.cuh"
 #include "nqs_tree.cuh"
+#include "nqs_fx.cuh"
 
 using namespace nqs;
 
@@ -21,6 +23,11 @@ namespace {
 // mixed form with an energy tolerance: samples re-evaluated in FP64 each call
 // to check the per-sample error factor (nqs_options.audit_samples = 0)
 constexpr int kDefaultAudit = 4;
+
+// chains: samples (determinants) from which the FP64 sweeps go site by site
+// through the fixed-point tensor-core steps (one launch per site) instead of
+// one block per sample
+constexpr int64_t kFxMinRows = 512;
 
 struct DevBuf {
     void* p = nullptr;
@@ -53,6 +60,9 @@ struct nqs_ctx {
     bool refine_df = false;   // FP64 tables of the error-budgeted re-evaluation: double-FP32 mat-vecs
     DevBuf tc_img, tc_exps;   // split-FP16 operand images for the tensor-core batches
     bool has_tc = false;
+    // fixed-point tensor-core steps (nqs_fx.cu): digit images, lists and rows of a call
+    DevBuf fx_img, fx_exps, fx_list, fx_rows;
+    bool has_fx = false;
 
     // staging and workspace
     DevBuf st_samples, st_counts, st_u, st_out0, st_out1, st_out2, st_out3, st_out4;
@@ -419,8 +429,85 @@ int env_pass(nqs_ctx* c, const uint64_t* samples, int64_t Ns, bool adjoints, int
     e.psi_mant = (double*)c->pmant.p;
     e.psi_exp = (int*)c->pexp.p;
     e.h_diag = (double*)c->hdiag.p;
+    const bool fx = tn == 1 && c->has_fx && Ns >= kFxMinRows;
+    if (fx) {
+        // both sweeps of all samples site by site on the tensor cores: step i takes
+        // the left states through site i and the right ones through site K - 1 - i
+        e.tn = 0;
+        TRY(ensure(c, c->fx_list, (size_t)K * Ns * 4 + (size_t)K * 5 * 8 + 256));
+        int64_t* off = (int64_t*)c->fx_list.p;
+        int32_t* list = (int32_t*)((char*)c->fx_list.p + (((size_t)K * 5 * 8 + 255) & ~(size_t)255));
+        LAUNCH(NQS_STAGE_ENV, launch_group_by_state(samples, Ns, K, list, off, c->stream));
+        LAUNCH(NQS_STAGE_ENV, launch_fx_unit_rows(e.Lenv, e.Lexp, Ns, K + 1, 0, D, c->stream));
+        LAUNCH(NQS_STAGE_ENV, launch_fx_unit_rows(e.Renv, e.Rexp, Ns, K + 1, K, D, c->stream));
+        FxStep x{};
+        x.K = K;
+        x.img = (const unsigned char*)c->fx_img.p;
+        x.exps = (const int*)c->fx_exps.p;
+        x.pool[0] = e.Lenv; x.pool[1] = e.Renv;
+        x.pool_e[0] = e.Lexp; x.pool_e[1] = e.Rexp;
+        x.stride = K + 1;
+        x.n = Ns;
+        x.sides = 2;
+        x.err = (DevError*)c->derr.p;
+        for (int i = 0; i < K; ++i) {
+            const int t = K - 1 - i;
+            x.mat[0] = i * 4;
+            x.mat[1] = (K + t) * 4;
+            x.list[0] = list + (size_t)i * Ns; x.list[1] = list + (size_t)t * Ns;
+            x.off[0] = off + (size_t)i * 5; x.off[1] = off + (size_t)t * 5;
+            x.src[0] = i; x.dst[0] = i + 1;
+            x.src[1] = t + 1; x.dst[1] = t;
+            LAUNCH(NQS_STAGE_ENV, launch_fx_step(x, D, c->n_sm, c->stream));
+        }
+        LAUNCH(NQS_STAGE_ENV, launch_fx_first(e.Lenv, e.Lexp, Ns, K + 1, K, D, e.psi_mant, e.psi_exp, c->stream));
+        CK(cudaGetLastError());
+    }
     LAUNCH(NQS_STAGE_ENV, launch_env_fp64(e, c->stream));
     CK(cudaGetLastError());
+    return NQS_OK;
+}
+
+// log|psi| of n determinants of a chain, site by site on the tensor cores, in
+// batches whose two alternating rows per determinant stay within 1 GiB
+int fx_amplitude(nqs_ctx* c, const uint64_t* dets, int64_t n, double* log_abs, int8_t* sign)
+{
+    const int K = c->K, D = c->av.D;
+    const int64_t per = std::min<int64_t>(n, ((int64_t)1 << 30) / (16 * D));
+    TRY(ensure(c, c->fx_list, (size_t)K * per * 4 + (size_t)K * 5 * 8 + 256));
+    TRY(ensure(c, c->fx_rows, (size_t)per * (2 * (D * 8 + 4) + 12) + 1024));
+    int64_t* off = (int64_t*)c->fx_list.p;
+    int32_t* list = (int32_t*)((char*)c->fx_list.p + (((size_t)K * 5 * 8 + 255) & ~(size_t)255));
+    double* rows = (double*)c->fx_rows.p;
+    double* mant = rows + (size_t)per * 2 * D;
+    int* exps = (int*)(mant + per);
+    int* ex = exps + 2 * per;
+    for (int64_t i0 = 0; i0 < n; i0 += per) {
+        const int64_t m = std::min(per, n - i0);
+        LAUNCH(NQS_STAGE_OTHER, launch_group_by_state(dets + 2 * i0, m, K, list, off, c->stream));
+        LAUNCH(NQS_STAGE_OTHER, launch_fx_unit_rows(rows, exps, m, 2, 0, D, c->stream));
+        FxStep x{};
+        x.K = K;
+        x.img = (const unsigned char*)c->fx_img.p;
+        x.exps = (const int*)c->fx_exps.p;
+        x.pool[0] = x.pool[1] = rows;
+        x.pool_e[0] = x.pool_e[1] = exps;
+        x.stride = 2;
+        x.n = m;
+        x.sides = 1;
+        x.err = (DevError*)c->derr.p;
+        for (int i = 0; i < K; ++i) {
+            x.mat[0] = i * 4;
+            x.list[0] = list + (size_t)i * m;
+            x.off[0] = off + (size_t)i * 5;
+            x.src[0] = i & 1;
+            x.dst[0] = (i + 1) & 1;
+            LAUNCH(NQS_STAGE_OTHER, launch_fx_step(x, D, c->n_sm, c->stream));
+        }
+        LAUNCH(NQS_STAGE_OTHER, launch_fx_first(rows, exps, m, 2, K & 1, D, mant, ex, c->stream));
+        LAUNCH(NQS_STAGE_OTHER, launch_fx_log_psi(c->av, dets + 2 * i0, m, mant, ex, log_abs + i0, sign + i0, c->stream));
+        CK(cudaGetLastError());
+    }
     return NQS_OK;
 }
 
@@ -508,6 +595,24 @@ int site_tables(nqs_ctx* c, const FamArgs<T>& f, int nbb)
     TRY(ensure(c, c->site_items, (size_t)(bounds.back() + 1) * sizeof(SiteItem)));
     sb.items = c->site_items.p;
     LAUNCH(NQS_STAGE_TABLES, fam_site_fill(f, sb, nbb, c->stream));
+    if (std::is_same<T, double>::value && c->has_fx && !f.df) {
+        FxStep x{};
+        x.K = K;
+        x.img = (const unsigned char*)c->fx_img.p;
+        x.exps = (const int*)c->fx_exps.p;
+        x.pool[0] = x.pool[1] = (double*)f.pool;
+        x.pool_e[0] = x.pool_e[1] = f.pool_e;
+        x.items = (const uint2*)sb.items;
+        x.err = (DevError*)c->derr.p;
+        for (int tau = 0; tau < K; ++tau) {
+            x.mat[0] = tau * 4;
+            x.mat[1] = (K + K - 1 - tau) * 4;
+            for (int g = 0; g < 8; ++g) { x.gbeg[g] = bounds[(size_t)tau * 8 + g]; x.gend[g] = bounds[(size_t)tau * 8 + g + 1]; }
+            LAUNCH(NQS_STAGE_TABLES, launch_fx_step(x, f.D, c->n_sm, c->stream));
+        }
+        CK(cudaGetLastError());
+        return NQS_OK;
+    }
     for (int tau = 0; tau < K; ++tau)
         LAUNCH(NQS_STAGE_TABLES, fam_site_step(f, sb, tau, bounds.data(), c->tile_bps * c->n_sm, c->stream));
     CK(cudaGetLastError());
@@ -1101,7 +1206,8 @@ extern "C" int nqs_destroy(nqs_ctx* c)
                       &c->grad_scr, &c->u_dev, &c->ebar_dev, &c->smp_cand, &c->smp_ccnt, &c->smp_cpos,
                       &c->smp_tabs, &c->smp_tree, &c->tk_rank, &c->tk_off, &c->tk, &c->g_img, &c->g_bexp,
                       &c->g_col0, &c->mv_det, &c->mv_draw, &c->g_tts, &c->tr_rows, &c->tr_build, &c->tr_items,
-                      &c->tr_pool, &c->tr_close, &c->g_live, &c->cexp, &c->corr_ab};
+                      &c->tr_pool, &c->tr_close, &c->g_live, &c->cexp, &c->corr_ab, &c->fx_img,
+                      &c->fx_exps, &c->fx_list, &c->fx_rows};
     for (DevBuf* b : more) release(*b);
     for (auto* v : {&c->smp_pa, &c->smp_pb, &c->smp_off, &c->smp_cnt, &c->smp_par, &c->smp_cell})
         for (DevBuf& b : *v) release(b);
@@ -1360,6 +1466,13 @@ extern "C" int nqs_set_ansatz(nqs_ctx* c, const double* site_tensors, int n_edge
         }
     }
     LAUNCH(NQS_STAGE_OTHER, launch_ansatz_forms(fm, c->stream));
+    c->has_fx = chain && fx_fits(D);
+    if (c->has_fx) {
+        TRY(ensure(c, c->fx_img, fx_image_bytes(fm.n_mats, D)));
+        TRY(ensure(c, c->fx_exps, (size_t)2 * fm.n_mats * D * 4));
+        LAUNCH(NQS_STAGE_OTHER, launch_fx_images(fm.A, fm.n_mats, D, (unsigned char*)c->fx_img.p, (int*)c->fx_exps.p,
+                                                 c->stream));
+    }
     CK(cudaGetLastError());
     if (n_hidden > 0) {
         const size_t nw = (size_t)n_hidden * 2 * K, np = (size_t)((n_hidden + 3) & ~3);
@@ -1585,6 +1698,14 @@ extern "C" int nqs_amplitude(nqs_ctx* c, const uint64_t* dets, int64_t n, double
     bool h0, h1;
     TRY(stage_out(c, c->st_out0, log_abs, (size_t)n, &dla, &h0));
     TRY(stage_out(c, c->st_out1, sign, (size_t)n, &dsg, &h1));
+    if (c->av.readout == 0 && c->has_fx && n >= kFxMinRows) {
+        TRY(fx_amplitude(c, dd, n, dla, dsg));
+        TRY(read_dev_error(c));       // the determinants' check and the tiles' bounded waits
+        TRY(copy_back(c, log_abs, dla, (size_t)n, h0));
+        TRY(copy_back(c, sign, dsg, (size_t)n, h1));
+        if (h0 || h1) CK(cudaStreamSynchronize(c->stream));
+        return NQS_OK;
+    }
     TRY(read_dev_error(c));
     if (c->av.readout == 1) LAUNCH(NQS_STAGE_OTHER, launch_rnn_full(c->av, dd, n, dla, dsg, c->stream));
     else LAUNCH(NQS_STAGE_OTHER, launch_full_amp_fp64(c->av, dd, n, dla, dsg, c->stream));

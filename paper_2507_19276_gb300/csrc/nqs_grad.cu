@@ -56,20 +56,20 @@ size_t grad_corr_offset(const AnsatzView& an, int64_t Ns)
 }
 
 // Stable grouping of the sample indices of vertex i (blockIdx.x) by local state.
-__global__ void __launch_bounds__(1024) k_grad_sort(GradArgs a)
+__global__ void __launch_bounds__(1024) k_group_by_state(const uint64_t* samples, int64_t Ns, int32_t* sidx, int64_t* soff)
 {
     __shared__ int wsum[32];
     __shared__ int64_t base;
     const int i = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    int32_t* out = a.sidx + (size_t)i * a.Ns;
+    int32_t* out = sidx + (size_t)i * Ns;
     if (threadIdx.x == 0) base = 0;
     __syncthreads();
     for (int sg = 0; sg < 4; ++sg) {
-        if (threadIdx.x == 0) a.soff[(size_t)i * 5 + sg] = base;
-        for (int64_t t0 = 0; t0 < a.Ns; t0 += blockDim.x) {
+        if (threadIdx.x == 0) soff[(size_t)i * 5 + sg] = base;
+        for (int64_t t0 = 0; t0 < Ns; t0 += blockDim.x) {
             const int64_t s = t0 + threadIdx.x;
-            const bool f = s < a.Ns && sigma_at(a.samples[2 * s], a.samples[2 * s + 1], i) == sg;
+            const bool f = s < Ns && sigma_at(samples[2 * s], samples[2 * s + 1], i) == sg;
             const unsigned bal = __ballot_sync(kFull, f);
             if (lane == 0) wsum[warp] = __popc(bal);
             __syncthreads();
@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(1024) k_grad_sort(GradArgs a)
             __syncthreads();
         }
     }
-    if (threadIdx.x == 0) a.soff[(size_t)i * 5 + 4] = base;
+    if (threadIdx.x == 0) soff[(size_t)i * 5 + 4] = base;
 }
 
 // One (edge, local state, chunk, output tile): partial sum over the chunk's samples.
@@ -287,12 +287,18 @@ int launch_energy_weights(const double* e_loc, const double* counts, const doubl
     return 1;
 }
 
+int launch_group_by_state(const uint64_t* samples, int64_t Ns, int K, int32_t* sidx, int64_t* soff, cudaStream_t st)
+{
+    k_group_by_state<<<K, 1024, 0, st>>>(samples, Ns, sidx, soff);
+    return 1;
+}
+
 int launch_grad_fp64(const GradArgs& a, cudaStream_t st)
 {
     const int D = a.an.D;
     int n = 0;
     if (a.grad_sites && a.Ns > 0) {
-        k_grad_sort<<<a.an.K, 1024, 0, st>>>(a);
+        launch_group_by_state(a.samples, a.Ns, a.an.K, a.sidx, a.soff, st);
         const int nt = (D + kTile - 1) / kTile;
         dim3 grid((unsigned)(nt * nt), (unsigned)grad_chunks(a.Ns), (unsigned)(a.an.n_edges * 4));
         k_grad_tn<<<grid, 256, 0, st>>>(a, nt);

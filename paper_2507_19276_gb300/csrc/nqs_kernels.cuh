@@ -380,6 +380,8 @@ struct GradArgs {
 size_t grad_scratch_bytes(const AnsatzView& an, int64_t Ns);
 size_t grad_corr_offset(const AnsatzView& an, int64_t Ns);
 int launch_grad_fp64(const GradArgs& a, cudaStream_t st);
+// per vertex the sample indices grouped by local state, stable: sidx [K][Ns], soff [K][5]
+int launch_group_by_state(const uint64_t* samples, int64_t Ns, int K, int32_t* sidx, int64_t* soff, cudaStream_t st);
 
 // d log|f| / d theta_k of the correlator: tanh (2cosh), -tan (cos, Ising)
 __device__ __forceinline__ double corr_dlog(int corr, double theta)
