@@ -29,6 +29,10 @@ constexpr int kDefaultAudit = 4;
 // one block per sample
 constexpr int64_t kFxMinRows = 512;
 
+// nodes of a level from which the prefix trees' FP64 steps take 128-node
+// fixed-point tiles (about half a tile per SM) instead of 32-node FP64 ones
+constexpr int64_t kFxMinNodes = 8192;
+
 struct DevBuf {
     void* p = nullptr;
     size_t n = 0;
@@ -63,6 +67,8 @@ struct nqs_ctx {
     // fixed-point tensor-core steps (nqs_fx.cu): digit images, lists and rows of a call
     DevBuf fx_img, fx_exps, fx_list, fx_rows;
     bool has_fx = false;
+    DevBuf fx_rimg, fx_rexps;   // of the normalised readout
+    bool has_fx_rnn = false;
 
     // staging and workspace
     DevBuf st_samples, st_counts, st_u, st_out0, st_out1, st_out2, st_out3, st_out4;
@@ -429,7 +435,7 @@ int env_pass(nqs_ctx* c, const uint64_t* samples, int64_t Ns, bool adjoints, int
     e.psi_mant = (double*)c->pmant.p;
     e.psi_exp = (int*)c->pexp.p;
     e.h_diag = (double*)c->hdiag.p;
-    const bool fx = tn == 1 && c->has_fx && Ns >= kFxMinRows;
+    const bool fx = tn == 1 && c->av.chain && c->has_fx && Ns >= kFxMinRows;
     if (fx) {
         // both sweeps of all samples site by site on the tensor cores: step i takes
         // the left states through site i and the right ones through site K - 1 - i
@@ -1048,7 +1054,14 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
             g.an.pred_ptr = (const int*)c->pred_ptr.p;
             g.an.pred_idx = (const int*)c->pred_idx.p;
             g.items = a.items;
-            for (int t = 0; t < K; ++t) LAUNCH(stage, launch_tree_graph64(g, t, lv, bounds.data(), c->stream));
+            for (int t = 0; t < K; ++t) {
+                // 128-node tensor-core tiles once a level fills the SMs with them
+                if (c->has_fx && (int64_t)lv.n[t] >= kFxMinNodes)
+                    LAUNCH(stage, launch_fx_graph(g, (const unsigned char*)c->fx_img.p, (const int*)c->fx_exps.p,
+                                                  (DevError*)c->derr.p, t, c->deg_h[(size_t)t], lv, bounds.data(), c->n_sm,
+                                                  c->stream));
+                else LAUNCH(stage, launch_tree_graph64(g, t, lv, bounds.data(), c->stream));
+            }
             q.an = g.an;
             q.samples = ds;
             q.s0 = s0;
@@ -1137,7 +1150,12 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
             rn.t = a;
             rn.n_nodes = (uint32_t)nodes;
             rn.cells = (const double*)c->rnn_cells.p;
-            for (int t = 0; t < K; ++t) LAUNCH(stage, launch_tree_rnn(rn, t, lv, bounds.data(), c->n_sm, c->stream));
+            for (int t = 0; t < K; ++t) {
+                if (c->has_fx_rnn && (int64_t)lv.n[t] >= kFxMinNodes)
+                    LAUNCH(stage, launch_fx_rnn(rn, (const unsigned char*)c->fx_rimg.p, (const int*)c->fx_rexps.p,
+                                                (DevError*)c->derr.p, t, lv, bounds.data(), c->n_sm, c->stream));
+                else LAUNCH(stage, launch_tree_rnn(rn, t, lv, bounds.data(), c->n_sm, c->stream));
+            }
             TreeRowsRnn r{};
             r.r = rn;
             r.lp = (const double*)c->rnn_lp.p;
@@ -1207,7 +1225,7 @@ extern "C" int nqs_destroy(nqs_ctx* c)
                       &c->smp_tabs, &c->smp_tree, &c->tk_rank, &c->tk_off, &c->tk, &c->g_img, &c->g_bexp,
                       &c->g_col0, &c->mv_det, &c->mv_draw, &c->g_tts, &c->tr_rows, &c->tr_build, &c->tr_items,
                       &c->tr_pool, &c->tr_close, &c->g_live, &c->cexp, &c->corr_ab, &c->fx_img,
-                      &c->fx_exps, &c->fx_list, &c->fx_rows};
+                      &c->fx_exps, &c->fx_list, &c->fx_rows, &c->fx_rimg, &c->fx_rexps};
     for (DevBuf* b : more) release(*b);
     for (auto* v : {&c->smp_pa, &c->smp_pb, &c->smp_off, &c->smp_cnt, &c->smp_par, &c->smp_cell})
         for (DevBuf& b : *v) release(b);
@@ -1466,11 +1484,12 @@ extern "C" int nqs_set_ansatz(nqs_ctx* c, const double* site_tensors, int n_edge
         }
     }
     LAUNCH(NQS_STAGE_OTHER, launch_ansatz_forms(fm, c->stream));
-    c->has_fx = chain && fx_fits(D);
+    c->has_fx = fx_fits(D);
     if (c->has_fx) {
-        TRY(ensure(c, c->fx_img, fx_image_bytes(fm.n_mats, D)));
-        TRY(ensure(c, c->fx_exps, (size_t)2 * fm.n_mats * D * 4));
-        LAUNCH(NQS_STAGE_OTHER, launch_fx_images(fm.A, fm.n_mats, D, (unsigned char*)c->fx_img.p, (int*)c->fx_exps.p,
+        const int sides = chain ? 2 : 1;
+        TRY(ensure(c, c->fx_img, fx_image_bytes(fm.n_mats, D, sides)));
+        TRY(ensure(c, c->fx_exps, (size_t)sides * fm.n_mats * 2 * D * 4));
+        LAUNCH(NQS_STAGE_OTHER, launch_fx_images(fm.A, fm.n_mats, D, sides, (unsigned char*)c->fx_img.p, (int*)c->fx_exps.p,
                                                  c->stream));
     }
     CK(cudaGetLastError());
@@ -1543,6 +1562,15 @@ extern "C" int nqs_set_readout(nqs_ctx* c, const double* v, const double* eta, c
     c->av.reta = (const double*)c->reta.p;
     c->av.rw = (const double*)c->rw.p;
     c->av.rc = (const double*)c->rc.p;
+    c->has_fx_rnn = c->av.chain && D <= kFxRnnMaxD;
+    if (c->has_fx_rnn) {
+        TRY(ensure(c, c->fx_rimg, fx_rnn_image_bytes(K, D)));
+        TRY(ensure(c, c->fx_rexps, fx_rnn_exps(K, D) * 4));
+        LAUNCH(NQS_STAGE_OTHER, launch_fx_rnn_images(c->av.A, K, D, (unsigned char*)c->fx_rimg.p, (int*)c->fx_rexps.p,
+                                                     c->stream));
+        CK(cudaGetLastError());
+        CK(cudaStreamSynchronize(c->stream));
+    }
     c->av.mask_na = constrained ? c->na : -1;
     c->av.mask_nb = constrained ? c->nb : -1;
     c->av.readout = 1;
@@ -1698,7 +1726,7 @@ extern "C" int nqs_amplitude(nqs_ctx* c, const uint64_t* dets, int64_t n, double
     bool h0, h1;
     TRY(stage_out(c, c->st_out0, log_abs, (size_t)n, &dla, &h0));
     TRY(stage_out(c, c->st_out1, sign, (size_t)n, &dsg, &h1));
-    if (c->av.readout == 0 && c->has_fx && n >= kFxMinRows) {
+    if (c->av.readout == 0 && c->av.chain && c->has_fx && n >= kFxMinRows) {
         TRY(fx_amplitude(c, dd, n, dla, dsg));
         TRY(read_dev_error(c));       // the determinants' check and the tiles' bounded waits
         TRY(copy_back(c, log_abs, dla, (size_t)n, h0));
@@ -1937,7 +1965,8 @@ int le_core(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, uint64
         LAUNCH(NQS_STAGE_FINAL, launch_finalize(f, c->stream));
     }
     CK(cudaGetLastError());
-    if (shared || gtc) TRY(read_dev_error(c));
+    // tiles with bounded waits ran: the tensor-core forms and the fixed-point steps
+    if (shared || gtc || (tree && (c->has_fx || c->has_fx_rnn))) TRY(read_dev_error(c));
     return NQS_OK;
 }
 

@@ -1594,25 +1594,49 @@ __global__ void __launch_bounds__(kFamRows, MB) k_fam_rows(FamArgs<T> f, RowSet 
             ratio = sum + comp;
             if (NH > 0) {
                 typedef typename Vec4<T>::type V4;
-                T X = T(0);                            // product of (1 + x_k) minus 1
-                if (live) {
-                    const V4* l4 = (const V4*)ltq;
-                    const V4* r4 = (const V4*)rsq;
-                    for (int k4 = sub; k4 <= NP / 4; k4 += 8) {
-                        const V4 t = l4[k4], u = r4[k4];
-                        T x;
-                        // the last group holds PL - 1 and PR - 1 (then zeros): (1 + a)(1 + b) - 1
-                        x = k4 == NP / 4 ? fma(t.x, u.x, t.x + u.x) : t.x * u.x; X = fma(X, x, X + x);
-                        x = t.y * u.y; X = fma(X, x, X + x);
-                        x = t.z * u.z; X = fma(X, x, X + x);
-                        x = t.w * u.w; X = fma(X, x, X + x);
+                if constexpr (dbl) {
+                    // FP64 runs at two operations per clock and SM: the product itself
+                    // (two operations per unit, pairs of units dealt over the lanes)
+                    // instead of the product minus one (three) -- its rounding,
+                    // ~sqrt(N_h) 2^-53, is that of the dot product
+                    double P = 1.0;
+                    if (live) {
+                        const double2* l2 = (const double2*)ltq;
+                        const double2* r2 = (const double2*)rsq;
+                        for (int k2 = sub; k2 <= NP / 2; k2 += 8) {
+                            const double2 t = l2[k2], u = r2[k2];
+                            if (k2 == NP / 2) {          // PL - 1 and PR - 1 (then a zero)
+                                P = fma(P, t.x, P);
+                                P = fma(P, u.x, P);
+                            } else {
+                                P = fma(P, t.x * u.x, P);
+                                P = fma(P, t.y * u.y, P);
+                            }
+                        }
                     }
+                    for (int o = 4; o; o >>= 1) P *= __shfl_xor_sync(kFull, P, o);
+                    if (live) ratio *= P;
+                } else {
+                    T X = T(0);                        // product of (1 + x_k) minus 1
+                    if (live) {
+                        const V4* l4 = (const V4*)ltq;
+                        const V4* r4 = (const V4*)rsq;
+                        for (int k4 = sub; k4 <= NP / 4; k4 += 8) {
+                            const V4 t = l4[k4], u = r4[k4];
+                            T x;
+                            // the last group holds PL - 1 and PR - 1 (then zeros): (1 + a)(1 + b) - 1
+                            x = k4 == NP / 4 ? fma(t.x, u.x, t.x + u.x) : t.x * u.x; X = fma(X, x, X + x);
+                            x = t.y * u.y; X = fma(X, x, X + x);
+                            x = t.z * u.z; X = fma(X, x, X + x);
+                            x = t.w * u.w; X = fma(X, x, X + x);
+                        }
+                    }
+                    for (int o = 4; o; o >>= 1) {
+                        const T Y = __shfl_xor_sync(kFull, X, o);
+                        X = fma(X, Y, X + Y);
+                    }
+                    if (live) ratio *= T(1) + X;
                 }
-                for (int o = 4; o; o >>= 1) {
-                    const T Y = __shfl_xor_sync(kFull, X, o);
-                    X = fma(X, Y, X + Y);
-                }
-                if (live) ratio *= T(1) + X;
             }
         }
         if (live && sub == 0) s_ratio[wbase + q] = ratio;

@@ -1,24 +1,28 @@
 // nqs_fx.cu -- FP64-accurate matrix steps on the tensor cores in fixed point.
 //
 // GB300 executes two FP64 FMAs per clock and SM; its tensor cores ~3600 FP16
-// products. A step y = M x on vectors scaled to a largest magnitude in [0.5, 1)
-// is therefore formed from exact integer products, the error-free splitting of
-// Ozaki, Ogita, Oishi and Rump (Numer. Algorithms 59, 2012): every entry becomes
-// a 56-bit fixed-point number (per vector, and per output row of the matrix),
-// cut into seven signed base-256 digits. Digits are exact in FP16, a product of
-// two is at most 2^14, and the sum over D <= 64 terms and the up to seven digit
-// pairs of one significance stays below 2^23, so the FP32 accumulators of
-// tensor memory hold exact integers. The 28 digit products down to significance
-// 2^-62 are kept; the seven sums of a result are joined in 64-bit integers (unit
-// 2^-56 of the scale) and rounded to FP64 once. The dropped products and the
-// input rounding are ~2^-53 of the scale; a chain of FP64 FMAs over D = 64
-// terms rounds its partial sums 64 times.
+// products. A step y = M x is therefore formed from exact integer products, the
+// error-free splitting of Ozaki, Ogita, Oishi and Rump (Numer. Algorithms 59,
+// 2012). The matrix is equilibrated by powers of two, first its columns, then
+// its rows; the vector takes the column powers and is scaled to a largest
+// magnitude in [0.5, 1) (so a power-of-two change of basis between two sites
+// changes nothing). Every entry becomes a 56-bit fixed-point number, cut into
+// seven signed base-256 digits. Digits are exact in FP16, a product of two is at
+// most 2^14, and the sum over D <= 64 terms and the up to seven digit pairs of
+// one significance stays below 2^23, so the FP32 accumulators of tensor memory
+// hold exact integers. The 34 digit products down to significance 2^-70 are
+// kept; the eight sums of a result are joined in 64-bit integers (unit 2^-56 of
+// the scale) and rounded to FP64 once. The remaining error, the rounding of the
+// entries and of the result, is ~2^-56 sqrt(D) of the scale; a chain of FP64
+// FMAs rounds its partial sums D times at 2^-53.
 //
-// A tile is 128 items of one matrix (256 threads, two per row): gather and cut
+// A tile is 128 items of one matrix (two or four threads per row): gather and cut
 // the rows into digits (bytes of x + 0x80..80, turned into FP16 by PRMT and one
-// packed subtraction), 28 x D/16 MMAs, then the integer epilogue. Per tile at
-// D = 64 that is ~20 k warp instructions and 112 MMAs, against 301 k cycles of
-// the FP64 pipe for the same products.
+// packed subtraction), 34 x D/16 MMAs, then the integer epilogue. Per tile at
+// D = 64 that is ~20 k warp instructions and 136 MMAs, against 301 k cycles of
+// the FP64 pipe for the same products. H50 tables of 200 samples (5 M products):
+// 45 ms on the FP64 pipe, 5.0 ms here; issue and latency of the digit and
+// epilogue chains bound it (one block per SM at D = 64).
 #include "nqs_fx.cuh"
 #include "nqs_tc.cuh"
 
@@ -29,21 +33,36 @@ namespace nqs {
 namespace {
 
 constexpr int kFxRows = 128;
-constexpr int kFxThreads = 256;
+constexpr int kFxSums = 8;                // significances kept
+// threads per row: four at D = 64, where one block fills the SM
+// (more warps hide the digit and epilogue chains), else two
+constexpr int fx_split(int D) { return D == 64 ? 4 : 2; }
 
-// x 2^55 rounded to an integer, |x| < 1, plus 0x80 in each of the seven bytes:
-// byte i (the top one nine bits wide) is digit i + 128.
-__device__ __forceinline__ uint64_t fx_code(double x)
+// x 2^(55 + off) rounded to an integer, |x 2^off| < 1, plus 0x80 in each of the
+// seven bytes: byte i (the top one nine bits wide) is digit i + 128.
+__device__ __forceinline__ uint64_t fx_code(double x, int off)
 {
     const uint64_t b = (uint64_t)__double_as_longlong(x);
     const int e = (int)((b >> 52) & 0x7FF);
-    uint64_t m = (b & 0xFFFFFFFFFFFFFull) | (e ? 1ull << 52 : 0ull);
-    const int sh = 1020 - e;                  // x 2^55 = m 2^-sh
+    uint64_t m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    const int sh = 1020 - e - off;            // x 2^(55 + off) = m 2^-sh
     if (sh <= 0) m <<= (-sh) & 3;
     else m = sh > 54 ? 0ull : (m + (1ull << (sh - 1))) >> sh;
+    if (e == 0) m = 0;
     const int64_t v = (int64_t)b < 0 ? -(int64_t)m : (int64_t)m;
     return (uint64_t)(v + 0x80808080808080ll);
 }
+
+constexpr int kFxNoExp = -(1 << 20);          // power of two of a zero
+
+// e with |x| in [2^(e-1), 2^e)
+__device__ __forceinline__ int fx_exp(double x)
+{
+    const int e = (__double2hiint(x) >> 20) & 0x7FF;
+    return e ? e - 1022 : kFxNoExp;
+}
+
+__device__ __forceinline__ bool fx_not_finite(double x) { return (__double2hiint(x) & 0x7FF00000) == 0x7FF00000; }
 
 // digit `i` (0 = least significant) of two codes as FP16
 __device__ __forceinline__ __half2 fx_digit2(uint64_t c0, uint64_t c1, int i)
@@ -60,42 +79,62 @@ __device__ __forceinline__ __half2 fx_digit2(uint64_t c0, uint64_t c1, int i)
     return __hsub2(*reinterpret_cast<const __half2*>(&w), k);
 }
 
-// One block per (side, matrix): the rows' powers of two, then their digits.
-__global__ void __launch_bounds__(256) k_fx_images(const double* __restrict__ A, int n_mats, int D, unsigned char* img,
-                                                   int* exps)
+// One block per (matrix, side): the columns' powers of two, the rows' after them,
+// then the digits. The operand has `rows` rows of D entries (columns past D, up
+// to C, and rows past `rows`, up to R, are zero) in blocks of R rows:
+// entry(n, k) of the matrix.
+template <class Entry>
+__device__ void fx_image(const Entry& entry, int rows, int D, int R, int C, unsigned char* img, int* cexp, int* rexp,
+                         int* sc, int* sr)
 {
-    __shared__ int se[kFxMaxD];
-    const int m = blockIdx.x, side = blockIdx.y, lane = threadIdx.x & 31;
-    const double* M = A + (size_t)m * D * D;
-    const size_t id = (size_t)side * n_mats + m;
-    for (int n = threadIdx.x >> 5; n < D; n += 8) {
-        double mx = 0.0;
-        int bad = 0;
-        for (int k = lane; k < D; k += 32) {
-            const double v = fabs(side == 0 ? __ldg(M + (size_t)n * D + k) : __ldg(M + (size_t)k * D + n));
-            mx = fmax(mx, v);
-            bad |= !(v <= 1.7976931348623157e308);
+    const int lane = threadIdx.x & 31;
+    for (int k = threadIdx.x; k < C; k += blockDim.x) {
+        int e = kFxNoExp;
+        if (k < D)
+            for (int n = 0; n < rows; ++n) {
+                const double v = entry(n, k);
+                if (!fx_not_finite(v)) e = max(e, fx_exp(v));
+            }
+        sc[k] = e == kFxNoExp ? 0 : e;
+        cexp[k] = sc[k];
+    }
+    __syncthreads();
+    const int RT = (rows + R - 1) / R * R;
+    for (int n = threadIdx.x >> 5; n < RT; n += blockDim.x >> 5) {
+        int e = kFxNoExp, bad = 0;
+        for (int k = lane; k < D && n < rows; k += 32) {
+            const double v = entry(n, k);
+            if (fx_not_finite(v)) bad = 1;
+            else if (v != 0.0) e = max(e, fx_exp(v) - sc[k]);
         }
-        mx = warp_max_f64(mx);
+        e = __reduce_max_sync(kFull, e);
         bad = __any_sync(kFull, bad);
-        int e = 0;
-        if (mx > 0.0) frexp(mx, &e);
         if (lane == 0) {
-            se[n] = bad ? 0 : e;
-            exps[id * D + n] = bad ? kFxNotFinite : e;
+            sr[n] = e <= kFxNoExp / 2 ? 0 : e;
+            rexp[n] = bad ? kFxNotFinite : sr[n];
         }
     }
     __syncthreads();
-    unsigned char* out = img + id * kFxDigits * 2 * D * D;
-    for (int q = threadIdx.x; q < D * (D / 2); q += 256) {
-        const int n = q / (D / 2), k = 2 * (q - n * (D / 2));
-        const double v0 = side == 0 ? __ldg(M + (size_t)n * D + k) : __ldg(M + (size_t)k * D + n);
-        const double v1 = side == 0 ? __ldg(M + (size_t)n * D + k + 1) : __ldg(M + (size_t)(k + 1) * D + n);
-        const uint64_t c0 = fx_code(ldexp(v0, -se[n])), c1 = fx_code(ldexp(v1, -se[n]));
+    for (int q = threadIdx.x; q < RT * (C / 2); q += blockDim.x) {
+        const int n = q / (C / 2), k = 2 * (q - n * (C / 2));
+        const double v0 = n < rows && k < D ? entry(n, k) : 0.0, v1 = n < rows && k + 1 < D ? entry(n, k + 1) : 0.0;
+        const uint64_t c0 = fx_code(v0, -sc[k] - sr[n]), c1 = fx_code(v1, -sc[k + 1] - sr[n]);
+        unsigned char* out = img + (size_t)(n / R) * kFxDigits * 2 * R * C;
         #pragma unroll
         for (int i = 0; i < kFxDigits; ++i)
-            *(__half2*)(out + (size_t)(kFxDigits - 1 - i) * 2 * D * D + tc::op_offset(n, k, D)) = fx_digit2(c0, c1, i);
+            *(__half2*)(out + (size_t)(kFxDigits - 1 - i) * 2 * R * C + tc::op_offset(n % R, k, C)) = fx_digit2(c0, c1, i);
     }
+}
+
+__global__ void __launch_bounds__(256) k_fx_images(const double* __restrict__ A, int n_mats, int D, unsigned char* img,
+                                                   int* exps)
+{
+    __shared__ int sc[kFxMaxD], sr[kFxMaxD];
+    const int m = blockIdx.x, side = blockIdx.y;
+    const double* M = A + (size_t)m * D * D;
+    const size_t id = (size_t)side * n_mats + m;
+    fx_image([&](int n, int k) { return side == 0 ? __ldg(M + (size_t)n * D + k) : __ldg(M + (size_t)k * D + n); }, D, D, D, D,
+             img + id * kFxDigits * 2 * D * D, exps + id * 2 * D, exps + id * 2 * D + D, sc, sr);
 }
 
 // an FP32 accumulator that holds an integer; small: |v| <= 2^22
@@ -105,8 +144,115 @@ __device__ __forceinline__ int fx_int(uint32_t w, bool small)
     return small ? __float_as_int(v + 12582912.f) - 0x4B400000 : __float2int_rn(v);
 }
 
+// the eight sums of a result as an integer of unit 2^-(56 - drop)
+__device__ __forceinline__ int64_t fx_join(const int* s, int drop)
+{
+    const int64_t hi = (int64_t)(s[0] * 256 + s[1]) * 65536 + (s[2] * 256 + s[3]);
+    const int64_t lo = ((int64_t)(s[4] * 256 + s[5]) * 256 + s[6]) * 256 + s[7];
+    return (hi << (18 - drop)) + ((lo + (1 << (13 + drop))) >> (14 + drop));
+}
+
+// V 2^q as a double with its exponent field f relative to the row's largest:
+// f = 1022 + (bits of |V|) + power - emax
+__device__ __forceinline__ double fx_double(int64_t v, int power, int emax)
+{
+    const uint64_t mag = (uint64_t)(v < 0 ? -v : v);
+    const int L = 64 - __clzll((long long)mag);
+    const int f = 1022 + L + power - emax;
+    const uint64_t m = L <= 53 ? mag << (53 - L) : (mag + (1ull << (L - 54))) >> (L - 53);
+    uint64_t bits = ((uint64_t)(f - 1) << 52) + m;
+    if (mag == 0 || f <= 0) bits = 0;
+    else if (f >= 2047) bits = 0x7FF0000000000000ull;
+    return __longlong_as_double((long long)(bits | ((uint64_t)v & 0x8000000000000000ull)));
+}
+
+// the digit products of significance 0..7 of one operand pair into eight
+// accumulators of N columns (one thread)
+template <int KS>
+__device__ __forceinline__ void fx_mma(uint32_t tmem, uint32_t N, uint64_t dA, uint64_t dB, uint32_t kA, uint32_t kB,
+                                       uint32_t idesc)
+{
+    for (int l = 0; l < kFxSums; ++l)             // digits a of the rows, l - a of the matrix
+        for (int a = max(0, l - kFxDigits + 1); a <= min(l, kFxDigits - 1); ++a)
+            #pragma unroll
+            for (int ks = 0; ks < KS; ++ks)
+                tc::mma_f16(tmem + (uint32_t)l * N, dA + (uint64_t)(a * (kA >> 4) + 16 * ks),
+                            dB + (uint64_t)((l - a) * (kB >> 4) + 16 * ks), idesc,
+                            (a != max(0, l - kFxDigits + 1) || ks) ? 1u : 0u);
+}
+
+// The digits of a tile's rows (row r at pool + src[r] * D, times the column powers
+// cm, scaled by 2^-ea[r]) into the operand buffers: eight entries of a row per
+// task, eight rows x four tasks per warp (shared memory in whole core matrices).
+// ea[r] must hold kFxNoExp; contains a block barrier.
+template <int D, int SP>
+__device__ __forceinline__ void fx_rows(const double* __restrict__ pool, const int64_t* src_row, const int* cm, int* ea_row,
+                                        int* bad_row, unsigned char* A)
+{
+    constexpr int NW = kFxRows * SP / 32;
+    constexpr uint32_t kA = kFxRows * D * 2;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int TASKS = D / 8 / SP;         // per thread: 128 D / 8 in all
+    double v[TASKS][8];
+    int rows[TASKS], pcs[TASKS];
+    #pragma unroll
+    for (int u = 0; u < TASKS; ++u) {
+        const int q = warp + NW * u;          // (row group, 4 pieces)
+        constexpr int PG = D / 8 < 4 ? 1 : D / 32;                   // groups of four pieces per row
+        int row, pc;
+        if constexpr (D == 16) {              // two pieces per row: sixteen rows per warp
+            row = q * 16 + (lane & 7) + 8 * (lane >> 4);
+            pc = (lane >> 3) & 1;
+        } else if constexpr (D == 48) {       // six pieces per row, row-major over the tasks
+            const int x = q * 32 + lane;      // 768 tasks
+            row = (x / 48) * 8 + (x & 7);
+            pc = (x % 48) >> 3;
+        } else {
+            row = (q / PG) * 8 + (lane & 7);
+            pc = (q % PG) * 4 + (lane >> 3);
+        }
+        rows[u] = row;
+        pcs[u] = pc;
+        const double* src = pool + (size_t)src_row[row] * D + 8 * pc;
+        #pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const double2 w = *(const double2*)(src + 2 * k);
+            v[u][2 * k] = w.x;
+            v[u][2 * k + 1] = w.y;
+        }
+    }
+    #pragma unroll
+    for (int u = 0; u < TASKS; ++u) {
+        int e = kFxNoExp;
+        bool bad = false;
+        #pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            e = max(e, fx_exp(v[u][k]) + cm[8 * pcs[u] + k]);
+            bad |= fx_not_finite(v[u][k]);
+        }
+        atomicMax(&ea_row[rows[u]], e);
+        if (bad) bad_row[rows[u]] = 1;
+    }
+    __syncthreads();
+    #pragma unroll
+    for (int u = 0; u < TASKS; ++u) {
+        const int ea = ea_row[rows[u]];
+        uint64_t c[8];
+        #pragma unroll
+        for (int k = 0; k < 8; ++k) c[k] = fx_code(v[u][k], cm[8 * pcs[u] + k] - ea);
+        const uint32_t off = tc::op_offset(rows[u], 8 * pcs[u], D);
+        #pragma unroll
+        for (int i = 0; i < kFxDigits; ++i) {
+            __align__(16) __half2 d[4];
+            #pragma unroll
+            for (int k = 0; k < 4; ++k) d[k] = fx_digit2(c[2 * k], c[2 * k + 1], i);
+            *(uint4*)(A + (kFxDigits - 1 - i) * kA + off) = *(const uint4*)d;
+        }
+    }
+}
+
 template <int D>
-__global__ void __launch_bounds__(kFxThreads, D <= 32 ? 2 : 1) k_fx_step(FxStep st)
+__global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1) k_fx_step(FxStep st)
 {
     extern __shared__ __align__(1024) unsigned char smraw[];
     __shared__ uint32_t tmem_slot;
@@ -114,13 +260,16 @@ __global__ void __launch_bounds__(kFxThreads, D <= 32 ? 2 : 1) k_fx_step(FxStep 
     __shared__ int64_t s_src[kFxRows], s_dst[kFxRows];
     __shared__ int64_t s_gb[8], s_ge[8];
     __shared__ int s_tile[9];
-    __shared__ int s_eb[D];
-    __shared__ int s_max[2][kFxRows];
+    __shared__ int s_eb[D], s_cm[D];
+    __shared__ int s_ea[kFxRows];                     // power of two taken out of each scaled row
+    constexpr int SP = fx_split(D);                   // threads per row
+    __shared__ int s_max[SP][kFxRows];
     __shared__ int s_bad[kFxRows];
-    constexpr int H = D / 2;                          // columns per thread in the epilogue
+    constexpr int NW = kFxRows * SP / 32;             // warps
+    constexpr int H = D / SP;                         // columns per thread in the epilogue
     constexpr uint32_t kA = kFxRows * D * 2;          // one digit of the rows
     constexpr uint32_t kB = 2 * D * D;                // one digit of the matrix
-    constexpr uint32_t kCols = kFxDigits * D <= 128 ? 128 : kFxDigits * D <= 256 ? 256 : 512;
+    constexpr uint32_t kCols = kFxSums * D <= 128 ? 128 : kFxSums * D <= 256 ? 256 : 512;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     unsigned char* const Bs = smraw + kFxDigits * kA;
     if (warp == 0) { tc::tmem_alloc(&tmem_slot, kCols); tc::tmem_relinquish(); }
@@ -175,6 +324,7 @@ __global__ void __launch_bounds__(kFxThreads, D <= 32 ? 2 : 1) k_fx_step(FxStep 
             s_src[tid] = a;
             s_dst[tid] = b;
             s_bad[tid] = 0;
+            s_ea[tid] = kFxNoExp;
         }
         const size_t mat = (size_t)st.mat[side] + (g & 3);
         if (held != g) {
@@ -182,51 +332,10 @@ __global__ void __launch_bounds__(kFxThreads, D <= 32 ? 2 : 1) k_fx_step(FxStep 
                 tc::mbar_expect_tx(&mb_b, kFxDigits * kB);
                 tc::bulk_g2s(Bs, st.img + mat * kFxDigits * kB, kFxDigits * kB, &mb_b);
             }
-            if (tid < D) s_eb[tid] = __ldg(st.exps + mat * D + tid);
+            if (tid < 2 * D) (tid < D ? s_cm : s_eb - D)[tid] = __ldg(st.exps + mat * 2 * D + tid);
         }
         __syncthreads();
-        // the rows' digits: eight entries of a row per task, eight rows x four tasks
-        // per warp (shared memory in whole core matrices)
-        {
-            const double* pool = st.pool[side];
-            constexpr int TASKS = D / 16;             // per thread: 128 D / 8 / 256
-            #pragma unroll
-            for (int u = 0; u < TASKS; ++u) {
-                const int q = warp + 8 * u;           // (row group, 4 pieces)
-                constexpr int PG = D / 8 < 4 ? 1 : D / 32;                   // groups of four pieces per row
-                int row, pc;
-                if constexpr (D == 16) {              // two pieces per row: sixteen rows per warp
-                    row = q * 16 + (lane & 7) + 8 * (lane >> 4);
-                    pc = (lane >> 3) & 1;
-                } else if constexpr (D == 48) {       // six pieces per row, row-major over the tasks
-                    const int x = q * 32 + lane;      // 768 tasks
-                    row = (x / 48) * 8 + (x & 7);
-                    pc = (x % 48) >> 3;
-                } else {
-                    row = (q / PG) * 8 + (lane & 7);
-                    pc = (q % PG) * 4 + (lane >> 3);
-                }
-                const double* src = pool + (size_t)s_src[row] * D + 8 * pc;
-                uint64_t c[8];
-                int bad = 0;
-                #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const double2 v = *(const double2*)(src + 2 * k);
-                    bad |= ((__double2hiint(v.x) & 0x7FF00000) == 0x7FF00000) | ((__double2hiint(v.y) & 0x7FF00000) == 0x7FF00000);
-                    c[2 * k] = fx_code(v.x);
-                    c[2 * k + 1] = fx_code(v.y);
-                }
-                if (bad) s_bad[row] = 1;
-                const uint32_t off = tc::op_offset(row, 8 * pc, D);
-                #pragma unroll
-                for (int i = 0; i < kFxDigits; ++i) {
-                    __align__(16) __half2 d[4];
-                    #pragma unroll
-                    for (int k = 0; k < 4; ++k) d[k] = fx_digit2(c[2 * k], c[2 * k + 1], i);
-                    *(uint4*)(smraw + (kFxDigits - 1 - i) * kA + off) = *(const uint4*)d;
-                }
-            }
-        }
+        fx_rows<D, SP>(st.pool[side], s_src, s_cm, s_ea, s_bad, smraw);
         tc::fence_proxy_async();
         tc::fence_before_sync();
         __syncthreads();
@@ -235,12 +344,7 @@ __global__ void __launch_bounds__(kFxThreads, D <= 32 ? 2 : 1) k_fx_step(FxStep 
             if (held != g) ok = tc::mbar_wait(&mb_b, ph_b, kPoll) && ok;
             const uint64_t d0 = tc::desc(0, 128, 16 * D);
             const uint64_t dA = d0 + (tc::smem_addr(smraw) >> 4), dB = d0 + (tc::smem_addr(Bs) >> 4);
-            for (int l = 0; l < kFxDigits; ++l)       // significance l: digits a of the row, l - a of the matrix
-                for (int a = 0; a <= l; ++a)
-                    #pragma unroll
-                    for (int ks = 0; ks < D / 16; ++ks)
-                        tc::mma_f16(tmem + (uint32_t)(l * D), dA + (uint64_t)(a * (kA >> 4) + 16 * ks),
-                                    dB + (uint64_t)((l - a) * (kB >> 4) + 16 * ks), idesc, (a | ks) ? 1u : 0u);
+            fx_mma<D / 16>(tmem, D, dA, dB, kA, kB, idesc);
             tc::mma_commit(&mb_mma);
         }
         if (held != g) ph_b ^= 1u;
@@ -248,23 +352,21 @@ __global__ void __launch_bounds__(kFxThreads, D <= 32 ? 2 : 1) k_fx_step(FxStep 
         ok = tc::mbar_wait(&mb_mma, ph_mma, kPoll) && ok;
         ph_mma ^= 1u;
         tc::fence_after_sync();
-        // join the seven sums: V = y 2^56 / 2^eb, and the row's largest exponent
+        // join the sums: V = y 2^(56 - ea - eb), and the row's largest exponent
         int64_t V[H];
         int emax = -(1 << 29);
         #pragma unroll
         for (int c0 = 0; c0 < H; c0 += 8) {
-            uint32_t w[kFxDigits][8];
+            uint32_t w[kFxSums][8];
             #pragma unroll
-            for (int l = 0; l < kFxDigits; ++l) tc::tmem_ld8u(tlane + (uint32_t)(l * D + c0), w[l]);
+            for (int l = 0; l < kFxSums; ++l) tc::tmem_ld8u(tlane + (uint32_t)(l * D + c0), w[l]);
             tc::tmem_wait_ld();
             #pragma unroll
             for (int c = 0; c < 8; ++c) {
-                int s[kFxDigits];
+                int s[kFxSums];
                 #pragma unroll
-                for (int l = 0; l < kFxDigits; ++l) s[l] = fx_int(w[l][c], (l + 1) * D <= 256);
-                const int64_t hi = (int64_t)(s[0] * 256 + s[1]) * 65536 + (s[2] * 256 + s[3]);
-                const int64_t lo = (int64_t)(s[4] * 256 + s[5]) * 256 + s[6];
-                const int64_t v = (hi << 18) + ((lo + 32) >> 6);
+                for (int l = 0; l < kFxSums; ++l) s[l] = fx_int(w[l][c], (l + 1) * D <= 256);
+                const int64_t v = fx_join(s, 0);
                 V[c0 + c] = v;
                 const int eb = s_eb[h * H + c0 + c];
                 if (v != 0) emax = max(emax, 64 - __clzll(v < 0 ? -v : v) + eb);
@@ -273,31 +375,21 @@ __global__ void __launch_bounds__(kFxThreads, D <= 32 ? 2 : 1) k_fx_step(FxStep 
         }
         s_max[h][r] = emax;
         tc::fence_before_sync();
-        __syncthreads();                              // the two halves of each row meet
-        emax = max(s_max[0][r], s_max[1][r]);
+        __syncthreads();                              // the parts of each row meet
+        #pragma unroll
+        for (int k = 0; k < SP; ++k) emax = max(emax, s_max[k][r]);
         if (r < n) {
             double* dst = st.pool[side] + (size_t)s_dst[r] * D + h * H;
             const bool bad = s_bad[r] != 0 || emax >= kFxNotFinite;
+            const double nan = __longlong_as_double(0x7FF8000000000000ll);
             #pragma unroll
             for (int c = 0; c < H; c += 2) {
-                double o[2];
-                #pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    const int64_t v = V[c + k];
-                    const uint64_t mag = (uint64_t)(v < 0 ? -v : v);
-                    const int L = 64 - __clzll((long long)mag);
-                    const int f = 1022 + L + s_eb[h * H + c + k] - emax;       // exponent field
-                    uint64_t m = L <= 53 ? mag << (53 - L) : (mag + (1ull << (L - 54))) >> (L - 53);
-                    uint64_t bits = ((uint64_t)(f - 1) << 52) + m;
-                    if (mag == 0 || f <= 0) bits = 0;
-                    bits |= (uint64_t)v & 0x8000000000000000ull;
-                    o[k] = bad ? __longlong_as_double(0x7FF8000000000000ll) : __longlong_as_double((long long)bits);
-                }
-                *(double2*)(dst + c) = make_double2(o[0], o[1]);
+                const double o0 = fx_double(V[c], s_eb[h * H + c], emax), o1 = fx_double(V[c + 1], s_eb[h * H + c + 1], emax);
+                *(double2*)(dst + c) = bad ? make_double2(nan, nan) : make_double2(o0, o1);
             }
             if (h == 0) {
                 const int* se = st.pool_e[side] + s_src[r];
-                st.pool_e[side][s_dst[r]] = *se + (emax < -(1 << 28) || bad ? 0 : emax - 56);
+                st.pool_e[side][s_dst[r]] = *se + (emax < -(1 << 28) || bad ? 0 : emax - 56 + s_ea[r]);
             }
         }
         __syncthreads();                              // the lists, maxima and digits are free
@@ -307,6 +399,393 @@ __global__ void __launch_bounds__(kFxThreads, D <= 32 ? 2 : 1) k_fx_step(FxStep 
     __syncthreads();
     tc::fence_after_sync();
     if (warp == 0) tc::tmem_dealloc(tmem, kCols);
+}
+
+// ---------------------------------------------------------------------------
+// Graph states over the prefix trees: vertex t of a level's nodes. Per in-edge
+// with a vertex source the tile's rows are cut and multiplied as above; the
+// edges' 64-bit results are aligned by their powers of two and added as
+// integers (log2 of the in-degree bits of the unit are given up for the sum).
+// H18 (D = 32, 2.5 in-edges): 128 nodes took 188 k cycles of the FP64 pipe.
+// ---------------------------------------------------------------------------
+
+// v 2^-d rounded, d >= 0
+__device__ __forceinline__ int64_t fx_shift(int64_t v, int d)
+{
+    if (d <= 0) return v;
+    return d > 62 ? 0 : (v + (1ll << (d - 1))) >> d;
+}
+
+template <int D>
+__global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1)
+k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __restrict__ exps, DevError* err, int t, int deg,
+           uint32_t at, uint32_t nl, TreeGroups gr, int drop)
+{
+    extern __shared__ __align__(1024) unsigned char smraw[];
+    __shared__ uint32_t tmem_slot;
+    __shared__ __align__(8) uint64_t mb_mma, mb_b;
+    __shared__ int64_t s_src[kFxRows];
+    __shared__ int s_eb[D], s_cm[D], s_ea[kFxRows], s_es[kFxRows], s_bad[kFxRows];
+    constexpr int SP = fx_split(D), H = D / SP;
+    __shared__ int s_max[SP][kFxRows];
+    __shared__ int t_e[kGtMaxDeg];                    // edges with a vertex source, then the e_0 ones
+    constexpr uint32_t kA = kFxRows * D * 2, kB = 2 * D * D;
+    constexpr uint32_t kCols = kFxSums * D <= 128 ? 128 : kFxSums * D <= 256 ? 256 : 512;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    unsigned char* const Bs = smraw + kFxDigits * kA;
+    if (warp == 0) { tc::tmem_alloc(&tmem_slot, kCols); tc::tmem_relinquish(); }
+    if (tid == 0) { tc::mbar_init(&mb_mma, 1); tc::mbar_init(&mb_b, 1); }
+    const int e0 = a.an.pred_ptr[t];
+    int nv = 0;                                       // in-edges with a vertex source
+    for (int e = e0; e < e0 + deg; ++e) nv += a.an.pred_idx[e] >= 0;
+    if (tid < deg) {
+        const bool vs = a.an.pred_idx[e0 + tid] >= 0;
+        int before = 0;
+        for (int e = e0; e < e0 + tid; ++e) before += (a.an.pred_idx[e] >= 0) == vs;
+        t_e[(vs ? 0 : nv) + before] = e0 + tid;
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = tmem_slot;
+    const int r = 32 * (warp & 3) + lane, h = warp >> 2;
+    const uint32_t tlane = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(h * H);
+    const uint32_t idesc = tc::idesc_f16(kFxRows, D);
+    uint32_t ph_mma = 0, ph_b = 0;
+    bool ok = true;
+    int64_t held = -1;
+    constexpr uint32_t kPoll = 1u << 24;
+    const int nt = gr.tile[4];
+    const int tile0 = (int)((int64_t)nt * blockIdx.x / gridDim.x);
+    const int tile1 = (int)((int64_t)nt * (blockIdx.x + 1) / gridDim.x);
+    for (int tile = tile0; tile < tile1; ++tile) {
+        int g = 0;
+        while (g < 3 && tile >= gr.tile[g + 1]) ++g;
+        const uint32_t i0 = gr.b[g] + (uint32_t)(tile - gr.tile[g]) * kFxRows;
+        const int n = (int)min(gr.b[g + 1] - i0, (uint32_t)kFxRows);
+        int64_t acc[H];
+        int X[H];
+        #pragma unroll
+        for (int c = 0; c < H; ++c) { acc[c] = 0; X[c] = kFxNoExp; }
+        bool bad = false;
+        for (int k = 0; k < nv; ++k) {
+            const int64_t mat = (int64_t)t_e[k] * 4 + g;
+            if (tid < kFxRows) {                      // rows past n repeat the first
+                const uint32_t row = __ldg(a.items + at + (size_t)(k + 1) * nl + i0 + (tid < n ? tid : 0));
+                s_src[tid] = row;
+                s_es[tid] = a.pool_e[row];
+                s_ea[tid] = kFxNoExp;
+                s_bad[tid] = 0;
+            }
+            if (held != mat) {
+                if (tid == 0) {
+                    tc::mbar_expect_tx(&mb_b, kFxDigits * kB);
+                    tc::bulk_g2s(Bs, img + (size_t)mat * kFxDigits * kB, kFxDigits * kB, &mb_b);
+                }
+                if (tid < 2 * D) (tid < D ? s_cm : s_eb - D)[tid] = __ldg(exps + (size_t)mat * 2 * D + tid);
+            }
+            __syncthreads();
+            fx_rows<D, SP>(a.pool, s_src, s_cm, s_ea, s_bad, smraw);
+            tc::fence_proxy_async();
+            tc::fence_before_sync();
+            __syncthreads();
+            if (tid == 0) {
+                tc::fence_after_sync();
+                if (held != mat) ok = tc::mbar_wait(&mb_b, ph_b, kPoll) && ok;
+                const uint64_t d0 = tc::desc(0, 128, 16 * D);
+                fx_mma<D / 16>(tmem, D, d0 + (tc::smem_addr(smraw) >> 4), d0 + (tc::smem_addr(Bs) >> 4), kA, kB, idesc);
+                tc::mma_commit(&mb_mma);
+            }
+            if (held != mat) ph_b ^= 1u;
+            held = mat;
+            ok = tc::mbar_wait(&mb_mma, ph_mma, kPoll) && ok;
+            ph_mma ^= 1u;
+            tc::fence_after_sync();
+            const int ex = s_ea[r] + s_es[r];
+            bad |= s_bad[r] != 0;
+            #pragma unroll
+            for (int c0 = 0; c0 < H; c0 += 8) {
+                uint32_t w[kFxSums][8];
+                #pragma unroll
+                for (int l = 0; l < kFxSums; ++l) tc::tmem_ld8u(tlane + (uint32_t)(l * D + c0), w[l]);
+                tc::tmem_wait_ld();
+                #pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    int s[kFxSums];
+                    #pragma unroll
+                    for (int l = 0; l < kFxSums; ++l) s[l] = fx_int(w[l][c], (l + 1) * D <= 256);
+                    const int64_t v = fx_join(s, drop);
+                    const int eb = s_eb[h * H + c0 + c];
+                    bad |= eb == kFxNotFinite;
+                    if (v != 0) {
+                        const int x = ex + eb;
+                        int64_t& A = acc[c0 + c];
+                        int& XA = X[c0 + c];
+                        if (x > XA) { A = fx_shift(A, x - XA) + v; XA = x; }
+                        else A += fx_shift(v, XA - x);
+                    }
+                }
+            }
+            tc::fence_before_sync();
+            __syncthreads();                          // accumulators, digits and lists are free
+        }
+        for (int k = nv; k < deg; ++k) {              // M e_0: column 0 of the matrix
+            const double* col = a.an.AT + ((size_t)t_e[k] * 4 + g) * D * D + h * H;
+            #pragma unroll
+            for (int c = 0; c < H; ++c) {
+                const double m = __ldg(col + c);
+                if (fx_not_finite(m)) bad = true;
+                const int x = fx_exp(m);
+                int64_t v = (int64_t)fx_code(m, -x) - 0x80808080808080ll;             // unit 2^-55
+                v = drop ? fx_shift(v, drop - 1) : v * 2;
+                if (v != 0) {
+                    if (x > X[c]) { acc[c] = fx_shift(acc[c], x - X[c]) + v; X[c] = x; }
+                    else acc[c] += fx_shift(v, X[c] - x);
+                }
+            }
+        }
+        int emax = bad ? kFxNotFinite : -(1 << 29);
+        #pragma unroll
+        for (int c = 0; c < H; ++c)
+            if (acc[c] != 0) emax = max(emax, 64 - __clzll(acc[c] < 0 ? -acc[c] : acc[c]) + X[c]);
+        s_max[h][r] = emax;
+        __syncthreads();                              // the parts of each row meet
+        #pragma unroll
+        for (int k = 0; k < SP; ++k) emax = max(emax, s_max[k][r]);
+        if (r < n) {
+            const uint32_t out = __ldg(a.items + at + i0 + r);
+            double* dst = a.pool + (size_t)out * D + h * H;
+            const bool nf = emax >= kFxNotFinite;
+            const double nan = __longlong_as_double(0x7FF8000000000000ll);
+            #pragma unroll
+            for (int c = 0; c < H; c += 2) {
+                const double o0 = fx_double(acc[c], X[c], emax), o1 = fx_double(acc[c + 1], X[c + 1], emax);
+                *(double2*)(dst + c) = nf ? make_double2(nan, nan) : make_double2(o0, o1);
+            }
+            if (h == 0) a.pool_e[out] = emax < -(1 << 28) || nf ? 0 : emax - 56 + drop;
+        }
+        __syncthreads();                              // s_max is free
+    }
+    if (!ok && tid == 0) report(err, 5, 4, (long long)blockIdx.x);
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    if (warp == 0) tc::tmem_dealloc(tmem, kCols);
+}
+
+template <int D>
+void fx_graph_launch(const TreeGraph64& a, const unsigned char* img, const int* exps, DevError* err, int t, int deg,
+                     const TreeLevels& lv, const TreeGroups& g, int n_sm, cudaStream_t st)
+{
+    const size_t smem = (size_t)kFxDigits * (kFxRows * D * 2 + 2 * D * D);
+    allow_max_smem(k_fx_graph<D>);
+    int drop = -6;                                    // D deg <= 2^(6 + drop) keeps the sums in 63 bits
+    for (int x = 1; x < D; x <<= 1) ++drop;
+    for (int x = 1; x < deg; x <<= 1) ++drop;
+    k_fx_graph<D><<<(unsigned)std::min<int64_t>(g.tile[4], (int64_t)(D <= 32 ? 2 : 1) * n_sm), kFxRows * fx_split(D), smem, st>>>(
+        a, img, exps, err, t, deg, lv.at[t], lv.n[t], g, std::max(0, drop));
+}
+
+// ---------------------------------------------------------------------------
+// Normalised chain readout over the prefix trees (the steps of k_tree_rnn): the
+// 4 D candidate entries of 128 nodes as one product of the nodes' cells with the
+// vertex's four matrices, 32 rows of them at a time. FP64 work is what is left:
+// adding v, P and the choice (~3 operations per entry instead of D + 3).
+// ---------------------------------------------------------------------------
+
+template <int KP>
+__global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* __restrict__ img, const int* __restrict__ exps,
+                                                DevError* err, int t, uint32_t at, uint32_t nl, TreeGroups gr)
+{
+    extern __shared__ __align__(1024) unsigned char smraw[];
+    __shared__ uint32_t tmem_slot;
+    __shared__ __align__(8) uint64_t mb_mma, mb_b;
+    __shared__ const double* s_src[kFxRows];
+    __shared__ double s_prod[kFxRows];
+    __shared__ int s_pex[kFxRows], s_sig[kFxRows], s_ea[kFxRows], s_bad[kFxRows];
+    __shared__ uint32_t s_flag[kFxRows], s_node[kFxRows];
+    __shared__ int s_cm[KP], s_eb[128];
+    constexpr uint32_t kA = kFxRows * KP * 2, kB = 32 * KP * 2;
+    constexpr uint32_t kCols = kFxSums * 32;
+    const AnsatzView& an = a.an;
+    const int K = an.K, D = an.D, DP = D | 1, nch = (4 * D + 31) / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    unsigned char* const Bs = smraw + kFxDigits * kA;                       // [nch][digits][32][KP]
+    double* rv = (double*)(Bs + (size_t)nch * kFxDigits * kB);              // [4][D]
+    double* eta = rv + 4 * D;
+    double* rw = eta + D;
+    double* cand = rw + D;                                                  // [rows][4][DP]
+    double* Pv = cand + (size_t)kFxRows * 4 * DP;                           // [rows][4]
+    if (warp == 0) { tc::tmem_alloc(&tmem_slot, kCols); tc::tmem_relinquish(); }
+    if (tid == 0) { tc::mbar_init(&mb_mma, 1); tc::mbar_init(&mb_b, 1); }
+    for (int q = tid; q < 4 * D; q += 256) rv[q] = __ldg(an.rv + (size_t)t * 4 * D + q);
+    for (int q = tid; q < D; q += 256) { eta[q] = __ldg(an.reta + (size_t)t * D + q); rw[q] = __ldg(an.rw + (size_t)t * D + q); }
+    for (int q = tid; q < KP + 128; q += 256) (q < KP ? s_cm : s_eb - KP)[q] = __ldg(exps + (size_t)t * (KP + 128) + q);
+    const double rc = __ldg(an.rc + t);
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = tmem_slot;
+    const uint32_t b_bytes = (uint32_t)nch * kFxDigits * kB;
+    bool ok = true;
+    constexpr uint32_t kPoll = 1u << 24;
+    if (tid == 0) {
+        tc::mbar_expect_tx(&mb_b, b_bytes);
+        tc::bulk_g2s(Bs, img + (size_t)t * b_bytes, b_bytes, &mb_b);
+        ok = tc::mbar_wait(&mb_b, 0, kPoll);
+    }
+    const int r = 32 * (warp & 3) + lane, h = warp >> 2;                    // row and half of a 32-entry chunk
+    const uint32_t tlane = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(h * 16);
+    const uint32_t idesc = tc::idesc_f16(kFxRows, 32);
+    uint32_t ph_mma = 0;
+    const size_t cur = (size_t)(t & 1) * a.n_nodes, prv = (size_t)((t & 1) ^ 1) * a.n_nodes;
+    const uint32_t nt = (nl + kFxRows - 1) / kFxRows;
+    for (uint32_t tile = blockIdx.x; tile < nt; tile += gridDim.x) {
+        const uint32_t i0 = tile * (uint32_t)kFxRows;
+        const int n = (int)min(nl - i0, (uint32_t)kFxRows);
+        __syncthreads();
+        if (tid < kFxRows) {
+            const uint32_t i = i0 + (tid < n ? tid : 0), node = __ldg(a.t.items + at + i);
+            s_node[tid] = node;
+            s_sig[tid] = (i >= gr.b[1]) + (i >= gr.b[2]) + (i >= gr.b[3]);
+            s_ea[tid] = kFxNoExp;
+            s_bad[tid] = 0;
+            uint32_t src = node;
+            if ((int)(a.t.start[node] & 255u) == t) src = a.t.parent[node];
+            if (src < a.t.id1) {                      // n itself up to here
+                const int64_t s = a.t.s0 + src;
+                const uint64_t na = a.t.samples[2 * s], nb = a.t.samples[2 * s + 1];
+                s_src[tid] = t > 0 ? a.cells + ((size_t)s * K + t - 1) * D : nullptr;
+                s_prod[tid] = 1.0;
+                s_pex[tid] = 0;
+                s_flag[tid] = (uint32_t)__popcll(na & low_mask(t)) | ((uint32_t)__popcll(nb & low_mask(t)) << 8);
+            } else {
+                s_src[tid] = a.cell + (prv + src) * D;
+                s_prod[tid] = a.prod[prv + src];
+                s_pex[tid] = a.pex[prv + src];
+                s_flag[tid] = a.flag[prv + src];
+            }
+        }
+        __syncthreads();
+        {
+            // the cells' digits, eight entries per task (zeros past D)
+            constexpr int TASKS = KP / 16;
+            double v[TASKS][8];
+            int rows[TASKS], pcs[TASKS];
+            #pragma unroll
+            for (int u = 0; u < TASKS; ++u) {
+                const int q = warp + 8 * u;
+                const int row = KP == 16 ? q * 16 + (lane & 7) + 8 * (lane >> 4) : q * 8 + (lane & 7);
+                const int pc = KP == 16 ? (lane >> 3) & 1 : lane >> 3;
+                rows[u] = row;
+                pcs[u] = pc;
+                const double* src = s_src[row];
+                int e = kFxNoExp;
+                bool bad = false;
+                #pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int c = 8 * pc + k;
+                    v[u][k] = c < D ? (src ? src[c] : (c == 0 ? 1.0 : 0.0)) : 0.0;     // h_{-1} = e_0
+                    e = max(e, fx_exp(v[u][k]) + s_cm[c]);
+                    bad |= fx_not_finite(v[u][k]);
+                }
+                atomicMax(&s_ea[row], e);
+                if (bad) s_bad[row] = 1;
+            }
+            __syncthreads();
+            #pragma unroll
+            for (int u = 0; u < TASKS; ++u) {
+                const int ea = s_ea[rows[u]];
+                uint64_t c[8];
+                #pragma unroll
+                for (int k = 0; k < 8; ++k) c[k] = fx_code(v[u][k], s_cm[8 * pcs[u] + k] - ea);
+                const uint32_t off = tc::op_offset(rows[u], 8 * pcs[u], KP);
+                #pragma unroll
+                for (int i = 0; i < kFxDigits; ++i) {
+                    __align__(16) __half2 d[4];
+                    #pragma unroll
+                    for (int k = 0; k < 4; ++k) d[k] = fx_digit2(c[2 * k], c[2 * k + 1], i);
+                    *(uint4*)(smraw + (kFxDigits - 1 - i) * kA + off) = *(const uint4*)d;
+                }
+            }
+        }
+        const int ea = s_ea[r];
+        const bool row_bad = s_bad[r] != 0;
+        for (int ch = 0; ch < nch; ++ch) {
+            tc::fence_proxy_async();
+            tc::fence_before_sync();
+            __syncthreads();                          // digits written (first chunk), accumulators read (later ones)
+            if (tid == 0) {
+                tc::fence_after_sync();
+                const uint64_t d0 = tc::desc(0, 128, 16 * KP);
+                fx_mma<KP / 16>(tmem, 32, d0 + (tc::smem_addr(smraw) >> 4),
+                                d0 + (tc::smem_addr(Bs + (size_t)ch * kFxDigits * kB) >> 4), kA, kB, idesc);
+                tc::mma_commit(&mb_mma);
+            }
+            ok = tc::mbar_wait(&mb_mma, ph_mma, kPoll) && ok;
+            ph_mma ^= 1u;
+            tc::fence_after_sync();
+            #pragma unroll
+            for (int c0 = 0; c0 < 16; c0 += 8) {
+                const int col = 32 * ch + 16 * h + c0;
+                if (col >= 4 * D) break;              // uniform over the warp
+                uint32_t w[kFxSums][8];
+                #pragma unroll
+                for (int l = 0; l < kFxSums; ++l) tc::tmem_ld8u(tlane + (uint32_t)(l * 32 + c0), w[l]);
+                tc::tmem_wait_ld();
+                #pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    if (col + c >= 4 * D) break;
+                    int s[kFxSums];
+                    #pragma unroll
+                    for (int l = 0; l < kFxSums; ++l) s[l] = fx_int(w[l][c], (l + 1) * KP <= 256);
+                    const int64_t v = fx_join(s, 0);
+                    const int eb = s_eb[col + c];
+                    // fx_double scales by 2^-(emax): emax = 0 gives V 2^(56 - 56) at power - 56
+                    const double y = v == 0 ? 0.0 : fx_double(v, ea + eb - 56, 0);
+                    const int sg = (col + c) / D, cc = col + c - sg * D;
+                    cand[((size_t)r * 4 + sg) * DP + cc] =
+                        row_bad || eb == kFxNotFinite ? __longlong_as_double(0x7FF8000000000000ll) : rv[col + c] + y;
+                }
+            }
+        }
+        tc::fence_before_sync();
+        __syncthreads();
+        for (int q = tid; q < n * 4; q += 256) {
+            const double* x = cand + (size_t)q * DP;
+            double p = 0.0;
+            for (int c = 0; c < D; ++c) p = fma(eta[c] * x[c], x[c], p);
+            Pv[q] = p;
+        }
+        __syncthreads();
+        if (tid < n) tree_rnn_pick(a, t, tid, s_sig[tid], s_flag[tid], s_prod[tid], s_pex[tid], cur + s_node[tid], cand, DP, Pv, rw, rc);
+        if (t + 1 < K)
+            for (int q = tid; q < n * D; q += 256) {
+                const int it = q / D, c = q - it * D;
+                a.cell[(cur + s_node[it]) * D + c] = cand[(size_t)(it * 4 + s_sig[it]) * DP + c];
+            }
+    }
+    if (!ok && tid == 0) report(err, 5, 4, (long long)blockIdx.x);
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    if (warp == 0) tc::tmem_dealloc(tmem, kCols);
+}
+
+// per site: row s D + r of the operand is row r of M^s, in blocks of 32 rows
+__global__ void __launch_bounds__(256) k_fx_rnn_images(const double* __restrict__ A, int D, int KP, unsigned char* img, int* exps)
+{
+    __shared__ int sc[32], sr[128];
+    const int t = blockIdx.x, nch = (4 * D + 31) / 32;
+    const double* M = A + (size_t)t * 4 * D * D;
+    fx_image([&](int n, int k) { return __ldg(M + (size_t)n * D + k); }, 4 * D, D, 32, KP,
+             img + (size_t)t * nch * kFxDigits * 64 * KP, exps + (size_t)t * (KP + 128), exps + (size_t)t * (KP + 128) + KP, sc, sr);
+}
+
+size_t fx_rnn_smem(int D)
+{
+    const size_t KP = D <= 16 ? 16 : 32, nch = (4 * D + 31) / 32;
+    return kFxDigits * (kFxRows * KP * 2 + nch * 64 * KP) + (6 * D + (size_t)kFxRows * 4 * (D | 1) + 4 * kFxRows) * 8;
 }
 
 // rows of the unit vector e_0 with power 0
@@ -362,14 +841,52 @@ void fx_launch(const FxStep& s, int64_t tiles, int n_sm, cudaStream_t st)
     const size_t smem = (size_t)kFxDigits * (kFxRows * D * 2 + 2 * D * D);
     allow_max_smem(k_fx_step<D>);
     const int per = D <= 16 ? 2 : D <= 32 ? 2 : 1;    // 512 tensor-memory columns per SM
-    k_fx_step<D><<<(unsigned)std::min<int64_t>(tiles, (int64_t)per * n_sm), kFxThreads, smem, st>>>(s);
+    k_fx_step<D><<<(unsigned)std::min<int64_t>(tiles, (int64_t)per * n_sm), kFxRows * fx_split(D), smem, st>>>(s);
 }
 
 }  // namespace
 
-int launch_fx_images(const double* A, int n_mats, int D, unsigned char* img, int* exps, cudaStream_t st)
+int launch_fx_images(const double* A, int n_mats, int D, int sides, unsigned char* img, int* exps, cudaStream_t st)
 {
-    k_fx_images<<<dim3((unsigned)n_mats, 2), 256, 0, st>>>(A, n_mats, D, img, exps);
+    k_fx_images<<<dim3((unsigned)n_mats, (unsigned)sides), 256, 0, st>>>(A, n_mats, D, img, exps);
+    return 1;
+}
+
+int launch_fx_graph(const TreeGraph64& a, const unsigned char* img, const int* exps, DevError* err, int t, int deg,
+                    const TreeLevels& lv, const int64_t* bounds, int n_sm, cudaStream_t st)
+{
+    const TreeGroups g = tree_groups(t, bounds, kFxRows);
+    if (g.tile[4] == 0) return 0;
+    switch (a.an.D) {
+    case 16: fx_graph_launch<16>(a, img, exps, err, t, deg, lv, g, n_sm, st); break;
+    case 32: fx_graph_launch<32>(a, img, exps, err, t, deg, lv, g, n_sm, st); break;
+    case 48: fx_graph_launch<48>(a, img, exps, err, t, deg, lv, g, n_sm, st); break;
+    default: fx_graph_launch<64>(a, img, exps, err, t, deg, lv, g, n_sm, st); break;
+    }
+    return 1;
+}
+
+int launch_fx_rnn_images(const double* A, int K, int D, unsigned char* img, int* exps, cudaStream_t st)
+{
+    k_fx_rnn_images<<<(unsigned)K, 256, 0, st>>>(A, D, D <= 16 ? 16 : 32, img, exps);
+    return 1;
+}
+
+int launch_fx_rnn(const TreeRnn& a, const unsigned char* img, const int* exps, DevError* err, int t, const TreeLevels& lv,
+                  const int64_t* bounds, int n_sm, cudaStream_t st)
+{
+    if (lv.n[t] == 0) return 0;
+    const size_t smem = fx_rnn_smem(a.an.D);
+    const int64_t nt = (lv.n[t] + kFxRows - 1) / kFxRows;
+    const int per = smem <= 100 * 1024 ? 2 : 1;       // 256 tensor-memory columns each
+    const unsigned grid = (unsigned)std::min<int64_t>(nt, (int64_t)per * n_sm);
+    if (a.an.D <= 16) {
+        allow_max_smem(k_fx_rnn<16>);
+        k_fx_rnn<16><<<grid, 256, smem, st>>>(a, img, exps, err, t, lv.at[t], lv.n[t], tree_groups(t, bounds, kFxRows));
+    } else {
+        allow_max_smem(k_fx_rnn<32>);
+        k_fx_rnn<32><<<grid, 256, smem, st>>>(a, img, exps, err, t, lv.at[t], lv.n[t], tree_groups(t, bounds, kFxRows));
+    }
     return 1;
 }
 

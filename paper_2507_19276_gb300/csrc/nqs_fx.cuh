@@ -2,7 +2,7 @@
 // (see nqs_fx.cu).
 #pragma once
 
-#include "nqs_kernels.cuh"
+#include "nqs_tree.cuh"
 
 namespace nqs {
 
@@ -14,11 +14,12 @@ inline bool fx_fits(int D) { return D % 16 == 0 && D >= 16 && D <= kFxMaxD; }
 
 // Digit images of a chain's site matrices: per (side, site, local state) -- side
 // 0: y = M x, side 1: y = x^T M -- kFxDigits FP16 matrices of D x D (K-major
-// core matrices, most significant first), and per output row its power of two
-// (kFxNotFinite: the row holds an infinity or a NaN).
+// core matrices, most significant first), and the powers of two of its columns,
+// then of its rows ([2][D]; kFxNotFinite: the row holds an infinity or a NaN).
 constexpr int kFxNotFinite = 1 << 28;
-inline size_t fx_image_bytes(int n_mats, int D) { return (size_t)2 * n_mats * kFxDigits * 2 * D * D; }
-int launch_fx_images(const double* A, int n_mats, int D, unsigned char* img, int* exps, cudaStream_t st);
+// sides = 1: side 0 alone (a graph's edges).
+inline size_t fx_image_bytes(int n_mats, int D, int sides) { return (size_t)sides * n_mats * kFxDigits * 2 * D * D; }
+int launch_fx_images(const double* A, int n_mats, int D, int sides, unsigned char* img, int* exps, cudaStream_t st);
 
 // One product per item: row `src` times the group's matrix into row `dst`,
 // renormalised to a largest magnitude in [0.5, 1), its power of two added to the
@@ -40,6 +41,22 @@ struct FxStep {
     DevError* err;
 };
 int launch_fx_step(const FxStep& s, int D, int n_sm, cudaStream_t st);
+
+// vertex t of the nodes of level t (FP64 graph states, see TreeGraph64)
+int launch_fx_graph(const TreeGraph64& a, const unsigned char* img, const int* exps, DevError* err, int t, int deg,
+                    const TreeLevels& lv, const int64_t* bounds, int n_sm, cudaStream_t st);
+
+// the normalised readout's candidate cells (see TreeRnn): images of a site's four
+// matrices, widths whose tile fits shared memory
+constexpr int kFxRnnMaxD = 24;
+inline size_t fx_rnn_image_bytes(int K, int D)
+{
+    return (size_t)K * ((4 * D + 31) / 32) * kFxDigits * 64 * (D <= 16 ? 16 : 32);
+}
+inline size_t fx_rnn_exps(int K, int D) { return (size_t)K * ((D <= 16 ? 16 : 32) + 128); }
+int launch_fx_rnn_images(const double* A, int K, int D, unsigned char* img, int* exps, cudaStream_t st);
+int launch_fx_rnn(const TreeRnn& a, const unsigned char* img, const int* exps, DevError* err, int t, const TreeLevels& lv,
+                  const int64_t* bounds, int n_sm, cudaStream_t st);
 
 // row `at` of every sample (stride rows each) set to e_0 with power 0
 int launch_fx_unit_rows(double* rows, int* exps, int64_t n, int64_t stride, int64_t at, int D, cudaStream_t st);

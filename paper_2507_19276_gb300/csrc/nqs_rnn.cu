@@ -37,13 +37,6 @@ __device__ __forceinline__ double warp_allsum(double v)
     return v;
 }
 
-__device__ __forceinline__ bool rnn_allowed(const AnsatzView& an, int i, int nad, int nbd, int s)
-{
-    if (an.mask_na < 0) return true;
-    const int ea = nad + (s & 1), eb = nbd + (s >> 1), left = an.K - 1 - i;
-    return ea <= an.mask_na && eb <= an.mask_nb && an.mask_na - ea <= left && an.mask_nb - eb <= left;
-}
-
 // One warp: the four candidate cells of vertex i into cand[4][D] (shared
 // memory) and P_i(s) on every lane. src(j) gives the cell of vertex j >= 0;
 // the boundary source j = -1 is e_0 (M e_0 = column 0 of M).
@@ -279,8 +272,6 @@ __global__ void __launch_bounds__(256) k_rnn_amp(RnnAmpArgs a)
 // that re-ran every row took 420 ms for 300 H50 samples (chi = 10).
 // ---------------------------------------------------------------------------
 
-constexpr double kProdLow = 0x1p-500;
-
 __global__ void __launch_bounds__(256) k_tree_rnn(TreeRnn a, int t, uint32_t at, uint32_t nl, TreeGroups gr, int IT)
 {
     extern __shared__ double sm[];
@@ -358,31 +349,7 @@ __global__ void __launch_bounds__(256) k_tree_rnn(TreeRnn a, int t, uint32_t at,
             Pv[q] = p;
         }
         __syncthreads();
-        if (tid < n) {
-            const int sg = s_sig[tid];
-            uint32_t f = s_flag[tid];
-            const int nad = (int)(f & 255u), nbd = (int)((f >> 8) & 255u);
-            double Z = 0.0;
-            for (int q = 0; q < 4; ++q)
-                if (rnn_allowed(an, t, nad, nbd, q)) Z += Pv[tid * 4 + q];
-            const double P = Pv[tid * 4 + sg];
-            const double* h = cand + (size_t)(tid * 4 + sg) * DP;
-            double ph = rc;
-            for (int c = 0; c < D; ++c) ph = fma(rw[c], h[c], ph);
-            double prod = s_prod[tid];
-            int pex = s_pex[tid];
-            if (!rnn_allowed(an, t, nad, nbd, sg) || !(P > 0.0) || !(Z > 0.0)) f |= 1u << 17;
-            else {
-                prod *= P / Z;
-                if (prod < kProdLow) { prod *= 0x1p500; --pex; }
-                f ^= ph < 0.0 ? 1u << 16 : 0u;
-            }
-            f += (uint32_t)(sg & 1) + ((uint32_t)(sg >> 1) << 8);
-            const uint32_t node = s_node[tid];
-            a.prod[cur + node] = prod;
-            a.pex[cur + node] = pex;
-            a.flag[cur + node] = f;
-        }
+        if (tid < n) tree_rnn_pick(a, t, tid, s_sig[tid], s_flag[tid], s_prod[tid], s_pex[tid], cur + s_node[tid], cand, DP, Pv, rw, rc);
         if (t + 1 < K)
             for (int q = tid; q < n * D; q += 256) {
                 const int it = q / D, c = q - it * D;

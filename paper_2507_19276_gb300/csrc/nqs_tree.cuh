@@ -252,4 +252,37 @@ inline TreeGroups tree_groups(int t, const int64_t* bounds, int rows)
     return g;
 }
 
+__device__ __forceinline__ bool rnn_allowed(const AnsatzView& an, int i, int nad, int nbd, int s)
+{
+    if (an.mask_na < 0) return true;
+    const int ea = nad + (s & 1), eb = nbd + (s >> 1), left = an.K - 1 - i;
+    return ea <= an.mask_na && eb <= an.mask_nb && an.mask_na - ea <= left && an.mask_nb - eb <= left;
+}
+
+// Node `it` of a tile of level t chooses its local state sg: the normaliser over
+// the allowed states, the phase's sign, the running weight and electron counts
+// (cand [node][4][DP] the candidate cells, Pv [node][4] their weights).
+__device__ __forceinline__ void tree_rnn_pick(const TreeRnn& a, int t, int it, int sg, uint32_t f, double prod, int pex, size_t out,
+                                              const double* cand, int DP, const double* Pv, const double* rw, double rc)
+{
+    const AnsatzView& an = a.an;
+    const int nad = (int)(f & 255u), nbd = (int)((f >> 8) & 255u);
+    double Z = 0.0;
+    for (int q = 0; q < 4; ++q)
+        if (rnn_allowed(an, t, nad, nbd, q)) Z += Pv[it * 4 + q];
+    const double P = Pv[it * 4 + sg];
+    const double* h = cand + (size_t)(it * 4 + sg) * DP;
+    double ph = rc;
+    for (int c = 0; c < an.D; ++c) ph = fma(rw[c], h[c], ph);
+    if (!rnn_allowed(an, t, nad, nbd, sg) || !(P > 0.0) || !(Z > 0.0)) f |= 1u << 17;
+    else {
+        prod *= P / Z;
+        if (prod < 0x1p-500) { prod *= 0x1p500; --pex; }
+        f ^= ph < 0.0 ? 1u << 16 : 0u;
+    }
+    a.prod[out] = prod;
+    a.pex[out] = pex;
+    a.flag[out] = f + (uint32_t)(sg & 1) + ((uint32_t)(sg >> 1) << 8);
+}
+
 }  // namespace nqs

@@ -230,3 +230,33 @@ def test_fixed_point_steps_not_finite(ctx):
     occ = _occ(s.samples, s.K)
     hit = (occ[:, 10] + occ[:, 11]) == 2
     assert np.all(np.isnan(la[hit])) and np.all(np.isfinite(la[~hit]))
+
+
+@pytest.mark.parametrize("D,ns", [(16, 301), (32, 260), (48, 130), (64, 129)])
+@pytest.mark.parametrize("chain", [False, True])
+def test_prefix_tree_fixed_point(ctx, D, ns, chain):
+    """Levels large enough for the fixed-point tiles, chains and graphs with up to
+    four in-edges and e_0 sources, part tiles; the FP64 bar."""
+    from oracle import oracle as O
+    s = W.tiny_system(K=8, na=4, nb=4, D=D, n_hidden=3, seed=D, n_samples=ns, eps=0.01, n_draws=20) if chain \
+        else _dag(D, 8, D, n_samples=ns, eps=0.01, n_draws=20)
+    ctx.set_system(s)
+    ctx.set_precision(nqs.NQS_PREC_FP64)
+    ref = O.local_energy(O.Problem(s), cond=True)
+    e, summ = ctx.local_energy(s.samples, s.counts, s.eps, s.n_draws, s.seed)
+    scale = np.maximum(np.abs(ref["e_loc"]), ref["e_abs"]) + (2.0 ** -52 / 1e-12) * ref["e_cond"]
+    assert np.all(np.abs(e - ref["e_loc"]) <= 1e-12 * scale)
+    assert summ["n_det"] == int(ref["n_det"].sum())
+
+
+@pytest.mark.parametrize("D,ns", [(4, 300), (10, 301), (16, 129), (17, 200), (24, 128)])
+def test_normalised_chain_fixed_point(ctx, D, ns):
+    """The same for the normalised readout's candidate cells: one to three blocks of
+    32 entries, both reduction widths."""
+    from oracle import oracle as O
+    s = W.with_readout(W.tiny_system(K=8, na=4, nb=4, D=D, n_hidden=2, seed=D, eps=0.01, n_draws=20, n_samples=ns), seed=D)
+    ctx.set_system(s)
+    ctx.set_precision(nqs.NQS_PREC_FP64)
+    ref = O.local_energy(O.Problem(s))
+    e, _ = ctx.local_energy(s.samples, s.counts, s.eps, s.n_draws, s.seed)
+    assert np.all(np.abs(e - ref["e_loc"]) <= 1e-12 * np.maximum(np.abs(ref["e_loc"]), ref["e_abs"]))
