@@ -1566,8 +1566,8 @@ extern "C" int nqs_set_readout(nqs_ctx* c, const double* v, const double* eta, c
     if (c->has_fx_rnn) {
         TRY(ensure(c, c->fx_rimg, fx_rnn_image_bytes(K, D)));
         TRY(ensure(c, c->fx_rexps, fx_rnn_exps(K, D) * 4));
-        LAUNCH(NQS_STAGE_OTHER, launch_fx_rnn_images(c->av.A, K, D, (unsigned char*)c->fx_rimg.p, (int*)c->fx_rexps.p,
-                                                     c->stream));
+        LAUNCH(NQS_STAGE_OTHER, launch_fx_rnn_images(c->av.A, (const double*)c->rv.p, K, D, (unsigned char*)c->fx_rimg.p,
+                                                     (int*)c->fx_rexps.p, c->stream));
         CK(cudaGetLastError());
         CK(cudaStreamSynchronize(c->stream));
     }
@@ -2226,8 +2226,10 @@ int vjp_core(nqs_ctx* c, const uint64_t* ds, const double* du, int64_t Ns, doubl
         g.part = (double*)((char*)g.soff + (((size_t)K * 5 * 8 + 255) & ~(size_t)255));
         g.vcorr = (double*)(scr + ((grad_corr_offset(c->av, n) + 255) & ~(size_t)255));
         g.cpart = g.vcorr + (size_t)n * NH;
+        g.err = (DevError*)c->derr.p;
         LAUNCH(NQS_STAGE_OTHER, launch_grad_fp64(g, c->stream));
         CK(cudaGetLastError());
+        if (dg && c->has_fx) TRY(read_dev_error(c));
     }
     return NQS_OK;
 }

@@ -137,18 +137,24 @@ __global__ void __launch_bounds__(256) k_fx_images(const double* __restrict__ A,
              img + id * kFxDigits * 2 * D * D, exps + id * 2 * D, exps + id * 2 * D + D, sc, sr);
 }
 
-// an FP32 accumulator that holds an integer; small: |v| <= 2^22
-__device__ __forceinline__ int fx_int(uint32_t w, bool small)
+// The eight sums of a result (FP32 accumulators that hold integers) as an integer
+// of unit 2^-(56 - drop). A sum of at most 2^22 is read from the low bits of
+// v + 1.5 2^23 (their common offset comes off once per pair), a larger one converted.
+template <int RED>
+__device__ __forceinline__ int64_t fx_join(const uint32_t* w, int drop)
 {
-    const float v = __uint_as_float(w);
-    return small ? __float_as_int(v + 12582912.f) - 0x4B400000 : __float2int_rn(v);
-}
-
-// the eight sums of a result as an integer of unit 2^-(56 - drop)
-__device__ __forceinline__ int64_t fx_join(const int* s, int drop)
-{
-    const int64_t hi = (int64_t)(s[0] * 256 + s[1]) * 65536 + (s[2] * 256 + s[3]);
-    const int64_t lo = ((int64_t)(s[4] * 256 + s[5]) * 256 + s[6]) * 256 + s[7];
+    constexpr uint32_t kOff = 0x4B400000u;        // bits of 1.5 2^23
+    uint32_t s[kFxSums];
+    #pragma unroll
+    for (int l = 0; l < kFxSums; ++l) {
+        const float v = __uint_as_float(w[l]);
+        // (l + 1, at most 7) digit pairs of RED terms of at most 2^14 each
+        const bool small = (l < kFxDigits ? l + 1 : 2 * kFxDigits - 1 - l) * RED <= 256;
+        s[l] = small ? (uint32_t)__float_as_int(v + 12582912.f) : (uint32_t)__float2int_rn(v) + kOff;
+    }
+    const int a = (int)(s[0] * 256u + s[1] - 257u * kOff), b = (int)(s[2] * 256u + s[3] - 257u * kOff);
+    const int c = (int)(s[4] * 256u + s[5] - 257u * kOff), d = (int)(s[6] * 256u + s[7] - 257u * kOff);
+    const int64_t hi = (int64_t)a * 65536 + b, lo = (int64_t)c * 65536 + d;
     return (hi << (18 - drop)) + ((lo + (1 << (13 + drop))) >> (14 + drop));
 }
 
@@ -349,8 +355,21 @@ __global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1) k_fx_s
         }
         if (held != g) ph_b ^= 1u;
         held = g;
-        ok = tc::mbar_wait(&mb_mma, ph_mma, kPoll) && ok;
+        if (tile + 1 < tile1) {                       // the next tile's rows towards L2 meanwhile
+            int g2 = g;
+            while (g2 < 7 && tile + 1 >= s_tile[g2 + 1]) ++g2;
+            const int64_t i = s_gb[g2] + (int64_t)(tile + 1 - s_tile[g2]) * kFxRows + (tid & (kFxRows - 1));
+            if (i < s_ge[g2]) {
+                const int64_t row = st.items ? (int64_t)__ldg(st.items + i).x
+                                             : (int64_t)__ldg(st.list[g2 >> 2] + i) * st.stride + st.src[g2 >> 2];
+                const double* src = st.pool[g2 >> 2] + (size_t)row * D;
+                for (int c = 16 * (tid / kFxRows); c < D; c += 16 * SP)
+                    asm volatile("prefetch.global.L2 [%0];" :: "l"(src + c));
+            }
+        }
+        if (tid == 0) ok = tc::mbar_wait(&mb_mma, ph_mma, kPoll) && ok;
         ph_mma ^= 1u;
+        __syncthreads();
         tc::fence_after_sync();
         // join the sums: V = y 2^(56 - ea - eb), and the row's largest exponent
         int64_t V[H];
@@ -363,10 +382,8 @@ __global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1) k_fx_s
             tc::tmem_wait_ld();
             #pragma unroll
             for (int c = 0; c < 8; ++c) {
-                int s[kFxSums];
-                #pragma unroll
-                for (int l = 0; l < kFxSums; ++l) s[l] = fx_int(w[l][c], (l + 1) * D <= 256);
-                const int64_t v = fx_join(s, 0);
+                const uint32_t x[kFxSums] = {w[0][c], w[1][c], w[2][c], w[3][c], w[4][c], w[5][c], w[6][c], w[7][c]};
+                const int64_t v = fx_join<D>(x, 0);
                 V[c0 + c] = v;
                 const int eb = s_eb[h * H + c0 + c];
                 if (v != 0) emax = max(emax, 64 - __clzll(v < 0 ? -v : v) + eb);
@@ -498,8 +515,9 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
             }
             if (held != mat) ph_b ^= 1u;
             held = mat;
-            ok = tc::mbar_wait(&mb_mma, ph_mma, kPoll) && ok;
+            if (tid == 0) ok = tc::mbar_wait(&mb_mma, ph_mma, kPoll) && ok;
             ph_mma ^= 1u;
+            __syncthreads();
             tc::fence_after_sync();
             const int ex = s_ea[r] + s_es[r];
             bad |= s_bad[r] != 0;
@@ -511,10 +529,8 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
                 tc::tmem_wait_ld();
                 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
-                    int s[kFxSums];
-                    #pragma unroll
-                    for (int l = 0; l < kFxSums; ++l) s[l] = fx_int(w[l][c], (l + 1) * D <= 256);
-                    const int64_t v = fx_join(s, drop);
+                    const uint32_t x8[kFxSums] = {w[0][c], w[1][c], w[2][c], w[3][c], w[4][c], w[5][c], w[6][c], w[7][c]};
+                    const int64_t v = fx_join<D>(x8, drop);
                     const int eb = s_eb[h * H + c0 + c];
                     bad |= eb == kFxNotFinite;
                     if (v != 0) {
@@ -587,6 +603,187 @@ void fx_graph_launch(const TreeGraph64& a, const unsigned char* img, const int* 
 }
 
 // ---------------------------------------------------------------------------
+// Outer-product sums of the gradient, sum_n (w_n g_n) h_n^T over a chunk of one
+// local-state group (k_grad_tn's blocks), with the samples as the reduction:
+// 64 samples at a time, the operands' rows (components) scaled by powers of two
+// over those samples, the exact sums converted once and added in FP64. A
+// 64-sample product of 64 x 64 takes 150 k cycles of the FP64 pipe (1.95 ms for
+// H50, D = 64, 4096 samples).
+// ---------------------------------------------------------------------------
+
+constexpr int kGradRed = 64;              // samples per product
+
+template <int D>
+__global__ void __launch_bounds__(256) k_fx_grad(GradArgs a, int chunk_samples, DevError* err)
+{
+    extern __shared__ __align__(1024) unsigned char smraw[];
+    __shared__ uint32_t tmem_slot;
+    __shared__ __align__(8) uint64_t mb_mma;
+    __shared__ const double* s_g[kGradRed];
+    __shared__ const double* s_h[kGradRed];
+    __shared__ double s_w[kGradRed];
+    __shared__ int s_e[2 * D], s_bad[2 * D];
+    constexpr uint32_t kB = 2 * D * kGradRed;         // one digit of one operand
+    constexpr uint32_t kCols = kFxSums * D <= 128 ? 128 : kFxSums * D <= 256 ? 256 : 512;
+    constexpr int H = D / 2;
+    const int K = a.an.K, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int e = blockIdx.y >> 2, sg = blockIdx.y & 3, chunk = blockIdx.x;
+    int i, j;
+    if (a.an.chain) { i = e; j = e - 1; }
+    else {
+        j = a.an.pred_idx[e];
+        int lo = 0;
+        while (a.an.pred_ptr[lo + 1] <= e) ++lo;
+        i = lo;
+    }
+    const int64_t g0 = a.soff[(size_t)i * 5 + sg], g1 = a.soff[(size_t)i * 5 + sg + 1];
+    const int64_t c0 = g0 + (int64_t)chunk * chunk_samples;
+    if (c0 >= g1) return;                             // beyond this group's chunks
+    const int64_t c1 = c0 + chunk_samples < g1 ? c0 + chunk_samples : g1;
+    if (warp == 0) { tc::tmem_alloc(&tmem_slot, kCols); tc::tmem_relinquish(); }
+    if (tid == 0) tc::mbar_init(&mb_mma, 1);
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = tmem_slot;
+    // M = 128 rows of which the first D are components (the others read what
+    // follows in shared memory and are not used)
+    const int r = 32 * (warp & 3) + lane, h = warp >> 2;
+    const bool act = 32 * (warp & 3) < D;             // uniform over the warp
+    const uint32_t tlane = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(h * H);
+    const uint32_t idesc = tc::idesc_f16(kFxRows, D);
+    uint32_t ph = 0;
+    bool ok = true;
+    double acc[H];
+    #pragma unroll
+    for (int c = 0; c < H; ++c) acc[c] = 0.0;
+    for (int64_t k0 = c0; k0 < c1; k0 += kGradRed) {
+        const int nk = (int)(c1 - k0 < kGradRed ? c1 - k0 : kGradRed);
+        if (tid < kGradRed) {
+            const double *gp = nullptr, *hp = nullptr;
+            double w = 0.0;
+            if (tid < nk) {
+                const int64_t s = a.sidx[(size_t)i * a.Ns + k0 + tid];
+                int eg, eh;
+                if (a.an.chain) {
+                    gp = a.Renv + ((size_t)s * (K + 1) + i + 1) * D;
+                    eg = a.Rexp[(size_t)s * (K + 1) + i + 1];
+                    hp = a.Lenv + ((size_t)s * (K + 1) + i) * D;
+                    eh = a.Lexp[(size_t)s * (K + 1) + i];
+                } else {
+                    gp = a.Gst + ((size_t)s * K + i) * D;
+                    eg = a.Gexp[(size_t)s * K + i];
+                    hp = j < 0 ? nullptr : a.Hst + ((size_t)s * K + j) * D;
+                    eh = j < 0 ? 0 : a.Hexp[(size_t)s * K + j];
+                }
+                w = ldexp(a.u[s] / a.psi_mant[s], eg + eh - a.psi_exp[s]);
+            }
+            s_g[tid] = gp;
+            s_h[tid] = hp;
+            s_w[tid] = w;
+        }
+        if (tid < 2 * D) { s_e[tid] = kFxNoExp; s_bad[tid] = 0; }
+        __syncthreads();
+        // component c of operand o (0: w g, 1: h) over eight samples per task, the
+        // components across the lanes
+        constexpr int TASKS = 2 * D * (kGradRed / 8) / 256;
+        double v[TASKS][8];
+        #pragma unroll
+        for (int u = 0; u < TASKS; ++u) {
+            const int q = tid + 256 * u, c = q % (2 * D), n8 = q / (2 * D);
+            int ex = kFxNoExp;
+            bool bad = false;
+            #pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int n = 8 * n8 + k;
+                double x = 0.0;
+                if (n < nk) {
+                    if (c < D) x = s_w[n] * s_g[n][c];
+                    else x = s_h[n] ? s_h[n][c - D] : (c == D ? 1.0 : 0.0);
+                }
+                v[u][k] = x;
+                ex = max(ex, fx_exp(x));
+                bad |= fx_not_finite(x);
+            }
+            if (ex != kFxNoExp) atomicMax(&s_e[c], ex);
+            if (bad) s_bad[c] = 1;
+        }
+        __syncthreads();
+        #pragma unroll
+        for (int u = 0; u < TASKS; ++u) {
+            const int q = tid + 256 * u, c = q % (2 * D), n8 = q / (2 * D);
+            const int ex = s_e[c] == kFxNoExp ? 0 : s_e[c];
+            uint64_t cd[8];
+            #pragma unroll
+            for (int k = 0; k < 8; ++k) cd[k] = fx_code(v[u][k], -ex);
+            unsigned char* op = smraw + (c < D ? 0u : kFxDigits * kB);
+            const uint32_t off = tc::op_offset(c < D ? c : c - D, 8 * n8, kGradRed);
+            #pragma unroll
+            for (int d = 0; d < kFxDigits; ++d) {
+                __align__(16) __half2 w[4];
+                #pragma unroll
+                for (int k = 0; k < 4; ++k) w[k] = fx_digit2(cd[2 * k], cd[2 * k + 1], d);
+                *(uint4*)(op + (kFxDigits - 1 - d) * kB + off) = *(const uint4*)w;
+            }
+        }
+        tc::fence_proxy_async();
+        tc::fence_before_sync();
+        __syncthreads();
+        if (tid == 0) {
+            tc::fence_after_sync();
+            const uint64_t d0 = tc::desc(0, 128, 16 * kGradRed);
+            fx_mma<kGradRed / 16>(tmem, D, d0 + (tc::smem_addr(smraw) >> 4),
+                                  d0 + (tc::smem_addr(smraw + kFxDigits * kB) >> 4), kB, kB, idesc);
+            tc::mma_commit(&mb_mma);
+            ok = tc::mbar_wait(&mb_mma, ph, 1u << 24) && ok;
+        }
+        ph ^= 1u;
+        __syncthreads();
+        tc::fence_after_sync();
+        if (act) {
+            const int ea = r < D ? s_e[r] : 0;
+            const bool bad = r < D && s_bad[r];
+            #pragma unroll
+            for (int q0 = 0; q0 < H; q0 += 8) {
+                uint32_t w[kFxSums][8];
+                #pragma unroll
+                for (int l = 0; l < kFxSums; ++l) tc::tmem_ld8u(tlane + (uint32_t)(l * D + q0), w[l]);
+                tc::tmem_wait_ld();
+                #pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const uint32_t x[kFxSums] = {w[0][c], w[1][c], w[2][c], w[3][c], w[4][c], w[5][c], w[6][c], w[7][c]};
+                    const int col = D + h * H + q0 + c;
+                    double y = fx_double(fx_join<kGradRed>(x, 0), ea + s_e[col] - 56, 0);
+                    if (bad | s_bad[col]) y = __longlong_as_double(0x7FF8000000000000ll);
+                    acc[q0 + c] += y;
+                }
+            }
+        }
+        tc::fence_before_sync();
+        __syncthreads();                              // operands, accumulators and lists are free
+    }
+    if (act && r < D) {
+        double* out = a.part + (((size_t)chunk * a.an.n_edges + e) * 4 + sg) * D * D + (size_t)r * D + h * H;
+        #pragma unroll
+        for (int c = 0; c < H; c += 2) *(double2*)(out + c) = make_double2(acc[c], acc[c + 1]);
+    }
+    if (!ok && tid == 0) report(err, 5, 4, (long long)blockIdx.x);
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    if (warp == 0) tc::tmem_dealloc(tmem, kCols);
+}
+
+template <int D>
+void fx_grad_launch(const GradArgs& a, int64_t chunks, int chunk_samples, DevError* err, cudaStream_t st)
+{
+    allow_max_smem(k_fx_grad<D>);
+    // the MMAs read 128 rows of the last digit too: D and a spare 128 - D rows behind the operands
+    const size_t smem = (size_t)2 * kFxDigits * 2 * D * kGradRed + (size_t)2 * (128 - D) * kGradRed;
+    k_fx_grad<D><<<dim3((unsigned)chunks, (unsigned)(a.an.n_edges * 4)), 256, smem, st>>>(a, chunk_samples, err);
+}
+
+// ---------------------------------------------------------------------------
 // Normalised chain readout over the prefix trees (the steps of k_tree_rnn): the
 // 4 D candidate entries of 128 nodes as one product of the nodes' cells with the
 // vertex's four matrices, 32 rows of them at a time. FP64 work is what is left:
@@ -605,10 +802,12 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
     __shared__ int s_pex[kFxRows], s_sig[kFxRows], s_ea[kFxRows], s_bad[kFxRows];
     __shared__ uint32_t s_flag[kFxRows], s_node[kFxRows];
     __shared__ int s_cm[KP], s_eb[128];
+    __shared__ short s_pos[128];                      // candidate entry n at s DP + component
     constexpr uint32_t kA = kFxRows * KP * 2, kB = 32 * KP * 2;
     constexpr uint32_t kCols = kFxSums * 32;
     const AnsatzView& an = a.an;
     const int K = an.K, D = an.D, DP = D | 1, nch = (4 * D + 31) / 32;
+    const bool fold = D < KP;                         // v as one more column, against a cell entry of 1
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     unsigned char* const Bs = smraw + kFxDigits * kA;                       // [nch][digits][32][KP]
     double* rv = (double*)(Bs + (size_t)nch * kFxDigits * kB);              // [4][D]
@@ -621,6 +820,7 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
     for (int q = tid; q < 4 * D; q += 256) rv[q] = __ldg(an.rv + (size_t)t * 4 * D + q);
     for (int q = tid; q < D; q += 256) { eta[q] = __ldg(an.reta + (size_t)t * D + q); rw[q] = __ldg(an.rw + (size_t)t * D + q); }
     for (int q = tid; q < KP + 128; q += 256) (q < KP ? s_cm : s_eb - KP)[q] = __ldg(exps + (size_t)t * (KP + 128) + q);
+    for (int q = tid; q < 4 * D; q += 256) s_pos[q] = (short)((q / D) * DP + q % D);
     const double rc = __ldg(an.rc + t);
     tc::fence_before_sync();
     __syncthreads();
@@ -685,7 +885,7 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
                 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     const int c = 8 * pc + k;
-                    v[u][k] = c < D ? (src ? src[c] : (c == 0 ? 1.0 : 0.0)) : 0.0;     // h_{-1} = e_0
+                    v[u][k] = c < D ? (src ? src[c] : (c == 0 ? 1.0 : 0.0)) : (c == D ? 1.0 : 0.0);   // h_{-1} = e_0
                     e = max(e, fx_exp(v[u][k]) + s_cm[c]);
                     bad |= fx_not_finite(v[u][k]);
                 }
@@ -722,8 +922,9 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
                                 d0 + (tc::smem_addr(Bs + (size_t)ch * kFxDigits * kB) >> 4), kA, kB, idesc);
                 tc::mma_commit(&mb_mma);
             }
-            ok = tc::mbar_wait(&mb_mma, ph_mma, kPoll) && ok;
+            if (tid == 0) ok = tc::mbar_wait(&mb_mma, ph_mma, kPoll) && ok;
             ph_mma ^= 1u;
+            __syncthreads();
             tc::fence_after_sync();
             #pragma unroll
             for (int c0 = 0; c0 < 16; c0 += 8) {
@@ -736,16 +937,13 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
                 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
                     if (col + c >= 4 * D) break;
-                    int s[kFxSums];
-                    #pragma unroll
-                    for (int l = 0; l < kFxSums; ++l) s[l] = fx_int(w[l][c], (l + 1) * KP <= 256);
-                    const int64_t v = fx_join(s, 0);
+                    const uint32_t x[kFxSums] = {w[0][c], w[1][c], w[2][c], w[3][c], w[4][c], w[5][c], w[6][c], w[7][c]};
+                    const int64_t v = fx_join<KP>(x, 0);
                     const int eb = s_eb[col + c];
-                    // fx_double scales by 2^-(emax): emax = 0 gives V 2^(56 - 56) at power - 56
-                    const double y = v == 0 ? 0.0 : fx_double(v, ea + eb - 56, 0);
-                    const int sg = (col + c) / D, cc = col + c - sg * D;
-                    cand[((size_t)r * 4 + sg) * DP + cc] =
-                        row_bad || eb == kFxNotFinite ? __longlong_as_double(0x7FF8000000000000ll) : rv[col + c] + y;
+                    double y = fx_double(v, ea + eb - 56, 0);
+                    if (!fold) y += rv[col + c];
+                    cand[(size_t)r * 4 * DP + s_pos[col + c]] =
+                        row_bad || eb == kFxNotFinite ? __longlong_as_double(0x7FF8000000000000ll) : y;
                 }
             }
         }
@@ -772,13 +970,16 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
     if (warp == 0) tc::tmem_dealloc(tmem, kCols);
 }
 
-// per site: row s D + r of the operand is row r of M^s, in blocks of 32 rows
-__global__ void __launch_bounds__(256) k_fx_rnn_images(const double* __restrict__ A, int D, int KP, unsigned char* img, int* exps)
+// per site: row s D + r of the operand is row r of M^s and, where a column is free,
+// v^s[r], in blocks of 32 rows
+__global__ void __launch_bounds__(256) k_fx_rnn_images(const double* __restrict__ A, const double* __restrict__ v, int D, int KP,
+                                                       unsigned char* img, int* exps)
 {
     __shared__ int sc[32], sr[128];
     const int t = blockIdx.x, nch = (4 * D + 31) / 32;
     const double* M = A + (size_t)t * 4 * D * D;
-    fx_image([&](int n, int k) { return __ldg(M + (size_t)n * D + k); }, 4 * D, D, 32, KP,
+    const double* vt = v + (size_t)t * 4 * D;
+    fx_image([&](int n, int k) { return k < D ? __ldg(M + (size_t)n * D + k) : __ldg(vt + n); }, 4 * D, D < KP ? D + 1 : D, 32, KP,
              img + (size_t)t * nch * kFxDigits * 64 * KP, exps + (size_t)t * (KP + 128), exps + (size_t)t * (KP + 128) + KP, sc, sr);
 }
 
@@ -866,9 +1067,20 @@ int launch_fx_graph(const TreeGraph64& a, const unsigned char* img, const int* e
     return 1;
 }
 
-int launch_fx_rnn_images(const double* A, int K, int D, unsigned char* img, int* exps, cudaStream_t st)
+int launch_fx_grad(const GradArgs& a, int64_t chunks, int chunk_samples, DevError* err, cudaStream_t st)
 {
-    k_fx_rnn_images<<<(unsigned)K, 256, 0, st>>>(A, D, D <= 16 ? 16 : 32, img, exps);
+    switch (a.an.D) {
+    case 16: fx_grad_launch<16>(a, chunks, chunk_samples, err, st); break;
+    case 32: fx_grad_launch<32>(a, chunks, chunk_samples, err, st); break;
+    case 48: fx_grad_launch<48>(a, chunks, chunk_samples, err, st); break;
+    default: fx_grad_launch<64>(a, chunks, chunk_samples, err, st); break;
+    }
+    return 1;
+}
+
+int launch_fx_rnn_images(const double* A, const double* v, int K, int D, unsigned char* img, int* exps, cudaStream_t st)
+{
+    k_fx_rnn_images<<<(unsigned)K, 256, 0, st>>>(A, v, D, D <= 16 ? 16 : 32, img, exps);
     return 1;
 }
 

@@ -54,9 +54,12 @@ inline size_t fx_rnn_image_bytes(int K, int D)
     return (size_t)K * ((4 * D + 31) / 32) * kFxDigits * 64 * (D <= 16 ? 16 : 32);
 }
 inline size_t fx_rnn_exps(int K, int D) { return (size_t)K * ((D <= 16 ? 16 : 32) + 128); }
-int launch_fx_rnn_images(const double* A, int K, int D, unsigned char* img, int* exps, cudaStream_t st);
+int launch_fx_rnn_images(const double* A, const double* v, int K, int D, unsigned char* img, int* exps, cudaStream_t st);
 int launch_fx_rnn(const TreeRnn& a, const unsigned char* img, const int* exps, DevError* err, int t, const TreeLevels& lv,
                   const int64_t* bounds, int n_sm, cudaStream_t st);
+
+// outer-product partial sums of the gradient (k_grad_tn's, for the widths of fx_fits)
+int launch_fx_grad(const GradArgs& a, int64_t chunks, int chunk_samples, DevError* err, cudaStream_t st);
 
 // row `at` of every sample (stride rows each) set to e_0 with power 0
 int launch_fx_unit_rows(double* rows, int* exps, int64_t n, int64_t stride, int64_t at, int D, cudaStream_t st);

@@ -17,13 +17,14 @@
 // Correlator: d log|f| / d b_k = t_k, d / d W[k][s] = t_k n_s, d / d W2[k][s][t]
 // = t_k n_s n_t / 2, with t_k = tanh(theta_k) (2cosh) or -tan(theta_k) (cos,
 // Ising); one thread per parameter sums over the samples in index order.
-#include "nqs_kernels.cuh"
+#include "nqs_fx.cuh"
 
 namespace nqs {
 
 namespace {
 
 constexpr int kGradChunk = 256;   // samples per block (one chunk of a local-state group)
+constexpr int64_t kFxGradMin = 256;   // samples from which the fixed-point products run
 constexpr int kTile = 64;         // output tile edge
 constexpr int kStage = 16;        // samples staged per round
 
@@ -299,9 +300,15 @@ int launch_grad_fp64(const GradArgs& a, cudaStream_t st)
     int n = 0;
     if (a.grad_sites && a.Ns > 0) {
         launch_group_by_state(a.samples, a.Ns, a.an.K, a.sidx, a.soff, st);
-        const int nt = (D + kTile - 1) / kTile;
-        dim3 grid((unsigned)(nt * nt), (unsigned)grad_chunks(a.Ns), (unsigned)(a.an.n_edges * 4));
-        k_grad_tn<<<grid, 256, 0, st>>>(a, nt);
+        // fixed-point products where the width allows and the groups fill their
+        // 64-sample reductions (a quarter of the samples each)
+        if (fx_fits(D) && a.Ns >= kFxGradMin && a.err) {
+            launch_fx_grad(a, grad_chunks(a.Ns), kGradChunk, a.err, st);
+        } else {
+            const int nt = (D + kTile - 1) / kTile;
+            dim3 grid((unsigned)(nt * nt), (unsigned)grad_chunks(a.Ns), (unsigned)(a.an.n_edges * 4));
+            k_grad_tn<<<grid, 256, 0, st>>>(a, nt);
+        }
         const int64_t tot = (int64_t)a.an.n_edges * 4 * D * D;
         k_grad_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(a);
         n += 3;

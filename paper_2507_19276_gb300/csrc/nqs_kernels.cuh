@@ -375,6 +375,7 @@ struct GradArgs {
     // of samples the partial sums of every (column, hidden unit)
     double* vcorr;                        // [Ns][n_hidden]
     double* cpart;                        // [chunks][2K + 1][n_hidden]
+    DevError* err;                        // of the fixed-point tiles' bounded waits
 };
 // scratch bytes of the gradient for Ns samples, and the offset of vcorr in them
 size_t grad_scratch_bytes(const AnsatzView& an, int64_t Ns);
