@@ -42,15 +42,17 @@ constexpr int fx_split(int D) { return D == 64 ? 4 : 2; }
 // seven bytes: byte i (the top one nine bits wide) is digit i + 128.
 __device__ __forceinline__ uint64_t fx_code(double x, int off)
 {
-    const uint64_t b = (uint64_t)__double_as_longlong(x);
-    const int e = (int)((b >> 52) & 0x7FF);
-    uint64_t m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-    const int sh = 1020 - e - off;            // x 2^(55 + off) = m 2^-sh
-    if (sh <= 0) m <<= (-sh) & 3;
-    else m = sh > 54 ? 0ull : (m + (1ull << (sh - 1))) >> sh;
-    if (e == 0) m = 0;
-    const int64_t v = (int64_t)b < 0 ? -(int64_t)m : (int64_t)m;
-    return (uint64_t)(v + 0x80808080808080ll);
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t e = (hi >> 20) & 0x7FFu;
+    const uint32_t mh = (hi & 0xFFFFFu) | (min(e, 1u) << 20);
+    // the mantissa left-justified, x = m 2^(e - 1086), then x 2^(56 + off) (0 where
+    // the shift passes the word), rounded by its last bit
+    const uint64_t m = ((uint64_t)__funnelshift_l(lo, mh, 11) << 32) | (lo << 11);
+    uint64_t v;
+    asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"(1030u - e - (uint32_t)off));
+    v = (v + 1) >> 1;
+    const uint64_t sg = (uint64_t)((int64_t)(int32_t)hi >> 31);
+    return (v ^ sg) + (0x80808080808080ull - sg);
 }
 
 constexpr int kFxNoExp = -(1 << 20);          // power of two of a zero
@@ -73,7 +75,7 @@ __device__ __forceinline__ __half2 fx_digit2(uint64_t c0, uint64_t c1, int i)
         const uint32_t p = __byte_perm(a, b, (uint32_t)((i & 3) | ((4 + (i & 3)) << 8)));   // a's byte, x, b's byte, x
         w = (p & 0x00FF00FFu) | 0x64006400u;
     } else {
-        w = (uint32_t)(c0 >> 48) | ((uint32_t)(c1 >> 48) << 16) | 0x64006400u;
+        w = __byte_perm((uint32_t)(c0 >> 32), (uint32_t)(c1 >> 32), 0x7632) | 0x64006400u;
     }
     const __half2 k = __half2half2(__ushort_as_half((unsigned short)0x6480));               // 1024 + 128
     return __hsub2(*reinterpret_cast<const __half2*>(&w), k);
@@ -170,6 +172,31 @@ __device__ __forceinline__ double fx_double(int64_t v, int power, int emax)
     if (mag == 0 || f <= 0) bits = 0;
     else if (f >= 2047) bits = 0x7FF0000000000000ull;
     return __longlong_as_double((long long)(bits | ((uint64_t)v & 0x8000000000000000ull)));
+}
+
+// A thread's H results of row r (column block h) into the staging rows (D + 2
+// doubles apart: no bank conflicts), which reuse the digits' shared memory...
+template <int D, int H>
+__device__ __forceinline__ void fx_put(const int64_t* V, const int* power, int emax, bool bad, double* rows, int r, int h)
+{
+    const double nan = __longlong_as_double(0x7FF8000000000000ll);
+    double* out = rows + (size_t)r * (D + 2) + h * H;
+    #pragma unroll
+    for (int c = 0; c < H; c += 2) {
+        const double o0 = fx_double(V[c], power[c], emax), o1 = fx_double(V[c + 1], power[c + 1], emax);
+        *(double2*)(out + c) = bad ? make_double2(nan, nan) : make_double2(o0, o1);
+    }
+}
+
+// ... and whole rows from there to dst(row) (16 bytes per lane: stored straight
+// from the threads, 32 rows per instruction, they took a third of a tile's time)
+template <int D, class Dst>
+__device__ __forceinline__ void fx_store(const double* rows, int n, const Dst& dst)
+{
+    for (int q = threadIdx.x; q < n * (D / 2); q += blockDim.x) {
+        const int row = q / (D / 2), c = 2 * (q - row * (D / 2));
+        *(double2*)(dst(row) + c) = *(const double2*)(rows + (size_t)row * (D + 2) + c);
+    }
 }
 
 // the digit products of significance 0..7 of one operand pair into eight
@@ -395,20 +422,13 @@ __global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1) k_fx_s
         __syncthreads();                              // the parts of each row meet
         #pragma unroll
         for (int k = 0; k < SP; ++k) emax = max(emax, s_max[k][r]);
-        if (r < n) {
-            double* dst = st.pool[side] + (size_t)s_dst[r] * D + h * H;
-            const bool bad = s_bad[r] != 0 || emax >= kFxNotFinite;
-            const double nan = __longlong_as_double(0x7FF8000000000000ll);
-            #pragma unroll
-            for (int c = 0; c < H; c += 2) {
-                const double o0 = fx_double(V[c], s_eb[h * H + c], emax), o1 = fx_double(V[c + 1], s_eb[h * H + c + 1], emax);
-                *(double2*)(dst + c) = bad ? make_double2(nan, nan) : make_double2(o0, o1);
-            }
-            if (h == 0) {
-                const int* se = st.pool_e[side] + s_src[r];
-                st.pool_e[side][s_dst[r]] = *se + (emax < -(1 << 28) || bad ? 0 : emax - 56 + s_ea[r]);
-            }
+        fx_put<D, H>(V, s_eb + h * H, emax, s_bad[r] != 0 || emax >= kFxNotFinite, (double*)smraw, r, h);
+        if (r < n && h == 0) {
+            const int* se = st.pool_e[side] + s_src[r];
+            st.pool_e[side][s_dst[r]] = *se + (emax < -(1 << 28) || emax >= kFxNotFinite ? 0 : emax - 56 + s_ea[r]);
         }
+        __syncthreads();
+        fx_store<D>((const double*)smraw, n, [&](int row) { return st.pool[side] + (size_t)s_dst[row] * D; });
         __syncthreads();                              // the lists, maxima and digits are free
     }
     if (!ok && tid == 0) report(st.err, 5, 4, (long long)blockIdx.x);
@@ -568,19 +588,15 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
         __syncthreads();                              // the parts of each row meet
         #pragma unroll
         for (int k = 0; k < SP; ++k) emax = max(emax, s_max[k][r]);
-        if (r < n) {
-            const uint32_t out = __ldg(a.items + at + i0 + r);
-            double* dst = a.pool + (size_t)out * D + h * H;
-            const bool nf = emax >= kFxNotFinite;
-            const double nan = __longlong_as_double(0x7FF8000000000000ll);
-            #pragma unroll
-            for (int c = 0; c < H; c += 2) {
-                const double o0 = fx_double(acc[c], X[c], emax), o1 = fx_double(acc[c + 1], X[c + 1], emax);
-                *(double2*)(dst + c) = nf ? make_double2(nan, nan) : make_double2(o0, o1);
-            }
-            if (h == 0) a.pool_e[out] = emax < -(1 << 28) || nf ? 0 : emax - 56 + drop;
+        const uint32_t out = __ldg(a.items + at + i0 + (r < n ? r : 0));
+        fx_put<D, H>(acc, X, emax, emax >= kFxNotFinite, (double*)smraw, r, h);
+        if (h == 0) {
+            s_src[r] = out;                           // the result rows (the sources are done with)
+            if (r < n) a.pool_e[out] = emax < -(1 << 28) || emax >= kFxNotFinite ? 0 : emax - 56 + drop;
         }
-        __syncthreads();                              // s_max is free
+        __syncthreads();
+        fx_store<D>((const double*)smraw, n, [&](int row) { return a.pool + (size_t)s_src[row] * D; });
+        __syncthreads();                              // s_max and the rows are free
     }
     if (!ok && tid == 0) report(err, 5, 4, (long long)blockIdx.x);
     tc::fence_before_sync();
@@ -889,7 +905,9 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
                     e = max(e, fx_exp(v[u][k]) + s_cm[c]);
                     bad |= fx_not_finite(v[u][k]);
                 }
-                atomicMax(&s_ea[row], e);
+                e = max(e, __shfl_xor_sync(kFull, e, 8));
+                if constexpr (KP == 32) e = max(e, __shfl_xor_sync(kFull, e, 16));
+                if (KP == 16 ? !(lane & 8) : lane < 8) atomicMax(&s_ea[row], e);
                 if (bad) s_bad[row] = 1;
             }
             __syncthreads();

@@ -2,7 +2,26 @@
 // energy summary (Sec. 2.1 weighted mean, Sec. 2.3 B and E~_loc).
 #include "nqs_kernels.cuh"
 
+#include <mutex>
+#include <set>
+#include <utility>
+
 namespace nqs {
+
+void allow_max_smem_fn(const void* kernel)
+{
+    static std::mutex mu;
+    static std::set<std::pair<int, const void*>> done;
+    int dev = 0, mx = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return;
+    std::lock_guard<std::mutex> lock(mu);
+    if (done.count({dev, kernel})) return;
+    cudaDeviceGetAttribute(&mx, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaFuncAttributes fa{};
+    if (cudaFuncGetAttributes(&fa, kernel) == cudaSuccess &&
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, mx - (int)fa.sharedSizeBytes) == cudaSuccess)
+        done.insert({dev, kernel});
+}
 
 // (pq|rs) = sum_x L[x][p][q] L[x][r][s], ascending x, fused multiply-add,
 // stored at [p][q][s][r] (the layout eri_at reads).
