@@ -52,6 +52,7 @@ struct DrawArgs {
     const uint64_t* chunk_pre;           // [Ns][n_chunks] inclusive prefix of weights
     int shift;                           // remainder weight shift
     int n_draws;
+    int64_t s0;                          // first sample of this launch (set by the launcher)
     uint64_t seed;
     int64_t index_base;                  // Philox sample counter of samples[0]
     const int64_t* index;                // per-sample Philox counters (NULL: index_base + s)

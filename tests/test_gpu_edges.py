@@ -260,3 +260,31 @@ def test_normalised_chain_fixed_point(ctx, D, ns):
     ref = O.local_energy(O.Problem(s))
     e, _ = ctx.local_energy(s.samples, s.counts, s.eps, s.n_draws, s.seed)
     assert np.all(np.abs(e - ref["e_loc"]) <= 1e-12 * np.maximum(np.abs(ref["e_loc"]), ref["e_abs"]))
+
+
+@pytest.mark.parametrize("K,na,nb", [(2, 1, 1), (3, 1, 2), (4, 0, 2), (5, 5, 1), (9, 4, 2), (13, 6, 7), (16, 2, 14), (24, 12, 11), (40, 3, 2)])
+def test_count_pass_and_draws(ctx, K, na, nb):
+    """Lists, weights and draws at block edges of the canonical order (empty and
+    one-chunk blocks, short (j, b) runs, every weight width) against the oracle,
+    bit by bit."""
+    import dataclasses
+    from oracle import oracle as O
+    rng = np.random.default_rng(K)
+    dec = W._decay_1d(K, 2.0)
+    h, L = W._banded_h(rng, K, dec), W._sym_chol(rng, 2 * K, K, 0.3, dec)
+    smp = W.random_dets(rng, K, na, nb, 3) if K > 5 else W.all_dets(K, na, nb)[:4]
+    base = W.tiny_system(K=4, D=1)
+    s = dataclasses.replace(base, K=K, n_alpha=na, n_beta=nb, h1e=h, chol=L, tensors=np.ones((K, 4, 1, 1)), samples=smp,
+                            counts=np.ones(len(smp)))
+    P = O.Problem(s)
+    ctx.set_system(s)
+    for eps in (0.0, 3e-3, 0.1, 1e3):
+        off, rank, dets, H, sg = ctx.connected(s.samples, eps)
+        ranks, w = ctx.draws(s.samples, eps, 300, 9)
+        for i, d in enumerate(s.samples):
+            od, oH, osg = O.connected(P, d)
+            keep = np.abs(oH) >= eps
+            assert np.array_equal(H[off[i]:off[i + 1]], oH[keep]) and np.array_equal(sg[off[i]:off[i + 1]], osg[keep])
+            assert np.array_equal(rank[off[i]:off[i + 1]], np.flatnonzero(keep).astype(np.uint32))
+            ref, rw, _ = O.draws(P, d, i, eps, 300, 9)
+            assert int(w[i]) == int(rw) and np.array_equal(ranks[i], ref)
