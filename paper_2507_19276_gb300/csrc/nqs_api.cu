@@ -685,7 +685,7 @@ int family_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, i
     f.D = D;
     f.tc = (sizeof(T) == 4 && c->has_tc) ? 1 : 0;
     if (f.tc) {
-        f.nmax = 128;                                  // one M = 128 tensor-core tile
+        f.nmax = 0;                                    // no CUDA-core batches
         int cols = 32;
         while (cols < D) cols <<= 1;
         f.tc_cols = cols;
@@ -697,7 +697,7 @@ int family_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, i
         nm = nm / 4 * 4;
         f.nmax = nm < 4 ? 4 : (nm > 64 ? 64 : nm);
     }
-    f.batch_bytes = fam_batch_bytes(D, f.nmax, sizeof(T), f.tc != 0);
+    f.batch_bytes = fam_batch_bytes(D, f.nmax, sizeof(T));
     f.err = (DevError*)c->derr.p;
     f.A = (const T*)(dbl ? c->A.p : c->Af.p);
     f.AT = (const T*)(dbl ? c->AT.p : c->ATf.p);

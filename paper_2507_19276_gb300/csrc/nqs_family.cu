@@ -91,30 +91,62 @@ __device__ void mv_block(const T* __restrict__ MT, int D, const T* X, T* Y, int 
     }
 }
 
+// hi + lo += m (xh + xl), the pair unnormalised: the error-free product by FMA
+// and Knuth's two-sum, as in the double-double algorithms of Hida, Li and Bailey
+__device__ __forceinline__ void fma_df(float& hi, float& lo, float2 m, float xh, float xl)
+{
+    const float p = m.x * xh;
+    const float pe = fmaf(m.x, xh, -p) + fmaf(m.x, xl, m.y * xh);
+    const float u = hi + p, z = u - hi;
+    lo += ((hi - (u - z)) + (p - z)) + pe;
+    hi = u;
+}
+
 // Block-wide y_i = M x_i as mv_block, in double-FP32 arithmetic: M as (hi, lo)
 // float pairs (MT[b][a] = M[a][b]), x_i split into float halves Xh + Xl, one
-// output per thread and pass accumulated as an unnormalised pair (the
-// error-free product by FMA and Knuth's two-sum, as in the double-double
-// algorithms of Hida, Li and Bailey; relative error about D 2^-48).
+// output row per thread and pass for four vectors at once (a D = 256 matrix,
+// 512 KB, does not stay in L1, so its reads are what four vectors share), each
+// accumulated as an unnormalised pair (relative error about D 2^-48). The steps
+// of the FP64 re-evaluation of the D = 256, K = 20 tables: a vector at a time
+// 9.2 ms, four 5.9 ms.
 __device__ void mv_block_df(const float2* __restrict__ MT, int D, const float* Xh, const float* Xl,
                             double* Y, int nv)
 {
     const int G = (int)blockDim.x >= D ? (int)blockDim.x / D : 1;
+    const bool vec = (D & 3) == 0;                        // the vectors' rows are 16-byte aligned
     for (int q = threadIdx.x; q < G * D; q += blockDim.x) {
         const int a = q % D, g = q / D;
-        for (int i = g; i < nv; i += G) {
-            float hi = 0.f, lo = 0.f;
+        for (int i = 4 * g; i < nv; i += 4 * G) {
+            const int n4 = nv - i < 4 ? nv - i : 4;
+            float hi[4] = {}, lo[4] = {};
             const float* xh = Xh + (size_t)i * D;
             const float* xl = Xl + (size_t)i * D;
-            for (int b = 0; b < D; ++b) {
+            int b = 0;
+            if (vec)
+                for (; b < D; b += 4) {
+                    float2 m[4];
+                    #pragma unroll
+                    for (int u = 0; u < 4; ++u) m[u] = __ldg(MT + (size_t)(b + u) * D + a);
+                    #pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        if (k < n4) {
+                            const float4 h = *(const float4*)(xh + k * D + b), l = *(const float4*)(xl + k * D + b);
+                            fma_df(hi[k], lo[k], m[0], h.x, l.x);
+                            fma_df(hi[k], lo[k], m[1], h.y, l.y);
+                            fma_df(hi[k], lo[k], m[2], h.z, l.z);
+                            fma_df(hi[k], lo[k], m[3], h.w, l.w);
+                        }
+                    }
+                }
+            for (; b < D; ++b) {
                 const float2 m = __ldg(MT + (size_t)b * D + a);
-                const float p = m.x * xh[b];
-                const float pe = fmaf(m.x, xh[b], -p) + fmaf(m.x, xl[b], m.y * xh[b]);
-                const float u = hi + p, z = u - hi;
-                lo += ((hi - (u - z)) + (p - z)) + pe;
-                hi = u;
+                #pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (k < n4) fma_df(hi[k], lo[k], m, xh[k * D + b], xl[k * D + b]);
             }
-            Y[(size_t)i * D + a] = (double)hi + (double)lo;
+            #pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (k < n4) Y[(size_t)(i + k) * D + a] = (double)hi[k] + (double)lo[k];
         }
     }
 }
@@ -155,224 +187,9 @@ __device__ __forceinline__ int tr_key(int K, int sA, int aA, int sB, int aB)
 // A_t^{sg} (side 0, column convention) or its transpose (side 1, row vectors).
 //  - FP32 with tensor-core images: tcgen05 MMAs, M = 128 rows, N = D,
 //    operands split into FP16 hi + lo (x_hi M_hi + x_lo M_hi + x_hi M_lo),
-//    FP32 accumulation in tensor memory (tc_apply);
-//  - otherwise: shared-memory CUDA-core products (mv_block).
+//    FP32 accumulation in tensor memory (k_site_tiles_pipe, k_site_tiles_ws);
+//  - otherwise: shared-memory CUDA-core products (k_site_tiles).
 // ---------------------------------------------------------------------------
-
-template <typename T>
-struct BatchSmem {
-    T* X; T* Y;                        // CUDA-core path: [nmax][D] each
-    unsigned char* Ah; unsigned char* Al; unsigned char* Bh;   // tensor path operands
-    float* rmax;                       // [2][128]
-    uint64_t* mbar;
-    uint32_t tmem;
-    uint32_t phase;
-    int cur_mat;
-};
-
-template <typename T>
-__device__ __forceinline__ bool use_tc(const FamArgs<T>& f)
-{
-    return std::is_same<T, float>::value && f.tc;
-}
-
-// One tensor-core batch (T = float) of n <= 128 rows through the matrix image
-// `mat`: y_r = M x_r with x_r = acc.src(r), y_r rescaled by a power of two and
-// written to acc.dst(r), acc.set_exp(r, e) receiving the exponent added (the
-// row's power of two plus the image's). Row sources and destinations come
-// from the accessor; results per row do not depend on the other rows of the
-// tile. The scaled rows leave through shared memory (see the epilogue).
-template <class Acc>
-__device__ void tc_apply(const FamArgs<float>& f, BatchSmem<float>& sm, const Acc& acc, int n, int mat)
-{
-    const int D = f.D;
-    // The reduction runs over D / KC chunks of KC columns (one chunk up to
-    // D = 128): per chunk the batch rows' columns are gathered and split
-    // into FP16 hi / lo, the matrix image's chunk is staged, and the MMAs
-    // accumulate into the same tensor-memory columns.
-    const int KC = fam_tc_kc(D), nck = D / KC;
-    const int cpr = KC >> 3;                      // 8-element units per row of a chunk
-    const int nun = n * cpr;
-    bool ok = true;
-    for (int ck = 0; ck < nck; ++ck) {
-        // gather: each thread takes up to 2 units per round and issues all
-        // their loads before splitting any (latency-bound otherwise)
-        for (int u0 = 0; u0 < nun; u0 += 2 * blockDim.x) {
-            float4 v4[2][2];
-            #pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const int u = u0 + k * blockDim.x + threadIdx.x;
-                if (u < nun) {
-                    const int r = u / cpr, c = u - r * cpr;
-                    const float4* p = (const float4*)(acc.src(r) + ck * KC + 8 * c);
-                    v4[k][0] = p[0];
-                    v4[k][1] = p[1];
-                }
-            }
-            #pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const int u = u0 + k * blockDim.x + threadIdx.x;
-                if (u < nun) {
-                    const int r = u / cpr, c = u - r * cpr;
-                    const float xs[8] = {v4[k][0].x, v4[k][0].y, v4[k][0].z, v4[k][0].w,
-                                         v4[k][1].x, v4[k][1].y, v4[k][1].z, v4[k][1].w};
-                    __align__(16) __half hi[8], lo[8];
-                    #pragma unroll
-                    for (int j = 0; j < 8; ++j) tc::split_half(xs[j], hi[j], lo[j]);
-                    const uint32_t off = tc::op_offset(r, 8 * c, KC);
-                    *(uint4*)(sm.Ah + off) = *(const uint4*)hi;
-                    *(uint4*)(sm.Al + off) = *(const uint4*)lo;
-                }
-            }
-        }
-        // the image chunk (kept across batches when one chunk holds the matrix)
-        if (nck > 1 || mat != sm.cur_mat) {
-            const int nimg = 4 * D * KC / 16;
-            const uint4* __restrict__ g = f.tc_mats + (size_t)mat * (4 * D * D / 16) + (size_t)ck * nimg;
-            uint4* d = (uint4*)sm.Bh;
-            for (int i0 = 0; i0 < nimg; i0 += 4 * blockDim.x) {
-                uint4 w[4];
-                #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int i = i0 + k * blockDim.x + threadIdx.x;
-                    if (i < nimg) w[k] = __ldg(g + i);
-                }
-                #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int i = i0 + k * blockDim.x + threadIdx.x;
-                    if (i < nimg) d[i] = w[k];
-                }
-            }
-            sm.cur_mat = nck > 1 ? -1 : mat;
-        }
-        tc::fence_proxy_async();
-        tc::fence_before_sync();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            tc::fence_after_sync();
-            const uint32_t idesc = tc::idesc_f16(128, D);
-            const uint32_t lbo = 128, sbo = 16 * KC;
-            const unsigned char* Bl = sm.Bh + 2 * D * KC;
-            const unsigned char* As[3] = {sm.Ah, sm.Al, sm.Ah};
-            const unsigned char* Bs[3] = {sm.Bh, sm.Bh, Bl};
-            uint32_t acc = ck > 0 ? 1u : 0u;
-            for (int term = 0; term < 3; ++term)
-                for (int ks = 0; ks < KC / 16; ++ks) {
-                    tc::mma_f16(sm.tmem, tc::desc(tc::smem_addr(As[term]) + ks * 256, lbo, sbo),
-                                tc::desc(tc::smem_addr(Bs[term]) + ks * 256, lbo, sbo), idesc, acc);
-                    acc = 1;
-                }
-            tc::mma_commit(sm.mbar);
-        }
-        // the chunk's operands may be overwritten once its MMAs are done (one
-        // warp polls the mbarrier, the others wait at the barrier)
-        if (threadIdx.x < 32) ok = tc::mbar_wait(sm.mbar, sm.phase, 1u << 24) && ok;
-        sm.phase ^= 1u;
-        tc::fence_before_sync();
-        __syncthreads();
-        tc::fence_after_sync();
-    }
-    if (!ok && threadIdx.x == 0) report(f.err, 5, 4, (long long)f.s0);
-    // tensor memory -> registers, twice (row maximum, then the scaled row), 8
-    // columns at a time so that nothing indexed by D lives in local memory.
-    // Warp w reads lanes 32 (w % 4) .. +31 and half (w / 4) of the columns.
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int q = warp & 3, h = warp >> 2, half = D >> 1;
-    const int r = 32 * q + lane;
-    const uint32_t trow = sm.tmem + ((uint32_t)(32 * q) << 16) + h * half;
-    if (warp < 8) {
-        float m = 0.f;
-        for (int c0 = 0; c0 < half; c0 += 8) {
-            float v[8];
-            tc::tmem_ld8(trow + c0, v);
-            tc::tmem_wait_ld();
-            #pragma unroll
-            for (int j = 0; j < 8; ++j) m = fmaxf(m, fabsf(v[j]));
-        }
-        sm.rmax[h * 128 + r] = m;
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    // the scaled rows leave through shared memory in column slices of up to 64
-    // (row stride 272 bytes: 8 consecutive rows fill the 32 banks), copied out
-    // row by row so that a warp's stores fill whole lines. The slice buffer
-    // overlays the operands (free now that the MMAs completed); for D > 128 it
-    // reaches into the matrix image, which is reloaded per chunk there anyway.
-    constexpr int kSRS = 272;
-    float mm = 0.f;
-    int e = 0;
-    if (warp < 8) {
-        mm = fmaxf(sm.rmax[r], sm.rmax[128 + r]);
-        if (mm > 0.f) frexpf(mm, &e);
-        if (h == 0 && r < n) acc.set_exp(r, e + f.tc_exp[mat]);
-    }
-    const bool pw = e >= -126 && e <= 126;
-    const float sc2 = pw ? __int_as_float((127 - e) << 23) : 0.f;
-    unsigned char* slice = sm.Ah;
-    for (int cs = 0; cs < D; cs += 64) {
-        const int sw = D - cs < 64 ? D - cs : 64, hw = sw >> 1;
-        if (warp < 8) {
-            float* o = (float*)(slice + r * kSRS) + h * hw;
-            const uint32_t tr = sm.tmem + ((uint32_t)(32 * q) << 16) + cs + h * hw;
-            for (int c0 = 0; c0 < hw; c0 += 8) {
-                float v[8];
-                tc::tmem_ld8(tr + c0, v);   // every lane of the warp takes part
-                tc::tmem_wait_ld();
-                #pragma unroll
-                for (int j = 0; j < 8; ++j) v[j] = pw ? v[j] * sc2 : ldexpf(v[j], -e);
-                *(float4*)(o + c0) = make_float4(v[0], v[1], v[2], v[3]);
-                *(float4*)(o + c0 + 4) = make_float4(v[4], v[5], v[6], v[7]);
-            }
-        }
-        __syncthreads();
-        const int qpr = sw >> 2;                  // 16-byte pieces per row of the slice
-        for (int v = threadIdx.x; v < n * qpr; v += blockDim.x) {
-            const int rr = v / qpr, qq = v - rr * qpr;
-            *(float4*)(acc.dst(rr) + cs + 4 * qq) = *(const float4*)(slice + rr * kSRS + qq * 16);
-        }
-        __syncthreads();
-    }
-    if (128 * kSRS > 4 * 128 * KC) sm.cur_mat = -1;   // the slice reached into the image
-    tc::fence_before_sync();
-    __syncthreads();
-}
-
-template <typename T>
-__device__ void batch_init(const FamArgs<T>& f, BatchSmem<T>& sm, unsigned char* base, uint32_t* tmem_slot,
-                           uint64_t* mbar)
-{
-    const int D = f.D;
-    if (!use_tc(f)) {
-        sm.X = (T*)base;
-        sm.Y = sm.X + (size_t)f.nmax * D;
-        return;
-    }
-    unsigned char* p = base;
-    const size_t kc = (size_t)fam_tc_kc(D);
-    sm.Ah = p; p += (size_t)128 * kc * 2;
-    sm.Al = p; p += (size_t)128 * kc * 2;
-    sm.Bh = p; p += (size_t)4 * D * kc;
-    sm.rmax = (float*)p;
-    sm.mbar = mbar;
-    sm.cur_mat = -1;
-    sm.phase = 0;
-    if ((threadIdx.x >> 5) == 0) { tc::tmem_alloc(tmem_slot, f.tc_cols); tc::tmem_relinquish(); }
-    if (threadIdx.x == 0) tc::mbar_init(mbar, 1);
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    sm.tmem = *tmem_slot;
-}
-
-template <typename T>
-__device__ void batch_fini(const FamArgs<T>& f, BatchSmem<T>& sm)
-{
-    if (!use_tc(f)) return;
-    tc::fence_before_sync();
-    __syncthreads();
-    if ((threadIdx.x >> 5) == 0) tc::tmem_dealloc(sm.tmem, f.tc_cols);
-}
 
 // fields of a key: first site, its alternative, second site, its alternative
 template <typename T>
@@ -945,17 +762,14 @@ template <typename T>
 __global__ void __launch_bounds__(256, 4) k_site_tiles(FamArgs<T> f, const SiteItem* items, SiteStep st)
 {
     extern __shared__ __align__(1024) unsigned char smraw[];
-    __shared__ uint32_t tmem_slot;
-    __shared__ __align__(8) uint64_t mbar;
     __shared__ const T* s_src[128];
     __shared__ T* s_dst[128];
     __shared__ const int* s_se[128];
     __shared__ int* s_de[128];
     __shared__ int s_eo[128];
-    BatchSmem<T> sm;
-    batch_init(f, sm, smraw, &tmem_slot, &mbar);
-    const bool tc = use_tc(f);
     const int rows = st.rows, D = f.D;
+    T* const X = (T*)smraw;
+    T* const Y = X + (size_t)f.nmax * D;
     const int ntiles = st.tbeg[8];
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         int g = 0;
@@ -970,56 +784,43 @@ __global__ void __launch_bounds__(256, 4) k_site_tiles(FamArgs<T> f, const SiteI
         }
         __syncthreads();
         const int mat = st.mat[g];
-        if constexpr (std::is_same<T, float>::value) {
-            if (tc) {
-                struct Acc {
-                    const float* const* s; float* const* d; const int* const* se; int* const* de;
-                    __device__ const float* src(int r) const { return s[r]; }
-                    __device__ float* dst(int r) const { return d[r]; }
-                    __device__ void set_exp(int r, int x) const { *de[r] = *se[r] + x; }
-                } acc{s_src, s_dst, s_se, s_de};
-                tc_apply(f, sm, acc, n, mat);          // ends with a block barrier
-                continue;
-            }
-        }
-        // CUDA-core batch: gather, y = M x with the FP32/FP64 matrices, rescale, scatter
+        // gather, y = M x with the FP32/FP64 matrices, rescale, scatter
         const int side = mat / (4 * f.K), t = (mat >> 2) % f.K, sg = mat & 3;
         for (int q = threadIdx.x; q < n * D; q += blockDim.x) {
             const int i = q / D, c = q - i * D;
-            sm.X[q] = s_src[i][c];
+            X[q] = s_src[i][c];
         }
         __syncthreads();
         if constexpr (std::is_same<T, double>::value) {
             if (f.df) {
                 // the gathered rows as float halves in Y, the products back into X
-                float* Xh = (float*)sm.Y;
+                float* Xh = (float*)Y;
                 float* Xl = Xh + (size_t)n * D;
                 for (int q = threadIdx.x; q < n * D; q += blockDim.x) {
-                    const float h = (float)sm.X[q];
+                    const float h = (float)X[q];
                     Xh[q] = h;
-                    Xl[q] = (float)(sm.X[q] - (double)h);
+                    Xl[q] = (float)(X[q] - (double)h);
                 }
                 __syncthreads();
-                mv_block_df((side == 0 ? f.ATdf : f.Adf) + ((size_t)t * 4 + sg) * D * D, D, Xh, Xl, sm.X, n);
+                mv_block_df((side == 0 ? f.ATdf : f.Adf) + ((size_t)t * 4 + sg) * D * D, D, Xh, Xl, X, n);
                 __syncthreads();
-                for (int q = threadIdx.x; q < n * D; q += blockDim.x) sm.Y[q] = sm.X[q];
+                for (int q = threadIdx.x; q < n * D; q += blockDim.x) Y[q] = X[q];
             } else {
-                mv_block<T>((side == 0 ? f.AT : f.A) + ((size_t)t * 4 + sg) * D * D, D, sm.X, sm.Y, n);
+                mv_block<T>((side == 0 ? f.AT : f.A) + ((size_t)t * 4 + sg) * D * D, D, X, Y, n);
             }
         } else {
-            mv_block<T>((side == 0 ? f.AT : f.A) + ((size_t)t * 4 + sg) * D * D, D, sm.X, sm.Y, n);
+            mv_block<T>((side == 0 ? f.AT : f.A) + ((size_t)t * 4 + sg) * D * D, D, X, Y, n);
         }
         __syncthreads();
-        renorm_rows<T>(sm.Y, D, n, s_eo);
+        renorm_rows<T>(Y, D, n, s_eo);
         __syncthreads();
         for (int q = threadIdx.x; q < n * D; q += blockDim.x) {
             const int i = q / D, c = q - i * D;
-            s_dst[i][c] = sm.Y[q];
+            s_dst[i][c] = Y[q];
         }
         for (int i = threadIdx.x; i < n; i += blockDim.x) *s_de[i] = *s_se[i] + s_eo[i];
         __syncthreads();
     }
-    batch_fini(f, sm);
 }
 
 // ---------------------------------------------------------------------------
@@ -1031,9 +832,7 @@ __global__ void __launch_bounds__(256, 4) k_site_tiles(FamArgs<T> f, const SiteI
 // registers, so that each SM keeps two tiles' gathers in flight. A stage holds
 // the raw FP32 rows (stride 4D + 16 bytes, so that the split's reads fall on
 // distinct banks) and, once split in place, the A operand (hi then lo, in the
-// core-matrix layout). Per row the arithmetic is that of tc_apply (same split,
-// same MMAs in the same order, same rescaling), so the results are bitwise
-// those of the unpipelined kernel.
+// core-matrix layout). A row's result depends on no other row of its tile.
 // ---------------------------------------------------------------------------
 constexpr int kPipeRows = 128;
 
@@ -1264,6 +1063,330 @@ __global__ void __launch_bounds__(256, 2) k_site_tiles_pipe(FamArgs<float> f, co
     if (tid < 32) tc::tmem_dealloc(tmem, f.tc_cols);
 }
 
+// ---------------------------------------------------------------------------
+// Warp-specialised tensor-core site step (FP32 tables, 64 < D <= 256). The
+// image of one matrix (4 D^2 bytes) no longer fits beside the rows' operands, so
+// the reduction runs in chunks of KC columns. One block per SM walks the tiles:
+//  - warps 0-7 gather: a lane reads 32 bytes of a row (eight lanes eight rows, so
+//    a warp reads whole 128-byte lines and each group of eight stores fills one
+//    128-byte core matrix), splits them into FP16 hi / lo and stores them into
+//    one of two chunk stages; the next chunk's loads are in flight while the
+//    warp waits for the stage to come free;
+//  - warps 8-11 take the finished accumulator (two of them in tensor memory)
+//    twice, 32 rows each: the row maximum, then the scaled row, transposed
+//    through shared memory 32 columns at a time so that the stores fill lines;
+//  - one thread of warp 12 starts the copies of the matrix chunks (two stages;
+//    one that stays while the matrix does where KC = D) and issues the MMAs,
+//    x_hi M_hi + x_lo M_hi + x_hi M_lo per chunk into the same columns.
+// Bounds: the rows' DRAM traffic (2 KB per row at D = 256), then the shared-memory
+// bandwidth that the MMAs share with the staging. With one warp role for all of it
+// (two blocks per SM, each in step with its own MMAs and with eight-way bank
+// conflicts in the operand stores) the 19 steps of the D = 256, K = 20 tables of
+// 8192 samples took 38.0 ms; now 16.9 ms.
+// Rows past the end of a tile repeat its last one. Every wait gives up after a
+// while; then all roles leave, the outstanding copies and MMAs are waited for
+// (bounded) and the tensor memory is freed.
+// ---------------------------------------------------------------------------
+constexpr int kWsThreads = 13 * 32;
+
+template <int D>
+struct WsCfg {
+    static constexpr int KC = D <= 128 ? D : 64;          // = fam_tc_kc(D)
+    static constexpr int NCK = D / KC;                    // chunks of a matrix
+    static constexpr int NB = NCK > 1 ? 2 : 1;            // matrix chunk stages
+    static constexpr uint32_t kA = 4 * 128 * KC;          // bytes of a row stage: hi, lo
+    static constexpr uint32_t kB = 4 * D * KC;            // bytes of a matrix chunk: hi, lo
+    static constexpr int NI = KC / 16;                    // 32-byte pieces per lane and chunk
+    static constexpr int NBT = NI > 4 && NI % 2 == 0 ? 2 : 1;     // batches that they are read in
+    static constexpr int NL = NI / NBT;
+    static constexpr uint32_t kAccCols = D <= 128 ? 128 : 256;    // columns of an accumulator
+    static constexpr int kSliceRow = 36;                  // floats per row of a 32-column slice
+    static constexpr size_t kSmem = 2 * (size_t)kA + NB * (size_t)kB + 4 * 32 * kSliceRow * 4;
+};
+
+__device__ __forceinline__ void ld_row32(const float* p, float* v)
+{
+    asm volatile("ld.global.nc.L1::no_allocate.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "l"(p));
+}
+
+// wait with a limit; false once any role of the block has given up
+__device__ __forceinline__ bool ws_wait(uint64_t* bar, uint32_t parity, volatile int* bad)
+{
+    for (int n = 0; n < 1024; ++n) {
+        if (tc::mbar_wait(bar, parity, 1u << 14)) return true;
+        if (*bad) return false;
+    }
+    *bad = 1;
+    return false;
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(tc::smem_addr(bar)) : "memory");
+}
+
+template <int D>
+__global__ void __launch_bounds__(kWsThreads, 1) k_site_tiles_ws(FamArgs<float> f, const SiteItem* items, SiteStep st)
+{
+    using C = WsCfg<D>;
+    constexpr int KC = C::KC, NCK = C::NCK;
+    extern __shared__ __align__(1024) unsigned char smraw[];
+    __shared__ uint32_t tmem_slot;
+    // stage of rows written / stage and matrix chunk read by its MMAs / matrix
+    // chunk landed / accumulator complete / accumulator read
+    __shared__ __align__(8) uint64_t b_rows[2], b_used[2], b_mat[2], b_full[2], b_free[2];
+    __shared__ volatile int s_bad;
+    unsigned char* const sA = smraw;
+    unsigned char* const sB = smraw + 2 * C::kA;
+    float* const slices = (float*)(sB + C::NB * (size_t)C::kB);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int ntiles = st.tbeg[8];
+    if (warp == 12) { tc::tmem_alloc(&tmem_slot, 2 * C::kAccCols); tc::tmem_relinquish(); }
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < 2; ++s) {
+            tc::mbar_init(&b_rows[s], 8);
+            tc::mbar_init(&b_used[s], 1);
+            tc::mbar_init(&b_mat[s], 1);
+            tc::mbar_init(&b_full[s], 1);
+            tc::mbar_init(&b_free[s], 4);
+        }
+        s_bad = 0;
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = tmem_slot;
+    int g = 0;
+    // tile -> group (the blocks' tiles ascend), first item, rows
+    auto tile_info = [&](int tile, int64_t& i0, int& n) {
+        while (g < 7 && tile >= st.tbeg[g + 1]) ++g;
+        i0 = st.gbeg[g] + (int64_t)(tile - st.tbeg[g]) * 128;
+        const int64_t left = st.gend[g] - i0;
+        n = (int)(left < 128 ? left : 128);
+    };
+
+    if (warp < 8) {
+        // this lane's rows of the warp's 16 (one of each eight) and its pieces
+        const int r8 = 16 * warp + (lane & 7);
+        const float* row[2];
+        float v[C::NL][8];
+        uint32_t src[2];                                  // pool rows, read a tile ahead
+        auto rows_of = [&](int tile) {
+            int64_t i0;
+            int n;
+            tile_info(tile, i0, n);
+            #pragma unroll
+            for (int o = 0; o < 2; ++o) {
+                const int r = r8 + 8 * o;
+                src[o] = items[i0 + (r < n ? r : n - 1)].src;
+            }
+        };
+        auto turn = [&]() { row[0] = f.pool + (size_t)src[0] * D; row[1] = f.pool + (size_t)src[1] * D; };
+        // piece i of a chunk: rest = (32 i + lane) / 8 is column unit rest % (KC / 8)
+        // of the rest / (KC / 8)-th row
+        auto load = [&](int ck, int b) {
+            #pragma unroll
+            for (int i = 0; i < C::NL; ++i) {
+                const int rest = 4 * (b * C::NL + i) + (lane >> 3);
+                const int o = rest / (KC / 8), c = rest - o * (KC / 8);
+                ld_row32((o ? row[1] : row[0]) + ck * KC + 8 * c, v[i]);
+            }
+        };
+        auto store = [&](unsigned char* a, int b) {
+            #pragma unroll
+            for (int i = 0; i < C::NL; ++i) {
+                const int rest = 4 * (b * C::NL + i) + (lane >> 3);
+                const int o = rest / (KC / 8), c = rest - o * (KC / 8);
+                __align__(16) __half2 hi[4], lo[4];
+                #pragma unroll
+                for (int j = 0; j < 4; ++j) tc::split_half2(v[i][2 * j], v[i][2 * j + 1], hi[j], lo[j]);
+                const uint32_t off = tc::op_offset(r8 + 8 * o, 8 * c, KC);
+                *(uint4*)(a + off) = *(const uint4*)hi;
+                *(uint4*)(a + 2 * 128 * KC + off) = *(const uint4*)lo;
+            }
+        };
+        uint32_t j = 0;                                   // chunks so far
+        rows_of(blockIdx.x);
+        turn();
+        load(0, 0);
+        bool ok = true;
+        for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
+            const bool more = tile + (int)gridDim.x < ntiles;
+            if (more) rows_of(tile + gridDim.x);
+            #pragma unroll
+            for (int ck = 0; ck < NCK; ++ck) {
+                const uint32_t s = j & 1;
+                if (j >= 2) ok = __all_sync(kFull, ok && ws_wait(&b_used[s], ((j - 2) >> 1) & 1, &s_bad));
+                if (!ok) break;
+                #pragma unroll
+                for (int b = 0; b < C::NBT; ++b) {
+                    store(sA + s * C::kA, b);
+                    if (b == C::NBT - 1) {
+                        tc::fence_proxy_async();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&b_rows[s]);
+                        if (ck < NCK - 1) load(ck + 1, 0);
+                        else if (more) { turn(); load(0, 0); }
+                    } else {
+                        load(ck, b + 1);
+                    }
+                }
+                ++j;
+            }
+        }
+    } else if (warp < 12) {
+        const int q = warp - 8;                           // tensor-memory lanes 32 q .. (q = warp % 4)
+        float* const sl = slices + q * 32 * C::kSliceRow;
+        uint32_t it = 0;
+        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
+            int64_t i0;
+            int n;
+            tile_info(tile, i0, n);
+            const int mat = st.mat[g], r = 32 * q + lane;
+            SiteItem item{};
+            int se = 0;
+            if (r < n) { item = items[i0 + r]; se = f.pool_e[item.src] + f.tc_exp[mat]; }
+            // destinations of the rows that this lane copies out
+            uint32_t dk[8];
+            #pragma unroll
+            for (int k = 0; k < 8; ++k) dk[k] = __shfl_sync(kFull, item.dst, 4 * k + (lane >> 3));
+            const uint32_t buf = it & 1;
+            if (!__all_sync(kFull, ws_wait(&b_full[buf], (it >> 1) & 1, &s_bad))) break;
+            tc::fence_after_sync();
+            const uint32_t tr = tmem + ((uint32_t)(32 * q) << 16) + buf * C::kAccCols;
+            float m = 0.f;
+            #pragma unroll
+            for (int c0 = 0; c0 < D; c0 += 16) {
+                uint32_t w[16];
+                tc::tmem_ld16(tr + c0, w);
+                tc::tmem_wait_ld();
+                #pragma unroll
+                for (int u = 0; u < 16; ++u) m = fmaxf(m, fabsf(__uint_as_float(w[u])));
+            }
+            int e = 0;
+            if (m > 0.f) frexpf(m, &e);
+            if (r < n) f.pool_e[item.dst] = se + e;
+            // 2^-e in two factors (e reaches -148 .. 128): the first is exact, or the
+            // result is zero either way
+            const int ea = -e / 2, eb = -e - ea;
+            const float f0 = __int_as_float((127 + ea) << 23), f1 = __int_as_float((127 + eb) << 23);
+            const bool one = e >= -126 && e <= 126;
+            const float s0 = one ? __int_as_float((127 - e) << 23) : f0, s1 = one ? 1.f : f1;
+            #pragma unroll
+            for (int cs = 0; cs < D; cs += 32) {
+                constexpr int kTail = D % 32;             // 0 or 16
+                const int wd = cs + 32 <= D ? 32 : kTail;
+                __syncwarp();
+                #pragma unroll
+                for (int h = 0; h < 32; h += 16) {
+                    if (h >= wd) continue;
+                    uint32_t w[16];
+                    tc::tmem_ld16(tr + cs + h, w);
+                    tc::tmem_wait_ld();
+                    #pragma unroll
+                    for (int u = 0; u < 16; u += 4)
+                        *(float4*)(sl + lane * C::kSliceRow + h + u) =
+                            make_float4(__uint_as_float(w[u]) * s0 * s1, __uint_as_float(w[u + 1]) * s0 * s1,
+                                        __uint_as_float(w[u + 2]) * s0 * s1, __uint_as_float(w[u + 3]) * s0 * s1);
+                }
+                __syncwarp();
+                #pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int rr = 4 * k + (lane >> 3), pc = lane & 7;
+                    if (4 * pc < wd && 32 * q + rr < n)
+                        *(float4*)(f.pool + (size_t)dk[k] * D + cs + 4 * pc) =
+                            *(const float4*)(sl + rr * C::kSliceRow + 4 * pc);
+                }
+            }
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&b_free[buf]);
+        }
+    } else if (lane == 0) {
+        const uint32_t idesc = tc::idesc_f16(128, D), lbo = 128, sbo = 16 * KC;
+        uint32_t j = 0, it = 0, nm = 0, seen = 0;         // chunks, tiles, matrix chunks copied / landed
+        int cur = -1;
+        bool ok = true;
+        auto fetch = [&](int mat, int ck) {
+            const uint32_t s = nm % C::NB;
+            tc::mbar_expect_tx(&b_mat[s], C::kB);
+            tc::bulk_g2s(sB + s * C::kB, (const unsigned char*)f.tc_mats + (size_t)mat * 4 * D * D + (size_t)ck * C::kB,
+                         C::kB, &b_mat[s]);
+            ++nm;
+        };
+        auto landed = [&]() {
+            const uint32_t s = seen % C::NB, p = (seen / C::NB) & 1;
+            ++seen;
+            return ws_wait(&b_mat[s], p, &s_bad);
+        };
+        int64_t i0;
+        int n;
+        tile_info(blockIdx.x, i0, n);
+        int mat = st.mat[g];
+        if (NCK > 1) fetch(mat, 0);
+        for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x, ++it) {
+            const uint32_t buf = it & 1;
+            // the next tile's matrix, for its first chunk
+            int next = -1;
+            if (tile + (int)gridDim.x < ntiles) { tile_info(tile + gridDim.x, i0, n); next = st.mat[g]; }
+            if (NCK == 1 && mat != cur) {
+                if (j > 0) ok = ws_wait(&b_used[(j - 1) & 1], ((j - 1) >> 1) & 1, &s_bad);
+                if (!ok) break;
+                fetch(mat, 0);
+                ok = landed();
+                cur = mat;
+            }
+            if (ok && it >= 2) ok = ws_wait(&b_free[buf], ((it - 2) >> 1) & 1, &s_bad);
+            for (int ck = 0; ok && ck < NCK; ++ck, ++j) {
+                const uint32_t s = j & 1;
+                if (NCK > 1) ok = landed();
+                ok = ok && ws_wait(&b_rows[s], (j >> 1) & 1, &s_bad);
+                if (!ok) break;
+                tc::fence_after_sync();
+                const unsigned char* Ah = sA + s * C::kA;
+                const unsigned char* Bh = sB + (C::NB > 1 ? s : 0) * C::kB;
+                const unsigned char* As[3] = {Ah, Ah + 2 * 128 * KC, Ah};
+                const unsigned char* Bs[3] = {Bh, Bh, Bh + 2 * D * KC};
+                uint32_t acc = ck > 0 ? 1u : 0u;
+                #pragma unroll
+                for (int term = 0; term < 3; ++term)
+                    #pragma unroll
+                    for (int ks = 0; ks < KC / 16; ++ks) {
+                        tc::mma_f16(tmem + buf * C::kAccCols, tc::desc(tc::smem_addr(As[term]) + ks * 256, lbo, sbo),
+                                    tc::desc(tc::smem_addr(Bs[term]) + ks * 256, lbo, sbo), idesc, acc);
+                        acc = 1;
+                    }
+                tc::mma_commit(&b_used[s]);
+                if (ck == NCK - 1) tc::mma_commit(&b_full[buf]);
+                // the next matrix chunk goes where the previous chunk's MMAs read
+                if (NCK > 1 && (ck < NCK - 1 || next >= 0)) {
+                    if (j > 0) ok = ws_wait(&b_used[(j - 1) & 1], ((j - 1) >> 1) & 1, &s_bad);
+                    if (ok) fetch(ck < NCK - 1 ? mat : next, ck < NCK - 1 ? ck + 1 : 0);
+                }
+            }
+            mat = next;
+        }
+        if (!ok) report(f.err, 5, 4, (long long)f.s0);
+        // nothing in flight when the block ends
+        if (seen < nm) tc::mbar_wait(&b_mat[seen % C::NB], (seen / C::NB) & 1, 1u << 24);
+        if (j > 0) tc::mbar_wait(&b_used[(j - 1) & 1], ((j - 1) >> 1) & 1, 1u << 24);
+    }
+    __syncwarp();
+    tc::fence_before_sync();
+    __syncthreads();
+    if (s_bad && threadIdx.x == 0) report(f.err, 5, 4, (long long)f.s0);
+    if (warp == 12) tc::tmem_dealloc(tmem, 2 * C::kAccCols);
+}
+
+template <int D>
+void launch_site_tiles_ws(const FamArgs<float>& f, const SiteItem* items, const SiteStep& ss, int grid, cudaStream_t st)
+{
+    allow_max_smem(k_site_tiles_ws<D>);
+    k_site_tiles_ws<D><<<grid, kWsThreads, WsCfg<D>::kSmem, st>>>(f, items, ss);
+}
+
 template <typename T>
 int fam_site_count(const FamArgs<T>& f, const SiteBufs& b, int nbb, cudaStream_t st)
 {
@@ -1334,10 +1457,27 @@ int fam_site_step(const FamArgs<T>& f, const SiteBufs& b, int tau, const int64_t
             return 1;
         }
     }
+    if constexpr (std::is_same<T, float>::value) {
+        if (tc) {
+            int dev = 0, n_sm = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+            const int grid = tiles < n_sm ? tiles : n_sm;
+            const SiteItem* it = (const SiteItem*)b.items;
+            switch (f.D) {            // every D > 64 that has images
+                case 80: launch_site_tiles_ws<80>(f, it, ss, grid, st); break;
+                case 96: launch_site_tiles_ws<96>(f, it, ss, grid, st); break;
+                case 112: launch_site_tiles_ws<112>(f, it, ss, grid, st); break;
+                case 128: launch_site_tiles_ws<128>(f, it, ss, grid, st); break;
+                case 192: launch_site_tiles_ws<192>(f, it, ss, grid, st); break;
+                default: launch_site_tiles_ws<256>(f, it, ss, grid, st); break;
+            }
+            return 1;
+        }
+    }
     allow_max_smem(k_site_tiles<T>);
-    const size_t smem = f.batch_bytes;
     const int grid = tiles < max_ctas ? tiles : max_ctas;
-    k_site_tiles<T><<<grid, 256, smem, st>>>(f, (const SiteItem*)b.items, ss);
+    k_site_tiles<T><<<grid, 256, f.batch_bytes, st>>>(f, (const SiteItem*)b.items, ss);
     return 1;
 }
 

@@ -105,16 +105,12 @@ template <typename T> int fam_launch_rbm(const FamArgs<T>& f, int nb, cudaStream
 // past n_hidden); returns launches
 int fam_corr_sites(const double* W, int K, int n_hidden, float4* out, double4_32a* out64, cudaStream_t st);
 
-// shared memory of the batch buffers of the site tiles
-// width of the reduction chunks of a tensor-core batch: the whole D up to 128,
-// else 64 (the operands of one chunk then fit shared memory)
+// shared memory of one CUDA-core batch of the site tiles (rows and products)
+inline size_t fam_batch_bytes(int D, int nmax, size_t elem) { return (size_t)2 * nmax * D * elem; }
+
+// width of the reduction chunks of a matrix image: the whole D up to 128, else 64
+// (the operands of one chunk then fit shared memory)
 __host__ __device__ inline int fam_tc_kc(int D) { return D <= 128 ? D : 64; }
-__host__ __device__ inline size_t fam_batch_bytes(int D, int nmax, size_t elem, bool tc)
-{
-    if (!tc) return (size_t)2 * nmax * D * elem;
-    const size_t kc = (size_t)fam_tc_kc(D);
-    return (size_t)4 * 128 * kc + (size_t)4 * D * kc + 2 * 128 * 4;
-}
 
 // Split-FP16 operand images of the chain's site tensors for the tensor-core
 // batches: for side 0 the matrix A_t^s, for side 1 its transpose, each scaled

@@ -288,3 +288,23 @@ def test_count_pass_and_draws(ctx, K, na, nb):
             assert np.array_equal(rank[off[i]:off[i + 1]], np.flatnonzero(keep).astype(np.uint32))
             ref, rw, _ = O.draws(P, d, i, eps, 300, 9)
             assert int(w[i]) == int(rw) and np.array_equal(ranks[i], ref)
+
+
+@pytest.mark.parametrize("D,ns", [(80, 131), (96, 5), (96, 300), (112, 131), (128, 300), (192, 130), (256, 1), (256, 130)])
+def test_site_steps_of_wide_bonds(ctx, D, ns):
+    """Site steps of 64 < D <= 256: one reduction chunk or several, tiles of one
+    row to full ones, several matrices per block. Mixed bar, and 2^-20 of the
+    rows' conditioning: both operands of a product carry 22 bits, lo x lo is left
+    out, and the sums are FP32 (about 4 x 2^-22 a product)."""
+    from oracle import oracle as O
+    s = W.tiny_system(K=7, na=3, nb=4, D=D, n_hidden=5, seed=90 + D, eps=0.01, n_draws=20, n_samples=ns)
+    ctx.set_system(s)
+    ctx.set_precision(nqs.NQS_PREC_MIXED)
+    try:
+        e, summ = ctx.local_energy(s.samples, s.counts, s.eps, s.n_draws, s.seed)
+    finally:
+        ctx.set_precision(nqs.NQS_PREC_FP64)
+    ref = O.local_energy(O.Problem(s), cond=True)
+    bar = 1e-6 * np.maximum(np.abs(ref["e_loc"]), ref["e_abs"]) + 2.0 ** -20 * ref["e_cond"]
+    assert np.all(np.abs(e - ref["e_loc"]) <= bar)
+    assert summ["n_det"] == int(ref["n_det"].sum())
