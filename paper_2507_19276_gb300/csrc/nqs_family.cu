@@ -678,24 +678,29 @@ __global__ void __launch_bounds__(256) k_site_build(FamArgs<T> f, SiteBufs sb)
 // group of S samples, steps in order: at each site the four matrices
 // [A^0; A^1; A^2; A^3] are read once per block and applied to the S samples'
 // vectors (every sample needs all four: its three alternatives and its own
-// state), one output row per thread and pass with an fma over the input index
-// in ascending order (the order of mv_block, so the results are the same bit
-// for bit).
-template <typename T, int S>
+// state), with an fma over the input index in ascending order (the order of
+// mv_block, so the results are the same bit for bit).
+// With S > 1 a thread takes row r of NS of the four products (as many as leave all
+// threads a row) of all S samples, so that a vector element read from shared
+// memory serves NS matrices and a matrix element S samples, four input indices at
+// a time: with scalar vector reads and one product per thread the FP32 tables of
+// 8192 samples at D = 256, K = 20 took 13.4 ms, now 6.1 ms. A block of one sample
+// keeps an output row of one product per thread.
+template <typename T, int S, int NS>
 __global__ void __launch_bounds__(256) k_site_boundary(FamArgs<T> f)
 {
-    extern __shared__ __align__(16) unsigned char smb[];
+    extern __shared__ __align__(32) unsigned char smb[];
     __shared__ int eo[S * 4];
     __shared__ int eL[S];
     __shared__ int own_s[S];
     const int nbb = (int)(f.s1 - f.s0);
     const int side = blockIdx.x & 1, g0 = (blockIdx.x >> 1) * S;
     const int ns = nbb - g0 < S ? nbb - g0 : S;
-    const int K = f.K, D = f.D;
-    T* X = (T*)smb;                               // [S][D] the samples' vectors
-    T* Z = X + (size_t)S * D;                     // [S][4][D] their four products
+    const int K = f.K, D = f.D, DP = (D + 3) & ~3;
+    T* X = (T*)smb;                               // [S][DP] the samples' vectors
+    T* Z = X + (size_t)S * DP;                    // [S][4][D] their four products
     const T* Mats = side == 0 ? f.AT : f.A;       // column convention left, row vectors right
-    for (int q = threadIdx.x; q < S * D; q += blockDim.x) X[q] = (q % D) == 0 ? T(1) : T(0);
+    for (int q = threadIdx.x; q < S * DP; q += blockDim.x) X[q] = (q % DP) == 0 ? T(1) : T(0);
     if (threadIdx.x < S) eL[threadIdx.x] = 0;
     __syncthreads();
     for (int step = 0; step < K; ++step) {
@@ -704,20 +709,59 @@ __global__ void __launch_bounds__(256) k_site_boundary(FamArgs<T> f)
             const int64_t s = f.s0 + g0 + threadIdx.x;
             own_s[threadIdx.x] = sigma_at(f.samples[2 * s], f.samples[2 * s + 1], t);
         }
-        for (int q = threadIdx.x; q < 4 * D; q += blockDim.x) {
-            const int sg = q / D, r = q - sg * D;
-            const T* MT = Mats + ((size_t)t * 4 + sg) * D * D;
-            T acc[S];
-            #pragma unroll
-            for (int j = 0; j < S; ++j) acc[j] = T(0);
-            for (int c = 0; c < D; ++c) {
-                const T m = __ldg(MT + (size_t)c * D + r);
-                #pragma unroll
-                for (int j = 0; j < S; ++j) acc[j] = fma(m, X[j * D + c], acc[j]);
+        const T* MT = Mats + (size_t)t * 4 * D * D;
+        if constexpr (S == 1) {
+            for (int q = threadIdx.x; q < 4 * D; q += blockDim.x) {
+                const int sg = q / D, r = q - sg * D;
+                const T* M = MT + (size_t)sg * D * D + r;
+                T acc = T(0);
+                #pragma unroll 8
+                for (int c = 0; c < D; ++c) acc = fma(__ldg(M + (size_t)c * D), X[c], acc);
+                Z[(size_t)sg * D + r] = acc;
             }
-            #pragma unroll
-            for (int j = 0; j < S; ++j)
-                if (j < ns) Z[((size_t)j * 4 + sg) * D + r] = acc[j];
+        } else {
+            constexpr int RT = 64 * NS;                   // threads per NS products
+            typedef typename Vec4<T>::type V4;
+            const int sg0 = (int)(threadIdx.x / RT) * NS;
+            const T* M = MT + (size_t)sg0 * D * D;
+            for (int r = threadIdx.x % RT; r < D; r += RT) {
+                T acc[NS][S];
+                #pragma unroll
+                for (int k = 0; k < NS; ++k)
+                    #pragma unroll
+                    for (int j = 0; j < S; ++j) acc[k][j] = T(0);
+                int c = 0;
+                for (; c + 4 <= D; c += 4) {
+                    T m[4][NS];
+                    #pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        #pragma unroll
+                        for (int k = 0; k < NS; ++k) m[u][k] = __ldg(M + ((size_t)k * D + c + u) * D + r);
+                    #pragma unroll
+                    for (int j = 0; j < S; ++j) {
+                        const V4 x = *(const V4*)(X + (size_t)j * DP + c);
+                        #pragma unroll
+                        for (int k = 0; k < NS; ++k) {
+                            acc[k][j] = fma(m[0][k], x.x, acc[k][j]);
+                            acc[k][j] = fma(m[1][k], x.y, acc[k][j]);
+                            acc[k][j] = fma(m[2][k], x.z, acc[k][j]);
+                            acc[k][j] = fma(m[3][k], x.w, acc[k][j]);
+                        }
+                    }
+                }
+                for (; c < D; ++c)
+                    #pragma unroll
+                    for (int k = 0; k < NS; ++k) {
+                        const T m = __ldg(M + ((size_t)k * D + c) * D + r);
+                        #pragma unroll
+                        for (int j = 0; j < S; ++j) acc[k][j] = fma(m, X[(size_t)j * DP + c], acc[k][j]);
+                    }
+                #pragma unroll
+                for (int j = 0; j < S; ++j)
+                    if (j < ns)
+                        #pragma unroll
+                        for (int k = 0; k < NS; ++k) Z[((size_t)j * 4 + sg0 + k) * D + r] = acc[k][j];
+            }
         }
         __syncthreads();
         renorm_rows<T>(Z, D, ns * 4, eo);
@@ -737,7 +781,7 @@ __global__ void __launch_bounds__(256) k_site_boundary(FamArgs<T> f)
         }
         for (int q = threadIdx.x; q < ns * D; q += blockDim.x) {
             const int j = q / D, c = q - j * D;
-            X[q] = Z[((size_t)j * 4 + own_s[j]) * D + c];
+            X[(size_t)j * DP + c] = Z[((size_t)j * 4 + own_s[j]) * D + c];
         }
         __syncthreads();
         if (threadIdx.x < ns) eL[threadIdx.x] += eo[threadIdx.x * 4 + own_s[threadIdx.x]];
@@ -1397,13 +1441,15 @@ int fam_site_count(const FamArgs<T>& f, const SiteBufs& b, int nbb, cudaStream_t
     int dev = 0, n_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (nbb >= 8 * n_sm) {
-        const size_t smem = (size_t)5 * 8 * f.D * sizeof(T);
-        allow_max_smem(k_site_boundary<T, 8>);
-        k_site_boundary<T, 8><<<(unsigned)((nbb + 7) / 8) * 2, 256, smem, st>>>(f);
-    } else {
-        k_site_boundary<T, 1><<<(unsigned)nbb * 2, 256, (size_t)5 * f.D * sizeof(T), st>>>(f);
-    }
+    const int DP = (f.D + 3) & ~3;
+    auto launch = [&](void (*kernel)(FamArgs<T>), int S) {
+        allow_max_smem(kernel);
+        kernel<<<(unsigned)((nbb + S - 1) / S) * 2, 256, (size_t)S * (DP + 4 * f.D) * sizeof(T), st>>>(f);
+    };
+    if (nbb < 8 * n_sm) launch(k_site_boundary<T, 1, 1>, 1);
+    else if (f.D <= 64) launch(k_site_boundary<T, 8, 1>, 8);
+    else if (f.D <= 128) launch(k_site_boundary<T, 8, 2>, 8);
+    else launch(k_site_boundary<T, 8, 4>, 8);
     k_site_build<T, false><<<nbb, 256, 0, st>>>(f, b);
     const int ns = launch_scan_i64_wide(b.counts, b.offs, (int64_t)n * nbb, b.scan_tmp, st);
     k_site_bounds<<<1, 256, 0, st>>>(b.offs, n, nbb, b.bounds);

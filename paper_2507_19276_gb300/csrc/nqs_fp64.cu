@@ -13,6 +13,8 @@
 // vertex p with the stored h_j(n), j < p.
 #include "nqs_kernels.cuh"
 
+#include <algorithm>
+
 namespace nqs {
 
 // ---------------------------------------------------------------------------
@@ -70,6 +72,111 @@ __device__ __forceinline__ const double* tens(const double* base, int e, int sg,
 // Environments, psi(n), RBM angles, H_nn
 // ---------------------------------------------------------------------------
 
+// hi + lo += m (xh + xl), the pair unnormalised: the error-free product by FMA
+// and Knuth's two-sum, as in the double-double algorithms of Hida, Li and Bailey
+__device__ __forceinline__ void fma_df(float& hi, float& lo, float2 m, float xh, float xl)
+{
+    const float ph = m.x * xh;
+    const float pl = fmaf(m.x, xh, -ph) + fmaf(m.x, xl, m.y * xh);
+    const float u = hi + ph, z = u - hi;
+    lo += ((hi - (u - z)) + (ph - z)) + pl;
+    hi = u;
+}
+
+// psi(n) of a chain in double-FP32 arithmetic, S <= 32 samples per block: the samples
+// that share a site's local state are taken four at a time, so that a matrix is
+// read once or twice per site and block where a block per sample reads it once
+// per sample (86 GB from L2 for 8192 samples at D = 256, K = 20: 7.6 ms, now
+// 6.6 ms; at D = 64, where the matrices stay in L1, both take 1.0 ms). G groups of threads take every G-th four where D leaves room. Per sample
+// the steps and their order are those of k_env_fp64 with tn = 3.
+template <int G>
+__global__ void __launch_bounds__(256, 5) k_psi_df(EnvArgs a, int S)
+{
+    extern __shared__ __align__(16) double smp[];
+    __shared__ uint32_t s_mask[4];
+    __shared__ int s_ex[32];
+    const int D = a.an.D, K = a.an.K, DP = (D + 3) & ~3;
+    const int64_t s0 = (int64_t)blockIdx.x * S;
+    const int ns = a.Ns - s0 < S ? (int)(a.Ns - s0) : S;
+    float* xh = (float*)smp;                      // [S][DP] the states' halves
+    float* xl = xh + (size_t)S * DP;
+    double* y = (double*)(xl + (size_t)S * DP);   // [S][D] their products
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int q = threadIdx.x; q < S * DP; q += 256) { xh[q] = q % DP == 0 ? 1.f : 0.f; xl[q] = 0.f; }
+    if (threadIdx.x < 32) s_ex[threadIdx.x] = 0;
+    for (int t = 0; t < K; ++t) {
+        if (warp == 0) {
+            const int sg = lane < ns ? sigma_at(a.samples[2 * (s0 + lane)], a.samples[2 * (s0 + lane) + 1], t) : -1;
+            #pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                const uint32_t b = __ballot_sync(0xffffffffu, sg == g);
+                if (lane == 0) s_mask[g] = b;
+            }
+        }
+        __syncthreads();
+        int part = 0;
+        for (int sg = 0; sg < 4; ++sg) {
+            const float2* M = a.ATdf + ((size_t)t * 4 + sg) * D * D;
+            for (uint32_t m = s_mask[sg]; m; ++part) {
+                int js[4];                        // the four samples (the last one repeats)
+                int n4 = 0;
+                #pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if (m) { js[k] = __ffs(m) - 1; m &= m - 1; n4 = k + 1; }
+                    else js[k] = js[k > 0 ? k - 1 : 0];
+                }
+                if (part % G != (int)threadIdx.x / (256 / G)) continue;
+                for (int r = threadIdx.x % (256 / G); r < D; r += 256 / G) {
+                    float hi[4] = {}, lo[4] = {};
+                    int c = 0;
+                    for (; c + 4 <= D; c += 4) {
+                        float2 w[4];
+                        #pragma unroll
+                        for (int u = 0; u < 4; ++u) w[u] = __ldg(M + (size_t)(c + u) * D + r);
+                        #pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            if (k < n4) {
+                                const float4 h = *(const float4*)(xh + js[k] * DP + c);
+                                const float4 l = *(const float4*)(xl + js[k] * DP + c);
+                                fma_df(hi[k], lo[k], w[0], h.x, l.x);
+                                fma_df(hi[k], lo[k], w[1], h.y, l.y);
+                                fma_df(hi[k], lo[k], w[2], h.z, l.z);
+                                fma_df(hi[k], lo[k], w[3], h.w, l.w);
+                            }
+                        }
+                    }
+                    for (; c < D; ++c) {
+                        const float2 w = __ldg(M + (size_t)c * D + r);
+                        #pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (k < n4) fma_df(hi[k], lo[k], w, xh[js[k] * DP + c], xl[js[k] * DP + c]);
+                    }
+                    #pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (k < n4) y[(size_t)js[k] * D + r] = (double)hi[k] + (double)lo[k];
+                }
+            }
+        }
+        __syncthreads();
+        for (int j = warp; j < ns; j += 8) {      // rescaled by a power of two, split again
+            const int e = warp_renorm(y + (size_t)j * D, D, lane);
+            if (lane == 0) s_ex[j] += e;
+            for (int c = lane; c < D; c += 32) {
+                const double v = y[(size_t)j * D + c];
+                const float h = (float)v;
+                xh[j * DP + c] = h;
+                xl[j * DP + c] = (float)(v - (double)h);
+            }
+        }
+        __syncthreads();
+    }
+    if ((int)threadIdx.x < ns) {
+        const int j = threadIdx.x;
+        a.psi_mant[s0 + j] = (double)xh[j * DP] + (double)xl[j * DP];
+        a.psi_exp[s0 + j] = s_ex[j];
+    }
+}
+
 __global__ void k_env_fp64(EnvArgs a)
 {
     extern __shared__ double sm[];
@@ -86,9 +193,7 @@ __global__ void k_env_fp64(EnvArgs a)
     if (!a.tn) {
         // tensor-network part done elsewhere
     } else if (a.an.chain && a.tn == 3) {
-        // psi(n) alone in double-FP32 arithmetic (the error-free product by FMA
-        // and Knuth's two-sum, as in the double-double algorithms of Hida, Li and
-        // Bailey), on the FP32 pipe: the state as (hi, lo) float pairs in place of
+        // psi(n) alone in double-FP32 arithmetic (fma_df), on the FP32 pipe: the state as (hi, lo) float pairs in place of
         // x, the site matrices as pairs, each output accumulated as an
         // unnormalised pair (relative error about D 2^-48), then rounded to FP64
         // for the exact power-of-two rescaling and split again
@@ -101,15 +206,8 @@ __global__ void k_env_fp64(EnvArgs a)
             const float2* M = a.ATdf + ((size_t)t * 4 + sigma_at(na, nb, t)) * D * D;
             for (int r = threadIdx.x; r < D; r += blockDim.x) {
                 float hi = 0.f, lo = 0.f;
-                for (int c = 0; c < D; ++c) {
-                    const float2 m = __ldg(M + (size_t)c * D + r);
-                    const float ah = xh[c], al = xl[c];
-                    const float ph = m.x * ah;
-                    const float pl = fmaf(m.x, ah, -ph) + fmaf(m.x, al, m.y * ah);
-                    const float u = hi + ph, z = u - hi;
-                    lo += ((hi - (u - z)) + (ph - z)) + pl;
-                    hi = u;
-                }
+                #pragma unroll 4
+                for (int c = 0; c < D; ++c) fma_df(hi, lo, __ldg(M + (size_t)c * D + r), xh[c], xl[c]);
                 y[r] = (double)hi + (double)lo;
             }
             __syncthreads();
@@ -312,13 +410,39 @@ __global__ void k_env_fp64(EnvArgs a)
     }
 }
 
-int launch_env_fp64(const EnvArgs& a, cudaStream_t st)
+int launch_env_fp64(const EnvArgs& args, cudaStream_t st)
 {
-    if (a.Ns == 0) return 0;
+    if (args.Ns == 0) return 0;
+    EnvArgs a = args;
+    int n = 1;
+    if (a.an.chain && a.tn == 3) {
+        // one wave of blocks: as many samples per block as that takes, up to 32 and
+        // to 72 KB of shared memory (three blocks per SM); with fewer than four
+        // there is little to share and a block per sample stays
+        int dev = 0, n_sm = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+        const int D = a.an.D;
+        const size_t per = (size_t)(((D + 3) & ~3) + D) * 8;
+        const int fit = std::min<int>(32, (int)(72 * 1024 / per));
+        const int bps = std::min<int>(5, (int)(216 * 1024 / (fit > 0 ? fit * per : per)));
+        const int S = (int)std::min<int64_t>(fit, (a.Ns + (int64_t)bps * n_sm - 1) / ((int64_t)bps * n_sm));
+        if (S >= 4) {
+            auto launch = [&](void (*kernel)(EnvArgs, int)) {
+                allow_max_smem(kernel);
+                kernel<<<(unsigned)((a.Ns + S - 1) / S), 256, S * per, st>>>(a, S);
+            };
+            if (D > 128) launch(k_psi_df<1>);
+            else if (D > 64) launch(k_psi_df<2>);
+            else launch(k_psi_df<4>);
+            a.tn = 0;
+            ++n;
+        }
+    }
     const int threads = a.an.D >= 256 ? 256 : (a.an.D > 64 ? 128 : 64);
     const size_t smem = (2 * a.an.D + 34 + a.an.tk_zy) * sizeof(double) + 2 * kMaxOrb * sizeof(int);
     k_env_fp64<<<(unsigned)a.Ns, threads, smem, st>>>(a);
-    return 1;
+    return n;
 }
 
 // ---------------------------------------------------------------------------

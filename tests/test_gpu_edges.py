@@ -308,3 +308,26 @@ def test_site_steps_of_wide_bonds(ctx, D, ns):
     bar = 1e-6 * np.maximum(np.abs(ref["e_loc"]), ref["e_abs"]) + 2.0 ** -20 * ref["e_cond"]
     assert np.all(np.abs(e - ref["e_loc"]) <= bar)
     assert summ["n_det"] == int(ref["n_det"].sum())
+
+
+@pytest.mark.parametrize("D,nh", [(5, 0), (16, 3), (50, 0), (64, 3), (80, 3), (130, 0), (256, 3)])
+def test_full_batches_equal_small_ones(ctx, D, nh):
+    """Boundary vectors and psi(n) of batches that fill the GPU (several samples
+    per block, the last block short) against the same samples in small calls
+    (one per block): every row's arithmetic is the same, so are the results (without
+    a tolerance: which samples are re-evaluated depends on the batch)."""
+    s = W.tiny_system(K=8, na=4, nb=4, D=D, n_hidden=nh, seed=70 + D, eps=0.02, n_draws=10, n_samples=4900)
+    n = 4133
+    ctx.set_system(s)
+    parts = (0, 2000, n - 500)
+    try:
+        ctx.set_precision(nqs.NQS_PREC_MIXED)
+        e, _ = ctx.local_energy(s.samples[:n], s.counts[:n], s.eps, s.n_draws, s.seed)
+        got = []
+        for i in parts:
+            ctx.set_precision(nqs.NQS_PREC_MIXED, sample_index_base=i)
+            got.append(ctx.local_energy(s.samples[i:i + 500], s.counts[i:i + 500], s.eps, s.n_draws, s.seed)[0])
+    finally:
+        ctx.set_precision(nqs.NQS_PREC_FP64)
+    for i, p in zip(parts, got):
+        assert np.array_equal(p, e[i:i + 500])
