@@ -18,12 +18,19 @@
 // of the mixed form) and writes it back split. Every node's arithmetic is its
 // own, whatever tile it is in.
 //
-// A tile's chain (resolve, gather, MMA, read-back, store) is latency-bound, so
-// the tiles are small enough for three per SM. The form before this one ran 128
-// rows of one sample through all their vertices with the states in shared
-// memory, one tile per SM, all four local states' products per edge (N = 4D) and
-// no sharing between rows: 417 ms for the tiles of H18 (D = 32, 16 384 samples),
-// tensor pipe 14% busy.
+// A tile's chain (items, gather, MMA, read-back, store) is all latency, so one
+// block per SM runs its parts in warps of their own: four warps copy source
+// states into a ring of slots, an in-edge of a tile each; two warps make finished
+// slots visible to the tensor cores; one thread issues the MMAs of each slot into
+// one of four accumulators; four groups of four warps drain every fourth tile, a
+// node per thread. H18 (D = 32, 16 384 samples): 97 ms. With the proxy fence in the
+// copying warps (it drains their copies) and three groups 111 ms, with it in the
+// MMA thread 123 ms. Three blocks per SM that each ran the chain in step took
+// 170 ms (1.1 instructions per cycle, 2.2 TB/s); running 128 rows of one sample
+// through all their vertices, states in shared memory, all four local states'
+// products per edge and no sharing between rows, 417 ms. What is left is the drain
+// groups' instructions and the gathers' latency: without any gather, power or
+// store the kernel's chain alone takes about half of it.
 //
 // The ratio psi(m)/psi(n) = psi_TN(m)/psi_TN(n) f(m)/f(n) is formed in FP64
 // from the FP32 result, with the correlator ratio of Eq. (RBM) (2cosh, or the
@@ -44,7 +51,13 @@ namespace nqs {
 namespace {
 
 constexpr int kGtRows = 128;
-constexpr int kGtThreads = 2 * kGtRows;   // two per node: halves of its D columns
+// groups of four warps that drain accumulators (a thread holds a row of D values)
+constexpr int gt_groups(int D) { return D <= 32 ? 4 : 2; }
+constexpr int kGtFence = 2;               // warps that pass the slots on to the MMAs
+constexpr int gt_threads(int D) { return (4 + 4 * gt_groups(D) + 1 + kGtFence) * 32; }
+// slots of the ring of source states; more take shared memory from the L1 that the
+// item lists and shared ancestors hit (twelve: 102 ms where six take 97)
+constexpr int kGtRing = 6;
 
 // 2^d for d <= 0 in FP32 (0 below the normal range)
 __device__ __forceinline__ float pow2_neg(int d)
@@ -95,32 +108,61 @@ __global__ void k_tree_graph_prep(const double* __restrict__ Hst, const int* __r
     }
 }
 
-// Vertex t of the nodes of level t (see the file header).
-template <int D>
-__global__ void __launch_bounds__(kGtThreads, D <= 32 ? 3 : 2) k_tree_graph_tc(TreeGraphTc a, int t, int deg, uint32_t at,
-                                                                                       uint32_t nl, TreeGroups gr)
+__device__ __forceinline__ void gt_arrive(uint64_t* bar)
 {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(tc::smem_addr(bar)) : "memory");
+}
+
+// wait with a limit; false once any role of the block has given up
+__device__ __forceinline__ bool gt_wait(uint64_t* bar, uint32_t parity, volatile int* bad)
+{
+    for (int n = 0; n < 1024; ++n) {
+        if (tc::mbar_wait(bar, parity, 1u << 14)) return true;
+        if (*bad) return false;
+    }
+    *bad = 1;
+    return false;
+}
+
+// 32 bytes to global memory (32-byte aligned)
+__device__ __forceinline__ void st_32(void* p, const uint32_t* v)
+{
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                 :: "l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
+
+// Vertex t of the nodes of level t (see the file header). Every wait gives up
+// after a while; then all roles leave, what is in flight is waited for (bounded)
+// and the tensor memory is freed.
+template <int D>
+__global__ void __launch_bounds__(gt_threads(D), 1) k_tree_graph_tc(TreeGraphTc a, int t, int deg, uint32_t at, uint32_t nl,
+                                                                 TreeGroups gr, int n_slots)
+{
+    constexpr int NG = gt_groups(D);
     extern __shared__ __align__(1024) unsigned char smraw[];
     __shared__ uint32_t tmem_slot;
-    __shared__ __align__(8) uint64_t mb_mma, mb_b;
-    __shared__ uint32_t s_src[kGtMaxDeg][kGtRows];
-    __shared__ int s_es[kGtMaxDeg][kGtRows];
-    __shared__ uint32_t s_out[kGtRows];           // pool row of the result (level K - 1: the node)
-    __shared__ float s_max[2][kGtRows];
-    __shared__ int t_e[kGtMaxDeg];                // edges with a vertex source, then the e_0 ones
-    constexpr int H = D / 2;                      // columns per thread
-    constexpr int EP = D <= 32 ? 3 : 1;           // edges per tensor-memory round trip
+    // ring slot written / passed on / read by its MMAs; accumulator complete / read; images landed
+    __shared__ __align__(8) uint64_t b_full[kGtRing], b_ready[kGtRing], b_used[kGtRing];
+    __shared__ __align__(8) uint64_t b_acc[NG], b_free[NG], b_mat;
+    __shared__ volatile int s_bad;
+    constexpr int MD = 128 / D < kGtMaxDeg ? 128 / D : kGtMaxDeg;     // largest in-degree (see graph_tc_fits)
+    __shared__ int t_e[MD];                       // edges with a vertex source, then the e_0 ones
     constexpr uint32_t kSlot = kGtRows * D * 4;   // hi then lo, 128 x D FP16 each
     constexpr uint32_t kLo = kGtRows * D * 2;
     constexpr uint32_t kMat = 2 * D * D;          // one half of one matrix image
+    constexpr uint32_t kAcc = 128;                // columns of a tile's accumulators
     const int K = a.an.K;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int r = 32 * (warp & 3) + lane, h = warp >> 2;
-    unsigned char* const Bs = smraw + (size_t)deg * kSlot;
-    uint32_t cols = 32;
-    while (cols < (uint32_t)(deg * D)) cols <<= 1;
-    if (warp == 0) { tc::tmem_alloc(&tmem_slot, cols); tc::tmem_relinquish(); }
-    if (tid == 0) { tc::mbar_init(&mb_mma, 1); tc::mbar_init(&mb_b, 1); }
+    constexpr int kMmaWarp = 4 + 4 * NG;
+    unsigned char* const Bs = smraw + (size_t)n_slots * kSlot;
+    if (warp == kMmaWarp) { tc::tmem_alloc(&tmem_slot, 512); tc::tmem_relinquish(); }
+    if (tid == 0) {
+        for (int s = 0; s < kGtRing; ++s) { tc::mbar_init(&b_full[s], 128); tc::mbar_init(&b_ready[s], 1); tc::mbar_init(&b_used[s], 1); }
+        for (int s = 0; s < NG; ++s) { tc::mbar_init(&b_acc[s], 1); tc::mbar_init(&b_free[s], 4); }
+        tc::mbar_init(&b_mat, 1);
+        s_bad = 0;
+    }
     const int e0 = a.an.pred_ptr[t];
     int nv = 0;                                   // in-edges with a vertex source
     for (int e = e0; e < e0 + deg; ++e) nv += a.an.pred_idx[e] >= 0;
@@ -134,19 +176,9 @@ __global__ void __launch_bounds__(kGtThreads, D <= 32 ? 3 : 2) k_tree_graph_tc(T
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = tmem_slot;
-    const uint32_t tlane = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(h * H);
-    const uint32_t idesc = tc::idesc_f16(kGtRows, D);
-    uint32_t ph_mma = 0, ph_b = 0;
-    bool ok = true;
-    int held = -1;                                // local state whose images are in Bs
-    constexpr uint32_t kPoll = 1u << 24;
     const int nt = gr.tile[4];
     const int tile0 = (int)((int64_t)nt * blockIdx.x / gridDim.x);
     const int tile1 = (int)((int64_t)nt * (blockIdx.x + 1) / gridDim.x);
-    // this thread's part of a tile's items: node rr's result row (first half of the
-    // block) and the sources of its every other in-edge; loaded one tile ahead
-    const int rr = tid & (kGtRows - 1);
-    uint32_t pre[kGtMaxDeg / 2] = {0, 0, 0, 0}, pre_out = 0;
     auto place = [&](int tile, int& sg, uint32_t& i0, int& n) {
         sg = 0;
         while (sg < 3 && tile >= gr.tile[sg + 1]) ++sg;
@@ -156,173 +188,223 @@ __global__ void __launch_bounds__(kGtThreads, D <= 32 ? 3 : 2) k_tree_graph_tc(T
         i0 = b0 + (uint32_t)(tile - f) * kGtRows;
         n = (int)min(b1 - i0, (uint32_t)kGtRows);
     };
-    auto fetch = [&](int tile) {
+    // row r of a tile: its result row and the sources of its in-edges (rows past
+    // the tile's repeat the first)
+    auto fetch = [&](int tile, int r, uint32_t& out, uint32_t* src) {
         int sg, n;
         uint32_t i0;
         place(tile, sg, i0, n);
-        const uint32_t* it = a.items + at + i0 + (rr < n ? rr : 0);   // rows past n repeat the first
-        if (tid < kGtRows) pre_out = __ldg(it);
+        const uint32_t* it = a.items + at + i0 + (r < n ? r : 0);
+        out = __ldg(it);
         #pragma unroll
-        for (int u = 0; u < kGtMaxDeg / 2; ++u) {
-            const int k = 2 * u + (tid >> 7);
-            if (k < nv) pre[u] = __ldg(it + (size_t)(k + 1) * nl);
-        }
+        for (int k = 0; k < MD; ++k)
+            if (k < nv) src[k] = __ldg(it + (size_t)(k + 1) * nl);
     };
-    if (tile0 < tile1) fetch(tile0);
-    for (int tile = tile0; tile < tile1; ++tile) {
-        int sg, n;
-        uint32_t i0;
-        place(tile, sg, i0, n);
-        if (tid < kGtRows) s_out[rr] = pre_out;
-        uint32_t mine[kGtMaxDeg / 2];
-        #pragma unroll
-        for (int u = 0; u < kGtMaxDeg / 2; ++u) {
-            const int k = 2 * u + (tid >> 7);
-            mine[u] = pre[u];
-            if (k < nv) s_src[k][rr] = pre[u];
-        }
-        if (tid == 0 && sg != held && nv > 0) {
-            tc::mbar_expect_tx(&mb_b, (uint32_t)nv * 2 * kMat);
-            for (int k = 0; k < nv; ++k) {
-                const unsigned char* src = a.bimg + (size_t)t_e[k] * 8 * kMat + (size_t)sg * kMat;
-                tc::bulk_g2s(Bs + (size_t)k * 2 * kMat, src, kMat, &mb_b);
-                tc::bulk_g2s(Bs + (size_t)k * 2 * kMat + kMat, src + 4 * kMat, kMat, &mb_b);
-            }
-        }
-        __syncthreads();
-        // the sources' states: 16-byte pieces, eight nodes x four pieces per warp so
-        // that shared memory is written in whole core matrices and global memory
-        // read in 64-byte runs
-        for (int k = 0; k < nv; ++k) {
-            unsigned char* slot = smraw + (size_t)k * kSlot;
-            constexpr int CG = D / 16;            // groups of four pieces per row
-            for (int q = warp; q < 16 * CG; q += 8) {
-                const int rr = (q / CG) * 8 + (lane & 7), pc = (q % CG) * 4 + (lane >> 3);
-                const bool lo = pc >= D / 8;
-                const int c8 = lo ? pc - D / 8 : pc;
-                tc::cp_async16(slot + (lo ? kLo : 0) + tc::op_offset(rr, 8 * c8, D),
-                               a.pool + (size_t)s_src[k][rr] * 4 * D + 16 * pc);
+
+    if (warp < 4) {
+        // the sources' states, an in-edge of a tile per slot: 16-byte pieces, eight
+        // nodes x four pieces per warp so that shared memory is written in whole core
+        // matrices and global memory read in 64-byte runs; the copies announce themselves
+        uint32_t nxt[MD] = {}, out;
+        uint32_t slot = 0, round = 0;
+        bool ok = true;
+        if (tile0 < tile1) fetch(tile0, 32 * warp + lane, out, nxt);
+        for (int tile = tile0; ok && tile < tile1 && nv > 0; ++tile) {
+            uint32_t cur[MD];
+            #pragma unroll
+            for (int k = 0; k < MD; ++k) cur[k] = nxt[k];
+            if (tile + 1 < tile1) fetch(tile + 1, 32 * warp + lane, out, nxt);
+            #pragma unroll
+            for (int k = 0; k < MD; ++k) {
+                if (k >= nv) break;
+                if (round > 0) ok = __all_sync(kFull, ok && gt_wait(&b_used[slot], (round - 1) & 1, &s_bad));
+                if (!ok) break;
+                unsigned char* to = smraw + (size_t)slot * kSlot;
+                #pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int rr = 8 * j + (lane & 7);
+                    const unsigned char* row = a.pool + (size_t)__shfl_sync(kFull, cur[k], rr) * 4 * D;
+                    #pragma unroll
+                    for (int p = 0; p < D / 16; ++p) {
+                        const int pc = 4 * p + (lane >> 3);
+                        const bool lo = pc >= D / 8;
+                        const int c8 = lo ? pc - D / 8 : pc;
+                        tc::cp_async16(to + (lo ? kLo : 0) + tc::op_offset(32 * warp + rr, 8 * c8, D), row + 16 * pc);
+                    }
+                }
+                tc::cp_async_arrive(&b_full[slot]);
+                if (++slot == (uint32_t)n_slots) { slot = 0; ++round; }
             }
         }
         tc::cp_async_commit();
-        // meanwhile the sources' powers of two, and the next tile's items
-        #pragma unroll
-        for (int u = 0; u < kGtMaxDeg / 2; ++u) {
-            const int k = 2 * u + (tid >> 7);
-            if (k < nv) s_es[k][rr] = a.pool_e[mine[u]] + __ldg(a.bexp + t_e[k] * 4 + sg);
-        }
-        if (tile + 1 < tile1) fetch(tile + 1);
         tc::cp_async_wait<0>();
-        tc::fence_proxy_async();
-        tc::fence_before_sync();
-        __syncthreads();
-        if (nv > 0) {
-            if (tid == 0) {
-                tc::fence_after_sync();
-                if (sg != held) ok = tc::mbar_wait(&mb_b, ph_b, kPoll) && ok;
-                const uint64_t d0 = tc::desc(0, 128, 16 * D);
-                for (int k = 0; k < nv; ++k) {
-                    const uint64_t dA = d0 + (tc::smem_addr(smraw + (size_t)k * kSlot) >> 4);
-                    const uint64_t dB = d0 + (tc::smem_addr(Bs + (size_t)k * 2 * kMat) >> 4);
-                    #pragma unroll
-                    for (int term = 0; term < 3; ++term)
-                        #pragma unroll
-                        for (int ks = 0; ks < D / 16; ++ks) {
-                            const uint64_t ao = term == 1 ? (kLo >> 4) : 0;
-                            const uint64_t bo = term == 2 ? (kMat >> 4) : 0;
-                            tc::mma_f16(tmem + (uint32_t)(k * D), dA + ao + 16 * ks, dB + bo + 16 * ks, idesc,
-                                        (term | ks) ? 1u : 0u);
-                        }
-                }
-                tc::mma_commit(&mb_mma);
-            }
-            if (sg != held) ph_b ^= 1u;
-            held = sg;
-            ok = tc::mbar_wait(&mb_mma, ph_mma, kPoll) && ok;
-            ph_mma ^= 1u;
-            tc::fence_after_sync();
-        }
-        int eref = nv < deg ? 0 : -(1 << 30);       // an e_0 source has power 0
-        for (int k = 0; k < nv; ++k) eref = max(eref, s_es[k][r]);
-        float y[H];
-        #pragma unroll
-        for (int c = 0; c < H; ++c) y[c] = 0.f;
-        #pragma unroll
-        for (int k0 = 0; k0 < kGtMaxDeg; k0 += EP) {
-            if (k0 >= nv) break;
-            uint32_t v[EP][H];
+    } else if (warp < kMmaWarp) {
+        // group gq drains every NG-th tile, a node per thread
+        const int gq = (warp - 4) >> 2, r = 32 * (warp & 3) + lane;
+        const uint32_t tlane = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + gq * kAcc;
+        uint32_t src[MD] = {}, out = 0;           // of the group's next tile, and its sources' powers of two
+        int es[MD] = {};
+        auto powers = [&]() {
             #pragma unroll
-            for (int q = 0; q < EP; ++q) {
-                const int k = k0 + q;
+            for (int k = 0; k < MD; ++k)
+                if (k < nv) es[k] = a.pool_e[src[k]];
+        };
+        if (tile0 + gq < tile1) { fetch(tile0 + gq, r, out, src); powers(); }
+        uint32_t use = 0;
+        for (int tile = tile0 + gq; tile < tile1; tile += NG, ++use) {
+            int sg, n;
+            uint32_t i0;
+            place(tile, sg, i0, n);
+            const uint32_t dst = out;
+            const bool more = tile + NG < tile1;
+            int se[MD];
+            int eref = nv < deg ? 0 : -(1 << 30);     // an e_0 source has power 0
+            #pragma unroll
+            for (int k = 0; k < MD; ++k)
+                if (k < nv) { se[k] = es[k] + __ldg(a.bexp + t_e[k] * 4 + sg); eref = max(eref, se[k]); }
+            if (more) fetch(tile + NG, r, out, src);
+            if (nv > 0) {
+                if (!__all_sync(kFull, gt_wait(&b_acc[gq], use & 1, &s_bad))) break;
+                tc::fence_after_sync();
+            }
+            float y[D];
+            #pragma unroll
+            for (int c = 0; c < D; ++c) y[c] = 0.f;
+            constexpr int CW = 16;                // columns read at a time
+            #pragma unroll
+            for (int k = 0; k < MD; ++k) {
                 if (k < nv) {
-                    const uint32_t ta = tlane + (uint32_t)(k * D);
-                    if constexpr (H >= 16) {
+                    const float f = pow2_neg(se[k] - eref);
+                    #pragma unroll
+                    for (int c0 = 0; c0 < D; c0 += CW) {
+                        uint32_t v[CW];
                         #pragma unroll
-                        for (int c0 = 0; c0 < H; c0 += 16) tc::tmem_ld16(ta + c0, v[q] + c0);
-                    } else {
-                        tc::tmem_ld8u(ta, v[q]);
+                        for (int c1 = 0; c1 < CW; c1 += 16) tc::tmem_ld16(tlane + (uint32_t)(k * D + c0 + c1), v + c1);
+                        tc::tmem_wait_ld();
+                        #pragma unroll
+                        for (int c = 0; c < CW; ++c) y[c0 + c] = fmaf(__uint_as_float(v[c]), f, y[c0 + c]);
                     }
                 }
             }
-            tc::tmem_wait_ld();
-            #pragma unroll
-            for (int q = 0; q < EP; ++q) {
-                const int k = k0 + q;
-                if (k < nv && k < kGtMaxDeg) {
-                    const float f = pow2_neg(s_es[k][r] - eref);
-                    #pragma unroll
-                    for (int c = 0; c < H; ++c) y[c] = fmaf(__uint_as_float(v[q][c]), f, y[c]);
-                }
+            if (nv > 0) {
+                tc::fence_before_sync();
+                __syncwarp();
+                if (lane == 0) gt_arrive(&b_free[gq]);
             }
-        }
-        for (int k = nv; k < deg; ++k) {
-            // M e_0: column 0 of the matrix
-            const float f = pow2_neg(-eref);
-            const float* col = a.col0 + ((size_t)t_e[k] * 4 + sg) * D + h * H;
-            #pragma unroll
-            for (int c = 0; c < H; ++c) y[c] = fmaf(__ldg(col + c), f, y[c]);
-        }
-        float mx = 0.f;
-        #pragma unroll
-        for (int c = 0; c < H; ++c) mx = fmaxf(mx, fabsf(y[c]));
-        s_max[h][r] = mx;
-        tc::fence_before_sync();
-        __syncthreads();                          // the two halves of each row meet
-        if (r < n) {
-            mx = fmaxf(s_max[0][r], s_max[1][r]);
-            int ge = 0;
-            if (mx > 0.f) frexpf(mx, &ge);
-            const bool pw = ge >= -126 && ge <= 126;
-            const float sc = pw ? __int_as_float((127 - ge) << 23) : 0.f;
-            #pragma unroll
-            for (int c = 0; c < H; ++c) y[c] = pw ? y[c] * sc : ldexpf(y[c], -ge);
-            const int ex = eref + ge;
-            if (t == K - 1) {
-                if (h == 0) {
-                    a.mant[s_out[r]] = y[0];
-                    a.mexp[s_out[r]] = ex;
-                }
-            } else {
-                unsigned char* out = a.pool + (size_t)s_out[r] * 4 * D;
+            if (more) powers();
+            for (int k = nv; k < deg; ++k) {
+                // M e_0: column 0 of the matrix
+                const float f = pow2_neg(-eref);
+                const float* col = a.col0 + ((size_t)t_e[k] * 4 + sg) * D;
                 #pragma unroll
-                for (int c8 = 0; c8 < H / 8; ++c8) {
-                    __align__(16) __half2 hi[4], lo[4];
+                for (int c = 0; c < D; ++c) y[c] = fmaf(__ldg(col + c), f, y[c]);
+            }
+            float mx = 0.f;
+            #pragma unroll
+            for (int c = 0; c < D; ++c) mx = fmaxf(mx, fabsf(y[c]));
+            if (r < n) {
+                int ge = 0;
+                if (mx > 0.f) frexpf(mx, &ge);
+                const int ex = eref + ge;
+                // 2^-ge, in two factors where one would not be a normal number (the first
+                // is exact, or the result is zero either way)
+                const bool one = ge >= -126 && ge <= 126;
+                const float f0 = __int_as_float((127 + (one ? -ge : -ge / 2)) << 23);
+                #pragma unroll
+                for (int c = 0; c < D; ++c) y[c] *= f0;
+                if (!one) {
+                    const float f1 = __int_as_float((127 - ge + ge / 2) << 23);
                     #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        tc::split_half2(y[8 * c8 + 2 * q], y[8 * c8 + 2 * q + 1], hi[q], lo[q]);
-                    *(uint4*)(out + 2 * (h * H + 8 * c8)) = *(const uint4*)hi;
-                    *(uint4*)(out + 2 * D + 2 * (h * H + 8 * c8)) = *(const uint4*)lo;
+                    for (int c = 0; c < D; ++c) y[c] *= f1;
                 }
-                if (h == 0) a.pool_e[s_out[r]] = ex;
+                if (t == K - 1) {
+                    a.mant[dst] = y[0];
+                    a.mexp[dst] = ex;
+                } else {
+                    unsigned char* row = a.pool + (size_t)dst * 4 * D;
+                    #pragma unroll
+                    for (int c0 = 0; c0 < D; c0 += 16) {
+                        __align__(16) __half2 hi[8], lo[8];
+                        #pragma unroll
+                        for (int q = 0; q < 8; ++q)
+                            tc::split_half2(y[c0 + 2 * q], y[c0 + 2 * q + 1], hi[q], lo[q]);
+                        st_32(row + 2 * c0, (const uint32_t*)hi);
+                        st_32(row + 2 * D + 2 * c0, (const uint32_t*)lo);
+                    }
+                    a.pool_e[dst] = ex;
+                }
             }
         }
-        __syncthreads();                          // s_out, s_es and s_max are free
+    } else if (warp > kMmaWarp) {
+        // the copies of every kGtFence-th slot, made visible to the MMAs: the proxy
+        // fence takes a few hundred cycles, which neither the MMA thread nor the
+        // copying warps (it drains all that they have in flight) should wait for
+        const uint32_t total = nv > 0 && tile0 < tile1 ? (uint32_t)(tile1 - tile0) * nv : 0;
+        uint32_t slot = warp - kMmaWarp - 1, round = 0;
+        for (uint32_t i = slot; lane == 0 && i < total; i += kGtFence) {
+            if (!gt_wait(&b_full[slot], round & 1, &s_bad)) break;
+            tc::fence_proxy_async();
+            gt_arrive(&b_ready[slot]);
+            slot += kGtFence;
+            if (slot >= (uint32_t)n_slots) { slot -= n_slots; ++round; }
+        }
+    } else if (lane == 0 && nv > 0) {
+        const uint32_t idesc = tc::idesc_f16(kGtRows, D);
+        const uint64_t d0 = tc::desc(0, 128, 16 * D);
+        uint32_t slot = 0, round = 0, n_mat = 0, last = 0, last_p = 0;
+        int held = -1;                            // local state whose images are in Bs
+        bool ok = true, any = false;
+        uint32_t it = 0;
+        for (int tile = tile0; ok && tile < tile1; ++tile, ++it) {
+            int sg, n;
+            uint32_t i0;
+            place(tile, sg, i0, n);
+            if (sg != held) {
+                if (any) ok = gt_wait(&b_used[last], last_p, &s_bad);     // the images' last readers
+                if (!ok) break;
+                tc::mbar_expect_tx(&b_mat, (uint32_t)nv * 2 * kMat);
+                for (int k = 0; k < nv; ++k) {
+                    const unsigned char* src = a.bimg + (size_t)t_e[k] * 8 * kMat + (size_t)sg * kMat;
+                    tc::bulk_g2s(Bs + (size_t)k * 2 * kMat, src, kMat, &b_mat);
+                    tc::bulk_g2s(Bs + (size_t)k * 2 * kMat + kMat, src + 4 * kMat, kMat, &b_mat);
+                }
+                ok = tc::mbar_wait(&b_mat, n_mat & 1, 1u << 24);          // not cut short: a copy in flight
+                if (!ok) { s_bad = 1; break; }
+                ++n_mat;
+                held = sg;
+            }
+            const uint32_t buf = it % NG;
+            if (it >= NG) ok = gt_wait(&b_free[buf], (it / NG - 1) & 1, &s_bad);
+            for (int k = 0; ok && k < nv; ++k) {
+                ok = gt_wait(&b_ready[slot], round & 1, &s_bad);
+                if (!ok) break;
+                tc::fence_after_sync();
+                const uint64_t dA = d0 + (tc::smem_addr(smraw + (size_t)slot * kSlot) >> 4);
+                const uint64_t dB = d0 + (tc::smem_addr(Bs + (size_t)k * 2 * kMat) >> 4);
+                #pragma unroll
+                for (int term = 0; term < 3; ++term)
+                    #pragma unroll
+                    for (int ks = 0; ks < D / 16; ++ks) {
+                        const uint64_t ao = term == 1 ? (kLo >> 4) : 0;
+                        const uint64_t bo = term == 2 ? (kMat >> 4) : 0;
+                        tc::mma_f16(tmem + buf * kAcc + (uint32_t)(k * D), dA + ao + 16 * ks, dB + bo + 16 * ks, idesc,
+                                    (term | ks) ? 1u : 0u);
+                    }
+                tc::mma_commit(&b_used[slot]);
+                if (k == nv - 1) tc::mma_commit(&b_acc[buf]);
+                any = true;
+                last = slot;
+                last_p = round & 1;
+                if (++slot == (uint32_t)n_slots) { slot = 0; ++round; }
+            }
+        }
+        if (any) tc::mbar_wait(&b_used[last], last_p, 1u << 24);          // nothing in flight at the end
     }
-    if (!ok) report(a.err, 5, 6, (long long)blockIdx.x);
+    __syncwarp();
     tc::fence_before_sync();
     __syncthreads();
-    tc::fence_after_sync();
-    if (warp == 0) tc::tmem_dealloc(tmem, cols);
+    if (s_bad && tid == 0) report(a.err, 5, 6, (long long)blockIdx.x);
+    if (warp == kMmaWarp) tc::tmem_dealloc(tmem, 512);
 }
 
 // Terms of the rows, one thread per row: psi_TN(m) from the row's node, the
@@ -456,28 +538,18 @@ int launch_tree_graph_tc(const TreeGraphTc& a, int t, int deg, const TreeLevels&
     const int D = a.an.D;
     const TreeGroups g = tree_groups(t, bounds, kGtRows);
     if (g.tile[4] == 0) return 0;
-    // resident CTAs per SM: bounded by registers (launch bounds), shared memory
-    // and the 512 tensor-memory columns (a CTA holds its own for the whole launch)
-    const size_t smem = (size_t)deg * ((size_t)kGtRows * D * 4 + (size_t)4 * D * D);
-    int cols = 32;
-    while (cols < deg * D) cols <<= 1;
-    int per = std::min(D <= 32 ? 3 : 2, 512 / cols);
-    per = std::max(1, std::min<int>(per, (int)((200u << 10) / (smem + 12 * 1024))));
-    const unsigned grid = (unsigned)std::min<int>(g.tile[4], per * n_sm);
-    switch (D) {
-    case 16:
-        allow_max_smem(k_tree_graph_tc<16>);
-        k_tree_graph_tc<16><<<grid, kGtThreads, smem, st>>>(a, t, deg, lv.at[t], lv.n[t], g);
-        break;
-    case 32:
-        allow_max_smem(k_tree_graph_tc<32>);
-        k_tree_graph_tc<32><<<grid, kGtThreads, smem, st>>>(a, t, deg, lv.at[t], lv.n[t], g);
-        break;
-    default:
-        allow_max_smem(k_tree_graph_tc<64>);
-        k_tree_graph_tc<64><<<grid, kGtThreads, smem, st>>>(a, t, deg, lv.at[t], lv.n[t], g);
-        break;
-    }
+    // one block per SM; its ring takes the shared memory that the images leave
+    const size_t slot = (size_t)kGtRows * D * 4, images = (size_t)deg * 4 * D * D;
+    const int n_slots = (int)std::min<size_t>(kGtRing, ((size_t)220 * 1024 - images) / slot);
+    const size_t smem = n_slots * slot + images;
+    const unsigned grid = (unsigned)std::min<int>(g.tile[4], n_sm);
+    auto launch = [&](void (*kernel)(TreeGraphTc, int, int, uint32_t, uint32_t, TreeGroups, int)) {
+        allow_max_smem(kernel);
+        kernel<<<grid, gt_threads(D), smem, st>>>(a, t, deg, lv.at[t], lv.n[t], g, n_slots);
+    };
+    if (D == 16) launch(k_tree_graph_tc<16>);
+    else if (D == 32) launch(k_tree_graph_tc<32>);
+    else launch(k_tree_graph_tc<64>);
     return 1;
 }
 

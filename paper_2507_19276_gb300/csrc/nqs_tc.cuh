@@ -161,6 +161,12 @@ __device__ __forceinline__ void cp_async4(void* sdst, const void* gsrc)
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"(smem_addr(sdst)), "l"(gsrc) : "memory");
 }
 
+// arrive on an mbarrier (one of its counted arrivals) once this thread's cp_async
+// copies so far have completed
+__device__ __forceinline__ void cp_async_arrive(uint64_t* mbar)
+{
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" :: "r"(smem_addr(mbar)) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 
 // wait until at most N of this thread's most recent groups are pending

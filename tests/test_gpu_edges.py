@@ -331,3 +331,30 @@ def test_full_batches_equal_small_ones(ctx, D, nh):
         ctx.set_precision(nqs.NQS_PREC_FP64)
     for i, p in zip(parts, got):
         assert np.array_equal(p, e[i:i + 500])
+
+
+@pytest.mark.parametrize("D", [16, 32, 64])
+def test_graph_tiles_beyond_the_ring(ctx, D):
+    """Vertex steps with many tiles per block (the ring of source states and the
+    accumulators go round several times) against the same samples in small calls;
+    a node's arithmetic is its own, so the results are equal."""
+    import dataclasses
+    s = _dag(40 + D, 8, D, n_samples=4800, eps=0.0, n_draws=0)
+    if D == 64:                                    # one in-edge (two matrices' images are refused)
+        ptr, idx, keep = [0], [], []
+        for i in range(s.K):
+            e = list(range(s.pred_ptr[i], s.pred_ptr[i + 1]))[-1:]
+            keep += e
+            idx += [int(s.pred_idx[x]) for x in e]
+            ptr.append(len(idx))
+        s = dataclasses.replace(s, pred_ptr=np.array(ptr, np.int32), pred_idx=np.array(idx, np.int32),
+                                tensors=np.ascontiguousarray(s.tensors[keep]))
+    ctx.set_system(s)
+    ctx.set_precision(nqs.NQS_PREC_MIXED)
+    try:
+        e, _ = ctx.local_energy(s.samples, s.counts, 0.0, 0, 1)
+        for i in (0, len(e) // 2, len(e) - 40):
+            p, _ = ctx.local_energy(s.samples[i:i + 40], s.counts[i:i + 40], 0.0, 0, 1)
+            assert np.array_equal(p, e[i:i + 40])
+    finally:
+        ctx.set_precision(nqs.NQS_PREC_FP64)
