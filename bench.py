@@ -400,17 +400,17 @@ def run(args):
         roof = {"bound": "tensor", "unit": "TFLOP/s", "achieved": achieved,
                 "peak": peaks["bf16_tflops_sustained"],
                 "peak_source": f"{src} dense bf16 (sustained; f16 has the same nominal rate)",
-                "kernel": ("k_graph_tiles (tcgen05, 128-row tiles re-running the vertices from "
-                           "each row's first change)" if graph else
+                "kernel": ("k_tree_graph_tc (tcgen05, 128-node tiles of the rows' prefix trees), "
+                           "k_tree_rows_tc" if graph else
                            "amplitude stage: k_fam_mark, k_fam_compact, k_site_boundary, "
-                           "k_site_build, k_site_tiles_pipe (tcgen05), k_fam_rbm, k_fam_rows")}
+                           "k_site_build, k_site_tiles_pipe / k_site_tiles_ws (tcgen05), k_fam_rbm, k_fam_rows")}
     else:
         roof = {"bound": "alu", "unit": "TFLOP/s", "achieved": achieved,
                 "peak": live["fma64_tflops"] if live else 1.056,
                 "peak_source": ("FP64 FMA rate measured before the timed region (peaks probe)" if live
                                 else "FP64 FMA rate of an earlier peaks-probe run on a GB300"),
                 "kernel": ("amplitude stage (shared prefixes, FP64)" if prec == nqs.NQS_PREC_FP64_SHARED
-                           else "k_amp_chain_fp64 / k_amp_graph_fp64 (one amplitude per row)")}
+                           else "k_tree_graph64 / k_fx_graph (prefix trees of the rows), k_tree_rows64")}
     roof["frac"] = roof["achieved"] / roof["peak"]
     # the same stage against the work the shared-prefix form executes
     roof["executed_frac"] = executed / (amp_ms / 1e3) / 1e12 / roof["peak"]
@@ -592,7 +592,7 @@ def run_rnn(args):
     roof = {"bound": "alu", "unit": "TFLOP/s", "achieved": flops / (amp_ms / 1e3) / 1e12, "peak": peak,
             "peak_source": "FP64 FMA rate measured before the timed region (peaks probe)" if live
             else "FP64 FMA rate of an earlier probe run on this pool's GB300",
-            "kernel": "k_rnn_amp (normalised readout, FP64, one warp per row)", "traffic": None,
+            "kernel": "k_tree_rnn / k_fx_rnn (normalised readout over the rows' prefix trees)", "traffic": None,
             "algorithmic_flops_per_step": flops, "stage_ms_per_step": amp_ms}
     roof["frac"] = roof["achieved"] / roof["peak"]
     # end to end: the same step with host-side outputs (samples back to the host,

@@ -60,9 +60,14 @@ typedef enum {
 } nqs_status;
 
 typedef enum {
-    NQS_PREC_FP64 = 0,        /* the plain form: every amplitude psi(m) is its own
-                                 FP64 product over the sites where m differs from n
-                                 (cached left/right environments outside that span) */
+    NQS_PREC_FP64 = 0,        /* the plain form: the FP64 recursion of the connected
+                                 m continued from n's states over each sample's prefix
+                                 tree (rows with the same first changes share their
+                                 steps; linear readouts close with n's adjoint
+                                 covectors after the last change; the tensor term
+                                 runs row by row). Levels with many nodes take their
+                                 matrix products in fixed point on the tensor cores,
+                                 with an error no larger than FP64's */
     NQS_PREC_MIXED = 1,       /* contractions on the tensor cores (split FP16
                                  operands, FP32 accumulation, per-site power-of-two
                                  rescaling); H_nm, psi(n), the ratios and the E_loc
@@ -70,8 +75,9 @@ typedef enum {
                                  evaluation (partial products common to many m of
                                  one n are formed once and each psi(m) is one dot
                                  product). Graph ansatz: the vertices from each
-                                 row's first changed site on are re-run for 128 rows
-                                 of one sample at a time; needs D in {16, 32, 64},
+                                 row's first changed site on are re-run over the
+                                 samples' prefix trees, 128 nodes at a time; needs
+                                 D in {16, 32, 64},
                                  in-degree x 4 x D <= 512, at most 16 vertex states
                                  live at once, the linear readout, no tensor term
                                  and the 2cosh or cos correlator (otherwise
@@ -170,8 +176,8 @@ typedef struct {
                                chains, plain form: span_sites; graphs (linear
                                readout): the in-edges with a vertex source of
                                every re-run vertex, summed over the amplitudes
-                               (the tensor-core tiles also run rows and local
-                               states a tile shares, not counted here);
+                               (rows that share a prefix share its products:
+                               fewer are executed than counted here);
                                shared-prefix form: one-change families plus
                                two-change clusters of the pass over the whole
                                batch */

@@ -21,7 +21,7 @@
 // packed subtraction), 34 x D/16 MMAs, then the integer epilogue. Per tile at
 // D = 64 that is ~20 k warp instructions and 136 MMAs, against 301 k cycles of
 // the FP64 pipe for the same products. H50 tables of 200 samples (5 M products):
-// 45 ms on the FP64 pipe, 5.0 ms here; issue and latency of the digit and
+// 45 ms on the FP64 pipe, 4.7 ms here; issue and latency of the digit and
 // epilogue chains bound it (one block per SM at D = 64).
 #include "nqs_fx.cuh"
 #include "nqs_tc.cuh"
