@@ -410,7 +410,9 @@ def run(args):
                 "peak_source": ("FP64 FMA rate measured before the timed region (peaks probe)" if live
                                 else "FP64 FMA rate of an earlier peaks-probe run on a GB300"),
                 "kernel": ("amplitude stage (shared prefixes, FP64)" if prec == nqs.NQS_PREC_FP64_SHARED
-                           else "k_tree_graph64 / k_fx_graph (prefix trees of the rows), k_tree_rows64")}
+                           else "k_tree_graph64 / k_fx_graph (prefix trees of the rows), k_tree_rows64"),
+                "note": ("frac counts a per-amplitude evaluation's products against the FP64 pipe; shared "
+                         "prefixes execute fewer, and large steps run in fixed point on the tensor cores")}
     roof["frac"] = roof["achieved"] / roof["peak"]
     # the same stage against the work the shared-prefix form executes
     roof["executed_frac"] = executed / (amp_ms / 1e3) / 1e12 / roof["peak"]
@@ -593,6 +595,8 @@ def run_rnn(args):
             "peak_source": "FP64 FMA rate measured before the timed region (peaks probe)" if live
             else "FP64 FMA rate of an earlier probe run on this pool's GB300",
             "kernel": "k_tree_rnn / k_fx_rnn (normalised readout over the rows' prefix trees)", "traffic": None,
+            "note": "frac counts a per-row evaluation against the FP64 pipe; rows share their prefixes and "
+                    "large levels run in fixed point on the tensor cores",
             "algorithmic_flops_per_step": flops, "stage_ms_per_step": amp_ms}
     roof["frac"] = roof["achieved"] / roof["peak"]
     # end to end: the same step with host-side outputs (samples back to the host,

@@ -26,12 +26,17 @@ constexpr int kDefaultAudit = 4;
 
 // chains: samples (determinants) from which the FP64 sweeps go site by site
 // through the fixed-point tensor-core steps (one launch per site) instead of
-// one block per sample
-constexpr int64_t kFxMinRows = 512;
+// one block per sample. log|psi| and its gradient at D = 64, K = 50, fixed-point /
+// block per sample: 512 determinants 3.03 / 2.00 ms, 1024 3.14 / 3.01, 2048 3.49 /
+// 4.62
+constexpr int64_t kFxMinRows = 1100;
 
 // nodes of a level from which the prefix trees' FP64 steps take 128-node
-// fixed-point tiles (about half a tile per SM) instead of 32-node FP64 ones
-constexpr int64_t kFxMinNodes = 8192;
+// fixed-point tiles instead of 32-node FP64 ones. All levels in fixed point / none,
+// H18 graph (D = 32): 2 samples 1.28 / 1.45 ms, 10 samples 1.55 / 2.38, 100 samples
+// 4.45 / 12.2; normalised readout (D = 10): 2 samples 3.44 / 3.76, 50 samples 15.5 /
+// 26.7. A level of a few tiles is latency either way, so those stay in FP64
+constexpr int64_t kFxMinNodes = 1024;
 
 struct DevBuf {
     void* p = nullptr;
@@ -888,11 +893,6 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
     if (kind != kTreeRnn) TRY(ensure(c, c->mv_det, (size_t)(chunks_all + 1) * 8));
     if (want_abs) TRY(ensure(c, c->part_det_abs, (size_t)(chunks_all + 1) * 8));
 
-    size_t free_b = 0, total_b = 0;
-    cudaMemGetInfo(&free_b, &total_b);
-    free_b += c->tr_build.n + c->tr_pool.n + c->tr_items.n;     // kept from earlier calls
-    size_t budget = std::min<size_t>(c->table_mb > 0 ? (size_t)c->table_mb << 20 : (size_t)16 << 30, free_b / 3);
-    if (c->fam_budget > 0) budget = std::min(budget, c->fam_budget);
     const int n2max = 9 * K * (K - 1) / 2 > 0 ? 9 * K * (K - 1) / 2 : 1, W = (T + 31) / 32;
     const size_t state = kind == kTreeGraph64 ? (size_t)D * 8 + 4 : (size_t)D * 4 + 4;
     const size_t node_b = kind == kTreeRnn ? 16 + 2 * ((size_t)D * 8 + 16) : 16 + (full ? 8 : 0);
@@ -903,6 +903,18 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
         return (size_t)4 * T * (T + 1) + (size_t)8 * n2max * W + nodes * node_b + (size_t)8 * r +
                lv * (4 + (kind == kTreeRnn ? 0 : state)) + (kind == kTreeGraph64 ? (size_t)3 * c->n_live * (D * 8 + 4) : 0);
     };
+    // a small call that the buffers kept from earlier calls already hold does not
+    // ask the driver for the free memory (25 us of a 0.4 ms call)
+    const size_t kept = c->tr_build.n + c->tr_pool.n + c->tr_items.n;
+    const size_t all = (size_t)Ns * bytes_of(rows_bound / Ns + 1);
+    size_t budget = (size_t)64 << 20;
+    if (all > budget || all > kept || c->table_mb > 0) {
+        size_t free_b = 0, total_b = 0;
+        cudaMemGetInfo(&free_b, &total_b);
+        free_b += kept;
+        budget = std::min<size_t>(c->table_mb > 0 ? (size_t)c->table_mb << 20 : (size_t)16 << 30, free_b / 3);
+    }
+    if (c->fam_budget > 0) budget = std::min(budget, c->fam_budget);
     for (int64_t s0 = 0; s0 < Ns;) {
         int64_t s1 = s0;
         size_t want = 0;
@@ -950,7 +962,7 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
         a.id3 = a.id2 + (uint32_t)((int64_t)nb * n2max);
         a.id4 = a.id3 + (uint32_t)R;
         const int64_t ncnt = (int64_t)4 * K * nb;
-        int64_t *scan_tmp = nullptr, *pool_off = nullptr;
+        int64_t *scan_tmp = nullptr, *pool_off = nullptr, *head = nullptr;
         float* mant = nullptr;
         int* mexp = nullptr;
         uint32_t* perm = nullptr;
@@ -974,6 +986,7 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
             a.level_cnt = v.take<int64_t>((size_t)ncnt);
             a.level_off = v.take<int64_t>((size_t)ncnt + 1);
             scan_tmp = v.take<int64_t>((size_t)scan_i64_tmp_elems(ncnt));
+            head = v.take<int64_t>((size_t)4 * K + 2);
             if (kind == kTreeGraphTc) {
                 mant = v.take<float>((size_t)nodes);
                 mexp = v.take<int>((size_t)nodes);
@@ -991,12 +1004,13 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
         LAUNCH(stage, launch_scan_i64(a.pool_tot, pool_off, nb, c->stream));
         LAUNCH(stage, launch_scan_i64_wide(a.level_cnt, a.level_off, ncnt, scan_tmp, c->stream));
         CK(cudaGetLastError());
-        std::vector<int64_t> bounds((size_t)4 * K + 1);
-        int64_t pool_rows = 0;
-        CK(cudaMemcpy2DAsync(bounds.data(), 8, a.level_off, (size_t)nb * 8, 8, (size_t)4 * K + 1, cudaMemcpyDeviceToHost,
-                             c->stream));
-        CK(cudaMemcpyAsync(&pool_rows, pool_off + nb, 8, cudaMemcpyDeviceToHost, c->stream));
+        // the levels' item bounds and the pool's rows, in one copy
+        std::vector<int64_t> bounds((size_t)4 * K + 2);
+        LAUNCH(stage, launch_tree_head(a.level_off, nb, 4 * K + 1, pool_off + nb, head, c->stream));
+        CK(cudaMemcpyAsync(bounds.data(), head, ((size_t)4 * K + 2) * 8, cudaMemcpyDeviceToHost, c->stream));
         CK(cudaStreamSynchronize(c->stream));
+        const int64_t pool_rows = bounds.back();
+        bounds.pop_back();
         const int64_t rows_total = pool_rows + a.pool0;
         const size_t pool_b = kind == kTreeRnn ? 0 : (size_t)rows_total * state;
         if (nb > 1 && (rows_total >= ((int64_t)1 << 32) ||
@@ -1046,10 +1060,8 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
             const size_t srow = (size_t)K + (chain ? 1 : 0);
             const double* h0 = chain ? (const double*)c->Lenv.p + D : (const double*)c->Hst.p;
             const int* x0 = chain ? (const int*)c->Lexp.p + 1 : (const int*)c->Hexp.p;
-            CK(cudaMemcpy2DAsync(g.pool, (size_t)K * D * 8, h0 + (size_t)s0 * srow * D, srow * D * 8, (size_t)K * D * 8,
-                                 (size_t)nb, cudaMemcpyDeviceToDevice, c->stream));
-            CK(cudaMemcpy2DAsync(g.pool_e, (size_t)K * 4, x0 + (size_t)s0 * srow, srow * 4, (size_t)K * 4, (size_t)nb,
-                                 cudaMemcpyDeviceToDevice, c->stream));
+            LAUNCH(stage, launch_tree_roots(h0 + (size_t)s0 * srow * D, x0 + (size_t)s0 * srow, (int)srow, nb, K, D, g.pool,
+                                            g.pool_e, c->stream));
             g.an = c->av;
             g.an.pred_ptr = (const int*)c->pred_ptr.p;
             g.an.pred_idx = (const int*)c->pred_idx.p;

@@ -24,7 +24,9 @@ namespace nqs {
 namespace {
 
 constexpr int kGradChunk = 256;   // samples per block (one chunk of a local-state group)
-constexpr int64_t kFxGradMin = 256;   // samples from which the fixed-point products run
+// samples from which the fixed-point products run. H18 energy gradient (D = 32),
+// fixed-point / FP64: 32 samples 1.82 / 1.82 ms, 128 2.53 / 2.60, 512 5.73 / 6.18
+constexpr int64_t kFxGradMin = 64;
 constexpr int kTile = 64;         // output tile edge
 constexpr int kStage = 16;        // samples staged per round
 

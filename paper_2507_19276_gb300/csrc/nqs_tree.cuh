@@ -114,6 +114,13 @@ struct TreeRows64 {
 int launch_tree_rows64(const TreeRows64& a, int64_t max_chunks, cudaStream_t st);
 
 // Mixed form of a graph ansatz: split-FP16 states, one vertex per launch.
+// out[i] = off[i * stride] for i < n, then *last: what the host reads of a tree batch
+int launch_tree_head(const int64_t* off, int stride, int n, const int64_t* last, int64_t* out, cudaStream_t st);
+// the roots' states and powers of two (nb samples, K rows of D each out of src_rows
+// per sample) into the pool's first rows
+int launch_tree_roots(const double* h, const int* x, int src_rows, int nb, int K, int D, double* pool, int* pool_e,
+                      cudaStream_t st);
+
 struct TreeGraphTc {
     AnsatzView an;
     const uint32_t* items;

@@ -191,7 +191,7 @@ def _log_psi_ref(s, dets):
 
 
 @pytest.mark.parametrize("D", [16, 32, 48, 64])
-@pytest.mark.parametrize("n", [512, 777])
+@pytest.mark.parametrize("n", [512, 777, 1201])
 def test_fixed_point_steps(ctx, D, n):
     """Chains on the fixed-point tensor-core steps: every width, part tiles of
     every local state, entries over many powers of two. K (D + 1) 2^-53 of the
