@@ -82,7 +82,8 @@ __device__ __forceinline__ __half2 fx_digit2(uint64_t c0, uint64_t c1, int i)
 }
 
 // One block per (matrix, side): the columns' powers of two, the rows' after them,
-// then the digits. The operand has `rows` rows of D entries (columns past D, up
+// then the digits. A column without entries has the power kFxNoExp, so that the
+// vector's entry there, which meets only zeros, takes no part in its scale. The operand has `rows` rows of D entries (columns past D, up
 // to C, and rows past `rows`, up to R, are zero) in blocks of R rows:
 // entry(n, k) of the matrix.
 template <class Entry>
@@ -98,7 +99,7 @@ __device__ void fx_image(const Entry& entry, int rows, int D, int R, int C, unsi
                 if (!fx_not_finite(v)) e = max(e, fx_exp(v));
             }
         sc[k] = e == kFxNoExp ? 0 : e;
-        cexp[k] = sc[k];
+        cexp[k] = e;                              // kFxNoExp: an empty column, out of the vector's scale
     }
     __syncthreads();
     const int RT = (rows + R - 1) / R * R;
