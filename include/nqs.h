@@ -66,8 +66,12 @@ typedef enum {
                                  steps; linear readouts close with n's adjoint
                                  covectors after the last change; the tensor term
                                  runs row by row). Levels with many nodes take their
-                                 matrix products in fixed point on the tensor cores,
-                                 with an error no larger than FP64's */
+                                 matrix products in fixed point on the tensor cores:
+                                 56 bits of the product's scale, at most D 2^-47 of
+                                 its largest term (FP64: D 2^-53 of the sum of the
+                                 terms' magnitudes); a result whose terms may all be
+                                 below 2^-8 of the scale, or that an infinity or a
+                                 NaN enters, is redone in FP64 */
     NQS_PREC_MIXED = 1,       /* contractions on the tensor cores (split FP16
                                  operands, FP32 accumulation, per-site power-of-two
                                  rescaling); H_nm, psi(n), the ratios and the E_loc

@@ -455,6 +455,7 @@ int env_pass(nqs_ctx* c, const uint64_t* samples, int64_t Ns, bool adjoints, int
         x.K = K;
         x.img = (const unsigned char*)c->fx_img.p;
         x.exps = (const int*)c->fx_exps.p;
+        x.at[0] = c->av.AT; x.at[1] = c->av.A;
         x.pool[0] = e.Lenv; x.pool[1] = e.Renv;
         x.pool_e[0] = e.Lexp; x.pool_e[1] = e.Rexp;
         x.stride = K + 1;
@@ -501,6 +502,7 @@ int fx_amplitude(nqs_ctx* c, const uint64_t* dets, int64_t n, double* log_abs, i
         x.K = K;
         x.img = (const unsigned char*)c->fx_img.p;
         x.exps = (const int*)c->fx_exps.p;
+        x.at[0] = c->av.AT; x.at[1] = c->av.A;
         x.pool[0] = x.pool[1] = rows;
         x.pool_e[0] = x.pool_e[1] = exps;
         x.stride = 2;
@@ -611,6 +613,7 @@ int site_tables(nqs_ctx* c, const FamArgs<T>& f, int nbb)
         x.K = K;
         x.img = (const unsigned char*)c->fx_img.p;
         x.exps = (const int*)c->fx_exps.p;
+        x.at[0] = c->av.AT; x.at[1] = c->av.A;
         x.pool[0] = x.pool[1] = (double*)f.pool;
         x.pool_e[0] = x.pool_e[1] = f.pool_e;
         x.items = (const uint2*)sb.items;
@@ -1500,7 +1503,7 @@ extern "C" int nqs_set_ansatz(nqs_ctx* c, const double* site_tensors, int n_edge
     if (c->has_fx) {
         const int sides = chain ? 2 : 1;
         TRY(ensure(c, c->fx_img, fx_image_bytes(fm.n_mats, D, sides)));
-        TRY(ensure(c, c->fx_exps, (size_t)sides * fm.n_mats * 2 * D * 4));
+        TRY(ensure(c, c->fx_exps, (size_t)sides * fm.n_mats * fx_exp_stride(D) * 4));
         LAUNCH(NQS_STAGE_OTHER, launch_fx_images(fm.A, fm.n_mats, D, sides, (unsigned char*)c->fx_img.p, (int*)c->fx_exps.p,
                                                  c->stream));
     }

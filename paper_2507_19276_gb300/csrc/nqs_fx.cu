@@ -13,8 +13,10 @@
 // hold exact integers. The 34 digit products down to significance 2^-70 are
 // kept; the eight sums of a result are joined in 64-bit integers (unit 2^-56 of
 // the scale) and rounded to FP64 once. The remaining error, the rounding of the
-// entries and of the result, is ~2^-56 sqrt(D) of the scale; a chain of FP64
-// FMAs rounds its partial sums D times at 2^-53.
+// entries and of the result, is ~2^-56 sqrt(D) of the scale (at most ~D 2^-55);
+// a chain of FP64 FMAs rounds its partial sums D times at 2^-53. On dense random
+// matrices that is the smaller error. Results whose terms may all lie far below the
+// scale are found by bit masks and redone in FP64 (see kFxTerm).
 //
 // A tile is 128 items of one matrix (two or four threads per row): gather and cut
 // the rows into digits (bytes of x + 0x80..80, turned into FP16 by PRMT and one
@@ -65,6 +67,48 @@ __device__ __forceinline__ int fx_exp(double x)
 }
 
 __device__ __forceinline__ bool fx_not_finite(double x) { return (__double2hiint(x) & 0x7FF00000) == 0x7FF00000; }
+__device__ __forceinline__ bool fx_nonzero(double x) { return ((__double2hiint(x) << 1) | __double2loint(x)) != 0; }
+
+// The unit of a result is 2^-56 of (row scale) x (matrix row scale), so its digits
+// hold it as well as FP64 would only if one of its terms is near that scale: where
+// the large entries of a graded state meet the small ones of the matrix row, an FP64
+// chain keeps 53 bits of what is there and the digits few or none. A term of at least
+// 2^-kFxTerm of the scale is known to be there if entries of at least 2^-(kFxTerm / 2)
+// meet in the state and the matrix row (a bit mask each; for dense rows, also beside a
+// unit diagonal, that holds practically always), or if the result itself reaches
+// 2^-kFxTerm. Any other result with a nonzero term (two more masks) is redone with
+// FP64 FMAs, as are those that an infinity, a NaN or a denormal entry takes part in.
+// What stays errs by at most ~D 2^-55 of the scale, that is D 2^-47 of its largest
+// term where FP64 FMAs err by up to D 2^-53 of the sum of the terms. Of the results of
+// I + G / sqrt(D) matrices, kFxTerm = 4 redoes 5% (H50's log|psi| 4.2 -> 18 ms), 6
+// 0.6% (6.4 ms), 8 none but those of the first site's e_0.
+constexpr int kFxTerm = 8;
+__device__ __forceinline__ bool fx_is_big(int e) { return e > -(kFxTerm / 2); }      // e as fx_exp's: |x| >= 2^(e-1)
+
+// exponent as fx_exp's of any finite nonzero number, kFxNoExp of the others
+__device__ __forceinline__ int fx_top(double y)
+{
+    const int f = (__double2hiint(y) >> 20) & 0x7FF;
+    if (f > 0) return f < 0x7FF ? f - 1022 : kFxNoExp;
+    int e = kFxNoExp;
+    if (fx_nonzero(y)) frexp(y, &e);
+    return e;
+}
+
+// a thread's H bits of row r's marks
+template <int H>
+__device__ __forceinline__ void fx_mark(uint64_t* marks, int r, int h, uint32_t low)
+{
+    unsigned char* to = (unsigned char*)(marks + r) + h * (H / 8);
+    #pragma unroll
+    for (int b = 0; b < H / 8; ++b) to[b] = (unsigned char)(low >> (8 * b));
+}
+
+// |v| < 2^bits
+__device__ __forceinline__ bool fx_below(int64_t v, int bits)
+{
+    return (uint64_t)(v + (1ll << bits)) < (2ull << bits);
+}
 
 // digit `i` (0 = least significant) of two codes as FP16
 __device__ __forceinline__ __half2 fx_digit2(uint64_t c0, uint64_t c1, int i)
@@ -88,7 +132,7 @@ __device__ __forceinline__ __half2 fx_digit2(uint64_t c0, uint64_t c1, int i)
 // entry(n, k) of the matrix.
 template <class Entry>
 __device__ void fx_image(const Entry& entry, int rows, int D, int R, int C, unsigned char* img, int* cexp, int* rexp,
-                         int* sc, int* sr)
+                         uint64_t* big, uint64_t* nonzero, int* sc, int* sr)
 {
     const int lane = threadIdx.x & 31;
     for (int k = threadIdx.x; k < C; k += blockDim.x) {
@@ -112,9 +156,20 @@ __device__ void fx_image(const Entry& entry, int rows, int D, int R, int C, unsi
         }
         e = __reduce_max_sync(kFull, e);
         bad = __any_sync(kFull, bad);
+        e = e <= kFxNoExp / 2 ? 0 : e;
+        uint64_t mb = 0, mz = 0;
+        for (int k0 = 0; k0 < C; k0 += 32) {
+            const int k = k0 + lane;
+            const double v = n < rows && k < D ? entry(n, k) : 0.0;
+            const int x = k < C ? fx_exp(v) - sc[k] - e : kFxNoExp;
+            mb |= (uint64_t)__ballot_sync(kFull, !bad && fx_is_big(x)) << k0;
+            mz |= (uint64_t)__ballot_sync(kFull, fx_nonzero(v)) << k0;
+        }
         if (lane == 0) {
-            sr[n] = e <= kFxNoExp / 2 ? 0 : e;
-            rexp[n] = bad ? kFxNotFinite : sr[n];
+            sr[n] = e;
+            rexp[n] = bad ? kFxNotFinite : e;
+            big[n] = mb;
+            nonzero[n] = mz;
         }
     }
     __syncthreads();
@@ -136,8 +191,10 @@ __global__ void __launch_bounds__(256) k_fx_images(const double* __restrict__ A,
     const int m = blockIdx.x, side = blockIdx.y;
     const double* M = A + (size_t)m * D * D;
     const size_t id = (size_t)side * n_mats + m;
+    int* const x = exps + id * fx_exp_stride(D);
+    uint64_t* const masks = (uint64_t*)(x + 2 * D);
     fx_image([&](int n, int k) { return side == 0 ? __ldg(M + (size_t)n * D + k) : __ldg(M + (size_t)k * D + n); }, D, D, D, D,
-             img + id * kFxDigits * 2 * D * D, exps + id * 2 * D, exps + id * 2 * D + D, sc, sr);
+             img + id * kFxDigits * 2 * D * D, x, x + D, masks, masks + D, sc, sr);
 }
 
 // The eight sums of a result (FP32 accumulators that hold integers) as an integer
@@ -176,16 +233,27 @@ __device__ __forceinline__ double fx_double(int64_t v, int power, int emax)
 }
 
 // A thread's H results of row r (column block h) into the staging rows (D + 2
-// doubles apart: no bank conflicts), which reuse the digits' shared memory...
+// doubles apart: no bank conflicts), which reuse the digits' shared memory; those
+// marked in `low` are there already, redone in FP64, and are scaled by 2^shift ...
 template <int D, int H>
-__device__ __forceinline__ void fx_put(const int64_t* V, const int* power, int emax, bool bad, double* rows, int r, int h)
+__device__ __forceinline__ void fx_put(const int64_t* V, const int* power, int emax, uint32_t low, int shift, double* rows,
+                                       int r, int h)
 {
-    const double nan = __longlong_as_double(0x7FF8000000000000ll);
     double* out = rows + (size_t)r * (D + 2) + h * H;
     #pragma unroll
     for (int c = 0; c < H; c += 2) {
         const double o0 = fx_double(V[c], power[c], emax), o1 = fx_double(V[c + 1], power[c + 1], emax);
-        *(double2*)(out + c) = bad ? make_double2(nan, nan) : make_double2(o0, o1);
+        const uint32_t m = (low >> c) & 3u;
+        if (m == 0) {
+            *(double2*)(out + c) = make_double2(o0, o1);
+        } else {
+            if (!(m & 1u)) out[c] = o0;
+            if (!(m & 2u)) out[c + 1] = o1;
+        }
+    }
+    for (; low; low &= low - 1) {
+        const int c = __ffs((int)low) - 1;
+        out[c] = scale_pow2(out[c], shift);
     }
 }
 
@@ -218,10 +286,11 @@ __device__ __forceinline__ void fx_mma(uint32_t tmem, uint32_t N, uint64_t dA, u
 // The digits of a tile's rows (row r at pool + src[r] * D, times the column powers
 // cm, scaled by 2^-ea[r]) into the operand buffers: eight entries of a row per
 // task, eight rows x four tasks per warp (shared memory in whole core matrices).
-// ea[r] must hold kFxNoExp; contains a block barrier.
+// ea[r] must hold kFxNoExp; contains a block barrier. big and nonzero get each row's
+// masks of entries that are large after the scaling, and not zero (bits below D).
 template <int D, int SP>
 __device__ __forceinline__ void fx_rows(const double* __restrict__ pool, const int64_t* src_row, const int* cm, int* ea_row,
-                                        int* bad_row, unsigned char* A)
+                                        int* bad_row, uint64_t* big, uint64_t* nonzero, unsigned char* A)
 {
     constexpr int NW = kFxRows * SP / 32;
     constexpr uint32_t kA = kFxRows * D * 2;
@@ -272,8 +341,16 @@ __device__ __forceinline__ void fx_rows(const double* __restrict__ pool, const i
     for (int u = 0; u < TASKS; ++u) {
         const int ea = ea_row[rows[u]];
         uint64_t c[8];
+        uint32_t mb = 0, mz = 0;
         #pragma unroll
-        for (int k = 0; k < 8; ++k) c[k] = fx_code(v[u][k], cm[8 * pcs[u] + k] - ea);
+        for (int k = 0; k < 8; ++k) {
+            const int off = cm[8 * pcs[u] + k] - ea;
+            c[k] = fx_code(v[u][k], off);
+            mb |= (fx_is_big(fx_exp(v[u][k]) + off) ? 1u : 0u) << k;
+            mz |= (fx_nonzero(v[u][k]) ? 1u : 0u) << k;
+        }
+        ((unsigned char*)(big + rows[u]))[pcs[u]] = (unsigned char)mb;
+        ((unsigned char*)(nonzero + rows[u]))[pcs[u]] = (unsigned char)mz;
         const uint32_t off = tc::op_offset(rows[u], 8 * pcs[u], D);
         #pragma unroll
         for (int i = 0; i < kFxDigits; ++i) {
@@ -294,11 +371,17 @@ __global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1) k_fx_s
     __shared__ int64_t s_src[kFxRows], s_dst[kFxRows];
     __shared__ int64_t s_gb[8], s_ge[8];
     __shared__ int s_tile[9];
-    __shared__ int s_eb[D], s_cm[D];
+    __shared__ __align__(8) int s_x[fx_exp_stride(D)];         // the matrix's powers of two and masks
     __shared__ int s_ea[kFxRows];                     // power of two taken out of each scaled row
     constexpr int SP = fx_split(D);                   // threads per row
-    __shared__ int s_max[SP][kFxRows];
+    __shared__ int s_max[SP][kFxRows], s_top[kFxRows];
     __shared__ int s_bad[kFxRows];
+    __shared__ uint64_t s_big[kFxRows], s_nz[kFxRows];
+    __shared__ uint64_t s_low[kFxRows];               // results to be redone in FP64
+    int* const s_cm = s_x;
+    int* const s_eb = s_x + D;
+    const uint64_t* const s_mb = (const uint64_t*)(s_x + 2 * D);
+    const uint64_t* const s_mz = s_mb + D;
     constexpr int NW = kFxRows * SP / 32;             // warps
     constexpr int H = D / SP;                         // columns per thread in the epilogue
     constexpr uint32_t kA = kFxRows * D * 2;          // one digit of the rows
@@ -366,10 +449,10 @@ __global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1) k_fx_s
                 tc::mbar_expect_tx(&mb_b, kFxDigits * kB);
                 tc::bulk_g2s(Bs, st.img + mat * kFxDigits * kB, kFxDigits * kB, &mb_b);
             }
-            if (tid < 2 * D) (tid < D ? s_cm : s_eb - D)[tid] = __ldg(st.exps + mat * 2 * D + tid);
+            for (int q = tid; q < fx_exp_stride(D); q += kFxRows * SP) s_x[q] = __ldg(st.exps + mat * fx_exp_stride(D) + q);
         }
         __syncthreads();
-        fx_rows<D, SP>(st.pool[side], s_src, s_cm, s_ea, s_bad, smraw);
+        fx_rows<D, SP>(st.pool[side], s_src, s_cm, s_ea, s_bad, s_big, s_nz, smraw);
         tc::fence_proxy_async();
         tc::fence_before_sync();
         __syncthreads();
@@ -402,6 +485,8 @@ __global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1) k_fx_s
         // join the sums: V = y 2^(56 - ea - eb), and the row's largest exponent
         int64_t V[H];
         int emax = -(1 << 29);
+        uint32_t low = 0;
+        const uint64_t mb = s_big[r], mz = s_nz[r];
         #pragma unroll
         for (int c0 = 0; c0 < H; c0 += 8) {
             uint32_t w[kFxSums][8];
@@ -413,20 +498,40 @@ __global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1) k_fx_s
                 const uint32_t x[kFxSums] = {w[0][c], w[1][c], w[2][c], w[3][c], w[4][c], w[5][c], w[6][c], w[7][c]};
                 const int64_t v = fx_join<D>(x, 0);
                 V[c0 + c] = v;
-                const int eb = s_eb[h * H + c0 + c];
-                if (v != 0) emax = max(emax, 64 - __clzll(v < 0 ? -v : v) + eb);
-                if (eb == kFxNotFinite) emax = kFxNotFinite;
+                const int col = h * H + c0 + c, eb = s_eb[col];
+                if (!(s_mb[col] & mb) && ((fx_below(v, 56 - kFxTerm) && (s_mz[col] & mz)) || eb == kFxNotFinite))
+                    low |= 1u << (c0 + c);
+                else if (v != 0) emax = max(emax, 64 - __clzll(v < 0 ? -v : v) + eb);
             }
         }
+        if (s_bad[r]) { low = H < 32 ? (1u << (H & 31)) - 1u : ~0u; emax = -(1 << 29); }
+        if (r >= n) low = 0;
         s_max[h][r] = emax;
+        fx_mark<H>(s_low, r, h, low);
         tc::fence_before_sync();
-        __syncthreads();                              // the parts of each row meet
+        const bool redo = __syncthreads_or(low != 0);         // the parts of each row meet
         #pragma unroll
         for (int k = 0; k < SP; ++k) emax = max(emax, s_max[k][r]);
-        fx_put<D, H>(V, s_eb + h * H, emax, s_bad[r] != 0 || emax >= kFxNotFinite, (double*)smraw, r, h);
+        if (redo) {
+            if (tid < kFxRows) s_top[tid] = -(1 << 29);
+            __syncthreads();
+            const double* M = st.at[side] + (mat - (size_t)side * 4 * st.K) * D * D;
+            for (int q = warp; q < n * ((D + 31) / 32); q += NW) {     // a warp per row and 32 results
+                const int row = q / ((D + 31) / 32), c = (q - row * ((D + 31) / 32)) * 32 + lane;
+                if (c >= D) continue;
+                if (!((s_low[row] >> c) & 1u)) continue;
+                const double y = dot_col4(M, st.pool[side] + (size_t)s_src[row] * D, D, c);
+                ((double*)smraw)[(size_t)row * (D + 2) + c] = y;
+                const int e = fx_top(y);
+                if (e != kFxNoExp) atomicMax(&s_top[row], e - s_ea[row] + 56);
+            }
+            __syncthreads();
+            emax = max(emax, s_top[r]);
+        }
+        fx_put<D, H>(V, s_eb + h * H, emax, low, 56 - emax - s_ea[r], (double*)smraw, r, h);
         if (r < n && h == 0) {
             const int* se = st.pool_e[side] + s_src[r];
-            st.pool_e[side][s_dst[r]] = *se + (emax < -(1 << 28) || emax >= kFxNotFinite ? 0 : emax - 56 + s_ea[r]);
+            st.pool_e[side][s_dst[r]] = *se + (emax < -(1 << 28) ? 0 : emax - 56 + s_ea[r]);
         }
         __syncthreads();
         fx_store<D>((const double*)smraw, n, [&](int row) { return st.pool[side] + (size_t)s_dst[row] * D; });
@@ -463,9 +568,16 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
     __shared__ uint32_t tmem_slot;
     __shared__ __align__(8) uint64_t mb_mma, mb_b;
     __shared__ int64_t s_src[kFxRows];
-    __shared__ int s_eb[D], s_cm[D], s_ea[kFxRows], s_es[kFxRows], s_bad[kFxRows];
+    __shared__ __align__(8) int s_x[fx_exp_stride(D)];
+    __shared__ int s_ea[kFxRows], s_es[kFxRows], s_bad[kFxRows];
     constexpr int SP = fx_split(D), H = D / SP;
-    __shared__ int s_max[SP][kFxRows];
+    __shared__ int s_max[SP][kFxRows], s_top[kFxRows];
+    __shared__ uint64_t s_big[kFxRows], s_nz[kFxRows];
+    __shared__ uint64_t s_low[kFxRows];
+    int* const s_cm = s_x;
+    int* const s_eb = s_x + D;
+    const uint64_t* const s_mb = (const uint64_t*)(s_x + 2 * D);
+    const uint64_t* const s_mz = s_mb + D;
     __shared__ int t_e[kGtMaxDeg];                    // edges with a vertex source, then the e_0 ones
     constexpr uint32_t kA = kFxRows * D * 2, kB = 2 * D * D;
     constexpr uint32_t kCols = kFxSums * D <= 128 ? 128 : kFxSums * D <= 256 ? 256 : 512;
@@ -505,7 +617,7 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
         int X[H];
         #pragma unroll
         for (int c = 0; c < H; ++c) { acc[c] = 0; X[c] = kFxNoExp; }
-        bool bad = false;
+        uint32_t low = 0;                             // results to be redone in FP64, all edges
         for (int k = 0; k < nv; ++k) {
             const int64_t mat = (int64_t)t_e[k] * 4 + g;
             if (tid < kFxRows) {                      // rows past n repeat the first
@@ -520,10 +632,10 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
                     tc::mbar_expect_tx(&mb_b, kFxDigits * kB);
                     tc::bulk_g2s(Bs, img + (size_t)mat * kFxDigits * kB, kFxDigits * kB, &mb_b);
                 }
-                if (tid < 2 * D) (tid < D ? s_cm : s_eb - D)[tid] = __ldg(exps + (size_t)mat * 2 * D + tid);
+                for (int q = tid; q < fx_exp_stride(D); q += kFxRows * SP) s_x[q] = __ldg(exps + (size_t)mat * fx_exp_stride(D) + q);
             }
             __syncthreads();
-            fx_rows<D, SP>(a.pool, s_src, s_cm, s_ea, s_bad, smraw);
+            fx_rows<D, SP>(a.pool, s_src, s_cm, s_ea, s_bad, s_big, s_nz, smraw);
             tc::fence_proxy_async();
             tc::fence_before_sync();
             __syncthreads();
@@ -541,7 +653,8 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
             __syncthreads();
             tc::fence_after_sync();
             const int ex = s_ea[r] + s_es[r];
-            bad |= s_bad[r] != 0;
+            const uint64_t mb = s_big[r], mz = s_nz[r];
+            if (s_bad[r]) low = H < 32 ? (1u << (H & 31)) - 1u : ~0u;
             #pragma unroll
             for (int c0 = 0; c0 < H; c0 += 8) {
                 uint32_t w[kFxSums][8];
@@ -552,9 +665,10 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
                 for (int c = 0; c < 8; ++c) {
                     const uint32_t x8[kFxSums] = {w[0][c], w[1][c], w[2][c], w[3][c], w[4][c], w[5][c], w[6][c], w[7][c]};
                     const int64_t v = fx_join<D>(x8, drop);
-                    const int eb = s_eb[h * H + c0 + c];
-                    bad |= eb == kFxNotFinite;
-                    if (v != 0) {
+                    const int col = h * H + c0 + c, eb = s_eb[col];
+                    if (!(s_mb[col] & mb) && ((fx_below(v, 56 - kFxTerm - drop) && (s_mz[col] & mz)) || eb == kFxNotFinite)) {
+                        low |= 1u << (c0 + c);
+                    } else if (v != 0) {
                         const int x = ex + eb;
                         int64_t& A = acc[c0 + c];
                         int& XA = X[c0 + c];
@@ -571,8 +685,8 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
             #pragma unroll
             for (int c = 0; c < H; ++c) {
                 const double m = __ldg(col + c);
-                if (fx_not_finite(m)) bad = true;
                 const int x = fx_exp(m);
+                if (fx_not_finite(m) || (x == kFxNoExp && fx_nonzero(m))) low |= 1u << c;
                 int64_t v = (int64_t)fx_code(m, -x) - 0x80808080808080ll;             // unit 2^-55
                 v = drop ? fx_shift(v, drop - 1) : v * 2;
                 if (v != 0) {
@@ -581,19 +695,49 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
                 }
             }
         }
-        int emax = bad ? kFxNotFinite : -(1 << 29);
+        int emax = -(1 << 29);
         #pragma unroll
         for (int c = 0; c < H; ++c)
-            if (acc[c] != 0) emax = max(emax, 64 - __clzll(acc[c] < 0 ? -acc[c] : acc[c]) + X[c]);
+            if (acc[c] != 0 && !((low >> c) & 1u)) emax = max(emax, 64 - __clzll(acc[c] < 0 ? -acc[c] : acc[c]) + X[c]);
+        if (r >= n) low = 0;
         s_max[h][r] = emax;
-        __syncthreads();                              // the parts of each row meet
+        fx_mark<H>(s_low, r, h, low);
+        const bool redo = __syncthreads_or(low != 0);         // the parts of each row meet
         #pragma unroll
         for (int k = 0; k < SP; ++k) emax = max(emax, s_max[k][r]);
+        if (redo) {
+            if (tid < kFxRows) s_top[tid] = -(1 << 29);
+            __syncthreads();
+            for (int q = warp; q < n * ((D + 31) / 32); q += kFxRows * SP / 32) {
+                const int row = q / ((D + 31) / 32), c = (q - row * ((D + 31) / 32)) * 32 + lane;
+                if (c >= D) continue;
+                if (!((s_low[row] >> c) & 1u)) continue;
+                const uint32_t* it = a.items + at + i0 + row;
+                int er = nv < deg ? 0 : -(1 << 30);   // an e_0 source has power 0
+                for (int k = 0; k < nv; ++k) er = max(er, a.pool_e[__ldg(it + (size_t)(k + 1) * nl)]);
+                double y = 0.0;
+                for (int k = 0; k < deg; ++k) {
+                    const double* M = a.an.AT + ((size_t)t_e[k] * 4 + g) * D * D;
+                    if (k < nv) {
+                        const uint32_t sr = __ldg(it + (size_t)(k + 1) * nl);
+                        y += scale_pow2(dot_col4(M, a.pool + (size_t)sr * D, D, c), a.pool_e[sr] - er);
+                    } else {
+                        y += scale_pow2(__ldg(M + c), -er);
+                    }
+                }
+                ((double*)smraw)[(size_t)row * (D + 2) + c] = y;
+                s_es[row] = er;                       // (the same from every result of the row)
+                const int e = fx_top(y);
+                if (e != kFxNoExp) atomicMax(&s_top[row], e + er + 56 - drop);
+            }
+            __syncthreads();
+            emax = max(emax, s_top[r]);
+        }
         const uint32_t out = __ldg(a.items + at + i0 + (r < n ? r : 0));
-        fx_put<D, H>(acc, X, emax, emax >= kFxNotFinite, (double*)smraw, r, h);
+        fx_put<D, H>(acc, X, emax, low, low ? s_es[r] + 56 - drop - emax : 0, (double*)smraw, r, h);
         if (h == 0) {
             s_src[r] = out;                           // the result rows (the sources are done with)
-            if (r < n) a.pool_e[out] = emax < -(1 << 28) || emax >= kFxNotFinite ? 0 : emax - 56 + drop;
+            if (r < n) a.pool_e[out] = emax < -(1 << 28) ? 0 : emax - 56 + drop;
         }
         __syncthreads();
         fx_store<D>((const double*)smraw, n, [&](int row) { return a.pool + (size_t)s_src[row] * D; });
@@ -819,6 +963,9 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
     __shared__ int s_pex[kFxRows], s_sig[kFxRows], s_ea[kFxRows], s_bad[kFxRows];
     __shared__ uint32_t s_flag[kFxRows], s_node[kFxRows];
     __shared__ int s_cm[KP], s_eb[128];
+    __shared__ uint64_t s_mb[128], s_mz[128];         // the operand rows' masks, the cells' below
+    __shared__ uint64_t s_big[kFxRows], s_nz[kFxRows];
+    __shared__ unsigned short s_low[3][2][kFxRows];   // entries to be redone in FP64, per chunk and half
     __shared__ short s_pos[128];                      // candidate entry n at s DP + component
     constexpr uint32_t kA = kFxRows * KP * 2, kB = 32 * KP * 2;
     constexpr uint32_t kCols = kFxSums * 32;
@@ -836,7 +983,12 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
     if (tid == 0) { tc::mbar_init(&mb_mma, 1); tc::mbar_init(&mb_b, 1); }
     for (int q = tid; q < 4 * D; q += 256) rv[q] = __ldg(an.rv + (size_t)t * 4 * D + q);
     for (int q = tid; q < D; q += 256) { eta[q] = __ldg(an.reta + (size_t)t * D + q); rw[q] = __ldg(an.rw + (size_t)t * D + q); }
-    for (int q = tid; q < KP + 128; q += 256) (q < KP ? s_cm : s_eb - KP)[q] = __ldg(exps + (size_t)t * (KP + 128) + q);
+    {
+        const int* x = exps + (size_t)t * fx_rnn_exp_stride(KP);
+        for (int q = tid; q < KP + 128; q += 256) (q < KP ? s_cm : s_eb - KP)[q] = __ldg(x + q);
+        const uint64_t* m = (const uint64_t*)(x + KP + 128);
+        (tid < 128 ? s_mb : s_mz - 128)[tid] = __ldg(m + tid);
+    }
     for (int q = tid; q < 4 * D; q += 256) s_pos[q] = (short)((q / D) * DP + q % D);
     const double rc = __ldg(an.rc + t);
     tc::fence_before_sync();
@@ -916,8 +1068,16 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
             for (int u = 0; u < TASKS; ++u) {
                 const int ea = s_ea[rows[u]];
                 uint64_t c[8];
+                uint32_t mb = 0, mz = 0;
                 #pragma unroll
-                for (int k = 0; k < 8; ++k) c[k] = fx_code(v[u][k], s_cm[8 * pcs[u] + k] - ea);
+                for (int k = 0; k < 8; ++k) {
+                    const int off = s_cm[8 * pcs[u] + k] - ea;
+                    c[k] = fx_code(v[u][k], off);
+                    mb |= (fx_is_big(fx_exp(v[u][k]) + off) ? 1u : 0u) << k;
+                    mz |= (fx_nonzero(v[u][k]) ? 1u : 0u) << k;
+                }
+                ((unsigned char*)(s_big + rows[u]))[pcs[u]] = (unsigned char)mb;
+                ((unsigned char*)(s_nz + rows[u]))[pcs[u]] = (unsigned char)mz;
                 const uint32_t off = tc::op_offset(rows[u], 8 * pcs[u], KP);
                 #pragma unroll
                 for (int i = 0; i < kFxDigits; ++i) {
@@ -930,6 +1090,8 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
         }
         const int ea = s_ea[r];
         const bool row_bad = s_bad[r] != 0;
+        uint64_t mb = 0, mz = 0;
+        bool any_low = false;
         for (int ch = 0; ch < nch; ++ch) {
             tc::fence_proxy_async();
             tc::fence_before_sync();
@@ -945,6 +1107,8 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
             ph_mma ^= 1u;
             __syncthreads();
             tc::fence_after_sync();
+            if (ch == 0) { mb = s_big[r]; mz = s_nz[r]; }
+            uint32_t low = 0;
             #pragma unroll
             for (int c0 = 0; c0 < 16; c0 += 8) {
                 const int col = 32 * ch + 16 * h + c0;
@@ -960,14 +1124,30 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
                     const int64_t v = fx_join<KP>(x, 0);
                     const int eb = s_eb[col + c];
                     double y = fx_double(v, ea + eb - 56, 0);
+                    if (!(s_mb[col + c] & mb) &&
+                        ((fx_below(v, 56 - kFxTerm) && (s_mz[col + c] & mz)) || eb == kFxNotFinite))
+                        low |= 1u << (c0 + c);
                     if (!fold) y += rv[col + c];
-                    cand[(size_t)r * 4 * DP + s_pos[col + c]] =
-                        row_bad || eb == kFxNotFinite ? __longlong_as_double(0x7FF8000000000000ll) : y;
+                    cand[(size_t)r * 4 * DP + s_pos[col + c]] = y;
                 }
             }
+            if (row_bad) low = 0xFFFFu;
+            s_low[ch][h][r] = (unsigned short)low;
+            any_low |= low != 0;
         }
         tc::fence_before_sync();
-        __syncthreads();
+        if (__syncthreads_or(any_low && r < n)) {
+            for (int q = warp; q < n * nch; q += 8) {
+                const int row = q / nch, e = (q - row * nch) * 32 + lane;
+                if (e >= 4 * D) continue;
+                if (!((s_low[e >> 5][(e >> 4) & 1][row] >> (e & 15)) & 1u)) continue;
+                const int sg = e / D, c = e - sg * D;
+                const double* M = an.AT + ((size_t)t * 4 + sg) * D * D;
+                const double* x = s_src[row];
+                cand[(size_t)row * 4 * DP + s_pos[e]] = rv[e] + (x ? dot_col4(M, x, D, c) : __ldg(M + c));
+            }
+            __syncthreads();
+        }
         for (int q = tid; q < n * 4; q += 256) {
             const double* x = cand + (size_t)q * DP;
             double p = 0.0;
@@ -998,8 +1178,10 @@ __global__ void __launch_bounds__(256) k_fx_rnn_images(const double* __restrict_
     const int t = blockIdx.x, nch = (4 * D + 31) / 32;
     const double* M = A + (size_t)t * 4 * D * D;
     const double* vt = v + (size_t)t * 4 * D;
+    int* const x = exps + (size_t)t * fx_rnn_exp_stride(KP);
+    uint64_t* const masks = (uint64_t*)(x + KP + 128);
     fx_image([&](int n, int k) { return k < D ? __ldg(M + (size_t)n * D + k) : __ldg(vt + n); }, 4 * D, D < KP ? D + 1 : D, 32, KP,
-             img + (size_t)t * nch * kFxDigits * 64 * KP, exps + (size_t)t * (KP + 128), exps + (size_t)t * (KP + 128) + KP, sc, sr);
+             img + (size_t)t * nch * kFxDigits * 64 * KP, x, x + KP, masks, masks + 128, sc, sr);
 }
 
 size_t fx_rnn_smem(int D)

@@ -15,8 +15,10 @@ inline bool fx_fits(int D) { return D % 16 == 0 && D >= 16 && D <= kFxMaxD; }
 // Digit images of a chain's site matrices: per (side, site, local state) -- side
 // 0: y = M x, side 1: y = x^T M -- kFxDigits FP16 matrices of D x D (K-major
 // core matrices, most significant first), and the powers of two of its columns,
-// then of its rows ([2][D]; kFxNotFinite: the row holds an infinity or a NaN).
+// then of its rows ([2][D]; kFxNotFinite: the row holds an infinity or a NaN), then
+// a mask per row of its large and of its nonzero entries ([2][D] words of 64 bits).
 constexpr int kFxNotFinite = 1 << 28;
+__host__ __device__ constexpr int fx_exp_stride(int D) { return 6 * D; }
 // sides = 1: side 0 alone (a graph's edges).
 inline size_t fx_image_bytes(int n_mats, int D, int sides) { return (size_t)sides * n_mats * kFxDigits * 2 * D * D; }
 int launch_fx_images(const double* A, int n_mats, int D, int sides, unsigned char* img, int* exps, cudaStream_t st);
@@ -28,6 +30,7 @@ struct FxStep {
     int K;
     int mat[2];                           // matrix block (side * K + site) * 4 of each side
     const unsigned char* img; const int* exps;
+    const double* at[2];                  // the FP64 matrices, by side: AT (y_c = sum_k x_k at[k][c]), A
     double* pool[2]; int* pool_e[2];      // by side: rows of D, their exponents
     // items of a group: (src, dst) rows ...
     const uint2* items;
@@ -53,7 +56,8 @@ inline size_t fx_rnn_image_bytes(int K, int D)
 {
     return (size_t)K * ((4 * D + 31) / 32) * kFxDigits * 64 * (D <= 16 ? 16 : 32);
 }
-inline size_t fx_rnn_exps(int K, int D) { return (size_t)K * ((D <= 16 ? 16 : 32) + 128); }
+__host__ __device__ constexpr int fx_rnn_exp_stride(int KP) { return KP + 128 + 2 * 2 * 128; }
+inline size_t fx_rnn_exps(int K, int D) { return (size_t)K * fx_rnn_exp_stride(D <= 16 ? 16 : 32); }
 int launch_fx_rnn_images(const double* A, const double* v, int K, int D, unsigned char* img, int* exps, cudaStream_t st);
 int launch_fx_rnn(const TreeRnn& a, const unsigned char* img, const int* exps, DevError* err, int t, const TreeLevels& lv,
                   const int64_t* bounds, int n_sm, cudaStream_t st);

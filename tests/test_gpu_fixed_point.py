@@ -62,9 +62,10 @@ def _assert_energy(e, ref):
     assert np.all(np.abs(e - ref["e_loc"]) <= 1e-12 * scale)
 
 
-def _assert_log_psi(ctx, s, dets):
-    """K (D + 1) 2^-53 of the running absolute product: the bound of an FP64 chain."""
-    ctx.set_system(s)
+def _assert_log_psi(ctx, s, dets, run=None):
+    """K (D + 1) 2^-53 of the running absolute product: the bound of an FP64 chain.
+    ``run``: the system handed to the library, where it is not the reference's."""
+    ctx.set_system(s if run is None else run)
     la, sg = ctx.amplitude(dets)
     ref, rs, cond = _log_psi_ref(s, dets)
     tol = s.K * (s.D + 1) * U * cond + 8 * U * np.abs(ref)
@@ -113,3 +114,108 @@ def test_empty_columns(ctx, D, graph):
     _assert_energy(_energy(ctx, s), ref)
     if not graph:
         _assert_energy(_energy(ctx, s, nqs.NQS_PREC_FP64_SHARED), ref)
+
+
+def _graded(rng, s, kind):
+    """Tensors whose states spread over many powers of two in a way that no scaling of
+    columns and rows takes out: the first cell falls by 2^-4 per component ("steps")
+    or the second half of the components by 2^-6 per site ("blocks"), the matrices in
+    between keep the components apart, and the last one weighs them all alike."""
+    E, D, K = s.n_edges, s.D, s.K
+    idx = s.pred_idx if s.pred_idx is not None else np.arange(-1, K - 1)
+    ptr = s.pred_ptr if s.pred_ptr is not None else np.arange(K + 1)
+    r = lambda *n: rng.uniform(0.5, 1.5, size=n) * rng.choice([-1.0, 1.0], size=n)  # noqa: E731
+    T = np.zeros((E, 4, D, D))
+    k = np.arange(D)
+    for e in range(E):
+        if kind == "steps":
+            T[e][:, k, k] = r(4, D)
+            if idx[e] < 0:
+                T[e][:, :, 0] = r(4, D) * np.exp2(-4.0 * k)
+        else:
+            h = D // 2
+            T[e][:, :h, :h] = rng.normal(size=(4, h, h)) / np.sqrt(h)
+            T[e][:, h:, h:] = rng.normal(size=(4, D - h, D - h)) / np.sqrt(D - h) * 2.0 ** -6
+            if idx[e] < 0:
+                T[e][:, :, 0] = r(4, D)
+    for e in range(ptr[K - 1], ptr[K]):          # every source's components count alike in psi
+        T[e][:, 0, :] = r(4, D) * (np.exp2(4.0 * k) if kind == "steps" else np.where(k < D // 2, 1.0, 2.0 ** (6 * K)))
+    return dataclasses.replace(s, tensors=np.ascontiguousarray(T))
+
+
+@pytest.mark.parametrize("D", [16, 32, 48, 64])
+@pytest.mark.parametrize("graph", [False, True])
+@pytest.mark.parametrize("kind", ["steps", "blocks"])
+def test_graded_states(ctx, D, graph, kind):
+    """Components far below their row's largest that a later site brings up again."""
+    rng = np.random.default_rng(D)
+    if graph:
+        s = _dag(D, 8, D, n_samples=150, eps=0.01, n_draws=20)
+    else:
+        s = W.tiny_system(K=8, na=4, nb=4, D=D, n_hidden=3, seed=D, n_samples=ROWS + 101, eps=0.01, n_draws=20)
+    s = _graded(rng, s, kind)
+    if not graph:
+        _assert_log_psi(ctx, dataclasses.replace(s, rbm_W=None, rbm_b=None), s.samples)
+        s = s.subset(np.arange(200))
+    ref = O.local_energy(O.Problem(s), cond=True)
+    _assert_energy(_energy(ctx, s), ref)
+    if not graph:
+        _assert_energy(_energy(ctx, s, nqs.NQS_PREC_FP64_SHARED), ref)
+
+
+@pytest.mark.parametrize("D", [5, 10, 16, 20, 24])
+@pytest.mark.parametrize("v", [0.0, 1e-3, 1.0])
+def test_graded_cells(ctx, D, v):
+    """The same for the normalised readout: cells that fall by 2^-4 per component, whose
+    weights and phases count every component alike; v of one local state alone."""
+    rng = np.random.default_rng(100 + D)
+    s = W.tiny_system(K=8, na=4, nb=4, D=D, n_hidden=2, seed=D, eps=0.01, n_draws=20, n_samples=200)
+    r = lambda *n: rng.uniform(0.5, 1.5, size=n) * rng.choice([-1.0, 1.0], size=n)  # noqa: E731
+    k = np.arange(D)
+    T = np.zeros((s.K, 4, D, D))
+    T[:, :, k, k] = r(s.K, 4, D)
+    T[0, :, :, 0] = r(4, D) * np.exp2(-4.0 * k)
+    vv = np.zeros((s.K, 4, D))
+    vv[:, 2] = v * r(s.K, D)
+    rnn = (vv, np.abs(r(s.K, D)) * np.exp2(8.0 * k), r(s.K, D) * np.exp2(4.0 * k), np.zeros(s.K))
+    s = dataclasses.replace(s, tensors=T, rnn=rnn)
+    ref = O.local_energy(O.Problem(s))
+    e = _energy(ctx, s)
+    assert np.all(np.abs(e - ref["e_loc"]) <= 1e-12 * np.maximum(np.abs(ref["e_loc"]), ref["e_abs"]))
+
+
+@pytest.mark.parametrize("D", [16, 64])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_not_finite_steps(ctx, D, bad):
+    """A NaN or an infinity in a site tensor reaches every amplitude whose local state
+    reads it, and none whose does not; the last site's unread rows reach none."""
+    s = W.tiny_system(K=8, na=4, nb=4, D=D, seed=1, n_samples=ROWS + 101)
+    occ = ((s.samples[:, None, :] >> np.arange(s.K, dtype=np.uint64)[None, :, None]) & np.uint64(1)).astype(int)
+    T = s.tensors.copy()
+    T[5, 3, 2, 7] = bad
+    ctx.set_system(dataclasses.replace(s, tensors=T))
+    la, _ = ctx.amplitude(s.samples)
+    hit = occ[:, 5].sum(1) == 2
+    assert not np.any(np.isfinite(la[hit])) and np.all(np.isfinite(la[~hit]))
+    T = s.tensors.copy()
+    T[-1, :, 1:, :] = bad
+    _assert_log_psi(ctx, s, s.samples, dataclasses.replace(s, tensors=T))
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_not_finite_levels(ctx, graph):
+    """The same for the levels of the prefix trees: an energy is NaN where the oracle's
+    is. Samples without the bad local state themselves; vertex 4, which the last one
+    reads in the graph too."""
+    s = W.tiny_system(K=8, na=4, nb=4, D=16, seed=2, n_samples=3000) if not graph else _dag(3, 8, 16, n_samples=3000)
+    occ = ((s.samples[:, None, :] >> np.arange(s.K, dtype=np.uint64)[None, :, None]) & np.uint64(1)).astype(int)
+    s = s.subset(np.flatnonzero(occ[:, 4].sum(1) < 2)[:300])
+    e = s.pred_ptr[4] if graph else 4
+    T = s.tensors.copy()
+    T[e, 3, 2, 0] = np.nan                         # (column 0: read from e_0 too)
+    s = dataclasses.replace(s, tensors=T, eps=0.3)
+    ref = O.local_energy(O.Problem(s))["e_loc"]
+    got = _energy(ctx, s)
+    assert np.isnan(ref).any() and np.array_equal(np.isnan(got), np.isnan(ref))
+    ok = ~np.isnan(ref)
+    assert np.all(np.abs(got - ref)[ok] <= 1e-9 * np.abs(ref[ok]).max(initial=1.0))
