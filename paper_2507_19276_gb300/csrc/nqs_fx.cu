@@ -767,7 +767,8 @@ void fx_graph_launch(const TreeGraph64& a, const unsigned char* img, const int* 
 // Outer-product sums of the gradient, sum_n (w_n g_n) h_n^T over a chunk of one
 // local-state group (k_grad_tn's blocks), with the samples as the reduction:
 // 64 samples at a time, the operands' rows (components) scaled by powers of two
-// over those samples, the exact sums converted once and added in FP64. A
+// over those samples, the exact sums converted once and added in FP64; entries without a
+// term near the scale (one sample's weight may set it) are redone as above. A
 // 64-sample product of 64 x 64 takes 150 k cycles of the FP64 pipe (1.95 ms for
 // H50, D = 64, 4096 samples).
 // ---------------------------------------------------------------------------
@@ -784,6 +785,10 @@ __global__ void __launch_bounds__(256) k_fx_grad(GradArgs a, int chunk_samples, 
     __shared__ const double* s_h[kGradRed];
     __shared__ double s_w[kGradRed];
     __shared__ int s_e[2 * D], s_bad[2 * D];
+    __shared__ uint64_t s_big[2 * D], s_nz[2 * D];    // per component, masks of samples
+    __shared__ int s_nlow;                            // entries to be redone in FP64: list, results
+    unsigned short* const s_low = (unsigned short*)(smraw + 8 * D * D);
+    double* const redone = (double*)smraw;            // [D][D] (both where the operands were)
     constexpr uint32_t kB = 2 * D * kGradRed;         // one digit of one operand
     constexpr uint32_t kCols = kFxSums * D <= 128 ? 128 : kFxSums * D <= 256 ? 256 : 512;
     constexpr int H = D / 2;
@@ -844,6 +849,7 @@ __global__ void __launch_bounds__(256) k_fx_grad(GradArgs a, int chunk_samples, 
             s_w[tid] = w;
         }
         if (tid < 2 * D) { s_e[tid] = kFxNoExp; s_bad[tid] = 0; }
+        if (tid == 0) s_nlow = 0;
         __syncthreads();
         // component c of operand o (0: w g, 1: h) over eight samples per task, the
         // components across the lanes
@@ -875,8 +881,15 @@ __global__ void __launch_bounds__(256) k_fx_grad(GradArgs a, int chunk_samples, 
             const int q = tid + 256 * u, c = q % (2 * D), n8 = q / (2 * D);
             const int ex = s_e[c] == kFxNoExp ? 0 : s_e[c];
             uint64_t cd[8];
+            uint32_t mb = 0, mz = 0;
             #pragma unroll
-            for (int k = 0; k < 8; ++k) cd[k] = fx_code(v[u][k], -ex);
+            for (int k = 0; k < 8; ++k) {
+                cd[k] = fx_code(v[u][k], -ex);
+                mb |= (fx_is_big(fx_exp(v[u][k]) - ex) ? 1u : 0u) << k;
+                mz |= (fx_nonzero(v[u][k]) ? 1u : 0u) << k;
+            }
+            ((unsigned char*)(s_big + c))[n8] = (unsigned char)mb;
+            ((unsigned char*)(s_nz + c))[n8] = (unsigned char)mz;
             unsigned char* op = smraw + (c < D ? 0u : kFxDigits * kB);
             const uint32_t off = tc::op_offset(c < D ? c : c - D, 8 * n8, kGradRed);
             #pragma unroll
@@ -901,9 +914,11 @@ __global__ void __launch_bounds__(256) k_fx_grad(GradArgs a, int chunk_samples, 
         ph ^= 1u;
         __syncthreads();
         tc::fence_after_sync();
+        uint32_t low = 0;
         if (act) {
             const int ea = r < D ? s_e[r] : 0;
             const bool bad = r < D && s_bad[r];
+            const uint64_t mb = s_big[r < D ? r : 0], mz = s_nz[r < D ? r : 0];
             #pragma unroll
             for (int q0 = 0; q0 < H; q0 += 8) {
                 uint32_t w[kFxSums][8];
@@ -914,14 +929,41 @@ __global__ void __launch_bounds__(256) k_fx_grad(GradArgs a, int chunk_samples, 
                 for (int c = 0; c < 8; ++c) {
                     const uint32_t x[kFxSums] = {w[0][c], w[1][c], w[2][c], w[3][c], w[4][c], w[5][c], w[6][c], w[7][c]};
                     const int col = D + h * H + q0 + c;
-                    double y = fx_double(fx_join<kGradRed>(x, 0), ea + s_e[col] - 56, 0);
-                    if (bad | s_bad[col]) y = __longlong_as_double(0x7FF8000000000000ll);
+                    const int64_t V = fx_join<kGradRed>(x, 0);
+                    double y = fx_double(V, ea + s_e[col] - 56, 0);
+                    if ((!(s_big[col] & mb) && fx_below(V, 56 - kFxTerm) && (s_nz[col] & mz)) || bad || s_bad[col]) {
+                        low |= 1u << (q0 + c);
+                        y = 0.0;
+                    }
                     acc[q0 + c] += y;
                 }
+            }
+            if (r >= D) low = 0;
+            if (low) {
+                int at = atomicAdd(&s_nlow, __popc(low));
+                for (uint32_t m = low; m; m &= m - 1) s_low[at++] = (unsigned short)(r * D + h * H + __ffs((int)m) - 1);
             }
         }
         tc::fence_before_sync();
         __syncthreads();                              // operands, accumulators and lists are free
+        if (s_nlow) {
+            const int nl = s_nlow;
+            for (int k = tid; k < nl; k += 256) {
+                const int q = s_low[k], row = q / D, c = q - row * D;
+                double y = 0.0;
+                #pragma unroll 4
+                for (int n = 0; n < nk; ++n)
+                    y = fma(s_w[n] * s_g[n][row], s_h[n] ? s_h[n][c] : (c == 0 ? 1.0 : 0.0), y);
+                redone[q] = y;
+            }
+            __syncthreads();
+            if (act && r < D) {
+                #pragma unroll
+                for (int c = 0; c < H; ++c)
+                    if ((low >> c) & 1u) acc[c] += redone[(size_t)r * D + h * H + c];
+            }
+            __syncthreads();
+        }
     }
     if (act && r < D) {
         double* out = a.part + (((size_t)chunk * a.an.n_edges + e) * 4 + sg) * D * D + (size_t)r * D + h * H;

@@ -219,3 +219,97 @@ def test_not_finite_levels(ctx, graph):
     assert np.isnan(ref).any() and np.array_equal(np.isnan(got), np.isnan(ref))
     ok = ~np.isnan(ref)
     assert np.all(np.abs(got - ref)[ok] <= 1e-9 * np.abs(ref[ok]).max(initial=1.0))
+
+
+GRAD = _const("kFxGradMin")           # samples from which the gradient takes the fixed-point products
+CHUNK = _const("kGradChunk")          # samples per block, in products of kGradRed
+RED = _const("kGradRed")
+
+
+def _grad_ref(s, u):
+    """sum_n u_n d log|psi_TN(n)| / d M_e^s in float64 over any graph, and 2 K (D + 1)
+    2^-53 times the same sum of magnitudes (of the products of absolute values, times
+    the conditioning of psi(n)): the rounding of FP64 recursions, both ways."""
+    E, K, D = s.n_edges, s.K, s.D
+    idx = s.pred_idx if s.pred_idx is not None else np.arange(-1, K - 1)
+    ptr = s.pred_ptr if s.pred_ptr is not None else np.arange(K + 1)
+    occ = ((s.samples[:, None, :] >> np.arange(K, dtype=np.uint64)[None, :, None]) & np.uint64(1)).astype(int)
+    sig = occ[:, :, 0] + 2 * occ[:, :, 1]
+    n = len(sig)
+    e0 = np.eye(1, D)[0][None, :].repeat(n, 0)
+    vert = np.repeat(np.arange(K), np.diff(ptr))
+    out = []
+    for T in (s.tensors, np.abs(s.tensors)):
+        M = [T[e][sig[:, vert[e]]] for e in range(E)]
+        h = {-1: e0}
+        for i in range(K):
+            h[i] = sum(np.einsum("nab,nb->na", M[e], h[idx[e]]) for e in range(ptr[i], ptr[i + 1]))
+        g = {i: np.zeros((n, D)) for i in range(-1, K)}
+        g[K - 1] = e0
+        for i in range(K - 1, -1, -1):
+            for e in range(ptr[i], ptr[i + 1]):
+                g[idx[e]] = g[idx[e]] + np.einsum("nab,na->nb", M[e], g[i])
+        out.append((h, g, h[K - 1][:, 0]))
+    (h, g, psi), (ha, ga, psia) = out
+    ref, mag = np.zeros(s.tensors.shape), np.zeros(s.tensors.shape)
+    w = u / psi
+    wa = np.abs(w) * (1.0 + psia / np.abs(psi))
+    for e in range(E):
+        for q in range(4):
+            k = sig[:, vert[e]] == q
+            ref[e, q] = (w[k, None] * g[vert[e]][k]).T @ h[idx[e]][k]
+            mag[e, q] = (wa[k, None] * ga[vert[e]][k]).T @ ha[idx[e]][k]
+    return ref, 2 * K * (D + 1) * U * mag
+
+
+@pytest.mark.parametrize("D", [16, 32, 48, 64])
+@pytest.mark.parametrize("graph", [False, True])
+@pytest.mark.parametrize("n", [GRAD - 1, GRAD, GRAD + 1, CHUNK - 1, CHUNK + 1, 4 * RED + 1, 4 * CHUNK + 3])
+def test_outer_products(ctx, D, graph, n):
+    """Groups around a product's samples and a block's, weights over 2^40."""
+    s = W.tiny_system(K=7, na=3, nb=4, D=D, seed=n, n_samples=n) if not graph else _dag(n, 7, D, n_hidden=0, n_samples=n)
+    rng = np.random.default_rng(D + n)
+    n = len(s.samples)
+    u = rng.normal(size=n) * np.exp2(rng.uniform(-20, 20, size=n))
+    ctx.set_system(s)
+    got = ctx.grad_log_psi_vjp(s.samples, u)[0]
+    ref, tol = _grad_ref(s, u)
+    assert np.all(np.abs(got - ref) <= tol)
+
+
+@pytest.mark.parametrize("D", [16, 64])
+def test_outer_products_of_sectors(ctx, D):
+    """States of two sectors of components, the samples of one with weights 2^45 times
+    the other's: the entries that only the light samples reach keep their digits."""
+    s = W.tiny_system(K=7, na=3, nb=4, D=D, seed=5, n_samples=600)
+    rng = np.random.default_rng(D)
+    h = D // 2
+    T = np.zeros_like(s.tensors)
+    T[:, :, :h, :h] = rng.normal(size=(s.K, 4, h, h)) / np.sqrt(h)
+    T[:, :, h:, h:] = rng.normal(size=(s.K, 4, D - h, D - h)) / np.sqrt(D - h)
+    T[0] = 0.0
+    T[0, 0::2, :h, 0] = rng.normal(size=(2, h))          # local states 0, 2: the first sector
+    T[0, 1::2, h:, 0] = rng.normal(size=(2, D - h))
+    T[-1, :, 0, :] = rng.normal(size=(4, D))
+    s = dataclasses.replace(s, tensors=T)
+    light = (s.samples[:, 0] & np.uint64(1)) == 1
+    u = rng.normal(size=len(light)) * np.where(light, 1.0, 2.0 ** 45)
+    ctx.set_system(s)
+    got = ctx.grad_log_psi_vjp(s.samples, u)[0]
+    ref, tol = _grad_ref(s, u)
+    assert np.all(np.abs(got - ref) <= tol)
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_outer_products_not_finite(ctx, bad):
+    """A weight that is not finite reaches the gradients of its sample's local states."""
+    s = W.tiny_system(K=7, na=3, nb=4, D=16, seed=5, n_samples=600)
+    u = np.random.default_rng(1).normal(size=600)
+    u[77] = bad
+    ctx.set_system(s)
+    got = ctx.grad_log_psi_vjp(s.samples, u)[0]
+    occ = ((s.samples[77] >> np.arange(s.K, dtype=np.uint64)[:, None]) & np.uint64(1)).astype(int)
+    hit = np.zeros((s.K, 4), bool)
+    hit[np.arange(s.K), occ[:, 0] + 2 * occ[:, 1]] = True
+    finite = np.isfinite(got)
+    assert np.all(finite[~hit]) and not np.any(finite[1:-1][hit[1:-1]])
