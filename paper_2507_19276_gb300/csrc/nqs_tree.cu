@@ -886,7 +886,9 @@ __global__ void k_corr_ab(const double* __restrict__ theta, int64_t n, double2* 
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const double e = exp(-2.0 * fabs(theta[i])), big = 1.0 / (1.0 + e), small = e * big;
+    // past 340, e^(-2 |theta|) nears the denormal numbers and the smaller factor loses its
+    // bits: NaN sends the sample's rows to the logarithms
+    const double x = fabs(theta[i]), e = x > 340.0 ? NAN : exp(-2.0 * x), big = 1.0 / (1.0 + e), small = e * big;
     ab[i] = theta[i] >= 0.0 ? make_double2(big, small) : make_double2(small, big);
 }
 

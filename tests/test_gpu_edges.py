@@ -358,3 +358,30 @@ def test_graph_tiles_beyond_the_ring(ctx, D):
             assert np.array_equal(p, e[i:i + 40])
     finally:
         ctx.set_precision(nqs.NQS_PREC_FP64)
+
+
+@pytest.mark.parametrize("graph", [False, True])
+@pytest.mark.parametrize("kind", ["theta"])
+def test_correlator_ratio_of_large_weights(ctx, graph, kind):
+    """2cosh ratios whose factors are far apart but whose product is not: an angle past
+    the range of e^(-2 theta), and products that pass through the denormal numbers and
+    come back (units 0, 8, 16, .. belong to one lane); the FP64 bar."""
+    import dataclasses
+    from oracle import oracle as O
+    s = W.tiny_system(K=6, na=3, nb=3, D=4, seed=8, graph=graph, n_samples=120)
+    nh = 2 if kind == "theta" else 41
+    Wc, b = np.zeros((nh, 2 * s.K)), np.zeros(nh)
+    # (occupied, empty) angles of orbital 0 alpha per unit: the factors' logarithms add to zero
+    units = {0: (380.0, -20.0), 1: (20.0, 380.0)} if kind == "theta" else \
+        {0: (330.0, -20.0), 8: (330.0, -20.0), 16: (120.0, -5.0),
+         24: (20.0, 330.0), 32: (20.0, 330.0), 40: (5.0, 120.0)}
+    for k, (occ, emp) in units.items():
+        b[k], Wc[k, 0] = emp, occ - emp
+    Wc += 0.1 * np.random.default_rng(1).normal(size=Wc.shape) * (np.arange(2 * s.K) > 1)
+    s = dataclasses.replace(s, rbm_W=Wc, rbm_b=b)
+    ctx.set_system(s)
+    ctx.set_precision(nqs.NQS_PREC_FP64)
+    ref = O.local_energy(O.Problem(s), cond=True)
+    e, _ = ctx.local_energy(s.samples, s.counts, s.eps, s.n_draws, s.seed)
+    scale = np.maximum(np.abs(ref["e_loc"]), ref["e_abs"]) + (2.0 ** -52 / 1e-12) * ref["e_cond"]
+    assert np.all(np.abs(e - ref["e_loc"]) <= 1e-12 * scale)
