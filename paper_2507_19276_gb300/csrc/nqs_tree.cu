@@ -762,8 +762,10 @@ constexpr int kRowLanes = 8;
 // Rows of the FP64 form: eight lanes per row dot the live states of the row's
 // node with the closing covectors and take the correlator ratio as a product
 // (9 FP64 operations per hidden unit; log 2cosh of every unit and row was ~80
-// and 40% of the H18 time). A ratio outside the normal range is redone as a sum
-// of logarithms, as the cos forms are.
+// and 40% of the H18 time). A row one of whose lanes leaves 2^-125 .. 2^125 on the
+// way is redone as a sum of logarithms, as the cos forms are: the eight lanes' product
+// then stays a normal number whatever the order, where one that passed through the
+// denormal numbers would come back with few bits.
 __global__ void __launch_bounds__(256) k_tree_rows64(TreeRows64 a)
 {
     __shared__ int64_t s_s;
@@ -788,6 +790,7 @@ __global__ void __launch_bounds__(256) k_tree_rows64(TreeRows64 a)
     for (int rr = threadIdx.x >> 3; rr < kTreeRows; rr += 32) {      // whole warps: the shuffles need them
         const bool on = rr < nr;
         double tn = 0.0, ratio = 1.0;
+        uint32_t top = 0x3FF00000u, bottom = 0x3FF00000u;            // of the running products' high words
         int er = 0;
         TreeWord w{};
         if (on) {
@@ -828,6 +831,9 @@ __global__ void __launch_bounds__(256) k_tree_rows64(TreeRows64 a)
                         e.y *= f.y;
                     }
                     ratio *= fma(h.x, e.x, h.y * e.y);
+                    const uint32_t hw = (uint32_t)__double2hiint(ratio);      // (not negative; or a NaN)
+                    top = max(top, hw);
+                    bottom = min(bottom, hw);
                 }
             }
         }
@@ -835,9 +841,11 @@ __global__ void __launch_bounds__(256) k_tree_rows64(TreeRows64 a)
             tn += __shfl_xor_sync(kFull, tn, o);
             ratio *= __shfl_xor_sync(kFull, ratio, o);
         }
+        const bool wide = top >= (1023u + 125u) << 20 || bottom < (1023u - 125u) << 20;
+        const unsigned wides = __ballot_sync(kFull, wide) >> (lane & 24) & 255u;
         if (on && l8 == 0) {
             const int p = w.x[0] / 3;
-            const bool by_log = NH > 0 && (!a.expd || !(ratio > 1e-290 && ratio < 1e290));
+            const bool by_log = NH > 0 && (!a.expd || wides);
             const double coef = tree_coef(t, s, r0 + rr);
             s_term[rr] = coef * scale_pow2(tn / mant, er - pex) * (by_log ? 1.0 : ratio);
             s_span[rr] = a.chain ? w.x[w.c - 1] / 3 - p + 1 : K - p;

@@ -361,7 +361,7 @@ def test_graph_tiles_beyond_the_ring(ctx, D):
 
 
 @pytest.mark.parametrize("graph", [False, True])
-@pytest.mark.parametrize("kind", ["theta"])
+@pytest.mark.parametrize("kind", ["theta", "path"])
 def test_correlator_ratio_of_large_weights(ctx, graph, kind):
     """2cosh ratios whose factors are far apart but whose product is not: an angle past
     the range of e^(-2 theta), and products that pass through the denormal numbers and
