@@ -283,7 +283,16 @@ __device__ __forceinline__ void tree_rnn_pick(const TreeRnn& a, int t, int it, i
     for (int c = 0; c < an.D; ++c) ph = fma(rw[c], h[c], ph);
     if (!rnn_allowed(an, t, nad, nbd, sg) || !(P > 0.0) || !(Z > 0.0)) f |= 1u << 17;
     else {
-        prod *= P / Z;
+        const double q = P / Z;
+        if (__double2hiint(q) >= 0x20B00000) {        // 2^-500 and above: the product stays normal
+            prod *= q;
+        } else {
+            int ep, ez;
+            const double m = frexp(P, &ep) / frexp(Z, &ez);
+            const int k = (ez - ep) / 500;
+            prod *= ldexp(m, ep - ez + 500 * k);
+            pex -= k;
+        }
         if (prod < 0x1p-500) { prod *= 0x1p500; --pex; }
         f ^= ph < 0.0 ? 1u << 16 : 0u;
     }

@@ -385,3 +385,32 @@ def test_correlator_ratio_of_large_weights(ctx, graph, kind):
     e, _ = ctx.local_energy(s.samples, s.counts, s.eps, s.n_draws, s.seed)
     scale = np.maximum(np.abs(ref["e_loc"]), ref["e_abs"]) + (2.0 ** -52 / 1e-12) * ref["e_cond"]
     assert np.all(np.abs(e - ref["e_loc"]) <= 1e-12 * scale)
+
+
+@pytest.mark.parametrize("D", [4, 28])
+def test_normalised_chain_tiny_conditionals(ctx, D):
+    """Conditionals of 1e-240 at two vertices (every local state is allowed there) whose
+    orbitals couple to no other, so that every m shares them with n: their product
+    leaves the range of a double, the ratio does not."""
+    import dataclasses
+    from oracle import oracle as O
+    s = W.with_readout(W.tiny_system(K=8, na=4, nb=4, D=D, seed=6), seed=4, v_std=1.0)
+    T, (v, eta, w, c) = s.tensors.copy(), s.rnn
+    v = v.copy()
+    for q in (1, 3):
+        T[q, 3] *= 1e-120
+        v[q, 3] = 0.0
+    h, L = s.h1e.copy(), s.chol.copy()
+    alone = np.ones((s.K, s.K), bool)
+    alone[[1, 3]], alone[:, [1, 3]] = False, False
+    alone |= np.eye(s.K, dtype=bool)
+    both = np.uint64((1 << 1) | (1 << 3))
+    s = dataclasses.replace(s, tensors=T, rnn=(v, eta, w, c), h1e=h * alone, chol=L * alone, eps=1e-9)
+    s = s.subset(np.flatnonzero(np.all((s.samples & both) == both, axis=1)))
+    ctx.set_system(s)
+    ctx.set_precision(nqs.NQS_PREC_FP64)
+    ref = O.local_energy(O.Problem(s))
+    first = (s.samples & np.uint64(1)).sum(1)          # one electron on orbital 0: m may change there
+    assert np.all(ref["n_det"] > 0) and np.any(first == 1) and np.all(ref["e_abs"] < 1e6)
+    e, _ = ctx.local_energy(s.samples, s.counts, s.eps, 0, 1)
+    assert np.all(np.abs(e - ref["e_loc"]) <= 1e-12 * np.maximum(np.abs(ref["e_loc"]), ref["e_abs"]))
