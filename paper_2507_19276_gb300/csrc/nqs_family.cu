@@ -1781,27 +1781,51 @@ __global__ void __launch_bounds__(kFamRows, MB) k_fam_rows(FamArgs<T> f, RowSet 
             if (NH > 0) {
                 typedef typename Vec4<T>::type V4;
                 if constexpr (dbl) {
-                    // FP64 runs at two operations per clock and SM: the product itself
-                    // (two operations per unit, pairs of units dealt over the lanes)
-                    // instead of the product minus one (three) -- its rounding,
-                    // ~sqrt(N_h) 2^-53, is that of the dot product
-                    double P = 1.0;
+                    // FP64 runs at two operations per clock and SM: two per unit, pairs of
+                    // units dealt over the lanes, on X = the product of (1 + t u) minus one,
+                    // X + t u (1 + X) = fma(fma(X, t, t), u, X): near 1 it rounds far less
+                    // than the product itself would. Where X falls below -3/4 on the way it
+                    // keeps too few bits of a small product: the group takes that instead.
+                    const double2* l2 = (const double2*)ltq;
+                    const double2* r2 = (const double2*)rsq;
+                    double X = 0.0;
+                    uint32_t low = 0;                        // largest high word: X negative and large
+                    auto follow = [&]() { low = max(low, (uint32_t)__double2hiint(X)); };
+                    // the last pair holds PL - 1 and PR - 1 (then zeros): t and u of 1 each
+                    auto factors = [&](int k2, double2& t, double2& u) {
+                        t = l2[k2];
+                        u = r2[k2];
+                        if (k2 == NP / 2) { t.y = u.x; u = make_double2(1.0, 1.0); }
+                    };
                     if (live) {
-                        const double2* l2 = (const double2*)ltq;
-                        const double2* r2 = (const double2*)rsq;
                         for (int k2 = sub; k2 <= NP / 2; k2 += 8) {
-                            const double2 t = l2[k2], u = r2[k2];
-                            if (k2 == NP / 2) {          // PL - 1 and PR - 1 (then a zero)
-                                P = fma(P, t.x, P);
-                                P = fma(P, u.x, P);
-                            } else {
+                            double2 t, u;
+                            factors(k2, t, u);
+                            X = fma(fma(X, t.x, t.x), u.x, X);
+                            follow();
+                            X = fma(fma(X, t.y, t.y), u.y, X);
+                            follow();
+                        }
+                    }
+                    for (int o = 4; o; o >>= 1) {
+                        const double Y = __shfl_xor_sync(kFull, X, o);
+                        X = fma(X, Y, X + Y);
+                        follow();
+                    }
+                    const unsigned lost = __ballot_sync(kFull, low > 0xBFE80000u) >> (lane & 24) & 255u;   // X < -3/4
+                    if (__any_sync(kFull, lost)) {
+                        double P = 1.0;
+                        if (live)
+                            for (int k2 = sub; k2 <= NP / 2; k2 += 8) {
+                                double2 t, u;
+                                factors(k2, t, u);
                                 P = fma(P, t.x * u.x, P);
                                 P = fma(P, t.y * u.y, P);
                             }
-                        }
+                        for (int o = 4; o; o >>= 1) P *= __shfl_xor_sync(kFull, P, o);
+                        if (lost) { ratio *= P; X = 0.0; }
                     }
-                    for (int o = 4; o; o >>= 1) P *= __shfl_xor_sync(kFull, P, o);
-                    if (live) ratio *= P;
+                    if (live) ratio = fma(ratio, X, ratio);
                 } else {
                     T X = T(0);                        // product of (1 + x_k) minus 1
                     if (live) {

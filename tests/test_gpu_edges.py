@@ -414,3 +414,41 @@ def test_normalised_chain_tiny_conditionals(ctx, D):
     assert np.all(ref["n_det"] > 0) and np.any(first == 1) and np.all(ref["e_abs"] < 1e6)
     e, _ = ctx.local_energy(s.samples, s.counts, s.eps, 0, 1)
     assert np.all(np.abs(e - ref["e_loc"]) <= 1e-12 * np.maximum(np.abs(ref["e_loc"]), ref["e_abs"]))
+
+
+@pytest.mark.parametrize("kind", ["many weak units", "units that cancel"])
+def test_shared_correlator_product(ctx, kind):
+    """The product over hidden units in the shared FP64 form, alone: a chain of ones, one
+    electron, one-body elements between pairs of orbitals, so E_loc = H f(m)/f(n) of one m.
+    Weak units: each of the factors 1 + x_k and of the two outer products counts with four
+    roundings of its x, the rest with four (the two products, the sum, the outer ones).
+    Units that cancel: products of 2^-60 and 2^60 whose value is 1, 16 roundings per unit."""
+    import dataclasses
+    K, rng = 16, np.random.default_rng(5)
+    nh = 512 if kind == "many weak units" else 60
+    s = W.tiny_system(K=K, na=1, nb=0, D=1, n_hidden=nh, seed=3)
+    if kind == "many weak units":
+        Wc, b = 1e-3 * rng.normal(size=(nh, 2 * K)), 1e-3 * rng.normal(size=nh)
+    else:
+        Wc, b = 0.9 + 1e-3 * rng.normal(size=(nh, 2 * K)), -0.9 + 1e-3 * rng.normal(size=nh)
+    h = np.zeros((K, K))
+    h[np.arange(0, K, 2), np.arange(1, K, 2)] = h[np.arange(1, K, 2), np.arange(0, K, 2)] = rng.normal(size=K // 2)
+    s = dataclasses.replace(s, tensors=np.ones_like(s.tensors), rbm_W=Wc, rbm_b=b, h1e=h, chol=np.zeros_like(s.chol))
+    ctx.set_system(s)
+    ctx.set_precision(nqs.NQS_PREC_FP64_SHARED)
+    try:
+        e, _ = ctx.local_energy(s.samples, s.counts, 1e-9, 0, 1)
+    finally:
+        ctx.set_precision(nqs.NQS_PREC_FP64)
+    off, _, dets, H, _ = ctx.connected(s.samples, 1e-9)
+    assert np.array_equal(np.diff(off), np.ones(K))
+
+    def theta(d):
+        bits = (d[:, None, :] >> np.arange(K, dtype=np.uint64)[None, :, None]) & np.uint64(1)
+        return b.astype(np.longdouble) + bits.reshape(len(d), 2 * K).astype(np.longdouble) @ Wc.T.astype(np.longdouble)
+    tn, tm = theta(s.samples), theta(dets)
+    ref = H * np.exp(np.sum(np.log(np.cosh(tm)) - np.log(np.cosh(tn)), axis=1))
+    x = np.maximum(np.abs(tn), np.abs(tm)) + 2 * np.abs(Wc).max()
+    units = 4 * (1 + np.sum(x * x, axis=1).max()) if kind == "many weak units" else 16 * (1 + nh)
+    assert kind != "many weak units" or units < 5
+    assert np.all(np.abs(e - ref) <= float(units) * 2.0 ** -53 * np.abs(ref))
