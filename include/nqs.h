@@ -65,8 +65,9 @@ typedef enum {
                                  tree (rows with the same first changes share their
                                  steps; linear readouts close with n's adjoint
                                  covectors after the last change; the tensor term
-                                 runs row by row). Levels with many nodes take their
-                                 matrix products in fixed point on the tensor cores:
+                                 runs row by row). Where D is 16, 32, 48 or 64 (the
+                                 normalised readout of a chain: up to 24), the matrix
+                                 products run in fixed point on the tensor cores:
                                  56 bits of the product's scale, at most D 2^-47 of
                                  its largest term (FP64: D 2^-53 of the sum of the
                                  terms' magnitudes); a result whose terms may all be
@@ -87,7 +88,8 @@ typedef enum {
                                  and the 2cosh or cos correlator (otherwise
                                  NQS_ERR_UNSUPPORTED with the reason) */
     NQS_PREC_FP64_SHARED = 2  /* the shared-prefix evaluation with FP64
-                                 contractions (chain ansatz only) */
+                                 contractions (chain ansatz only; in fixed point
+                                 where NQS_PREC_FP64's are) */
 } nqs_precision;
 
 typedef struct nqs_ctx nqs_ctx;
@@ -132,8 +134,9 @@ typedef struct {
     int tile_blocks_per_sm;   /* shared-prefix forms: blocks per multiprocessor of
                              each site-step tile launch (0: the default, 4; at most
                              32). A schedule parameter: results do not depend on it */
-    int table_mb;         /* shared-prefix forms: cap (MiB) on the tables of one
-                             sample batch (0: the default, 32 GiB); never more
+    int table_mb;         /* shared-prefix forms and prefix trees: cap (MiB) on the
+                             tables of one sample batch (0: the default, 32 GiB,
+                             of trees 16 GiB); never more
                              than a third of the free device memory. Larger
                              batches mean fewer, fuller launches; results do not
                              depend on it */
@@ -300,7 +303,10 @@ int nqs_connected(nqs_ctx* ctx, const uint64_t* samples, int64_t Ns, double det_
                   int64_t capacity);
 
 /* log|psi| and sign of psi for n determinants (full K-site product, FP64
- * whatever the precision option). sign is 0 where psi = 0. */
+ * whatever the precision option). sign is 0 where psi = 0. Chains whose D is 16,
+ * 32, 48 or 64 take the fixed-point products of NQS_PREC_FP64 from 1100
+ * determinants per call on, so the last bits may differ between a large call and
+ * small ones. */
 int nqs_amplitude(nqs_ctx* ctx, const uint64_t* dets, int64_t n, double* log_abs,
                   int8_t* sign);
 
@@ -397,7 +403,9 @@ int nqs_local_energy_batch(nqs_ctx* const* ctxs, int n_sys, nqs_batch_item* item
  *  FP64. The site-tensor part is, per edge and local state, the sum over the
  *  samples of that local state of u_n / psi_TN(n) g_i(n) h_j(n)^T (adjoint
  *  times forward cell); nqs_options.grad_chunk bounds how many samples'
- *  environments are held at once. */
+ *  environments are held at once (the sums then round in another order, and a
+ *  width of 16, 32, 48 or 64 takes fixed-point products from 64 samples of a chunk
+ *  on, a chain's environments from 1100). */
 int nqs_grad_log_psi_vjp(nqs_ctx* ctx, const uint64_t* samples, const double* u, int64_t Ns,
                          double* grad_sites, double* grad_W, double* grad_b);
 

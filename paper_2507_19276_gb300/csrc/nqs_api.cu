@@ -31,13 +31,6 @@ constexpr int kDefaultAudit = 4;
 // 4.62
 constexpr int64_t kFxMinRows = 1100;
 
-// nodes of a level from which the prefix trees' FP64 steps take 128-node
-// fixed-point tiles instead of 32-node FP64 ones. All levels in fixed point / none,
-// H18 graph (D = 32): 2 samples 1.28 / 1.45 ms, 10 samples 1.55 / 2.38, 100 samples
-// 4.45 / 12.2; normalised readout (D = 10): 2 samples 3.44 / 3.76, 50 samples 15.5 /
-// 26.7. A level of a few tiles is latency either way, so those stay in FP64
-constexpr int64_t kFxMinNodes = 1024;
-
 struct DevBuf {
     void* p = nullptr;
     size_t n = 0;
@@ -398,8 +391,10 @@ int rnn_env_pass(nqs_ctx* c, const uint64_t* samples, int64_t Ns)
 
 // tn: 1 = psi(n) and the environments; 2 = psi(n) only (chain, shared-prefix
 // path: its FP64 value is the denominator of every ratio of the sample);
-// 0 = no tensor-network part (the normalised readout has its own pass)
-int env_pass(nqs_ctx* c, const uint64_t* samples, int64_t Ns, bool adjoints, int tn = 1)
+// 0 = no tensor-network part (the normalised readout has its own pass). by_site:
+// large batches of a chain may go site by site (not for energies: a sample's bits
+// do not depend on the batch it comes in)
+int env_pass(nqs_ctx* c, const uint64_t* samples, int64_t Ns, bool adjoints, int tn, bool by_site)
 {
     const int K = c->K, D = c->av.D, NH = c->av.n_hidden;
     EnvArgs e{};
@@ -440,7 +435,7 @@ int env_pass(nqs_ctx* c, const uint64_t* samples, int64_t Ns, bool adjoints, int
     e.psi_mant = (double*)c->pmant.p;
     e.psi_exp = (int*)c->pexp.p;
     e.h_diag = (double*)c->hdiag.p;
-    const bool fx = tn == 1 && c->av.chain && c->has_fx && Ns >= kFxMinRows;
+    const bool fx = by_site && tn == 1 && c->av.chain && c->has_fx && Ns >= kFxMinRows;
     if (fx) {
         // both sweeps of all samples site by site on the tensor cores: step i takes
         // the left states through site i and the right ones through site K - 1 - i
@@ -1070,8 +1065,11 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
             g.an.pred_idx = (const int*)c->pred_idx.p;
             g.items = a.items;
             for (int t = 0; t < K; ++t) {
-                // 128-node tensor-core tiles once a level fills the SMs with them
-                if (c->has_fx && (int64_t)lv.n[t] >= kFxMinNodes)
+                // by the width alone, whatever the level holds: a sample's bits do not
+                // depend on the batch it comes in. Levels of a few tiles are latency either
+                // way (fixed point / FP64 below 1024 nodes: H18 2 samples 1.29 / 1.26 ms,
+                // K = 8, D = 16, 100 samples 0.44 / 0.43, readout of H50, 2 samples 3.62 / 3.49)
+                if (c->has_fx)
                     LAUNCH(stage, launch_fx_graph(g, (const unsigned char*)c->fx_img.p, (const int*)c->fx_exps.p,
                                                   (DevError*)c->derr.p, t, c->deg_h[(size_t)t], lv, bounds.data(), c->n_sm,
                                                   c->stream));
@@ -1166,7 +1164,7 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
             rn.n_nodes = (uint32_t)nodes;
             rn.cells = (const double*)c->rnn_cells.p;
             for (int t = 0; t < K; ++t) {
-                if (c->has_fx_rnn && (int64_t)lv.n[t] >= kFxMinNodes)
+                if (c->has_fx_rnn)
                     LAUNCH(stage, launch_fx_rnn(rn, (const unsigned char*)c->fx_rimg.p, (const int*)c->fx_rexps.p,
                                                 (DevError*)c->derr.p, t, lv, bounds.data(), c->n_sm, c->stream));
                 else LAUNCH(stage, launch_tree_rnn(rn, t, lv, bounds.data(), c->n_sm, c->stream));
@@ -1888,7 +1886,7 @@ int le_core(nqs_ctx* c, const uint64_t* ds, const double* dc, int64_t Ns, uint64
         StageScope sc(c, NQS_STAGE_ENV);
         LAUNCH(NQS_STAGE_ENV, launch_validate(ds, Ns, c->K, c->na, c->nb, (DevError*)c->derr.p, c->stream));
         // the mixed form takes psi(n) in double-FP32 arithmetic, the FP64 forms in FP64
-        TRY(env_pass(c, ds, Ns, tree64, rnn ? 0 : (shared ? (prec == NQS_PREC_MIXED ? 3 : 2) : 1)));
+        TRY(env_pass(c, ds, Ns, tree64, rnn ? 0 : (shared ? (prec == NQS_PREC_MIXED ? 3 : 2) : 1), false));
         if (rnn) TRY(rnn_env_pass(c, ds, Ns));
         k_check_psi<<<(unsigned)((Ns + 255) / 256), 256, 0, c->stream>>>((const double*)c->pmant.p, Ns,
                                                                        (DevError*)c->derr.p);
@@ -2212,7 +2210,7 @@ int vjp_core(nqs_ctx* c, const uint64_t* ds, const double* du, int64_t Ns, doubl
         const uint64_t* cs = ds + 2 * s0;
         TRY(reset_dev_error(c));
         LAUNCH(NQS_STAGE_OTHER, launch_validate(cs, n, c->K, c->na, c->nb, (DevError*)c->derr.p, c->stream));
-        TRY(env_pass(c, cs, n, true, c->av.readout == 1 ? 0 : 1));
+        TRY(env_pass(c, cs, n, true, c->av.readout == 1 ? 0 : 1, true));
         if (c->av.readout == 1) TRY(rnn_env_pass(c, cs, n));
         k_check_psi<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>((const double*)c->pmant.p, n,
                                                                       (DevError*)c->derr.p, s0);

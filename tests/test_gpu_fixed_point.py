@@ -313,3 +313,28 @@ def test_outer_products_not_finite(ctx, bad):
     hit[np.arange(s.K), occ[:, 0] + 2 * occ[:, 1]] = True
     finite = np.isfinite(got)
     assert np.all(finite[~hit]) and not np.any(finite[1:-1][hit[1:-1]])
+
+
+@pytest.mark.parametrize("kind,D", [("chain", 16), ("chain", 64), ("graph", 32), ("readout", 10), ("readout", 20)])
+def test_energies_do_not_depend_on_the_split(ctx, kind, D):
+    """A sample's plain-form energy has the same bits in a large batch, in small calls and
+    under a table cap that cuts the batch (the levels' node counts differ a hundredfold)."""
+    n = ROWS + 101
+    if kind == "graph":
+        s = _dag(D, 8, D, n_samples=n, eps=0.02, n_draws=10)
+    else:
+        s = W.tiny_system(K=8, na=4, nb=4, D=D, n_hidden=3, seed=D, n_samples=n, eps=0.02, n_draws=10)
+    if kind == "readout":
+        s = W.with_readout(s, seed=3)
+    ctx.set_system(s)
+
+    def run(lo, hi, **options):
+        ctx.set_precision(nqs.NQS_PREC_FP64, sample_index_base=lo, **options)
+        return ctx.local_energy(s.samples[lo:hi], s.counts[lo:hi], s.eps, s.n_draws, s.seed)[0].view(np.uint64)
+    try:
+        e = run(0, n)
+        for lo, hi in [(0, 1), (3, 40), (500, 900), (n - 130, n)]:
+            assert np.array_equal(run(lo, hi), e[lo:hi])
+        assert np.array_equal(run(0, n, table_mb=1), e)
+    finally:
+        ctx.set_precision(nqs.NQS_PREC_FP64)
