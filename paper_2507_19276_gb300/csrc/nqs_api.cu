@@ -850,6 +850,14 @@ struct Carve {
 
 enum TreeKind { kTreeGraph64, kTreeGraphTc, kTreeRnn };
 
+constexpr int kRetry = -1;                // tree_pass: the batch was cut
+#define FIT(expr)                      \
+    do {                               \
+        int r_ = (expr);               \
+        if (r_ == kRetry) goto retry;  \
+        if (r_ != NQS_OK) return r_;   \
+    } while (0)
+
 // Amplitudes of the deterministic and drawn rows over the prefix trees of
 // sample batches: partial sums per kTreeRows-row chunk of a sample's rows
 // (deterministic, then drawn) into part_det, chunk bases in base_det.
@@ -928,6 +936,18 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
         if (parts > 1) s1 = s0 + std::max<int64_t>(1, std::min(s1 - s0, (Ns - s0 + parts - 1) / parts));
     retry:
         const int nb = (int)(s1 - s0);
+        // another context may have taken the memory since it was asked for: a batch
+        // that does not fit gives its buffers back and is halved, and so are those after it
+        auto fit = [&](DevBuf& b, size_t bytes) {
+            const int r = ensure(c, b, bytes);
+            if (r != NQS_ERR_OOM || nb == 1) return r;
+            for (DevBuf* q : {&c->tr_build, &c->tr_items, &c->tr_pool, &c->tr_close}) release(*q);
+            c->err[0] = 0;
+            s1 = s0 + (nb + 1) / 2;
+            budget = 0;
+            for (int64_t s = s0; s < s1; ++s) budget += bytes_of(c->det_off_h[s + 1] - c->det_off_h[s] + n_draws);
+            return kRetry;
+        };
         const int64_t R = c->det_off_h[s1] - c->det_off_h[s0] + (int64_t)nb * n_draws;
         const int64_t max_chunks = R / kTreeRows + nb;
         TreeArgs a{};
@@ -996,7 +1016,7 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
                 rn.pex = v.take<int>((size_t)2 * nodes);
                 rn.flag = v.take<uint32_t>((size_t)2 * nodes);
             }
-            if (!pass) TRY(ensure(c, c->tr_build, v.n));
+            if (!pass) FIT(fit(c->tr_build, v.n));
         }
         LAUNCH(stage, launch_tree_nodes(a, max_chunks, c->stream));
         LAUNCH(stage, launch_scan_i64(a.pool_tot, pool_off, nb, c->stream));
@@ -1032,7 +1052,7 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
             if (nb > 1) { s1 = s0 + (nb + 1) / 2; goto retry; }
             return set_err(c, NQS_ERR_UNSUPPORTED, "prefix trees of %lld items exceed 2^32", (long long)n_items);
         }
-        TRY(ensure(c, c->tr_items, (size_t)(n_items + 1) * 4));
+        FIT(fit(c->tr_items, (size_t)(n_items + 1) * 4));
         a.items = (uint32_t*)c->tr_items.p;
         a.pool_tot = pool_off;
         LAUNCH(stage, launch_tree_items(a, lv, (const int*)c->pred_ptr.p, (const int*)c->pred_idx.p, c->stream));
@@ -1043,7 +1063,7 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
                 Carve v{pass ? (char*)c->tr_pool.p : nullptr};
                 g.pool = v.take<double>((size_t)rows_total * D);
                 g.pool_e = v.take<int>((size_t)rows_total);
-                if (!pass) TRY(ensure(c, c->tr_pool, v.n));
+                if (!pass) FIT(fit(c->tr_pool, v.n));
             }
             for (int pass = 0; pass < 2; ++pass) {
                 Carve v{pass ? (char*)c->tr_close.p : nullptr};
@@ -1051,7 +1071,7 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
                 q.Qe = v.take<int>((size_t)nb * c->n_live * 3);
                 q.c = v.take<double>((size_t)nb * K * 3);
                 q.ce = v.take<int>((size_t)nb * K * 3);
-                if (!pass) TRY(ensure(c, c->tr_close, v.n));
+                if (!pass) FIT(fit(c->tr_close, v.n));
             }
             // the roots' states h_j(n): a chain keeps L_{j+1} behind L_0 and R_{i+1} as g_i
             const bool chain = c->av.chain != 0;
@@ -1113,7 +1133,7 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
                 Carve v{pass ? (char*)c->tr_pool.p : nullptr};
                 g.pool = v.take<unsigned char>((size_t)rows_total * 4 * D);
                 g.pool_e = v.take<int>((size_t)rows_total);
-                if (!pass) TRY(ensure(c, c->tr_pool, v.n));
+                if (!pass) FIT(fit(c->tr_pool, v.n));
             }
             TRY(ensure(c, c->g_tts, (size_t)nb * (np ? np : 1) * 4));
             LAUNCH(stage, launch_tree_graph_prep((const double*)c->Hst.p, (const int*)c->Hexp.p, (const double*)c->theta.p,

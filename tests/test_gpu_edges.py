@@ -452,3 +452,53 @@ def test_shared_correlator_product(ctx, kind):
     units = 4 * (1 + np.sum(x * x, axis=1).max()) if kind == "many weak units" else 16 * (1 + nh)
     assert kind != "many weak units" or units < 5
     assert np.all(np.abs(e - ref) <= float(units) * 2.0 ** -53 * np.abs(ref))
+
+
+_FAKE_MALLOC = """
+#define _GNU_SOURCE
+#include <dlfcn.h>
+#include <stddef.h>
+#include <stdlib.h>
+int cudaMalloc(void** p, size_t n)
+{
+    static int (*real)(void**, size_t);
+    if (n > strtoull(getenv("FAKE_MALLOC_LIMIT"), NULL, 10)) { *p = NULL; return 2; }
+    if (!real) real = (int (*)(void**, size_t))dlsym(RTLD_NEXT, "cudaMalloc");
+    return real(p, n);
+}
+"""
+
+_FAKE_MALLOC_RUN = """
+import sys
+import numpy as np
+from paper_2507_19276_gb300 import nqs, workloads as W
+kind, out = sys.argv[1:]
+s = W.tiny_system(K=8, na=4, nb=4, D=16, n_hidden=3, seed=4, graph=kind != "readout", n_samples=2500)
+if kind == "readout":
+    s = W.with_readout(s, seed=3)
+c = nqs.Context(0)
+c.set_system(s)
+c.set_precision(nqs.NQS_PREC_MIXED if kind == "mixed" else nqs.NQS_PREC_FP64)
+np.save(out, c.local_energy(s.samples, s.counts, 0.0, 0, 1)[0])
+"""
+
+
+@pytest.mark.parametrize("kind", ["plain", "mixed", "readout"])
+def test_tree_batches_shrink_to_the_memory(tmp_path, kind):
+    """An allocation refused by the runtime (a fake cudaMalloc in a child process: nothing
+    past 64 MiB) cuts the batch of the prefix trees, and the energies keep their bits."""
+    import os
+    import subprocess
+    import sys
+    src, so, root = tmp_path / "fake.c", tmp_path / "fake.so", os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    src.write_text(_FAKE_MALLOC)
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", str(so), str(src), "-ldl"], check=True)
+    got = []
+    for limit in (1 << 60, 64 << 20):
+        out = tmp_path / f"{limit}.npy"
+        env = dict(os.environ, LD_PRELOAD=str(so), FAKE_MALLOC_LIMIT=str(limit))
+        r = subprocess.run([sys.executable, "-c", _FAKE_MALLOC_RUN, kind, str(out)], cwd=root, env=env, capture_output=True,
+                           text=True, timeout=300)
+        assert r.returncode == 0, r.stderr[-2000:]
+        got.append(np.load(out))
+    assert np.array_equal(got[0].view(np.uint64), got[1].view(np.uint64))
