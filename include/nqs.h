@@ -84,7 +84,9 @@ typedef enum {
                                  samples' prefix trees, 128 nodes at a time; needs
                                  D in {16, 32, 64},
                                  in-degree x 4 x D <= 512, at most 16 vertex states
-                                 live at once, the linear readout, no tensor term
+                                 live at once (128 rows of them and the in-edges'
+                                 matrix images within a block's shared memory),
+                                 the linear readout, no tensor term
                                  and the 2cosh or cos correlator (otherwise
                                  NQS_ERR_UNSUPPORTED with the reason) */
     NQS_PREC_FP64_SHARED = 2  /* the shared-prefix evaluation with FP64

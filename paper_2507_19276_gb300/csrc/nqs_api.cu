@@ -1112,7 +1112,7 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
             r.chain = chain ? 1 : 0;
             r.pool = g.pool; r.pool_e = g.pool_e;
             if (NH > 0 && c->av.corr == NQS_CORR_COSH) {
-                TRY(ensure(c, c->corr_ab, (size_t)nb * NH * 16));
+                FIT(fit(c->corr_ab, (size_t)nb * NH * 16));
                 LAUNCH(stage, launch_corr_ab((const double*)c->theta.p + (size_t)s0 * NH, (int64_t)nb * NH,
                                              (double2*)c->corr_ab.p, c->stream));
                 r.expd = (const double2*)c->cexp.p;
@@ -1135,7 +1135,7 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
                 g.pool_e = v.take<int>((size_t)rows_total);
                 if (!pass) FIT(fit(c->tr_pool, v.n));
             }
-            TRY(ensure(c, c->g_tts, (size_t)nb * (np ? np : 1) * 4));
+            FIT(fit(c->g_tts, (size_t)nb * (np ? np : 1) * 4));
             LAUNCH(stage, launch_tree_graph_prep((const double*)c->Hst.p, (const int*)c->Hexp.p, (const double*)c->theta.p,
                                                  s0, nb, K, D, NH, np, c->av.corr, g.pool, g.pool_e, (float*)c->g_tts.p,
                                                  c->stream));

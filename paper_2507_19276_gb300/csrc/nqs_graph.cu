@@ -562,8 +562,10 @@ int launch_tree_rows_tc(const TreeRowsTc& a, int64_t max_chunks, int n_sm, cudaS
     return 1;
 }
 
-// shared memory of a tile that keeps every live state of 128 rows: the bound on
-// the graphs this form accepts
+// Which graphs the mixed form takes is part of the interface. Two of its limits, 16
+// live states and the bytes below (128 rows of every live state beside the matrix
+// images), are those of tiles that kept the states in shared memory; the steps over the
+// prefix trees keep none there and would need only the limit on D x in-degree.
 static size_t graph_tiles_smem(int D, int K, int n_slots, int max_deg, int n_hidden, int nbuf)
 {
     const size_t np = (size_t)((n_hidden + 3) & ~3);
@@ -596,13 +598,13 @@ bool graph_tc_fits(const int* ptr, const int* idx, int K, int D, int n_hidden, c
         busy[s] = i;
     }
     const int n_slots = std::max<int>(1, (int)busy.size());
-    if (n_slots > kGtMaxSlots) { *why = "more live vertex states than the tile's slots"; return false; }
+    if (n_slots > kGtMaxSlots) { *why = "more than 16 vertex states live at once"; return false; }
     int dev = 0, mx = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&mx, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     const size_t margin = 24576;
     if (mx > 0 && graph_tiles_smem(D, K, n_slots, max_deg, n_hidden, 1) + margin > (size_t)mx) {
-        *why = "the tile's states and matrix images exceed the shared memory";
+        *why = "128 rows of the live vertex states and the matrix images exceed a block's shared memory";
         return false;
     }
     return true;
