@@ -67,7 +67,7 @@ __device__ __forceinline__ int fx_exp(double x)
 }
 
 __device__ __forceinline__ bool fx_not_finite(double x) { return (__double2hiint(x) & 0x7FF00000) == 0x7FF00000; }
-__device__ __forceinline__ bool fx_nonzero(double x) { return ((__double2hiint(x) << 1) | __double2loint(x)) != 0; }
+__device__ __forceinline__ bool fx_nonzero(double x) { return ((__double2hiint(x) & 0x7FFFFFFF) | __double2loint(x)) != 0; }
 
 // The unit of a result is 2^-56 of (row scale) x (matrix row scale), so its digits
 // hold it as well as FP64 would only if one of its terms is near that scale: where
@@ -76,8 +76,9 @@ __device__ __forceinline__ bool fx_nonzero(double x) { return ((__double2hiint(x
 // 2^-kFxTerm of the scale is known to be there if entries of at least 2^-(kFxTerm / 2)
 // meet in the state and the matrix row (a bit mask each; for dense rows, also beside a
 // unit diagonal, that holds practically always), or if the result itself reaches
-// 2^-kFxTerm. Any other result with a nonzero term (two more masks) is redone with
-// FP64 FMAs, as are those that an infinity, a NaN or a denormal entry takes part in.
+// 2^-kFxTerm. Any other result is redone with FP64 FMAs, as are those that an
+// infinity or a NaN takes part in. The masks cost two instructions per entry and four
+// per result; what a result without such a term needs is looked at by its thread alone.
 // What stays errs by at most ~D 2^-55 of the scale, that is D 2^-47 of its largest
 // term where FP64 FMAs err by up to D 2^-53 of the sum of the terms. Of the results of
 // I + G / sqrt(D) matrices, kFxTerm = 4 redoes 5% (H50's log|psi| 4.2 -> 18 ms), 6
@@ -95,19 +96,50 @@ __device__ __forceinline__ int fx_top(double y)
     return e;
 }
 
-// a thread's H bits of row r's marks
-template <int H>
-__device__ __forceinline__ void fx_mark(uint64_t* marks, int r, int h, uint32_t low)
-{
-    unsigned char* to = (unsigned char*)(marks + r) + h * (H / 8);
-    #pragma unroll
-    for (int b = 0; b < H / 8; ++b) to[b] = (unsigned char)(low >> (8 * b));
-}
-
-// |v| < 2^bits
+// |v| < 2^bits (bits > 32; -2^bits passes too): the high word alone
 __device__ __forceinline__ bool fx_below(int64_t v, int bits)
 {
-    return (uint64_t)(v + (1ll << bits)) < (2ull << bits);
+    return (uint32_t)(v >> 32) + (1u << (bits - 32)) < 2u << (bits - 32);
+}
+
+// an entry's digits (see fx_code) are those of a large one, |x| >= 2^-(kFxTerm / 2) up to
+// 2^-19 of that: its high word is out of -2^h .. 2^h, h = 55 - kFxTerm / 2 - 32
+__device__ __forceinline__ bool fx_code_big(uint64_t c)
+{
+    constexpr uint32_t kBig = 1u << (55 - kFxTerm / 2 - 32);
+    return (uint32_t)(c >> 32) - 0x808080u + kBig >= 2u * kBig;
+}
+
+// the candidates among a thread's H results (columns h H ..) of a row with the mask mb of
+// large entries: those whose column of masks (s_mb) shares none, or is not finite
+template <int H>
+__device__ __forceinline__ uint32_t fx_low(uint32_t below, bool not_finite, uint64_t mb, const uint64_t* s_mb, const int* s_eb, int h)
+{
+    uint32_t low = 0;
+    // (a warp nearly always has one small result, a thread seldom two: a loop over them)
+    for (uint32_t m = not_finite ? (H < 32 ? (1u << (H & 31)) - 1u : ~0u) : below; m; m &= m - 1) {
+        const int c = __ffs((int)m) - 1;
+        if (!(s_mb[h * H + c] & mb) && (((below >> c) & 1u) || s_eb[h * H + c] == kFxNotFinite)) low |= 1u << c;
+    }
+    return low;
+}
+
+// mask of the nonzero entries of x
+__device__ __forceinline__ uint64_t fx_row_nonzero(const double* x, int D)
+{
+    uint64_t m = 0;
+    for (int k = 0; k < D; ++k) m |= (uint64_t)fx_nonzero(x[k]) << k;
+    return m;
+}
+
+// entry c of M x in FP64 (M by columns, as dot_col4): nz and mz are the masks of the
+// nonzero entries of x and of row c, `whole` where either holds an infinity or a NaN
+__device__ __forceinline__ double fx_dot(const double* M, const double* x, int D, int c, uint64_t nz, uint64_t mz, bool whole)
+{
+    if (!whole && !(nz & mz)) return 0.0;
+    if (whole || (nz & (nz - 1))) return dot_col4(M, x, D, c);
+    const int k = __ffsll((long long)nz) - 1;         // a state of one entry (the first site's e_0)
+    return __ldg(M + (size_t)k * D + c) * x[k];
 }
 
 // digit `i` (0 = least significant) of two codes as FP16
@@ -286,11 +318,11 @@ __device__ __forceinline__ void fx_mma(uint32_t tmem, uint32_t N, uint64_t dA, u
 // The digits of a tile's rows (row r at pool + src[r] * D, times the column powers
 // cm, scaled by 2^-ea[r]) into the operand buffers: eight entries of a row per
 // task, eight rows x four tasks per warp (shared memory in whole core matrices).
-// ea[r] must hold kFxNoExp; contains a block barrier. big and nonzero get each row's
-// masks of entries that are large after the scaling, and not zero (bits below D).
+// ea[r] must hold kFxNoExp; contains a block barrier. big gets each row's mask of the
+// entries that are large after the scaling (bits below D).
 template <int D, int SP>
 __device__ __forceinline__ void fx_rows(const double* __restrict__ pool, const int64_t* src_row, const int* cm, int* ea_row,
-                                        int* bad_row, uint64_t* big, uint64_t* nonzero, unsigned char* A)
+                                        int* bad_row, uint64_t* big, unsigned char* A)
 {
     constexpr int NW = kFxRows * SP / 32;
     constexpr uint32_t kA = kFxRows * D * 2;
@@ -341,16 +373,13 @@ __device__ __forceinline__ void fx_rows(const double* __restrict__ pool, const i
     for (int u = 0; u < TASKS; ++u) {
         const int ea = ea_row[rows[u]];
         uint64_t c[8];
-        uint32_t mb = 0, mz = 0;
+        uint32_t mb = 0;
         #pragma unroll
         for (int k = 0; k < 8; ++k) {
-            const int off = cm[8 * pcs[u] + k] - ea;
-            c[k] = fx_code(v[u][k], off);
-            mb |= (fx_is_big(fx_exp(v[u][k]) + off) ? 1u : 0u) << k;
-            mz |= (fx_nonzero(v[u][k]) ? 1u : 0u) << k;
+            c[k] = fx_code(v[u][k], cm[8 * pcs[u] + k] - ea);
+            mb |= (fx_code_big(c[k]) ? 1u : 0u) << k;
         }
         ((unsigned char*)(big + rows[u]))[pcs[u]] = (unsigned char)mb;
-        ((unsigned char*)(nonzero + rows[u]))[pcs[u]] = (unsigned char)mz;
         const uint32_t off = tc::op_offset(rows[u], 8 * pcs[u], D);
         #pragma unroll
         for (int i = 0; i < kFxDigits; ++i) {
@@ -374,15 +403,13 @@ __global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1) k_fx_s
     __shared__ __align__(8) int s_x[fx_exp_stride(D)];         // the matrix's powers of two and masks
     __shared__ int s_ea[kFxRows];                     // power of two taken out of each scaled row
     constexpr int SP = fx_split(D);                   // threads per row
-    __shared__ int s_max[SP][kFxRows], s_top[kFxRows];
-    __shared__ int s_bad[kFxRows];
-    __shared__ uint64_t s_big[kFxRows], s_nz[kFxRows];
-    __shared__ uint64_t s_low[kFxRows];               // results to be redone in FP64
+    __shared__ int s_max[SP][kFxRows];
+    __shared__ int s_bad[kFxRows], s_inf;             // rows, and the matrix, with an infinity or a NaN
+    __shared__ uint64_t s_big[kFxRows];
     int* const s_cm = s_x;
     int* const s_eb = s_x + D;
     const uint64_t* const s_mb = (const uint64_t*)(s_x + 2 * D);
     const uint64_t* const s_mz = s_mb + D;
-    constexpr int NW = kFxRows * SP / 32;             // warps
     constexpr int H = D / SP;                         // columns per thread in the epilogue
     constexpr uint32_t kA = kFxRows * D * 2;          // one digit of the rows
     constexpr uint32_t kB = 2 * D * D;                // one digit of the matrix
@@ -450,9 +477,15 @@ __global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1) k_fx_s
                 tc::bulk_g2s(Bs, st.img + mat * kFxDigits * kB, kFxDigits * kB, &mb_b);
             }
             for (int q = tid; q < fx_exp_stride(D); q += kFxRows * SP) s_x[q] = __ldg(st.exps + mat * fx_exp_stride(D) + q);
+            if (warp == 0) {
+                bool inf = false;
+                for (int q = lane; q < D; q += 32) inf |= __ldg(st.exps + mat * fx_exp_stride(D) + D + q) == kFxNotFinite;
+                inf = __any_sync(kFull, inf);
+                if (lane == 0) s_inf = inf;
+            }
         }
         __syncthreads();
-        fx_rows<D, SP>(st.pool[side], s_src, s_cm, s_ea, s_bad, s_big, s_nz, smraw);
+        fx_rows<D, SP>(st.pool[side], s_src, s_cm, s_ea, s_bad, s_big, smraw);
         tc::fence_proxy_async();
         tc::fence_before_sync();
         __syncthreads();
@@ -485,8 +518,7 @@ __global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1) k_fx_s
         // join the sums: V = y 2^(56 - ea - eb), and the row's largest exponent
         int64_t V[H];
         int emax = -(1 << 29);
-        uint32_t low = 0;
-        const uint64_t mb = s_big[r], mz = s_nz[r];
+        uint32_t below = 0;
         #pragma unroll
         for (int c0 = 0; c0 < H; c0 += 8) {
             uint32_t w[kFxSums][8];
@@ -498,36 +530,34 @@ __global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1) k_fx_s
                 const uint32_t x[kFxSums] = {w[0][c], w[1][c], w[2][c], w[3][c], w[4][c], w[5][c], w[6][c], w[7][c]};
                 const int64_t v = fx_join<D>(x, 0);
                 V[c0 + c] = v;
-                const int col = h * H + c0 + c, eb = s_eb[col];
-                if (!(s_mb[col] & mb) && ((fx_below(v, 56 - kFxTerm) && (s_mz[col] & mz)) || eb == kFxNotFinite))
-                    low |= 1u << (c0 + c);
-                else if (v != 0) emax = max(emax, 64 - __clzll(v < 0 ? -v : v) + eb);
+                if (v != 0) emax = max(emax, 64 - __clzll(v < 0 ? -v : v) + s_eb[h * H + c0 + c]);
+                below |= (fx_below(v, 56 - kFxTerm) ? 1u : 0u) << (c0 + c);
             }
         }
-        if (s_bad[r]) { low = H < 32 ? (1u << (H & 31)) - 1u : ~0u; emax = -(1 << 29); }
+        uint32_t low = fx_low<H>(below, s_inf != 0, s_big[r], s_mb, s_eb, h);
+        if (s_bad[r]) low = H < 32 ? (1u << (H & 31)) - 1u : ~0u;
         if (r >= n) low = 0;
+        if (low) {                                    // the others' largest, and these in FP64
+            emax = -(1 << 29);
+            #pragma unroll
+            for (int c = 0; c < H; ++c)
+                if (V[c] != 0 && !((low >> c) & 1u)) emax = max(emax, 64 - __clzll(V[c] < 0 ? -V[c] : V[c]) + s_eb[h * H + c]);
+            const double* M = st.at[side] + (mat - (size_t)side * 4 * st.K) * D * D;
+            const double* x = st.pool[side] + (size_t)s_src[r] * D;
+            const uint64_t nz = fx_row_nonzero(x, D);
+            for (uint32_t m = low; m; m &= m - 1) {
+                const int c = h * H + __ffs((int)m) - 1;
+                const double y = fx_dot(M, x, D, c, nz, s_mz[c], s_bad[r] || s_eb[c] == kFxNotFinite);
+                ((double*)smraw)[(size_t)r * (D + 2) + c] = y;
+                const int e = fx_top(y);
+                if (e != kFxNoExp) emax = max(emax, e - s_ea[r] + 56);
+            }
+        }
         s_max[h][r] = emax;
-        fx_mark<H>(s_low, r, h, low);
         tc::fence_before_sync();
-        const bool redo = __syncthreads_or(low != 0);         // the parts of each row meet
+        __syncthreads();                              // the parts of each row meet
         #pragma unroll
         for (int k = 0; k < SP; ++k) emax = max(emax, s_max[k][r]);
-        if (redo) {
-            if (tid < kFxRows) s_top[tid] = -(1 << 29);
-            __syncthreads();
-            const double* M = st.at[side] + (mat - (size_t)side * 4 * st.K) * D * D;
-            for (int q = warp; q < n * ((D + 31) / 32); q += NW) {     // a warp per row and 32 results
-                const int row = q / ((D + 31) / 32), c = (q - row * ((D + 31) / 32)) * 32 + lane;
-                if (c >= D) continue;
-                if (!((s_low[row] >> c) & 1u)) continue;
-                const double y = dot_col4(M, st.pool[side] + (size_t)s_src[row] * D, D, c);
-                ((double*)smraw)[(size_t)row * (D + 2) + c] = y;
-                const int e = fx_top(y);
-                if (e != kFxNoExp) atomicMax(&s_top[row], e - s_ea[row] + 56);
-            }
-            __syncthreads();
-            emax = max(emax, s_top[r]);
-        }
         fx_put<D, H>(V, s_eb + h * H, emax, low, 56 - emax - s_ea[r], (double*)smraw, r, h);
         if (r < n && h == 0) {
             const int* se = st.pool_e[side] + s_src[r];
@@ -559,6 +589,49 @@ __device__ __forceinline__ int64_t fx_shift(int64_t v, int d)
     return d > 62 ? 0 : (v + (1ll << (d - 1))) >> d;
 }
 
+// Results `low` (from column c0) of one node in FP64, into out[]: the power of two its
+// sums are aligned to goes to *power (the same from every part of the row), the largest
+// exponent is returned. AT and exps: matrices and powers of the node's local state, four
+// apart per edge. Out of line: the caller keeps its registers.
+template <int D>
+__device__ __noinline__ int fx_graph_redo(const uint32_t* it, uint32_t nl, const double* pool, const int* pool_e,
+                                          const double* __restrict__ AT, const int* __restrict__ exps, const int* t_e,
+                                          int nv, int deg, uint32_t low, int c0, double* out, int* power)
+{
+    uint64_t nz[kGtMaxDeg];
+    uint32_t whole = 0;
+    int er = nv < deg ? 0 : -(1 << 30);               // an e_0 source has power 0
+    for (int k = 0; k < nv; ++k) {
+        const uint32_t sr = __ldg(it + (size_t)(k + 1) * nl);
+        const double* x = pool + (size_t)sr * D;
+        er = max(er, pool_e[sr]);
+        nz[k] = fx_row_nonzero(x, D);
+        for (int c = 0; c < D; ++c) whole |= (fx_not_finite(x[c]) ? 1u : 0u) << k;
+    }
+    int top = -(1 << 29);
+    for (; low; low &= low - 1) {
+        const int c = c0 + __ffs((int)low) - 1;
+        double y = 0.0;
+        for (int k = 0; k < deg; ++k) {
+            const double* M = AT + (size_t)t_e[k] * 4 * D * D;
+            if (k < nv) {
+                const uint32_t sr = __ldg(it + (size_t)(k + 1) * nl);
+                const int* ex = exps + (size_t)t_e[k] * 4 * fx_exp_stride(D);
+                const uint64_t mz = __ldg((const uint64_t*)(ex + 2 * D) + D + c);
+                const bool all = ((whole >> k) & 1u) || __ldg(ex + D + c) == kFxNotFinite;
+                y += scale_pow2(fx_dot(M, pool + (size_t)sr * D, D, c, nz[k], mz, all), pool_e[sr] - er);
+            } else {
+                y += scale_pow2(__ldg(M + c), -er);
+            }
+        }
+        out[c] = y;
+        const int e = fx_top(y);
+        if (e != kFxNoExp) top = max(top, e + er);
+    }
+    *power = er;
+    return top;
+}
+
 template <int D>
 __global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1)
 k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __restrict__ exps, DevError* err, int t, int deg,
@@ -571,13 +644,12 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
     __shared__ __align__(8) int s_x[fx_exp_stride(D)];
     __shared__ int s_ea[kFxRows], s_es[kFxRows], s_bad[kFxRows];
     constexpr int SP = fx_split(D), H = D / SP;
-    __shared__ int s_max[SP][kFxRows], s_top[kFxRows];
-    __shared__ uint64_t s_big[kFxRows], s_nz[kFxRows];
-    __shared__ uint64_t s_low[kFxRows];
+    __shared__ int s_max[SP][kFxRows];
+    __shared__ int s_inf;
+    __shared__ uint64_t s_big[kFxRows];
     int* const s_cm = s_x;
     int* const s_eb = s_x + D;
     const uint64_t* const s_mb = (const uint64_t*)(s_x + 2 * D);
-    const uint64_t* const s_mz = s_mb + D;
     __shared__ int t_e[kGtMaxDeg];                    // edges with a vertex source, then the e_0 ones
     constexpr uint32_t kA = kFxRows * D * 2, kB = 2 * D * D;
     constexpr uint32_t kCols = kFxSums * D <= 128 ? 128 : kFxSums * D <= 256 ? 256 : 512;
@@ -633,9 +705,15 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
                     tc::bulk_g2s(Bs, img + (size_t)mat * kFxDigits * kB, kFxDigits * kB, &mb_b);
                 }
                 for (int q = tid; q < fx_exp_stride(D); q += kFxRows * SP) s_x[q] = __ldg(exps + (size_t)mat * fx_exp_stride(D) + q);
+                if (warp == 0) {
+                    bool inf = false;
+                    for (int q = lane; q < D; q += 32) inf |= __ldg(exps + (size_t)mat * fx_exp_stride(D) + D + q) == kFxNotFinite;
+                    inf = __any_sync(kFull, inf);
+                    if (lane == 0) s_inf = inf;
+                }
             }
             __syncthreads();
-            fx_rows<D, SP>(a.pool, s_src, s_cm, s_ea, s_bad, s_big, s_nz, smraw);
+            fx_rows<D, SP>(a.pool, s_src, s_cm, s_ea, s_bad, s_big, smraw);
             tc::fence_proxy_async();
             tc::fence_before_sync();
             __syncthreads();
@@ -653,7 +731,7 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
             __syncthreads();
             tc::fence_after_sync();
             const int ex = s_ea[r] + s_es[r];
-            const uint64_t mb = s_big[r], mz = s_nz[r];
+            uint32_t below = 0;
             if (s_bad[r]) low = H < 32 ? (1u << (H & 31)) - 1u : ~0u;
             #pragma unroll
             for (int c0 = 0; c0 < H; c0 += 8) {
@@ -665,11 +743,9 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
                 for (int c = 0; c < 8; ++c) {
                     const uint32_t x8[kFxSums] = {w[0][c], w[1][c], w[2][c], w[3][c], w[4][c], w[5][c], w[6][c], w[7][c]};
                     const int64_t v = fx_join<D>(x8, drop);
-                    const int col = h * H + c0 + c, eb = s_eb[col];
-                    if (!(s_mb[col] & mb) && ((fx_below(v, 56 - kFxTerm - drop) && (s_mz[col] & mz)) || eb == kFxNotFinite)) {
-                        low |= 1u << (c0 + c);
-                    } else if (v != 0) {
-                        const int x = ex + eb;
+                    below |= (fx_below(v, 56 - kFxTerm - drop) ? 1u : 0u) << (c0 + c);
+                    if (v != 0) {
+                        const int x = ex + s_eb[h * H + c0 + c];
                         int64_t& A = acc[c0 + c];
                         int& XA = X[c0 + c];
                         if (x > XA) { A = fx_shift(A, x - XA) + v; XA = x; }
@@ -677,6 +753,7 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
                     }
                 }
             }
+            low |= fx_low<H>(below, s_inf != 0, s_big[r], s_mb, s_eb, h);
             tc::fence_before_sync();
             __syncthreads();                          // accumulators, digits and lists are free
         }
@@ -700,39 +777,14 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
         for (int c = 0; c < H; ++c)
             if (acc[c] != 0 && !((low >> c) & 1u)) emax = max(emax, 64 - __clzll(acc[c] < 0 ? -acc[c] : acc[c]) + X[c]);
         if (r >= n) low = 0;
+        if (low)                                      // these in FP64, all edges
+            emax = max(emax, fx_graph_redo<D>(a.items + at + i0 + r, nl, a.pool, a.pool_e, a.an.AT + (size_t)g * D * D,
+                                              exps + (size_t)g * fx_exp_stride(D), t_e, nv, deg, low, h * H,
+                                              (double*)smraw + (size_t)r * (D + 2), s_es + r) + 56 - drop);
         s_max[h][r] = emax;
-        fx_mark<H>(s_low, r, h, low);
-        const bool redo = __syncthreads_or(low != 0);         // the parts of each row meet
+        __syncthreads();                              // the parts of each row meet
         #pragma unroll
         for (int k = 0; k < SP; ++k) emax = max(emax, s_max[k][r]);
-        if (redo) {
-            if (tid < kFxRows) s_top[tid] = -(1 << 29);
-            __syncthreads();
-            for (int q = warp; q < n * ((D + 31) / 32); q += kFxRows * SP / 32) {
-                const int row = q / ((D + 31) / 32), c = (q - row * ((D + 31) / 32)) * 32 + lane;
-                if (c >= D) continue;
-                if (!((s_low[row] >> c) & 1u)) continue;
-                const uint32_t* it = a.items + at + i0 + row;
-                int er = nv < deg ? 0 : -(1 << 30);   // an e_0 source has power 0
-                for (int k = 0; k < nv; ++k) er = max(er, a.pool_e[__ldg(it + (size_t)(k + 1) * nl)]);
-                double y = 0.0;
-                for (int k = 0; k < deg; ++k) {
-                    const double* M = a.an.AT + ((size_t)t_e[k] * 4 + g) * D * D;
-                    if (k < nv) {
-                        const uint32_t sr = __ldg(it + (size_t)(k + 1) * nl);
-                        y += scale_pow2(dot_col4(M, a.pool + (size_t)sr * D, D, c), a.pool_e[sr] - er);
-                    } else {
-                        y += scale_pow2(__ldg(M + c), -er);
-                    }
-                }
-                ((double*)smraw)[(size_t)row * (D + 2) + c] = y;
-                s_es[row] = er;                       // (the same from every result of the row)
-                const int e = fx_top(y);
-                if (e != kFxNoExp) atomicMax(&s_top[row], e + er + 56 - drop);
-            }
-            __syncthreads();
-            emax = max(emax, s_top[r]);
-        }
         const uint32_t out = __ldg(a.items + at + i0 + (r < n ? r : 0));
         fx_put<D, H>(acc, X, emax, low, low ? s_es[r] + 56 - drop - emax : 0, (double*)smraw, r, h);
         if (h == 0) {
@@ -885,7 +937,7 @@ __global__ void __launch_bounds__(256) k_fx_grad(GradArgs a, int chunk_samples, 
             #pragma unroll
             for (int k = 0; k < 8; ++k) {
                 cd[k] = fx_code(v[u][k], -ex);
-                mb |= (fx_is_big(fx_exp(v[u][k]) - ex) ? 1u : 0u) << k;
+                mb |= (fx_code_big(cd[k]) ? 1u : 0u) << k;
                 mz |= (fx_nonzero(v[u][k]) ? 1u : 0u) << k;
             }
             ((unsigned char*)(s_big + c))[n8] = (unsigned char)mb;
@@ -931,7 +983,7 @@ __global__ void __launch_bounds__(256) k_fx_grad(GradArgs a, int chunk_samples, 
                     const int col = D + h * H + q0 + c;
                     const int64_t V = fx_join<kGradRed>(x, 0);
                     double y = fx_double(V, ea + s_e[col] - 56, 0);
-                    if ((!(s_big[col] & mb) && fx_below(V, 56 - kFxTerm) && (s_nz[col] & mz)) || bad || s_bad[col]) {
+                    if ((fx_below(V, 56 - kFxTerm) && !(s_big[col] & mb) && (s_nz[col] & mz)) || bad || s_bad[col]) {
                         low |= 1u << (q0 + c);
                         y = 0.0;
                     }
@@ -1005,9 +1057,8 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
     __shared__ int s_pex[kFxRows], s_sig[kFxRows], s_ea[kFxRows], s_bad[kFxRows];
     __shared__ uint32_t s_flag[kFxRows], s_node[kFxRows];
     __shared__ int s_cm[KP], s_eb[128];
-    __shared__ uint64_t s_mb[128], s_mz[128];         // the operand rows' masks, the cells' below
-    __shared__ uint64_t s_big[kFxRows], s_nz[kFxRows];
-    __shared__ unsigned short s_low[3][2][kFxRows];   // entries to be redone in FP64, per chunk and half
+    __shared__ uint64_t s_mb[128];                    // masks of the operand rows, the cells' below
+    __shared__ uint64_t s_big[kFxRows];
     __shared__ short s_pos[128];                      // candidate entry n at s DP + component
     constexpr uint32_t kA = kFxRows * KP * 2, kB = 32 * KP * 2;
     constexpr uint32_t kCols = kFxSums * 32;
@@ -1025,16 +1076,20 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
     if (tid == 0) { tc::mbar_init(&mb_mma, 1); tc::mbar_init(&mb_b, 1); }
     for (int q = tid; q < 4 * D; q += 256) rv[q] = __ldg(an.rv + (size_t)t * 4 * D + q);
     for (int q = tid; q < D; q += 256) { eta[q] = __ldg(an.reta + (size_t)t * D + q); rw[q] = __ldg(an.rw + (size_t)t * D + q); }
+    bool inf = false;                                 // in the site's matrices or v
     {
         const int* x = exps + (size_t)t * fx_rnn_exp_stride(KP);
-        for (int q = tid; q < KP + 128; q += 256) (q < KP ? s_cm : s_eb - KP)[q] = __ldg(x + q);
-        const uint64_t* m = (const uint64_t*)(x + KP + 128);
-        (tid < 128 ? s_mb : s_mz - 128)[tid] = __ldg(m + tid);
+        for (int q = tid; q < KP + 128; q += 256) {
+            const int e = __ldg(x + q);
+            (q < KP ? s_cm : s_eb - KP)[q] = e;
+            inf |= q >= KP && q < KP + 32 * nch && e == kFxNotFinite;
+        }
+        if (tid < 128) s_mb[tid] = __ldg((const uint64_t*)(x + KP + 128) + tid);
     }
     for (int q = tid; q < 4 * D; q += 256) s_pos[q] = (short)((q / D) * DP + q % D);
     const double rc = __ldg(an.rc + t);
     tc::fence_before_sync();
-    __syncthreads();
+    const bool any_inf = __syncthreads_or(inf);
     tc::fence_after_sync();
     const uint32_t tmem = tmem_slot;
     const uint32_t b_bytes = (uint32_t)nch * kFxDigits * kB;
@@ -1110,16 +1165,13 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
             for (int u = 0; u < TASKS; ++u) {
                 const int ea = s_ea[rows[u]];
                 uint64_t c[8];
-                uint32_t mb = 0, mz = 0;
+                uint32_t mb = 0;
                 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    const int off = s_cm[8 * pcs[u] + k] - ea;
-                    c[k] = fx_code(v[u][k], off);
-                    mb |= (fx_is_big(fx_exp(v[u][k]) + off) ? 1u : 0u) << k;
-                    mz |= (fx_nonzero(v[u][k]) ? 1u : 0u) << k;
+                    c[k] = fx_code(v[u][k], s_cm[8 * pcs[u] + k] - ea);
+                    mb |= (fx_code_big(c[k]) ? 1u : 0u) << k;
                 }
                 ((unsigned char*)(s_big + rows[u]))[pcs[u]] = (unsigned char)mb;
-                ((unsigned char*)(s_nz + rows[u]))[pcs[u]] = (unsigned char)mz;
                 const uint32_t off = tc::op_offset(rows[u], 8 * pcs[u], KP);
                 #pragma unroll
                 for (int i = 0; i < kFxDigits; ++i) {
@@ -1132,8 +1184,7 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
         }
         const int ea = s_ea[r];
         const bool row_bad = s_bad[r] != 0;
-        uint64_t mb = 0, mz = 0;
-        bool any_low = false;
+        uint64_t mb = 0;
         for (int ch = 0; ch < nch; ++ch) {
             tc::fence_proxy_async();
             tc::fence_before_sync();
@@ -1149,8 +1200,8 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
             ph_mma ^= 1u;
             __syncthreads();
             tc::fence_after_sync();
-            if (ch == 0) { mb = s_big[r]; mz = s_nz[r]; }
-            uint32_t low = 0;
+            if (ch == 0) mb = s_big[r];
+            uint32_t below = 0;
             #pragma unroll
             for (int c0 = 0; c0 < 16; c0 += 8) {
                 const int col = 32 * ch + 16 * h + c0;
@@ -1164,32 +1215,25 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
                     if (col + c >= 4 * D) break;
                     const uint32_t x[kFxSums] = {w[0][c], w[1][c], w[2][c], w[3][c], w[4][c], w[5][c], w[6][c], w[7][c]};
                     const int64_t v = fx_join<KP>(x, 0);
-                    const int eb = s_eb[col + c];
-                    double y = fx_double(v, ea + eb - 56, 0);
-                    if (!(s_mb[col + c] & mb) &&
-                        ((fx_below(v, 56 - kFxTerm) && (s_mz[col + c] & mz)) || eb == kFxNotFinite))
-                        low |= 1u << (c0 + c);
+                    double y = fx_double(v, ea + s_eb[col + c] - 56, 0);
+                    below |= (fx_below(v, 56 - kFxTerm) ? 1u : 0u) << (c0 + c);
                     if (!fold) y += rv[col + c];
                     cand[(size_t)r * 4 * DP + s_pos[col + c]] = y;
                 }
             }
+            uint32_t low = fx_low<16>(below, any_inf, mb, s_mb + 32 * ch, s_eb + 32 * ch, h);
             if (row_bad) low = 0xFFFFu;
-            s_low[ch][h][r] = (unsigned short)low;
-            any_low |= low != 0;
-        }
-        tc::fence_before_sync();
-        if (__syncthreads_or(any_low && r < n)) {
-            for (int q = warp; q < n * nch; q += 8) {
-                const int row = q / nch, e = (q - row * nch) * 32 + lane;
-                if (e >= 4 * D) continue;
-                if (!((s_low[e >> 5][(e >> 4) & 1][row] >> (e & 15)) & 1u)) continue;
+            for (; low; low &= low - 1) {             // in FP64
+                const int e = 32 * ch + 16 * h + __ffs((int)low) - 1;
+                if (e >= 4 * D) break;
                 const int sg = e / D, c = e - sg * D;
                 const double* M = an.AT + ((size_t)t * 4 + sg) * D * D;
-                const double* x = s_src[row];
-                cand[(size_t)row * 4 * DP + s_pos[e]] = rv[e] + (x ? dot_col4(M, x, D, c) : __ldg(M + c));
+                const double* x = s_src[r];
+                cand[(size_t)r * 4 * DP + s_pos[e]] = rv[e] + (x ? dot_col4(M, x, D, c) : __ldg(M + c));
             }
-            __syncthreads();
         }
+        tc::fence_before_sync();
+        __syncthreads();
         for (int q = tid; q < n * 4; q += 256) {
             const double* x = cand + (size_t)q * DP;
             double p = 0.0;
