@@ -76,9 +76,9 @@ __device__ __forceinline__ bool fx_nonzero(double x) { return ((__double2hiint(x
 // 2^-kFxTerm of the scale is known to be there if entries of at least 2^-(kFxTerm / 2)
 // meet in the state and the matrix row (a bit mask each; for dense rows, also beside a
 // unit diagonal, that holds practically always), or if the result itself reaches
-// 2^-kFxTerm. Any other result is redone with FP64 FMAs, as are those that an
-// infinity or a NaN takes part in. The masks cost two instructions per entry and four
-// per result; what a result without such a term needs is looked at by its thread alone.
+// 2^-kFxTerm. Any other result with a nonzero term (two more masks) is redone with
+// FP64 FMAs, as are those that an infinity or a NaN takes part in. The masks cost four
+// instructions per entry and per result; a small result is looked at by its thread alone.
 // What stays errs by at most ~D 2^-55 of the scale, that is D 2^-47 of its largest
 // term where FP64 FMAs err by up to D 2^-53 of the sum of the terms. Of the results of
 // I + G / sqrt(D) matrices, kFxTerm = 4 redoes 5% (H50's log|psi| 4.2 -> 18 ms), 6
@@ -110,16 +110,18 @@ __device__ __forceinline__ bool fx_code_big(uint64_t c)
     return (uint32_t)(c >> 32) - 0x808080u + kBig >= 2u * kBig;
 }
 
-// the candidates among a thread's H results (columns h H ..) of a row with the mask mb of
-// large entries: those whose column of masks (s_mb) shares none, or is not finite
-template <int H>
-__device__ __forceinline__ uint32_t fx_low(uint32_t below, bool not_finite, uint64_t mb, const uint64_t* s_mb, const int* s_eb, int h)
+// the candidates among a thread's H results (columns h H ..), small (`below`) or not finite,
+// of a row with the masks mb and mz of its large and nonzero entries (the columns' in s_m,
+// Z words apart): those that share a nonzero entry and no large one
+template <int H, int Z>
+__device__ __forceinline__ uint32_t fx_low(uint32_t below, bool not_finite, uint64_t mb, uint64_t mz, const uint64_t* s_m,
+                                           const int* s_eb, int h)
 {
     uint32_t low = 0;
     // (a warp nearly always has one small result, a thread seldom two: a loop over them)
     for (uint32_t m = not_finite ? (H < 32 ? (1u << (H & 31)) - 1u : ~0u) : below; m; m &= m - 1) {
-        const int c = __ffs((int)m) - 1;
-        if (!(s_mb[h * H + c] & mb) && (((below >> c) & 1u) || s_eb[h * H + c] == kFxNotFinite)) low |= 1u << c;
+        const int c = __ffs((int)m) - 1, col = h * H + c;
+        if (!(s_m[col] & mb) && ((((below >> c) & 1u) && (s_m[col + Z] & mz)) || s_eb[col] == kFxNotFinite)) low |= 1u << c;
     }
     return low;
 }
@@ -318,11 +320,11 @@ __device__ __forceinline__ void fx_mma(uint32_t tmem, uint32_t N, uint64_t dA, u
 // The digits of a tile's rows (row r at pool + src[r] * D, times the column powers
 // cm, scaled by 2^-ea[r]) into the operand buffers: eight entries of a row per
 // task, eight rows x four tasks per warp (shared memory in whole core matrices).
-// ea[r] must hold kFxNoExp; contains a block barrier. big gets each row's mask of the
-// entries that are large after the scaling (bits below D).
+// ea[r] must hold kFxNoExp; contains a block barrier. big and nonzero get each row's
+// masks of entries that are large after the scaling, and not zero (bits below D).
 template <int D, int SP>
 __device__ __forceinline__ void fx_rows(const double* __restrict__ pool, const int64_t* src_row, const int* cm, int* ea_row,
-                                        int* bad_row, uint64_t* big, unsigned char* A)
+                                        int* bad_row, uint64_t* big, uint64_t* nonzero, unsigned char* A)
 {
     constexpr int NW = kFxRows * SP / 32;
     constexpr uint32_t kA = kFxRows * D * 2;
@@ -373,13 +375,15 @@ __device__ __forceinline__ void fx_rows(const double* __restrict__ pool, const i
     for (int u = 0; u < TASKS; ++u) {
         const int ea = ea_row[rows[u]];
         uint64_t c[8];
-        uint32_t mb = 0;
+        uint32_t mb = 0, mz = 0;
         #pragma unroll
         for (int k = 0; k < 8; ++k) {
             c[k] = fx_code(v[u][k], cm[8 * pcs[u] + k] - ea);
             mb |= (fx_code_big(c[k]) ? 1u : 0u) << k;
+            mz |= (fx_nonzero(v[u][k]) ? 1u : 0u) << k;
         }
         ((unsigned char*)(big + rows[u]))[pcs[u]] = (unsigned char)mb;
+        ((unsigned char*)(nonzero + rows[u]))[pcs[u]] = (unsigned char)mz;
         const uint32_t off = tc::op_offset(rows[u], 8 * pcs[u], D);
         #pragma unroll
         for (int i = 0; i < kFxDigits; ++i) {
@@ -405,11 +409,10 @@ __global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1) k_fx_s
     constexpr int SP = fx_split(D);                   // threads per row
     __shared__ int s_max[SP][kFxRows];
     __shared__ int s_bad[kFxRows], s_inf;             // rows, and the matrix, with an infinity or a NaN
-    __shared__ uint64_t s_big[kFxRows];
+    __shared__ uint64_t s_big[kFxRows], s_nz[kFxRows];
     int* const s_cm = s_x;
     int* const s_eb = s_x + D;
-    const uint64_t* const s_mb = (const uint64_t*)(s_x + 2 * D);
-    const uint64_t* const s_mz = s_mb + D;
+    const uint64_t* const s_m = (const uint64_t*)(s_x + 2 * D);
     constexpr int H = D / SP;                         // columns per thread in the epilogue
     constexpr uint32_t kA = kFxRows * D * 2;          // one digit of the rows
     constexpr uint32_t kB = 2 * D * D;                // one digit of the matrix
@@ -485,7 +488,7 @@ __global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1) k_fx_s
             }
         }
         __syncthreads();
-        fx_rows<D, SP>(st.pool[side], s_src, s_cm, s_ea, s_bad, s_big, smraw);
+        fx_rows<D, SP>(st.pool[side], s_src, s_cm, s_ea, s_bad, s_big, s_nz, smraw);
         tc::fence_proxy_async();
         tc::fence_before_sync();
         __syncthreads();
@@ -534,7 +537,7 @@ __global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1) k_fx_s
                 below |= (fx_below(v, 56 - kFxTerm) ? 1u : 0u) << (c0 + c);
             }
         }
-        uint32_t low = fx_low<H>(below, s_inf != 0, s_big[r], s_mb, s_eb, h);
+        uint32_t low = fx_low<H, D>(below, s_inf != 0, s_big[r], s_nz[r], s_m, s_eb, h);
         if (s_bad[r]) low = H < 32 ? (1u << (H & 31)) - 1u : ~0u;
         if (r >= n) low = 0;
         if (low) {                                    // the others' largest, and these in FP64
@@ -544,10 +547,10 @@ __global__ void __launch_bounds__(kFxRows * fx_split(D), D <= 32 ? 2 : 1) k_fx_s
                 if (V[c] != 0 && !((low >> c) & 1u)) emax = max(emax, 64 - __clzll(V[c] < 0 ? -V[c] : V[c]) + s_eb[h * H + c]);
             const double* M = st.at[side] + (mat - (size_t)side * 4 * st.K) * D * D;
             const double* x = st.pool[side] + (size_t)s_src[r] * D;
-            const uint64_t nz = fx_row_nonzero(x, D);
+            const uint64_t nz = s_nz[r] & (D < 64 ? (1ull << (D & 63)) - 1 : ~0ull);
             for (uint32_t m = low; m; m &= m - 1) {
                 const int c = h * H + __ffs((int)m) - 1;
-                const double y = fx_dot(M, x, D, c, nz, s_mz[c], s_bad[r] || s_eb[c] == kFxNotFinite);
+                const double y = fx_dot(M, x, D, c, nz, s_m[D + c], s_bad[r] || s_eb[c] == kFxNotFinite);
                 ((double*)smraw)[(size_t)r * (D + 2) + c] = y;
                 const int e = fx_top(y);
                 if (e != kFxNoExp) emax = max(emax, e - s_ea[r] + 56);
@@ -646,10 +649,10 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
     constexpr int SP = fx_split(D), H = D / SP;
     __shared__ int s_max[SP][kFxRows];
     __shared__ int s_inf;
-    __shared__ uint64_t s_big[kFxRows];
+    __shared__ uint64_t s_big[kFxRows], s_nz[kFxRows];
     int* const s_cm = s_x;
     int* const s_eb = s_x + D;
-    const uint64_t* const s_mb = (const uint64_t*)(s_x + 2 * D);
+    const uint64_t* const s_m = (const uint64_t*)(s_x + 2 * D);
     __shared__ int t_e[kGtMaxDeg];                    // edges with a vertex source, then the e_0 ones
     constexpr uint32_t kA = kFxRows * D * 2, kB = 2 * D * D;
     constexpr uint32_t kCols = kFxSums * D <= 128 ? 128 : kFxSums * D <= 256 ? 256 : 512;
@@ -713,7 +716,7 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
                 }
             }
             __syncthreads();
-            fx_rows<D, SP>(a.pool, s_src, s_cm, s_ea, s_bad, s_big, smraw);
+            fx_rows<D, SP>(a.pool, s_src, s_cm, s_ea, s_bad, s_big, s_nz, smraw);
             tc::fence_proxy_async();
             tc::fence_before_sync();
             __syncthreads();
@@ -753,7 +756,7 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
                     }
                 }
             }
-            low |= fx_low<H>(below, s_inf != 0, s_big[r], s_mb, s_eb, h);
+            low |= fx_low<H, D>(below, s_inf != 0, s_big[r], s_nz[r], s_m, s_eb, h);
             tc::fence_before_sync();
             __syncthreads();                          // accumulators, digits and lists are free
         }
@@ -1057,8 +1060,8 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
     __shared__ int s_pex[kFxRows], s_sig[kFxRows], s_ea[kFxRows], s_bad[kFxRows];
     __shared__ uint32_t s_flag[kFxRows], s_node[kFxRows];
     __shared__ int s_cm[KP], s_eb[128];
-    __shared__ uint64_t s_mb[128];                    // masks of the operand rows, the cells' below
-    __shared__ uint64_t s_big[kFxRows];
+    __shared__ uint64_t s_m[2 * 128];                 // masks of the operand rows, the cells' below
+    __shared__ uint64_t s_big[kFxRows], s_nz[kFxRows];
     __shared__ short s_pos[128];                      // candidate entry n at s DP + component
     constexpr uint32_t kA = kFxRows * KP * 2, kB = 32 * KP * 2;
     constexpr uint32_t kCols = kFxSums * 32;
@@ -1084,7 +1087,7 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
             (q < KP ? s_cm : s_eb - KP)[q] = e;
             inf |= q >= KP && q < KP + 32 * nch && e == kFxNotFinite;
         }
-        if (tid < 128) s_mb[tid] = __ldg((const uint64_t*)(x + KP + 128) + tid);
+        s_m[tid] = __ldg((const uint64_t*)(x + KP + 128) + tid);
     }
     for (int q = tid; q < 4 * D; q += 256) s_pos[q] = (short)((q / D) * DP + q % D);
     const double rc = __ldg(an.rc + t);
@@ -1165,13 +1168,15 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
             for (int u = 0; u < TASKS; ++u) {
                 const int ea = s_ea[rows[u]];
                 uint64_t c[8];
-                uint32_t mb = 0;
+                uint32_t mb = 0, mz = 0;
                 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     c[k] = fx_code(v[u][k], s_cm[8 * pcs[u] + k] - ea);
                     mb |= (fx_code_big(c[k]) ? 1u : 0u) << k;
+                    mz |= (fx_nonzero(v[u][k]) ? 1u : 0u) << k;
                 }
                 ((unsigned char*)(s_big + rows[u]))[pcs[u]] = (unsigned char)mb;
+                ((unsigned char*)(s_nz + rows[u]))[pcs[u]] = (unsigned char)mz;
                 const uint32_t off = tc::op_offset(rows[u], 8 * pcs[u], KP);
                 #pragma unroll
                 for (int i = 0; i < kFxDigits; ++i) {
@@ -1184,7 +1189,7 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
         }
         const int ea = s_ea[r];
         const bool row_bad = s_bad[r] != 0;
-        uint64_t mb = 0;
+        uint64_t mb = 0, mz = 0;
         for (int ch = 0; ch < nch; ++ch) {
             tc::fence_proxy_async();
             tc::fence_before_sync();
@@ -1200,7 +1205,7 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
             ph_mma ^= 1u;
             __syncthreads();
             tc::fence_after_sync();
-            if (ch == 0) mb = s_big[r];
+            if (ch == 0) { mb = s_big[r]; mz = s_nz[r]; }
             uint32_t below = 0;
             #pragma unroll
             for (int c0 = 0; c0 < 16; c0 += 8) {
@@ -1221,7 +1226,7 @@ __global__ void __launch_bounds__(256) k_fx_rnn(TreeRnn a, const unsigned char* 
                     cand[(size_t)r * 4 * DP + s_pos[col + c]] = y;
                 }
             }
-            uint32_t low = fx_low<16>(below, any_inf, mb, s_mb + 32 * ch, s_eb + 32 * ch, h);
+            uint32_t low = fx_low<16, 128>(below, any_inf, mb, mz, s_m + 32 * ch, s_eb + 32 * ch, h);
             if (row_bad) low = 0xFFFFu;
             for (; low; low &= low - 1) {             // in FP64
                 const int e = 32 * ch + 16 * h + __ffs((int)low) - 1;
