@@ -305,8 +305,8 @@ int nqs_connected(nqs_ctx* ctx, const uint64_t* samples, int64_t Ns, double det_
                   int64_t capacity);
 
 /* log|psi| and sign of psi for n determinants (full K-site product, FP64
- * whatever the precision option). sign is 0 where psi = 0. Chains whose D is 16,
- * 32, 48 or 64 take the fixed-point products of NQS_PREC_FP64 from 1100
+ * whatever the precision option). sign is 0 where psi = 0. Chains whose D is 48 or
+ * 64 (16 or 32) take the fixed-point products of NQS_PREC_FP64 from 1700 (3200)
  * determinants per call on, so the last bits may differ between a large call and
  * small ones. */
 int nqs_amplitude(nqs_ctx* ctx, const uint64_t* dets, int64_t n, double* log_abs,
@@ -407,7 +407,7 @@ int nqs_local_energy_batch(nqs_ctx* const* ctxs, int n_sys, nqs_batch_item* item
  *  times forward cell); nqs_options.grad_chunk bounds how many samples'
  *  environments are held at once (the sums then round in another order, and a
  *  width of 16, 32, 48 or 64 takes fixed-point products from 64 samples of a chunk
- *  on, a chain's environments from 1100). */
+ *  on, a chain's environments as nqs_amplitude). */
 int nqs_grad_log_psi_vjp(nqs_ctx* ctx, const uint64_t* samples, const double* u, int64_t Ns,
                          double* grad_sites, double* grad_W, double* grad_b);
 

@@ -26,10 +26,13 @@ constexpr int kDefaultAudit = 4;
 
 // chains: samples (determinants) from which the FP64 sweeps go site by site
 // through the fixed-point tensor-core steps (one launch per site) instead of
-// one block per sample. log|psi| and its gradient at D = 64, K = 50, fixed-point /
-// block per sample: 512 determinants 3.03 / 2.00 ms, 1024 3.14 / 3.01, 2048 3.49 /
-// 4.62
-constexpr int64_t kFxMinRows = 1100;
+// one block per sample, where both take as long (narrow: D < 48). log|psi| and its
+// gradient at K = 50, fixed-point / block per sample: D = 64 1024 determinants 3.24 / 2.29
+// ms, 1300 3.38 / 2.79, 2048 3.60 / 4.11; D = 48 1500 2.97 / 2.42, 1900 3.06 / 3.16; D = 32
+// 1100 2.35 / 1.31, 2600 2.66 / 2.41, 3800 2.91 / 3.13; D = 16 2600 2.15 / 1.92, 3800 2.33 /
+// 2.46; K = 24, D = 64 1500 1.91 / 1.62, 1900 1.98 / 2.07
+constexpr int64_t kFxMinRows = 1700, kFxMinRowsNarrow = 3200;
+int64_t fx_min_rows(int D) { return D >= 48 ? kFxMinRows : kFxMinRowsNarrow; }
 
 struct DevBuf {
     void* p = nullptr;
@@ -435,7 +438,7 @@ int env_pass(nqs_ctx* c, const uint64_t* samples, int64_t Ns, bool adjoints, int
     e.psi_mant = (double*)c->pmant.p;
     e.psi_exp = (int*)c->pexp.p;
     e.h_diag = (double*)c->hdiag.p;
-    const bool fx = by_site && tn == 1 && c->av.chain && c->has_fx && Ns >= kFxMinRows;
+    const bool fx = by_site && tn == 1 && c->av.chain && c->has_fx && Ns >= fx_min_rows(D);
     if (fx) {
         // both sweeps of all samples site by site on the tensor cores: step i takes
         // the left states through site i and the right ones through site K - 1 - i
@@ -1759,7 +1762,7 @@ extern "C" int nqs_amplitude(nqs_ctx* c, const uint64_t* dets, int64_t n, double
     bool h0, h1;
     TRY(stage_out(c, c->st_out0, log_abs, (size_t)n, &dla, &h0));
     TRY(stage_out(c, c->st_out1, sign, (size_t)n, &dsg, &h1));
-    if (c->av.readout == 0 && c->av.chain && c->has_fx && n >= kFxMinRows) {
+    if (c->av.readout == 0 && c->av.chain && c->has_fx && n >= fx_min_rows(c->av.D)) {
         TRY(fx_amplitude(c, dd, n, dla, dsg));
         TRY(read_dev_error(c));       // the determinants' check and the tiles' bounded waits
         TRY(copy_back(c, log_abs, dla, (size_t)n, h0));

@@ -25,7 +25,8 @@ namespace {
 
 constexpr int kGradChunk = 256;   // samples per block (one chunk of a local-state group)
 // samples from which the fixed-point products run. H18 energy gradient (D = 32),
-// fixed-point / FP64: 32 samples 1.82 / 1.82 ms, 128 2.53 / 2.60, 512 5.73 / 6.18
+// fixed-point / FP64: 32 samples 1.81 / 1.81 ms, 64 2.03 / 2.06, 128 2.52 / 2.59,
+// 512 5.75 / 6.18
 constexpr int64_t kFxGradMin = 64;
 constexpr int kTile = 64;         // output tile edge
 constexpr int kStage = 16;        // samples staged per round

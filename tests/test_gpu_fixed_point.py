@@ -27,16 +27,18 @@ U = 2.0 ** -53
 
 
 def _const(name):
-    """Value of `constexpr ... name = value;` in the CUDA sources."""
+    """Value of `constexpr ... name = value` in the CUDA sources."""
     for f in sorted(os.listdir(CSRC)):
         with open(os.path.join(CSRC, f)) as h:
-            m = re.search(r"constexpr\s+\w+\s+" + name + r"\s*=\s*(\d+)\s*;", h.read())
+            m = re.search(r"constexpr\s+\w+\s+(?:\w+\s*=\s*\d+\s*,\s*)*" + name + r"\s*=\s*(\d+)\s*[,;]", h.read())
         if m:
             return int(m.group(1))
     raise KeyError(name)
 
 
-ROWS = _const("kFxMinRows")          # determinants from which a chain's sweeps take the steps
+def _rows(D):
+    """Determinants from which a chain's sweeps take the steps."""
+    return _const("kFxMinRows" if D >= 48 else "kFxMinRowsNarrow")
 
 
 @pytest.fixture(scope="module")
@@ -74,6 +76,27 @@ def _assert_log_psi(ctx, s, dets, run=None):
     assert np.all(np.abs(la - ref)[ok] <= tol[ok]) and np.array_equal(sg[ok], rs[ok])
 
 
+@pytest.mark.parametrize("D", [16, 32, 48, 64])
+@pytest.mark.parametrize("over", [-1, 0, 1, 701])
+def test_log_psi_at_the_line(ctx, D, over):
+    """Dense rows of unlike size on both sides of the size from which the steps run, one
+    launch per site: every width, part tiles of every local state."""
+    n, rng = _rows(D) + over, np.random.default_rng(D)
+    s = W.tiny_system(K=8, na=4, nb=4, D=D, seed=D, n_samples=n)
+    s = dataclasses.replace(s, tensors=s.tensors * np.exp2(rng.integers(-20, 8, size=(s.K, 4, D, 1))))
+    ctx.set_system(s)
+    ctx.stage_times()
+    la, sg = ctx.amplitude(s.samples)
+    launches = sum(k for _, k in ctx.stage_times().values())
+    assert len(la) == n and (launches >= s.K) == (over >= 0)
+    pick = rng.choice(n, 500, replace=False)
+    ref, rs, cond = _log_psi_ref(s, s.samples[pick])
+    tol = s.K * (D + 1) * U * cond + 8 * U * np.abs(ref)
+    ok = tol < 1e-3
+    assert ok.sum() > 250
+    assert np.all(np.abs(la[pick] - ref)[ok] <= tol[ok]) and np.array_equal(sg[pick][ok], rs[ok])
+
+
 def _isometric(rng, K, D):
     """Site tensors with sum_s M^s^T M^s = 1."""
     q = [np.linalg.qr(rng.normal(size=(4 * D, D)))[0].reshape(4, D, D) for _ in range(K)]
@@ -98,7 +121,7 @@ def test_normalised_chain_without_v(ctx, D):
 def test_empty_columns(ctx, D, graph):
     """Columns and rows without entries in small site tensors (2^-40), the states'
     entries there of order one: they meet only zeros and must not set the scale."""
-    n = ROWS + 101
+    n = _rows(D) + 101
     if graph:
         s = _dag(D, 8, D, n_samples=150, eps=0.01, n_draws=20)
     else:
@@ -152,7 +175,7 @@ def test_graded_states(ctx, D, graph, kind):
     if graph:
         s = _dag(D, 8, D, n_samples=150, eps=0.01, n_draws=20)
     else:
-        s = W.tiny_system(K=8, na=4, nb=4, D=D, n_hidden=3, seed=D, n_samples=ROWS + 101, eps=0.01, n_draws=20)
+        s = W.tiny_system(K=8, na=4, nb=4, D=D, n_hidden=3, seed=D, n_samples=_rows(D) + 101, eps=0.01, n_draws=20)
     s = _graded(rng, s, kind)
     if not graph:
         _assert_log_psi(ctx, dataclasses.replace(s, rbm_W=None, rbm_b=None), s.samples)
@@ -189,7 +212,7 @@ def test_graded_cells(ctx, D, v):
 def test_not_finite_steps(ctx, D, bad):
     """A NaN or an infinity in a site tensor reaches every amplitude whose local state
     reads it, and none whose does not; the last site's unread rows reach none."""
-    s = W.tiny_system(K=8, na=4, nb=4, D=D, seed=1, n_samples=ROWS + 101)
+    s = W.tiny_system(K=8, na=4, nb=4, D=D, seed=1, n_samples=_rows(D) + 101)
     occ = ((s.samples[:, None, :] >> np.arange(s.K, dtype=np.uint64)[None, :, None]) & np.uint64(1)).astype(int)
     T = s.tensors.copy()
     T[5, 3, 2, 7] = bad
@@ -319,7 +342,7 @@ def test_outer_products_not_finite(ctx, bad):
 def test_energies_do_not_depend_on_the_split(ctx, kind, D):
     """A sample's plain-form energy has the same bits in a large batch, in small calls and
     under a table cap that cuts the batch (the levels' node counts differ a hundredfold)."""
-    n = ROWS + 101
+    n = 1201
     if kind == "graph":
         s = _dag(D, 8, D, n_samples=n, eps=0.02, n_draws=10)
     else:
