@@ -394,8 +394,12 @@ def run(args):
     mv_alg = work["span_sites"] if sys_.pred_ptr is None else work["matvecs"]
     flops = 2.0 * D * D * mv_alg + 2.0 * D * n_amp
     executed = 2.0 * D * D * work["matvecs"] + 2.0 * D * n_amp
-    achieved = flops / (amp_ms / 1e3) / 1e12
     graph = sys_.pred_ptr is not None
+    # rate and fraction count what runs (the shared-prefix forms report it; the prefix
+    # trees count their rows' products, of which they execute a part); a per-amplitude
+    # evaluation's products over the same time are given beside them
+    shared = not graph and prec != nqs.NQS_PREC_FP64
+    achieved = executed / (amp_ms / 1e3) / 1e12 if shared else None
     if prec == nqs.NQS_PREC_MIXED:
         roof = {"bound": "tensor", "unit": "TFLOP/s", "achieved": achieved,
                 "peak": peaks["bf16_tflops_sustained"],
@@ -405,17 +409,20 @@ def run(args):
                            "amplitude stage: k_fam_mark, k_fam_compact, k_site_boundary, "
                            "k_site_build, k_site_tiles_pipe / k_site_tiles_ws (tcgen05), k_fam_rbm, k_fam_rows")}
     else:
-        roof = {"bound": "alu", "unit": "TFLOP/s", "achieved": achieved,
-                "peak": live["fma64_tflops"] if live else 1.056,
-                "peak_source": ("FP64 FMA rate measured before the timed region (peaks probe)" if live
-                                else "FP64 FMA rate of an earlier peaks-probe run on a GB300"),
-                "kernel": ("amplitude stage (shared prefixes, FP64)" if prec == nqs.NQS_PREC_FP64_SHARED
-                           else "k_tree_graph64 / k_fx_graph (prefix trees of the rows), k_tree_rows64"),
-                "note": ("frac counts a per-amplitude evaluation's products against the FP64 pipe; shared "
-                         "prefixes execute fewer, and large steps run in fixed point on the tensor cores")}
-    roof["frac"] = roof["achieved"] / roof["peak"]
-    # the same stage against the work the shared-prefix form executes
-    roof["executed_frac"] = executed / (amp_ms / 1e3) / 1e12 / roof["peak"]
+        kernel = ("amplitude stage (shared prefixes, FP64)" if prec == nqs.NQS_PREC_FP64_SHARED
+                  else "k_tree_graph64 / k_fx_graph (prefix trees of the rows), k_tree_rows64")
+        if D % 16 == 0 and D <= 64:
+            roof = {"bound": "tensor", "unit": "TFLOP/s", "achieved": achieved, "peak": peaks["bf16_tflops_sustained"] / 34,
+                    "peak_source": f"{src} dense bf16 (sustained), 34 digit products per fixed-point product",
+                    "kernel": kernel}
+        else:
+            roof = {"bound": "alu", "unit": "TFLOP/s", "achieved": achieved,
+                    "peak": live["fma64_tflops"] if live else 1.056,
+                    "peak_source": ("FP64 FMA rate measured before the timed region (peaks probe)" if live
+                                    else "FP64 FMA rate of an earlier peaks-probe run on a GB300"),
+                    "kernel": kernel}
+    roof["frac"] = roof["executed_frac"] = achieved / roof["peak"] if shared else None
+    roof["per_amplitude_tflops"] = flops / (amp_ms / 1e3) / 1e12
     # the row kernel (k_fam_rows, the largest share of the mixed step) against the
     # on-chip rate it is bound by: per row it gathers the left and right vectors
     # (D floats each) and, with a correlator, one factor row per side (N_h
@@ -453,7 +460,7 @@ def run(args):
     roof["traffic"] = STAGE_TRAFFIC_PER_AMP.get(key, None)
     if roof["traffic"] is not None:
         roof["traffic"] *= n_amp
-    roof.update({"algorithmic_flops_per_step": flops, "executed_flops_per_step": executed,
+    roof.update({"algorithmic_flops_per_step": flops, "executed_flops_per_step": executed if shared else None,
                  "stage_ms_per_step": amp_ms, "launches_per_step": amp_launches,
                  "span_sites_per_step": work["span_sites"], "matvecs_per_step": work["matvecs"]})
 
@@ -595,10 +602,9 @@ def run_rnn(args):
             "peak_source": "FP64 FMA rate measured before the timed region (peaks probe)" if live
             else "FP64 FMA rate of an earlier probe run on this pool's GB300",
             "kernel": "k_tree_rnn / k_fx_rnn (normalised readout over the rows' prefix trees)", "traffic": None,
-            "note": "frac counts a per-row evaluation against the FP64 pipe; rows share their prefixes and "
-                    "large levels run in fixed point on the tensor cores",
-            "algorithmic_flops_per_step": flops, "stage_ms_per_step": amp_ms}
-    roof["frac"] = roof["achieved"] / roof["peak"]
+            "note": "achieved counts a per-row evaluation, of which rows that share prefixes execute a part "
+                    "(in fixed point on the tensor cores up to D = 24): no fraction of the peak",
+            "algorithmic_flops_per_step": flops, "stage_ms_per_step": amp_ms, "frac": None}
     # end to end: the same step with host-side outputs (samples back to the host,
     # then E_loc through host buffers)
     hs = np.empty((n_draw, 2), np.uint64)
@@ -773,8 +779,9 @@ def run_batch(args):
                 for s, r in zip(systems, res))
     executed = sum(2.0 * s.D * s.D * r[1]["matvecs"] + 2.0 * s.D * r[1]["n_amplitudes"]
                    for s, r in zip(systems, res))
-    achieved = flops / (ms / args.steps / 1e3) / 1e12
+    achieved = executed / (ms / args.steps / 1e3) / 1e12
     roof = {"bound": "tensor", "unit": "TFLOP/s", "achieved": achieved,
+            "per_amplitude_tflops": flops / (ms / args.steps / 1e3) / 1e12,
             "peak": peaks["bf16_tflops_sustained"],
             "peak_source": f"{src} dense bf16 (sustained; f16 has the same nominal rate)",
             "kernel": "whole batch step (all stages of 64 systems, overlapped on streams)",
