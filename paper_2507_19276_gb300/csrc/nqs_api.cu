@@ -870,31 +870,31 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
     const bool full = kind != kTreeGraph64;
     const int stage = NQS_STAGE_AMP_DET;
     StageScope sc(c, stage);
-    TRY(ensure(c, c->tr_rows, (size_t)(3 * Ns + 2) * 8));
+    TRY(ensure(c, c->tr_rows, (size_t)(2 * Ns + 2) * 8));
     TRY(ensure(c, c->base_det, (size_t)(Ns + 1) * 8));
-    int64_t* row_cnt = (int64_t*)c->tr_rows.p;
-    int64_t* row_base = row_cnt + Ns;
+    int64_t* row_base = (int64_t*)c->tr_rows.p;
+    const int64_t* det_cnt = (const int64_t*)c->det_tot.p;
     const int64_t* dcnt = n_draws > 0 ? (const int64_t*)c->n_unique.p : nullptr;
-    LAUNCH(stage, launch_tree_row_counts((const int64_t*)c->det_tot.p, dcnt, Ns, row_cnt, c->stream));
-    LAUNCH(stage, launch_scan_i64(row_cnt, row_base, Ns, c->stream));
     // the FP64 forms sum a sample's rows together, the mixed form the deterministic
     // and the drawn rows apart
     const bool apart = kind == kTreeGraphTc;
     int64_t* chunk_base = apart ? row_base + Ns + 1 : (int64_t*)c->base_det.p;
-    LAUNCH(stage, launch_chunk_base(row_cnt, kTreeRows, chunk_base, Ns, c->stream));
+    // a sample's rows and chunks, one launch
+    ScanJobs scans{{{det_cnt, dcnt, row_base, Ns, 0}, {det_cnt, dcnt, chunk_base, Ns, kTreeRows}}, 2};
     const int64_t det_chunks = total_det / kTreeRows + Ns;
     const int64_t draw_chunks = Ns * (((int64_t)n_draws + kTreeRows - 1) / kTreeRows);
     if (apart) {
-        LAUNCH(stage, launch_chunk_base((const int64_t*)c->det_tot.p, kTreeRows, (int64_t*)c->base_det.p, Ns, c->stream));
+        scans.job[scans.n++] = {det_cnt, nullptr, (int64_t*)c->base_det.p, Ns, kTreeRows};
         if (n_draws > 0) {
             TRY(ensure(c, c->base_draw, (size_t)(Ns + 1) * 8));
             TRY(ensure(c, c->part_draw, (size_t)(draw_chunks + 1) * 8));
             TRY(ensure(c, c->span_draw, (size_t)(draw_chunks + 1) * 8));
             TRY(ensure(c, c->mv_draw, (size_t)(draw_chunks + 1) * 8));
             if (want_abs) TRY(ensure(c, c->part_draw_abs, (size_t)(draw_chunks + 1) * 8));
-            LAUNCH(stage, launch_chunk_base(dcnt, kTreeRows, (int64_t*)c->base_draw.p, Ns, c->stream));
+            scans.job[scans.n++] = {dcnt, nullptr, (int64_t*)c->base_draw.p, Ns, kTreeRows};
         }
     }
+    LAUNCH(stage, launch_scan_jobs(scans, c->stream));
     const int64_t rows_bound = total_det + Ns * (int64_t)n_draws;
     const int64_t chunks_all = rows_bound / kTreeRows + Ns;
     TRY(ensure(c, c->part_det, (size_t)(chunks_all + 1) * 8));
@@ -1022,8 +1022,12 @@ int tree_pass(nqs_ctx* c, const uint64_t* ds, int64_t Ns, int64_t total_det, int
             if (!pass) FIT(fit(c->tr_build, v.n));
         }
         LAUNCH(stage, launch_tree_nodes(a, max_chunks, c->stream));
-        LAUNCH(stage, launch_scan_i64(a.pool_tot, pool_off, nb, c->stream));
-        LAUNCH(stage, launch_scan_i64_wide(a.level_cnt, a.level_off, ncnt, scan_tmp, c->stream));
+        ScanJobs sums{{{a.pool_tot, nullptr, pool_off, nb, 0}, {a.level_cnt, nullptr, a.level_off, ncnt, 0}}, 2};
+        if (ncnt > kScanOneBlock) {
+            sums.n = 1;
+            LAUNCH(stage, launch_scan_i64_wide(a.level_cnt, a.level_off, ncnt, scan_tmp, c->stream));
+        }
+        LAUNCH(stage, launch_scan_jobs(sums, c->stream));
         CK(cudaGetLastError());
         // the levels' item bounds and the pool's rows, in one copy
         std::vector<int64_t> bounds((size_t)4 * K + 2);

@@ -87,8 +87,15 @@ int launch_scan_chunks_u32(const uint32_t* cnt, uint32_t* off, int64_t* total, i
 // per sample: inclusive scan of u64 chunk weights (in place), totals -> W
 int launch_scan_chunks_u64(uint64_t* w, uint64_t* total, int64_t Ns, uint32_t n_chunks,
                             cudaStream_t st);
+// exclusive scans, one block each, of one launch: out[0..n] (out[n] = total) of the values
+// in[i] + add[i] (add may be NULL), of ceil(value / rows) if rows > 0
+struct ScanJob { const int64_t* in; const int64_t* add; int64_t* out; int64_t n; int rows; };
+struct ScanJobs { ScanJob job[4]; int n; };
+int launch_scan_jobs(const ScanJobs& jobs, cudaStream_t st);
 // exclusive scan of n values -> out[0..n] (out[n] = total); single block
 int launch_scan_i64(const int64_t* in, int64_t* out, int64_t n, cudaStream_t st);
+constexpr int kScanTile = 4096;                       // 1024 threads x 4 elements
+constexpr int64_t kScanOneBlock = 16 * kScanTile;     // values one block scans as fast as many
 // the same over many blocks for large n; tmp holds scan_i64_tmp_elems(n) values
 inline int64_t scan_i64_tmp_elems(int64_t n) { return 2 * (n / 4096 + 2); }
 int launch_scan_i64_wide(const int64_t* in, int64_t* out, int64_t n, int64_t* tmp, cudaStream_t st);

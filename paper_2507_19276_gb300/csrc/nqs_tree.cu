@@ -95,7 +95,8 @@ __device__ __forceinline__ int block_excl(int v, int* sh, int* tot)
 }
 
 // One block per sample: roots, one-change nodes, and the two-change nodes in
-// the order of their changes (their table entries become indices).
+// the order of their changes (their table entries become indices), and the third
+// changes' bits cleared.
 __global__ void __launch_bounds__(512) k_tree_two(TreeArgs a)
 {
     __shared__ int sh[16];
@@ -141,6 +142,8 @@ __global__ void __launch_bounds__(512) k_tree_two(TreeArgs a)
             e2[q] = at++;
         }
     }
+    uint32_t* bits = a.bits + (size_t)sl * a.n2max * a.W;
+    for (int q = threadIdx.x; q < carry * a.W; q += blockDim.x) bits[q] = 0;
     if (threadIdx.x == 0) a.n2[sl] = carry;
 }
 
@@ -452,12 +455,6 @@ __global__ void __launch_bounds__(256) k_tree_perm(TreeArgs a, uint32_t* perm)
     }
 }
 
-__global__ void k_tree_row_counts(const int64_t* det, const int64_t* draw, int64_t n, int64_t* cnt)
-{
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < n) cnt[s] = det[s] + (draw ? draw[s] : 0);
-}
-
 // 2^d as a double, 0 below the normal range (d <= 0)
 __device__ __forceinline__ double pow2_neg64(int d)
 {
@@ -466,19 +463,10 @@ __device__ __forceinline__ double pow2_neg64(int d)
 
 }  // namespace
 
-int launch_tree_row_counts(const int64_t* det_cnt, const int64_t* draw_cnt, int64_t Ns, int64_t* cnt, cudaStream_t st)
-{
-    if (Ns == 0) return 0;
-    k_tree_row_counts<<<(unsigned)((Ns + 255) / 256), 256, 0, st>>>(det_cnt, draw_cnt, Ns, cnt);
-    return 1;
-}
-
 int launch_tree_nodes(const TreeArgs& a, int64_t max_chunks, cudaStream_t st)
 {
     const size_t T = (size_t)3 * a.K;
-    cudaMemsetAsync(a.e1, 0xff, a.nb * T * 4, st);
-    cudaMemsetAsync(a.e2, 0xff, a.nb * T * T * 4, st);
-    cudaMemsetAsync(a.bits, 0, (size_t)a.nb * a.n2max * a.W * 4, st);
+    cudaMemsetAsync(a.e1, 0xff, (char*)(a.e2 + a.nb * T * T) - (char*)a.e1, st);
     if (max_chunks > 0) k_tree_mark<<<(unsigned)max_chunks, kTreeRows, 0, st>>>(a);
     k_tree_two<<<a.nb, 512, 0, st>>>(a);
     if (max_chunks > 0) k_tree_bits<<<(unsigned)max_chunks, kTreeRows, 0, st>>>(a);

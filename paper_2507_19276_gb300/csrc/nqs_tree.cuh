@@ -29,7 +29,7 @@ struct TreeArgs {
     uint32_t* word;                       // changes (see above)
     uint32_t* rnode;                      // the node the row ends on
     // per batch sample
-    int* e1;                              // [nb][3K] last level of the one-change nodes (-1 unused)
+    int* e1;                              // [nb][3K] last level of the one-change nodes (-1 unused); e2 right behind
     int* e2;                              // [nb][3K][3K] the same of two-change nodes, then their index
     int* n2; int* n3;                     // [nb] two- and three-change nodes
     uint32_t* bits;                       // [nb][n2max][W] third changes of each two-change node
@@ -60,8 +60,6 @@ struct TreeLevels {
     int sources;
 };
 
-// rows of every sample (deterministic + drawn)
-int launch_tree_row_counts(const int64_t* det_cnt, const int64_t* draw_cnt, int64_t Ns, int64_t* cnt, cudaStream_t st);
 // words, marks and nodes of the batch; fills pool_tot and level_cnt
 int launch_tree_nodes(const TreeArgs& a, int64_t max_chunks, cudaStream_t st);
 // pool rows of the nodes (pool_tot scanned) and the items (level_off scanned)

@@ -137,32 +137,38 @@ int launch_scan_chunks_u64(uint64_t* w, uint64_t* total, int64_t Ns, uint32_t n_
     return 1;
 }
 
-__global__ void __launch_bounds__(1024) k_scan_i64(const int64_t* in, int64_t* out, int64_t n, int rows)
+// one block per job
+__global__ void __launch_bounds__(1024) k_scan_i64(ScanJobs jobs)
 {
     __shared__ int64_t wt[32];
+    const ScanJob& s = jobs.job[blockIdx.x];
     int64_t carry = 0;
-    for (int64_t t0 = 0; t0 < n; t0 += blockDim.x) {
+    for (int64_t t0 = 0; t0 < s.n; t0 += blockDim.x) {
         const int64_t i = t0 + threadIdx.x;
-        int64_t v = i < n ? in[i] : 0;
-        if (rows > 0) v = (v + rows - 1) / rows;
+        int64_t v = i < s.n ? s.in[i] + (s.add ? s.add[i] : 0) : 0;
+        if (s.rows > 0) v = (v + s.rows - 1) / s.rows;
         const int64_t inc = block_incl_scan<int64_t>(v, wt);
-        if (i < n) out[i] = carry + inc - v;
+        if (i < s.n) s.out[i] = carry + inc - v;
         carry += wt[(blockDim.x >> 5) - 1];
         __syncthreads();
     }
-    if (threadIdx.x == 0) out[n] = carry;
+    if (threadIdx.x == 0) s.out[s.n] = carry;
+}
+
+int launch_scan_jobs(const ScanJobs& jobs, cudaStream_t st)
+{
+    k_scan_i64<<<(unsigned)jobs.n, 1024, 0, st>>>(jobs);
+    return 1;
 }
 
 int launch_scan_i64(const int64_t* in, int64_t* out, int64_t n, cudaStream_t st)
 {
-    k_scan_i64<<<1, 1024, 0, st>>>(in, out, n, 0);
-    return 1;
+    return launch_scan_jobs({{{in, nullptr, out, n, 0}}, 1}, st);
 }
 
 // Multi-block exclusive scan: sums of 4096-element tiles, one block scans the
 // sums, then every tile rescans its elements from its offset (integers: the
 // result does not depend on the tiling).
-constexpr int kScanTile = 4096;   // 1024 threads x 4 elements
 
 __global__ void __launch_bounds__(1024) k_scan_tile_sums(const int64_t* in, int64_t n, int64_t* sums)
 {
@@ -201,20 +207,19 @@ __global__ void __launch_bounds__(1024) k_scan_tiles(const int64_t* in, int64_t*
 
 int launch_scan_i64_wide(const int64_t* in, int64_t* out, int64_t n, int64_t* tmp, cudaStream_t st)
 {
-    if (n <= 16 * kScanTile || !tmp) return launch_scan_i64(in, out, n, st);
+    if (n <= kScanOneBlock || !tmp) return launch_scan_i64(in, out, n, st);
     const int64_t nt = (n + kScanTile - 1) / kScanTile;
     int64_t* sums = tmp;
     int64_t* offs = tmp + nt + 1;
     k_scan_tile_sums<<<(unsigned)nt, 1024, 0, st>>>(in, n, sums);
-    k_scan_i64<<<1, 1024, 0, st>>>(sums, offs, nt, 0);
+    launch_scan_i64(sums, offs, nt, st);
     k_scan_tiles<<<(unsigned)nt, 1024, 0, st>>>(in, out, n, offs);
     return 3;
 }
 
 int launch_chunk_base(const int64_t* cnt, int rows, int64_t* out, int64_t Ns, cudaStream_t st)
 {
-    k_scan_i64<<<1, 1024, 0, st>>>(cnt, out, Ns, rows);
-    return 1;
+    return launch_scan_jobs({{{cnt, nullptr, out, Ns, rows}}, 1}, st);
 }
 
 // ---------------------------------------------------------------------------
