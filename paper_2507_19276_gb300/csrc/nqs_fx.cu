@@ -126,14 +126,6 @@ __device__ __forceinline__ uint32_t fx_low(uint32_t below, bool not_finite, uint
     return low;
 }
 
-// mask of the nonzero entries of x
-__device__ __forceinline__ uint64_t fx_row_nonzero(const double* x, int D)
-{
-    uint64_t m = 0;
-    for (int k = 0; k < D; ++k) m |= (uint64_t)fx_nonzero(x[k]) << k;
-    return m;
-}
-
 // entry c of M x in FP64 (M by columns, as dot_col4): nz and mz are the masks of the
 // nonzero entries of x and of row c, `whole` where either holds an infinity or a NaN
 __device__ __forceinline__ double fx_dot(const double* M, const double* x, int D, int c, uint64_t nz, uint64_t mz, bool whole)
@@ -594,23 +586,15 @@ __device__ __forceinline__ int64_t fx_shift(int64_t v, int d)
 
 // Results `low` (from column c0) of one node in FP64, into out[]: the power of two its
 // sums are aligned to goes to *power (the same from every part of the row), the largest
-// exponent is returned. AT and exps: matrices and powers of the node's local state, four
-// apart per edge. Out of line: the caller keeps its registers.
+// exponent is returned. AT: the matrices of the node's local state, four apart per edge.
+// Out of line: the caller keeps its registers.
 template <int D>
 __device__ __noinline__ int fx_graph_redo(const uint32_t* it, uint32_t nl, const double* pool, const int* pool_e,
-                                          const double* __restrict__ AT, const int* __restrict__ exps, const int* t_e,
-                                          int nv, int deg, uint32_t low, int c0, double* out, int* power)
+                                          const double* __restrict__ AT, const int* t_e, int nv, int deg, uint32_t low,
+                                          int c0, double* out, int* power)
 {
-    uint64_t nz[kGtMaxDeg];
-    uint32_t whole = 0;
     int er = nv < deg ? 0 : -(1 << 30);               // an e_0 source has power 0
-    for (int k = 0; k < nv; ++k) {
-        const uint32_t sr = __ldg(it + (size_t)(k + 1) * nl);
-        const double* x = pool + (size_t)sr * D;
-        er = max(er, pool_e[sr]);
-        nz[k] = fx_row_nonzero(x, D);
-        for (int c = 0; c < D; ++c) whole |= (fx_not_finite(x[c]) ? 1u : 0u) << k;
-    }
+    for (int k = 0; k < nv; ++k) er = max(er, pool_e[__ldg(it + (size_t)(k + 1) * nl)]);
     int top = -(1 << 29);
     for (; low; low &= low - 1) {
         const int c = c0 + __ffs((int)low) - 1;
@@ -619,10 +603,7 @@ __device__ __noinline__ int fx_graph_redo(const uint32_t* it, uint32_t nl, const
             const double* M = AT + (size_t)t_e[k] * 4 * D * D;
             if (k < nv) {
                 const uint32_t sr = __ldg(it + (size_t)(k + 1) * nl);
-                const int* ex = exps + (size_t)t_e[k] * 4 * fx_exp_stride(D);
-                const uint64_t mz = __ldg((const uint64_t*)(ex + 2 * D) + D + c);
-                const bool all = ((whole >> k) & 1u) || __ldg(ex + D + c) == kFxNotFinite;
-                y += scale_pow2(fx_dot(M, pool + (size_t)sr * D, D, c, nz[k], mz, all), pool_e[sr] - er);
+                y += scale_pow2(dot_col4(M, pool + (size_t)sr * D, D, c), pool_e[sr] - er);
             } else {
                 y += scale_pow2(__ldg(M + c), -er);
             }
@@ -782,8 +763,7 @@ k_fx_graph(TreeGraph64 a, const unsigned char* __restrict__ img, const int* __re
         if (r >= n) low = 0;
         if (low)                                      // these in FP64, all edges
             emax = max(emax, fx_graph_redo<D>(a.items + at + i0 + r, nl, a.pool, a.pool_e, a.an.AT + (size_t)g * D * D,
-                                              exps + (size_t)g * fx_exp_stride(D), t_e, nv, deg, low, h * H,
-                                              (double*)smraw + (size_t)r * (D + 2), s_es + r) + 56 - drop);
+                                              t_e, nv, deg, low, h * H, (double*)smraw + (size_t)r * (D + 2), s_es + r) + 56 - drop);
         s_max[h][r] = emax;
         __syncthreads();                              // the parts of each row meet
         #pragma unroll
