@@ -23,7 +23,7 @@
 // packed subtraction), 34 x D/16 MMAs, then the integer epilogue. Per tile at
 // D = 64 that is ~20 k warp instructions and 136 MMAs, against 301 k cycles of
 // the FP64 pipe for the same products. H50 tables of 200 samples (5 M products):
-// 45 ms on the FP64 pipe, 4.7 ms here; issue and latency of the digit and
+// 45 ms on the FP64 pipe, 4.9 ms here; issue and latency of the digit and
 // epilogue chains bound it (one block per SM at D = 64).
 #include "nqs_fx.cuh"
 #include "nqs_tc.cuh"
@@ -153,9 +153,9 @@ __device__ __forceinline__ __half2 fx_digit2(uint64_t c0, uint64_t c1, int i)
 
 // One block per (matrix, side): the columns' powers of two, the rows' after them,
 // then the digits. A column without entries has the power kFxNoExp, so that the
-// vector's entry there, which meets only zeros, takes no part in its scale. The operand has `rows` rows of D entries (columns past D, up
-// to C, and rows past `rows`, up to R, are zero) in blocks of R rows:
-// entry(n, k) of the matrix.
+// vector's entry there, which meets only zeros, takes no part in its scale. The operand
+// has `rows` rows of D entries (columns past D, up to C, and rows past `rows`, up to R,
+// are zero) in blocks of R rows: entry(n, k) of the matrix.
 template <class Entry>
 __device__ void fx_image(const Entry& entry, int rows, int D, int R, int C, unsigned char* img, int* cexp, int* rexp,
                          uint64_t* big, uint64_t* nonzero, int* sc, int* sr)
